@@ -835,6 +835,8 @@ extern "C" ja_status_t ja_repartition_agg(const ja_relation_t* partials, ja_agg_
 struct ExecPlan {
     std::shared_ptr<GemmTcPlan> gemm;
     bool gemm_checked = false;
+    std::shared_ptr<ContractTcPlan> contract;
+    bool contract_checked = false, contract_first = false;   // contract_first: expected to be faster than the TMA form
     AttnTcCache attn;
     float2* rope_table = nullptr;
     int64_t* rope_splits = nullptr;  // split points of the collapsed (h d) index
@@ -923,17 +925,17 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
         if (A->dtype != B->dtype || A->dtype != out->dtype) return ja_fail(JA_ERR_DTYPE, "matmul operands must share one dtype");
         if (A->dtype != JA_F32) {   // bf16 or f16: tensor cores
             const int loader = ja_config().gemm_loader;
-            if (!plan->gemm_checked) {
+            if (!plan->contract_checked) {
                 bool ok = false;
+                double us = 0;
                 if ((st = ja_gemm_tc_plan(A, B, out, nullptr, &plan->gemm, &ok)) != JA_OK) return st;
                 if (!ok) plan->gemm.reset();
-                plan->gemm_checked = true;
+                if ((st = ja_contract_tc_plan(in[0], in[1], o, A, B, out, &plan->contract, &us)) != JA_OK) return st;
+                plan->contract_first = plan->contract && (!plan->gemm || us < 0.9 * ja_gemm_tc_estimate_us(*plan->gemm));
+                plan->contract_checked = true;
             }
-            if (plan->gemm && loader != 1) return ja_launch_gemm_tc(*plan->gemm, stream);
-            if (loader != 0) {   // tilings TMA cannot address: the tensor cores fed by plain loads
-                bool launched = false;
-                if ((st = ja_launch_gemm_ld(A, B, out, stream, &launched)) != JA_OK || launched) return st;
-            }
+            if (plan->gemm && loader != 1 && (loader == 0 || !plan->contract_first)) return ja_launch_gemm_tc(*plan->gemm, stream);
+            if (plan->contract && loader != 0) return ja_launch_contract_tc(*plan->contract, stream);
         }
         return ja_launch_matmul_simt(A, B, out, stream);
     }
@@ -1135,6 +1137,15 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                          V->splits[1] == K->splits[1] && V->bs[0] == K->bs[0] && V->bs[2] == K->bs[2] &&
                          out->splits[1] == Q->splits[1] && out->bs[0] == Q->bs[0] && out->bs[2] == Q->bs[2];
         return ja_launch_attention(aa, stream);
+    }
+
+    // ---- any other (batched, transposed) matrix product of two 16-bit relations -------------------------------------
+    if (n_outputs == 1 && fn == JA_FN_MUL && agg == JA_AGG_SUM && n_in == 2) {
+        if (!plan->contract_checked) {
+            if ((st = ja_contract_tc_plan(in[0], in[1], o, inputs[0], inputs[1], out, &plan->contract, nullptr)) != JA_OK) return st;
+            plan->contract_checked = true;
+        }
+        if (plan->contract) return ja_launch_contract_tc(*plan->contract, stream);
     }
 
     // ---- anything else whose operator is a scalar function of the joined cells: the definition, cell by cell --------

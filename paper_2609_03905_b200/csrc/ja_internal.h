@@ -117,9 +117,13 @@ ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inp
 ja_status_t ja_launch_matmul_simt(const ja_relation* A, const ja_relation* B, const ja_relation* C, cudaStream_t st,
                                   bool partials = false);
 
-// tcgen05 matmul join-agg for bf16 relations under any tiling, operands staged by plain loads (k_gemm_ld.cu); *launched
-// stays false when the blocks are too small for its tiles. Key tables must be on the device.
-ja_status_t ja_launch_gemm_ld(const ja_relation* A, const ja_relation* B, const ja_relation* C, cudaStream_t st, bool* launched);
+// tcgen05 contraction of two 16-bit relations under any tiling and index order, operands staged by cp.async (k_contract_tc.cu).
+// ta, tb, tc: the terms of A, B and the output. *out stays empty when the einsum is not a (batched) matrix product;
+// *est_us: what the launch is expected to take. Key tables must be on the device.
+struct ContractTcPlan;
+ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, const std::string& tc, const ja_relation* A, const ja_relation* B,
+                                const ja_relation* C, std::shared_ptr<ContractTcPlan>* out, double* est_us);
+ja_status_t ja_launch_contract_tc(const ContractTcPlan& plan, cudaStream_t st);
 
 // Memory-bound join-aggs: flat key-aligned maps and row-structured maps / reductions.
 enum RowOp {
@@ -175,6 +179,7 @@ struct GemmEpilogue {
 ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, const GemmEpilogue* ep,
                             std::shared_ptr<GemmTcPlan>* out, bool* eligible);
 ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st);
+double ja_gemm_tc_estimate_us(const GemmTcPlan& plan);
 
 // Attention join-agg (QK^T join, online-softmax aggregation, PV).
 // the four tensor maps (Q, K, V, O) of the tensor-memory kernels, encoded once per (spec, relations) tuple
