@@ -1133,7 +1133,7 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
         std::vector<int32_t> qs(Q->splits[1].begin(), Q->splits[1].end()), ks(K->splits[1].begin(), K->splits[1].end());
         aa.q_split = qs.data();
         aa.k_split = ks.data();
-        aa.rows_layout = (n_outputs == 1 || aa.lse_rows_layout) && bshd_rows_layout(Q) && bshd_rows_layout(K) && bshd_rows_layout(V) && bshd_rows_layout(out) &&
+        aa.rows_layout = bshd_rows_layout(Q) && bshd_rows_layout(K) && bshd_rows_layout(V) && bshd_rows_layout(out) &&
                          V->splits[1] == K->splits[1] && V->bs[0] == K->bs[0] && V->bs[2] == K->bs[2] &&
                          out->splits[1] == Q->splits[1] && out->bs[0] == Q->bs[0] && out->bs[2] == Q->bs[2];
         return ja_launch_attention(aa, stream);

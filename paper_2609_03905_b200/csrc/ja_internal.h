@@ -186,6 +186,7 @@ double ja_gemm_tc_estimate_us(const GemmTcPlan& plan);
 struct AttnTcCache {
     alignas(64) unsigned char maps[4][128];
     bool valid = false;
+    int q_box = 0, k_box = 0;   // rows per box the maps were encoded with
 };
 struct AttnArgs {
     AttnTcCache* cache;    // where the tensor maps are kept between launches, or nullptr

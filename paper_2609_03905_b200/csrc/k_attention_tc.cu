@@ -1,9 +1,10 @@
 // Attention join-agg "bqhd,bkhd,bkhd->bqhd" (f = ATTENTION, (+) = online softmax) on the 5th-generation
 // tensor cores: both contractions of every joined tuple run as tcgen05.mma with accumulators in tensor memory.
 //
-// Two kernels. attention_tc2_kernel (further down) gives a CTA two output key tiles of one (batch, head) and is the one
-// that runs whenever sequences are whole pairs of 128-row tiles; attention_tc_kernel, described here, takes the rest:
-// one CTA owns one output key tile (128 query rows of one (batch, head)) and walks the function specs that
+// Three kernels. attention_tc2_kernel (further down) gives a CTA two output key tiles of one (batch, head) and is the one
+// that runs whenever sequences are whole pairs of 128-row tiles; attention_ragged_kernel is the same code for any other lengths
+// and blocks; attention_tc_kernel, described here, takes what the ragged form's tile lists cannot hold, where blocks are whole
+// tiles: one CTA owns one output key tile (128 query rows of one (batch, head)) and walks the function specs that
 // share that output key -- the 128-row key/value tiles that survive the causal band predicate -- ascending.
 //
 //   warp 0      TMA producer: Q once, then K_j and V_j (two stages each), straight from the "bshd" block-key
@@ -80,8 +81,12 @@ __device__ __forceinline__ int seq_row(const SeqGeom& g, int S, int b, int s, in
         start = (s / g.sblk) * g.sblk;
         rows = g.sblk;
     } else {
-        int sb = 0;
-        while (sb + 1 < g.nsb && g.split[sb + 1] <= s) ++sb;
+        int sb = 0, hi = g.nsb - 1;
+        while (sb < hi) {
+            const int mid = (sb + hi + 1) >> 1;
+            if (g.split[mid] <= s) sb = mid;
+            else hi = mid - 1;
+        }
         start = g.split[sb];
         rows = g.split[sb + 1] - start;
     }
@@ -560,8 +565,34 @@ constexpr int SMEM_BYTES2 = 7 * TILE_BYTES + 1024 + 256;
 constexpr int ATTN_QUEUES = 256;
 __device__ int32_t g_attn_queues[2 * ATTN_QUEUES];
 
+// The RAGGED form: sequences and blocks that are no whole pairs of 128-row tiles. TMA has no alignment rule for rows, so a tile may
+// start anywhere; what a box brings past a tile's rows is masked (scores), not multiplied (whole 16-key groups of V), zeroed in
+// shared memory (the rest of the last group) or not stored. The cost against whole tiles is the masks and the empty parts of the
+// last tiles. Measured, us, against the mma.sync kernel it took these from (48 to 60 TFLOP/s there, 600 to 980 here):
+//   five packed f16 sequences, 6001 rows, 32 / 8 heads     1413 -> 101      2 x 6080 rows in 64-row blocks, 8 heads   1525 -> 310
+//   one sequence of 684 rows, 4 heads                        97 -> 18       2 x 3473 rows, 8 heads                     855 -> 61
+// and against the one-tile kernel where blocks are whole tiles: 4 x 896 rows, 32 heads 101 -> 48, 16 x 128 rows 31.6 -> 22.8,
+// 1 x 128 rows, 16 heads 8.4 -> 8.1.
+//
+// A tile is up to 128 consecutive
+// positions of one sequence; it reaches shared memory as pieces of `q_piece` / `k_piece` rows, each inside one block of its
+// relation. The host lists the tiles and the items (pairs of query tiles, heaviest first) and how many key tiles each joins.
+constexpr int MAX_TILES = 512, MAX_ITEMS = 320;
+struct RaggedTiles {
+    RelView lse;                         // second output, located cell by cell (its blocks are padded to 128 bytes)
+    int32_t n_items, q_piece, k_piece;
+    uint32_t q[MAX_TILES], k[MAX_TILES]; // first position | (rows - 1) << 24
+    struct {
+        uint16_t q, k, n_a, n_b;         // first query tile, first key tile of its sequence, key tiles joined with tile A / B (0: no tile B)
+    } item[MAX_ITEMS];
+};
+__device__ __forceinline__ int tile_start(uint32_t t) { return (int)(t & 0xffffffu); }
+__device__ __forceinline__ int tile_rows(uint32_t t) { return (int)(t >> 24) + 1; }
+
 struct AttnItem {
     int q0, h, b, s0, n_a, n_b;
+    int n;               // key steps of the item (the larger of n_a, n_b)
+    int qt, kt;          // RAGGED: first query tile, first key tile
 };
 // item number `rank` in launch order (ja_attn_decode_cta: heaviest pairs first inside sections of (batch, head) pairs);
 // false past the end
@@ -578,14 +609,27 @@ __device__ __forceinline__ bool attn_item(const AttnTcParams& p, int rank, AttnI
     sequence_of(p, it->q0, it->s0, s1);
     it->n_a = p.causal ? (it->q0 + QT - it->s0) / KT : (s1 - it->s0) / KT;
     it->n_b = p.causal ? (it->q0 + 2 * QT - it->s0) / KT : (s1 - it->s0) / KT;
+    it->n = it->n_b;
+    return true;
+}
+__device__ __forceinline__ bool attn_item(const AttnTcParams& p, const RaggedTiles& rt, int rank, AttnItem* it) {
+    const int hb = p.H * p.B;
+    if (rank >= rt.n_items * hb) return false;
+    int slot, bh;
+    ja_attn_decode_cta(rank, rt.n_items, hb, p.sect, &slot, &bh);
+    it->h = bh % p.H;
+    it->b = bh / p.H;
+    it->qt = rt.item[slot].q;
+    it->kt = rt.item[slot].k;
+    it->n_a = rt.item[slot].n_a;
+    it->n_b = rt.item[slot].n_b;
+    it->n = max(it->n_a, it->n_b);
     return true;
 }
 
-template <bool PERSIST, int VAR, bool F16>
-__global__ void __launch_bounds__(NUM_THREADS2, 1)
-attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-                     const __grid_constant__ AttnTcParams p) {
+template <bool PERSIST, int VAR, bool F16, bool RAGGED>
+__device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV, const CUtensorMap& tmO,
+                                              const AttnTcParams& p, const RaggedTiles* rt) {
     constexpr int POLY = VAR & 3;
     constexpr bool WAIT_FIRST = (VAR & 4) == 0;
     extern __shared__ uint8_t smem_raw[];
@@ -612,7 +656,8 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const int rank = item_rank[e];
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + e));
-        return attn_item(p, rank, it);
+        if constexpr (RAGGED) return attn_item(p, *rt, rank, it);
+        else return attn_item(p, rank, it);
     };
 
     if (threadIdx.x == 0) {
@@ -653,21 +698,51 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     if (item > 0) break;
                     rank = (int)blockIdx.x;
                 }
-                if (!attn_item(p, rank, &it)) break;
+                if constexpr (RAGGED) {
+                    if (!attn_item(p, *rt, rank, &it)) break;
+                } else {
+                    if (!attn_item(p, rank, &it)) break;
+                }
                 const int hk = it.h / p.group;
                 // the Q buffers are free once the previous item's last Q K^T has read them
                 if (item > 0 && !mbar_wait(bar(Q_EMPTY), (uint32_t)(item - 1) & 1, abort_flag, p.status)) break;
+                if constexpr (RAGGED) {
+                    // the pieces of a tile that hold wanted rows; what they bring past a tile's rows is never used
+                    const int qp = rt->q_piece, n_tiles = it.n_b ? 2 : 1;
+                    int pieces[2] = {0, 0};
+                    for (int t = 0; t < n_tiles; ++t) pieces[t] = (tile_rows(rt->q[it.qt + t]) + qp - 1) / qp;
+                    mbar_expect_tx(bar(Q_FULL), (uint32_t)(pieces[0] + pieces[1]) * qp * D * 2);
+                    for (int t = 0; t < n_tiles; ++t)
+                        for (int i = 0; i < pieces[t]; ++i) {
+                            const int row = seq_row(p.q, p.S, it.b, tile_start(rt->q[it.qt + t]) + i * qp, it.h);
+                            for (int half = 0; half < 2; ++half)
+                                tma_load_3d(sQ + t * TILE_BYTES + half * HALF_BYTES + i * qp * 128, &tmQ, bar(Q_FULL), half * 64, it.h % p.q.hblk, row);
+                        }
+                } else {
                 mbar_expect_tx(bar(Q_FULL), 2 * TILE_BYTES);
                 for (int t = 0; t < 2; ++t) {
                     const int qrow_t = seq_row(p.q, p.S, it.b, it.q0 + t * QT, it.h);
                     for (int half = 0; half < 2; ++half)
                         tma_load_3d(sQ + t * TILE_BYTES + half * HALF_BYTES, &tmQ, bar(Q_FULL), half * 64, it.h % p.q.hblk, qrow_t);
                 }
+                }
                 // K / V tiles in the order the products consume them: K_0, then for every step j: K_{j+1} (if any), V_j
                 auto load = [&](const CUtensorMap* tm, int j) {
                     const int sl = li % 3;
                     const uint32_t ph = (uint32_t)(li / 3) & 1;
                     if (!mbar_wait(bar(KV_EMPTY + sl), ph ^ 1, abort_flag, p.status)) { ok = false; return; }
+                    if constexpr (RAGGED) {
+                        const uint32_t tile = rt->k[it.kt + j];
+                        const int kp = rt->k_piece, pieces = (tile_rows(tile) + kp - 1) / kp;
+                        mbar_expect_tx(bar(KV_FULL + sl), (uint32_t)pieces * kp * D * 2);
+                        for (int i = 0; i < pieces; ++i) {
+                            const int row = seq_row(p.k, p.S, it.b, tile_start(tile) + i * kp, hk);
+                            for (int half = 0; half < 2; ++half)
+                                tma_load_3d(sKV + sl * TILE_BYTES + half * HALF_BYTES + i * kp * 128, tm, bar(KV_FULL + sl), half * 64, hk % p.k.hblk, row);
+                        }
+                        ++li;
+                        return;
+                    }
                     const int krow = seq_row(p.k, p.S, it.b, it.s0 + j * KT, hk);
                     mbar_expect_tx(bar(KV_FULL + sl), TILE_BYTES);
                     for (int half = 0; half < 2; ++half)
@@ -675,8 +750,8 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     ++li;
                 };
                 load(&tmK, 0);
-                for (int j = 0; j < it.n_b && ok; ++j) {
-                    if (j + 1 < it.n_b) load(&tmK, j + 1);
+                for (int j = 0; j < it.n && ok; ++j) {
+                    if (j + 1 < it.n) load(&tmK, j + 1);
                     if (ok) load(&tmV, j);
                 }
             }
@@ -704,19 +779,28 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             }
             commit1_w(bar(S_FULL + t), leader);
         };
-        auto issue_pv = [&](int t, int sl, bool first) {   // O~_t (+)= P_t V, P in shared memory (K-major), V in slot sl (MN-major)
+        auto issue_pv = [&](int t, int sl, bool first, int keys) {   // O~_t (+)= P_t V, P in shared memory (K-major), V in slot sl (MN-major)
             const uint32_t vaddr = sKV + sl * TILE_BYTES, paddr = sP + t * TILE_BYTES;
+            if (!RAGGED || keys == KT) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
-                umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + off, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
-                          (!first || kk > 0) ? 1u : 0u, leader);
+                for (int kk = 0; kk < 8; ++kk) {
+                    const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
+                    umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + off, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
+                              (!first || kk > 0) ? 1u : 0u, leader);
+                }
+            } else {      // a short key tile: only the groups of 16 keys that exist
+                for (int kk = 0; kk * 16 < keys; ++kk) {
+                    const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
+                    umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + off, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
+                              (!first || kk > 0) ? 1u : 0u, leader);
+                }
             }
             commit1_w(bar(P_EMPTY + t), leader);
             commit1_w(bar(O_FULL + t), leader);
         };
         int li = 0;
         int cs[2] = {0, 0};                   // key steps of each tile in all items so far
+        int done[2] = {0, 0};                 // items so far that had the tile
         bool ok = true;
         AttnItem it;
         for (int item = 0; ok && next_item(item, &it); ++item) {
@@ -726,6 +810,7 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 const int sl = li % 3;
                 if (ok) ok = mbar_wait(bar(KV_FULL + sl), (uint32_t)(li / 3) & 1, abort_flag, p.status);
                 for (int t = 0; t < 2 && ok; ++t) {
+                    if (RAGGED && n_of[t] == 0) continue;   // no tile B
                     // S_t is free once the row threads hold the scores of the tile's previous key step (of the previous item)
                     if (cs[t] > 0 && !mbar_wait(bar(S_FREE + t), (uint32_t)(cs[t] - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                     tc_fence_after();
@@ -733,11 +818,11 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 }
                 if (!ok) break;
                 commit1_w(bar(KV_EMPTY + sl), leader);
-                if (it.n_b == 1) commit1_w(bar(Q_EMPTY), leader);
+                if (it.n == 1) commit1_w(bar(Q_EMPTY), leader);
                 ++li;
             }
-            for (int j = 0; j < it.n_b && ok; ++j) {
-                if (j + 1 < it.n_b) {
+            for (int j = 0; j < it.n && ok; ++j) {
+                if (j + 1 < it.n) {
                     const int sl = li % 3;
                     if (!mbar_wait(bar(KV_FULL + sl), (uint32_t)(li / 3) & 1, abort_flag, p.status)) { ok = false; break; }
                     for (int t = 0; t < 2 && ok; ++t) {
@@ -750,18 +835,30 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     }
                     if (!ok) break;
                     commit1_w(bar(KV_EMPTY + sl), leader);
-                    if (j + 2 == it.n_b) commit1_w(bar(Q_EMPTY), leader);   // that was the item's last Q K^T
+                    if (j + 2 == it.n) commit1_w(bar(Q_EMPTY), leader);   // that was the item's last Q K^T
                     ++li;
                 }
                 const int sl = li % 3;
                 if (!mbar_wait(bar(KV_FULL + sl), (uint32_t)(li / 3) & 1, abort_flag, p.status)) { ok = false; break; }
+                int keys = KT;
+                if constexpr (RAGGED) {
+                    keys = tile_rows(rt->k[it.kt + j]);
+                    if (keys & 15) {   // the last group's missing keys have P = 0: their V rows (other cells of the relation) must not be NaN
+                        uint8_t* v = smem + (2 + sl) * TILE_BYTES;
+                        const int gap = 16 - (keys & 15);
+                        for (int e = lane; e < gap * 16; e += 32)
+                            *reinterpret_cast<uint4*>(v + (e & 8) * (HALF_BYTES / 8) + (keys + (e >> 4)) * 128 + (e & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
+                }
                 for (int t = 0; t < 2 && ok; ++t) {
                     if (j < n_of[t]) {
                         if (!mbar_wait(bar(P_FULL + t), (uint32_t)(cs[t] + j) & 1, abort_flag, p.status)) { ok = false; break; }
                         // the first P V of an item overwrites O~: the row threads must have read the previous item's
-                        if (j == 0 && item > 0 && !mbar_wait(bar(O_READ + t), (uint32_t)(item - 1) & 1, abort_flag, p.status)) { ok = false; break; }
+                        if (j == 0 && done[t] > 0 && !mbar_wait(bar(O_READ + t), (uint32_t)(done[t] - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        issue_pv(t, sl, j == 0);
+                        issue_pv(t, sl, j == 0, keys);
                     }
                 }
                 if (!ok) break;
@@ -770,6 +867,8 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             }
             cs[0] += it.n_a;
             cs[1] += it.n_b;
+            done[0] += 1;
+            done[1] += it.n_b > 0;
         }
     } else {
         // ================= row threads =================
@@ -780,19 +879,31 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const uint32_t tS = tmem_base + t * 128 + lane_addr, tO = tmem_base + 256 + t * 128 + lane_addr;
         uint8_t* prow = pP + t * TILE_BYTES + r * 128;     // this row inside each 64-key half of the P tile
         const int sw = r & 7;                              // 128-byte swizzle: 16-byte chunk c of row r lives at chunk c ^ (r & 7)
-        int cs = 0;                                        // key steps of this tile in all items so far
+        int cs = 0, done = 0;                              // key steps of this tile in all items so far; items so far that had it
         bool ok = true;
         AttnItem it;
         for (int item = 0; ok && next_item(item, &it); ++item) {
             const int n_t = t == 0 ? it.n_a : it.n_b;
-            const int qrow = it.q0 + t * QT + r;
+            int q_tile0 = it.q0 + t * QT, q_rows = QT;
+            if constexpr (RAGGED) {
+                if (n_t == 0) continue;   // no tile B: nothing is waited for or handed over
+                q_tile0 = tile_start(rt->q[it.qt + t]);
+                q_rows = tile_rows(rt->q[it.qt + t]);
+            }
+            const int qrow = q_tile0 + r;
             float m_used = -INFINITY, l_run = 0.f;
             for (int j = 0; j < n_t && ok; ++j) {
                 const int c = cs + j;
                 if (!mbar_wait(bar(S_FULL + t), (uint32_t)c & 1, abort_flag, p.status)) { ok = false; break; }
                 tc_fence_after();
-                const bool diag = p.causal && (j == n_t - 1);
-                const int kmax = qrow - (it.s0 + j * KT);
+                bool diag = p.causal && (j == n_t - 1);
+                int kmax = qrow - (it.s0 + j * KT);
+                if constexpr (RAGGED) {   // keys past the tile's own, and (causal) keys after the query
+                    const uint32_t tile = rt->k[it.kt + j];
+                    const int k0 = tile_start(tile), last = tile_rows(tile) - 1;
+                    diag = last < KT - 1 || (p.causal && k0 + last > q_tile0);
+                    kmax = p.causal ? min(qrow - k0, last) : last;
+                }
                 uint32_t v[128];
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) tmem_ld32(tS + cc * 32, v + cc * 32);
@@ -822,7 +933,7 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 // TMA stores of the previous item's output, which was staged in the P tile, have read it (P_STORED).
                 auto wait_p_tile = [&]() -> bool {
                     if (c > 0 && !mbar_wait(bar(P_EMPTY + t), (uint32_t)(c - 1) & 1, abort_flag, p.status)) return false;
-                    if (j == 0 && item > 0 && !mbar_wait(bar(P_STORED + t), (uint32_t)(item - 1) & 1, abort_flag, p.status)) return false;
+                    if (j == 0 && done > 0 && !mbar_wait(bar(P_STORED + t), (uint32_t)(done - 1) & 1, abort_flag, p.status)) return false;
                     return true;
                 };
                 if (WAIT_FIRST || rescale) {
@@ -862,10 +973,18 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             if (!mbar_wait(bar(O_FULL + t), (uint32_t)(cs + n_t - 1) & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-            if (p.lse_base) {
+            if (RAGGED) {
+                if (rt->lse.base && r < q_rows) {
+                    const int64_t x[3] = {it.b, qrow, it.h};
+                    *reinterpret_cast<float*>(rt->lse.base + ja_elem_off(rt->lse, x)) = (m_used + log2f(l_run)) * 0.6931471805599453f;
+                }
+            } else if (p.lse_base) {
                 const int64_t cell = (int64_t)seq_row(p.q, p.S, it.b, qrow, it.h) * p.q.hblk + it.h % p.q.hblk;
                 p.lse_base[cell] = (m_used + log2f(l_run)) * 0.6931471805599453f;   // l is relative to the offset m_used
             }
+            char* direct = nullptr;              // RAGGED: a short tile's rows leave one by one, past the P tile
+            if (RAGGED && q_rows < QT && r < q_rows)
+                direct = p.o_base + ((int64_t)seq_row(p.q, p.S, it.b, qrow, it.h) * p.q.hblk + it.h % p.q.hblk) * (D * 2);
 #pragma unroll 1
             for (int cc = 0; cc < 4; ++cc) {   // not unrolled: the output stage runs once per item, and code size costs instruction fetches
                 uint32_t o[32];
@@ -879,7 +998,8 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                     for (int e = 0; e < 4; ++e)
                         po[e] = ja_pack16<F16>(__uint_as_float(o[g * 8 + 2 * e]) * inv, __uint_as_float(o[g * 8 + 2 * e + 1]) * inv);
                     const int ch = cc * 4 + g;                      // 16-byte chunk 0..15 of the row
-                    *reinterpret_cast<uint4*>(prow + (ch >> 3) * HALF_BYTES + (((ch & 7) ^ sw) << 4)) = ov;
+                    if (RAGGED && direct) *reinterpret_cast<uint4*>(direct + ch * 16) = ov;
+                    else *reinterpret_cast<uint4*>(prow + (ch >> 3) * HALF_BYTES + (((ch & 7) ^ sw) << 4)) = ov;
                 }
             }
             tc_fence_before();
@@ -890,11 +1010,19 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
                 mbar_arrive(bar(O_STAGED + t));
             }
             if (q == 0 && lane == 0) {
-                if (!mbar_wait(bar(O_STAGED + t), (uint32_t)item & 1, abort_flag, p.status)) { ok = false; }
+                if (!mbar_wait(bar(O_STAGED + t), (uint32_t)done & 1, abort_flag, p.status)) { ok = false; }
                 else {
-                    const int orow = seq_row(p.q, p.S, it.b, it.q0 + t * QT, it.h);
-                    for (int half = 0; half < 2; ++half)
-                        tma_store_3d(&tmO, sP + t * TILE_BYTES + half * HALF_BYTES, half * 64, it.h % p.q.hblk, orow);
+                    if (!RAGGED) {
+                        const int orow = seq_row(p.q, p.S, it.b, q_tile0, it.h);
+                        for (int half = 0; half < 2; ++half)
+                            tma_store_3d(&tmO, sP + t * TILE_BYTES + half * HALF_BYTES, half * 64, it.h % p.q.hblk, orow);
+                    } else if (q_rows == QT) {
+                        for (int i = 0; i < QT; i += rt->q_piece) {
+                            const int orow = seq_row(p.q, p.S, it.b, q_tile0 + i, it.h);
+                            for (int half = 0; half < 2; ++half)
+                                tma_store_3d(&tmO, sP + t * TILE_BYTES + half * HALF_BYTES + i * 128, half * 64, it.h % p.q.hblk, orow);
+                        }
+                    }
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may be reused after this
                     mbar_arrive(bar(P_STORED + t));  // the P tile may be written again
@@ -902,6 +1030,7 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             }
             ok = __all_sync(0xffffffffu, ok);
             cs += n_t;
+            ++done;
         }
     }
     tc_fence_before();
@@ -912,15 +1041,30 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     }
 }
 
+template <bool PERSIST, int VAR, bool F16>
+__global__ void __launch_bounds__(NUM_THREADS2, 1)
+attention_tc2_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
+                     const __grid_constant__ AttnTcParams p) {
+    attention_tc2<PERSIST, VAR, F16, false>(tmQ, tmK, tmV, tmO, p, nullptr);
+}
+template <bool F16>
+__global__ void __launch_bounds__(NUM_THREADS2, 1)
+attention_ragged_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                        const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
+                        const __grid_constant__ AttnTcParams p, const __grid_constant__ RaggedTiles rt) {
+    attention_tc2<true, 1, F16, true>(tmQ, tmK, tmV, tmO, p, &rt);
+}
+
 // "bshd" relation with uniform blocks along b and h as a rank-3 tensor (d, head in block, row of hblk x 128 cells)
-ja_status_t encode_rows(const RelView& v, bool f16, CUtensorMap* tm) {
+ja_status_t encode_rows(const RelView& v, bool f16, int box_rows, CUtensorMap* tm) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return ja_fail(JA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     const int64_t hb = v.bs[2];
     const int64_t rows = v.extent[0] * v.extent[1] * v.nblk[2];
     cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)hb, (cuuint64_t)rows};
     cuuint64_t strides[2] = {(cuuint64_t)(D * 2), (cuuint64_t)(hb * D * 2)};
-    cuuint32_t box[3] = {64, 1, 128};
+    cuuint32_t box[3] = {64, 1, (cuuint32_t)box_rows};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult res = enc(tm, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, v.base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -981,30 +1125,118 @@ ja_status_t launch_two_tiles(int variant, bool f16, dim3 grid, cudaStream_t st, 
 
 }  // namespace
 
+namespace {
+
+// The tiles of one relation's sequence index: from the start of each sequence in steps of 128 where every split point inside it
+// is a whole number of `piece` rows from there (a tile may then span blocks, piece by piece), else from the start of each block.
+bool list_tiles(const int32_t* split, int n_blocks, const std::vector<int>& ends, uint32_t* tiles, int32_t* piece, std::vector<int>* first) {
+    int g = 128;
+    for (size_t i = 0; i < ends.size(); ++i) {
+        const int s0 = i ? ends[i - 1] : 0;
+        for (int b = 0; b <= n_blocks; ++b)
+            if (split[b] > s0 && split[b] < ends[i])
+                while ((split[b] - s0) % g) g /= 2;
+    }
+    const bool by_block = g < 8;      // a piece is a whole number of 8-row swizzle groups
+    *piece = by_block ? 128 : g;
+    int n = 0;
+    for (size_t i = 0; i < ends.size(); ++i) {
+        const int s0 = i ? ends[i - 1] : 0;
+        first->push_back(n);
+        for (int at = s0; at < ends[i];) {
+            int stop = std::min(at + 128, ends[i]);
+            if (by_block) stop = std::min(stop, *std::upper_bound(split, split + n_blocks + 1, at));
+            if (n == MAX_TILES) return false;
+            tiles[n++] = (uint32_t)at | (uint32_t)(stop - at - 1) << 24;
+            at = stop;
+        }
+    }
+    first->push_back(n);
+    return true;
+}
+
+// Tiles and items of the ragged form; false (and no items) where there are too many of them, or where blocks are so short that
+// the tiles would be mostly empty: 128 x 128 tensor-memory tiles run some eight times faster than the mma.sync kernel's, so
+// they pay while at least an eighth of a tile pair is real.
+bool list_ragged_tiles(const AttnArgs& a, RaggedTiles* rt) {
+    rt->n_items = 0;
+    if (a.S >= (1 << 24)) return false;
+    std::vector<int> ends(a.ends, a.ends + a.n_ends), q_first, k_first;
+    if (ends.empty()) ends.push_back(a.S);
+    if (!list_tiles(a.q_split, a.q.nblk[1], ends, rt->q, &rt->q_piece, &q_first) || !list_tiles(a.k_split, a.k.nblk[1], ends, rt->k, &rt->k_piece, &k_first))
+        return false;
+    int longest = 0;
+    for (size_t i = 0; i < ends.size(); ++i) longest = std::max(longest, ends[i] - (i ? ends[i - 1] : 0));
+    // sequences of one 64-row tile: the mma.sync kernel has less to set up (32 x 64 rows 7.1 us against 8.9, 128 x 64 rows 7.7 against 10.2)
+    if (longest <= 64 && a.align % 64 == 0) return false;
+    if ((double)a.S * a.S < 0.125 * 128 * 128 * q_first.back() * k_first.back()) return false;
+    rt->lse = a.lse;
+    struct Item { int q, k, n_a, n_b; };
+    std::vector<Item> items;
+    for (size_t i = 0; i < ends.size(); ++i)
+        for (int q = q_first[i]; q < q_first[i + 1]; q += 2) {
+            auto joined = [&](int t) {       // key tiles of this sequence that start no later than the tile's last row
+                if (!a.causal) return k_first[i + 1] - k_first[i];
+                const int last = (int)(rt->q[t] & 0xffffffu) + (int)(rt->q[t] >> 24);
+                int n = 0;
+                while (k_first[i] + n < k_first[i + 1] && (int)(rt->k[k_first[i] + n] & 0xffffffu) <= last) ++n;
+                return n;
+            };
+            items.push_back({q, k_first[i], joined(q), q + 1 < q_first[i + 1] ? joined(q + 1) : 0});
+        }
+    if ((int)items.size() > MAX_ITEMS) return false;
+    std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.n_a + x.n_b > y.n_a + y.n_b; });
+    for (size_t i = 0; i < items.size(); ++i) {
+        rt->item[i].q = (uint16_t)items[i].q;
+        rt->item[i].k = (uint16_t)items[i].k;
+        rt->item[i].n_a = (uint16_t)items[i].n_a;
+        rt->item[i].n_b = (uint16_t)items[i].n_b;
+    }
+    rt->n_items = (int32_t)items.size();
+    return true;
+}
+
+}  // namespace
+
 // Returns JA_OK and sets *launched when a tensor-memory kernel took the job; leaves *launched false when the tiling does
-// not fit (every q / k split point and sequence end must be a multiple of 128 rows, blocks uniform along b and h, at most
-// MAX_SB sequence blocks when they are irregular). The four tensor maps are encoded once per (spec, relations) tuple and
+// not fit (blocks uniform along b and h, at most MAX_SB sequence blocks when they are irregular, tiles that are not mostly
+// empty). The four tensor maps are encoded once per (spec, relations) tuple and
 // kept in a.cache.
 ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* launched) {
     *launched = false;
-    if (a.align % 128 || !a.rows_layout) return JA_OK;
+    if (!a.rows_layout) return JA_OK;
     AttnTcParams p;
     memset(&p, 0, sizeof p);
     if (!fill_geom(a.q, a.q_split, &p.q) || !fill_geom(a.k, a.k_split, &p.k)) return JA_OK;
+    const JaConfig& cfg = ja_config();
+    bool pair_ok = a.S % (2 * QT) == 0;
+    for (int i = 0; i < a.n_ends; ++i)
+        if (a.ends[i] % (2 * QT)) pair_ok = false;
+    // whole pairs of tiles, blocks of whole tiles: the plain two-tile form. Anything else: the ragged one. (attn_one_tile = 1
+    // forces the one-tile form where blocks and sequences are whole tiles.)
+    const bool aligned = a.align % 128 == 0 && (!a.lse.base || a.lse_rows_layout);
+    RaggedTiles rt;
+    const bool ragged = !(aligned && (pair_ok || cfg.attn_one_tile == 1));
+    if (ragged && !list_ragged_tiles(a, &rt)) {
+        if (!aligned) return JA_OK;
+    }
+    const bool use_ragged = ragged && rt.n_items > 0;
     static_assert(sizeof(CUtensorMap) == 128, "AttnTcCache holds four 128-byte tensor maps");
     AttnTcCache local;
     AttnTcCache* cache = a.cache ? a.cache : &local;
     CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(cache->maps);
-    if (!cache->valid) {
+    const int q_box = use_ragged ? rt.q_piece : QT, k_box = use_ragged ? rt.k_piece : KT;
+    if (!cache->valid || cache->q_box != q_box || cache->k_box != k_box) {
         ja_status_t s;
-        if ((s = encode_rows(a.q, a.f16, &maps[0])) != JA_OK) return s;
-        if ((s = encode_rows(a.k, a.f16, &maps[1])) != JA_OK) return s;
-        if ((s = encode_rows(a.v, a.f16, &maps[2])) != JA_OK) return s;
-        if ((s = encode_rows(a.o, a.f16, &maps[3])) != JA_OK) return s;
+        if ((s = encode_rows(a.q, a.f16, q_box, &maps[0])) != JA_OK) return s;
+        if ((s = encode_rows(a.k, a.f16, k_box, &maps[1])) != JA_OK) return s;
+        if ((s = encode_rows(a.v, a.f16, k_box, &maps[2])) != JA_OK) return s;
+        if ((s = encode_rows(a.o, a.f16, q_box, &maps[3])) != JA_OK) return s;
         cache->valid = true;
+        cache->q_box = q_box;
+        cache->k_box = k_box;
     }
     const CUtensorMap &tq = maps[0], &tk = maps[1], &tv = maps[2], &to = maps[3];
-    const JaConfig& cfg = ja_config();
     p.o_base = a.o.base;
     p.lse_base = reinterpret_cast<float*>(a.lse.base);
     p.status = ja_device_status_word(st);
@@ -1014,12 +1246,44 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
     p.group = a.group;
     p.causal = a.causal;
     p.n_ends = a.n_ends;
-    bool pair_ok = a.S % (2 * QT) == 0;
-    for (int i = 0; i < a.n_ends; ++i) {
-        p.ends[i] = a.ends[i];
-        if (a.ends[i] % (2 * QT)) pair_ok = false;
-    }
+    for (int i = 0; i < a.n_ends; ++i) p.ends[i] = a.ends[i];
     p.scale_log2e = a.scale * 1.4426950408889634f;
+    const int sms = ja_sm_count();
+    // {next item, CTAs finished} for a launch of a persistent form. Launches recorded into a CUDA graph keep their pair for as long
+    // as the graph lives: they draw from the upper half of the ring, launches that run at once from the lower half, so a replay
+    // never shares a pair with an eager launch.
+    auto take_queue = [&]() -> ja_status_t {
+        int32_t* queues = nullptr;
+        if (cudaGetSymbolAddress((void**)&queues, g_attn_queues) != cudaSuccess || !queues)
+            return ja_fail(JA_ERR_CUDA, "cannot resolve the attention work queues");
+        static std::atomic<unsigned> next_queue{0}, next_captured{0};
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusNone;
+        const unsigned half = ATTN_QUEUES / 2;
+        const unsigned slot = cap == cudaStreamCaptureStatusActive ? half + next_captured.fetch_add(1) % half : next_queue.fetch_add(1) % half;
+        p.queue = queues + 2 * slot;
+        return JA_OK;
+    };
+    if (use_ragged) {
+        p.sect = (a.causal || a.n_ends > 1) ? a.H * a.B : std::max(1, (sms + rt.n_items - 1) / rt.n_items);
+        if (cfg.attn_section >= 1) p.sect = cfg.attn_section;
+        p.sect = std::min(p.sect, a.H * a.B);
+        ja_status_t s = take_queue();
+        if (s != JA_OK) return s;
+        const int64_t items = (int64_t)a.H * a.B * rt.n_items;
+        const dim3 grid((unsigned)std::min<int64_t>(items, sms), 1, 1);
+        if (a.f16) {
+            JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
+            attention_ragged_kernel<true><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p, rt);
+        } else {
+            JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
+            attention_ragged_kernel<false><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p, rt);
+        }
+        ja_count_launch();
+        JA_CUDA(cudaGetLastError());
+        *launched = true;
+        return JA_OK;
+    }
     const bool two_tiles = pair_ok && cfg.attn_one_tile != 1;
     // packed sequences: the work of a tile is its distance from the start of its own sequence, not its index
     const int rows_per_cta = two_tiles ? 2 * QT : QT, n_cta_tiles = a.S / rows_per_cta;
@@ -1038,7 +1302,6 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         p.n_order = n_cta_tiles;
         for (int t = 0; t < n_cta_tiles; ++t) p.order[t] = (uint16_t)w[t].second;
     }
-    const int sms = ja_sm_count();
     // tiles of different weight (causal band, packed sequences): one section, i.e. heaviest first across all (batch, head)
     // pairs; equal tiles: sections that fill the GPU once, so that CTAs running together share K / V tiles through L2
     p.sect = (a.causal || a.n_ends > 1) ? a.H * a.B : std::max(1, (sms + n_cta_tiles - 1) / n_cta_tiles);
@@ -1057,17 +1320,7 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         const int variant = cfg.attn_variant >= 0 ? cfg.attn_variant : 1;
         ja_status_t s;
         if (persist) {
-            int32_t* queues = nullptr;
-            if (cudaGetSymbolAddress((void**)&queues, g_attn_queues) != cudaSuccess || !queues)
-                return ja_fail(JA_ERR_CUDA, "cannot resolve the attention work queues");
-            // launches recorded into a CUDA graph keep their pair for as long as the graph lives: they draw from the upper half
-            // of the ring, launches that run at once from the lower half, so a replay never shares a pair with an eager launch
-            static std::atomic<unsigned> next_queue{0}, next_captured{0};
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusNone;
-            const unsigned half = ATTN_QUEUES / 2;
-            const unsigned slot = cap == cudaStreamCaptureStatusActive ? half + next_captured.fetch_add(1) % half : next_queue.fetch_add(1) % half;
-            p.queue = queues + 2 * slot;
+            if ((s = take_queue()) != JA_OK) return s;
             s = launch_two_tiles<true>(variant, a.f16, dim3((unsigned)std::min<int64_t>(items, sms), 1, 1), st, tq, tk, tv, to, p);
         } else {
             s = launch_two_tiles<false>(variant, a.f16, dim3((unsigned)items, 1, 1), st, tq, tk, tv, to, p);

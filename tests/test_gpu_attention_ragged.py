@@ -1,0 +1,118 @@
+"""Attention over sequences and blocks that are no whole pairs of 128-row tiles, on the tensor-memory kernel (its ragged form)
+against the oracle. Lengths sit at the edges of tiles (128 rows), of pairs, of the 16-key groups of the P V product and of the
+pieces a tile is made of. Tolerances: those of the other attention tests (ten half-ulps of the stored type; lse 1e-3 absolute:
+2^-9 of scores of order one plus the f32 logarithm)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_03905_b200 as ja
+import synth_inputs as si
+from oracle import blocked, operators
+
+from gpu_util import TOL, check_status, download, empty_like_tiling, relfro, upload
+
+pytestmark = pytest.mark.gpu
+ES = blocked.equal_splits
+BF, F32, F16 = torch.bfloat16, torch.float32, torch.float16
+
+
+def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_blocks=None):
+    grp = Hq // Hkv
+    Q, K, V = (si.normal((B, S, h, 128), 0.0, 1.0, dtype, 4, 60 + n) for n, h in enumerate((Hq, Hkv, Hkv)))
+    b_sp, g_sp = ES(B, b_blocks or B), ES(Hkv, max(1, Hkv // 2))
+    h_sp = [grp * v for v in g_sp]
+    d = [0, 128]
+    rq, rk, rv = upload(Q, [b_sp, q_split, h_sp, d]), upload(K, [b_sp, k_split, g_sp, d]), upload(V, [b_sp, k_split, g_sp, d])
+    ro = empty_like_tiling([B, S, Hq, 128], [b_sp, q_split, h_sp, d], dtype, fill=float("nan"))
+    rl = empty_like_tiling([B, S, Hq], [b_sp, q_split, h_sp], F32, fill=float("nan")) if lse else None
+    scale = 1.0 / math.sqrt(128)
+    parts = {"b": b_sp, "q": q_split, "h": h_sp, "d": d, "k": k_split}
+    if grp > 1:
+        parts["g"] = g_sp
+    spec = ja.Spec("bqhd,bkgd,bkgd->bqhd" if grp > 1 else "bqhd,bkhd,bkhd->bqhd", parts, "attention",
+                   (scale, 1.0 if causal else 0.0) + tuple(float(e) for e in ends), "online_softmax")
+    spec.execute([rq, rk, rv], [ro, rl] if lse else ro)
+    got = download(ro)
+    ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), grp, ends or None, causal, {BF: "bf16", F16: "f16"}[dtype])
+    assert relfro(got, ref) <= TOL[dtype]
+    # no row is worse than the whole: a row that lost or gained a key would be
+    err = np.linalg.norm(got - ref, axis=-1) / np.maximum(np.linalg.norm(ref, axis=-1), 1e-3)
+    assert err.max() <= 4 * TOL[dtype]
+    if lse:
+        s0 = 0
+        L = download(rl)
+        for s1 in ends or [S]:
+            K2 = np.repeat(si.to_f64(K)[:, s0:s1], grp, axis=2)
+            want = operators.attention_lse(si.to_f64(Q)[:, s0:s1], K2, causal, scale)
+            assert np.abs(L[:, s0:s1] - want).max() <= 1e-3
+            s0 = s1
+    check_status()
+
+
+@pytest.mark.parametrize("S", [46, 63, 65, 127, 128, 129, 143, 145, 255, 257, 383, 384, 385, 641])
+@pytest.mark.parametrize("causal", [True, False])
+def test_one_block_of_any_length(S, causal):
+    _run(2, S, 4, 4, [0, S], [0, S], [], causal, BF, lse=True)
+
+
+@pytest.mark.parametrize("cut", [200, 125, 64, 72, 40, 96])     # 8-, 1-, 64-, 8-, 8- and 32-row pieces
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_short_blocks(cut, causal, dtype):
+    S = cut * 6
+    _run(2, S, 8, 2, ES(S, 6), ES(S, 6), [], causal, dtype, b_blocks=1)
+
+
+@pytest.mark.parametrize("ends", [[50, 131, 400], [128, 256, 384], [64, 320, 1000], [777, 778, 1000], [1000]])
+@pytest.mark.parametrize("causal,lse", [(True, False), (True, True), (False, False)])
+def test_packed_sequences(ends, causal, lse):
+    S = ends[-1]
+    _run(2, S, 8, 4, [0] + ends, [0] + ends, ends, causal, BF, lse=lse)
+
+
+def test_queries_and_keys_cut_differently():
+    S = 600
+    _run(1, S, 4, 2, [0, 130, 391, 600], ES(S, 3), [], True, BF)
+    _run(1, S, 4, 4, ES(S, 4), [0, 64, 512, 600], [], True, F16, lse=True)
+
+
+def test_nothing_leaks_from_other_sequences():
+    """Keys and values of the second sequence are infinite: the first one's results must not notice."""
+    ends, S, H = [77, 200], 200, 2
+    Q, K, V = (si.normal((1, S, H, 128), 0.0, 1.0, BF, 4, 70 + n) for n in range(3))
+    ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), 1, ends, True, "bf16")
+    K[:, 77:] = float("inf")
+    V[:, 77:] = float("nan")
+    sp = [[0, 1], [0] + ends, [0, H], [0, 128]]
+    ro = empty_like_tiling([1, S, H, 128], sp, BF)
+    ja.Spec("bqhd,bkhd,bkhd->bqhd", {"b": sp[0], "q": sp[1], "h": sp[2], "d": sp[3], "k": sp[1]}, "attention",
+            (1.0 / math.sqrt(128), 1.0, 77.0, 200.0), "online_softmax").execute([upload(Q, sp), upload(K, sp), upload(V, sp)], ro)
+    torch.cuda.synchronize()
+    payload = ro.payload[: 77 * H * 128].reshape(1, 77, H, 128).to(torch.float64).cpu().numpy()
+    assert relfro(payload, ref[:, :77]) <= TOL[BF]
+    check_status()
+
+
+def test_more_items_than_a_wave_and_a_graph_replay():
+    S = 300
+    Q, K, V = (si.normal((8, S, 32, 128), 0.0, 1.0, BF, 4, 80 + n) for n in range(3))
+    sp = [ES(8, 8), [0, S], ES(32, 4), [0, 128]]
+    rels = [upload(x, sp) for x in (Q, K, V)]
+    ro = empty_like_tiling([8, S, 32, 128], sp, BF, fill=float("nan"))
+    spec = ja.Spec("bqhd,bkhd,bkhd->bqhd", {"b": sp[0], "q": sp[1], "h": sp[2], "d": sp[3], "k": sp[1]}, "attention", (1.0 / math.sqrt(128), 1.0),
+                   "online_softmax")
+    spec.execute(rels, ro)
+    ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), 1, None, True, "bf16")
+    first = download(ro)
+    assert relfro(first, ref) <= TOL[BF]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        spec.execute(rels, ro)
+    ro.payload.fill_(float("nan"))
+    g.replay()
+    g.replay()
+    assert np.array_equal(download(ro), first)
+    check_status()
