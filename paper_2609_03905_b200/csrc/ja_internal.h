@@ -111,7 +111,7 @@ JaConfig& ja_config();
 // ---- kernel launchers (one per .cu file) ------------------------------------------------------------
 // Plain-ALU tiled matmul join-agg over arbitrary tilings (f32 or bf16 operands, f32 accumulate). The key tables of the
 // three relations must be on the device (ja_relation_to_device).
-// the definition in its relational form, one thread per output cell: any spec whose operator is a scalar function of the
+// the definition in its relational form, cell by cell: any spec whose operator is a scalar function of the
 // joined cells (*launched stays false otherwise)
 ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inputs, const ja_relation* out, cudaStream_t st, bool* launched);
 ja_status_t ja_launch_matmul_simt(const ja_relation* A, const ja_relation* B, const ja_relation* C, cudaStream_t st,
@@ -124,6 +124,11 @@ struct ContractTcPlan;
 ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, const std::string& tc, const ja_relation* A, const ja_relation* B,
                                 const ja_relation* C, std::shared_ptr<ContractTcPlan>* out, double* est_us);
 ja_status_t ja_launch_contract_tc(const ContractTcPlan& plan, cudaStream_t st);
+// the same products of f32 relations on the FMA pipe (k_contract_f32.cu)
+struct ContractF32Plan;
+ja_status_t ja_contract_f32_plan(const std::string& ta, const std::string& tb, const std::string& tc, const ja_relation* A, const ja_relation* B,
+                                 const ja_relation* C, std::shared_ptr<ContractF32Plan>* out);
+ja_status_t ja_launch_contract_f32(const ContractF32Plan& plan, cudaStream_t st);
 
 // Memory-bound join-aggs: flat key-aligned maps and row-structured maps / reductions.
 enum RowOp {

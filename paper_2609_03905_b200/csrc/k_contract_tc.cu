@@ -34,12 +34,14 @@
 
 #include "ja_device.cuh"
 #include "ja_ptx.cuh"
+#include "ja_walk.cuh"
 
 namespace {
 
 using namespace ja_ptx;
+using namespace ja_walk;
 
-constexpr int BM = 128, BK = 64, MAX_BATCH = 2;
+constexpr int BM = 128, BK = 64;
 // RAW: an operand has odd interval lengths (pieces of one cell); its stages carry a second 16-byte word per piece (see load_walk)
 template <int BN, bool RAW> struct Cfg {
     static constexpr int A_WARPS = 4, B_WARPS = BN / 32, WARPS = A_WARPS + B_WARPS + 1, THREADS = WARPS * 32;
@@ -50,25 +52,6 @@ template <int BN, bool RAW> struct Cfg {
     static constexpr int CTAS_PER_SM = BN == 256 || RAW ? 1 : 2;
 };
 
-// one index of one relation
-struct Dim {
-    const int64_t* splits;   // device
-    int64_t blk_bytes;       // bytes between neighbouring blocks along this index (relations of equal blocks)
-    int64_t cell_bytes;      // bytes between neighbouring cells inside a block (relations of equal blocks)
-    int32_t bs;              // uniform interval length or 0
-    uint32_t magic, shift;   // x / bs = umulhi(x, magic) >> shift for 0 <= x < 2^31 (bs > 1)
-    int32_t nblk, extent;
-    int32_t nb_stride;       // blocks between neighbouring blocks along this index, in key order
-    int32_t pos;             // position of the index in the relation's term; -1: the relation does not have it
-};
-struct Rel {
-    char* base;
-    const int64_t* blk_off;
-    Dim r, k, b[MAX_BATCH];  // row index (m of A, n of B; of the output: r = m, k = n), contracted index, batch indices
-    int32_t equal;           // all blocks have one shape
-    int32_t g;               // cells per piece of the contiguous index: 8, 4, 2 or 1
-    int32_t kc;              // k comes after r: the contracted index is the contiguous one (operands), n is (output)
-};
 struct Params {
     Rel A, B, C;
     int32_t* status;
@@ -79,80 +62,6 @@ struct Params {
     int32_t cut_m, cut_n;    // tiles per interval of m / n where tiles stay inside intervals, 0: tiles are cut from the whole index
     int32_t f16, c_esize;
 };
-
-// A position on one index: the interval [lo, hi) that holds it.
-struct Cursor {
-    int blk, lo, hi;
-};
-__device__ __forceinline__ Cursor seek(const Dim& d, int x) {
-    Cursor c;
-    if (d.bs) {
-        c.blk = d.bs > 1 ? (int)(__umulhi((uint32_t)x, d.magic) >> d.shift) : x;
-        c.lo = c.blk * d.bs;
-        c.hi = min(c.lo + d.bs, d.extent);
-    } else {
-        int lo = 0, hi = d.nblk - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (d.splits[mid] <= x) lo = mid;
-            else hi = mid - 1;
-        }
-        c.blk = lo;
-        c.lo = (int)d.splits[lo];
-        c.hi = (int)d.splits[lo + 1];
-    }
-    return c;
-}
-// forward to x (x < extent, never before the cursor's interval): positions along a loader's walk only grow
-__device__ __forceinline__ void advance(const Dim& d, Cursor& c, int x) {
-    while (x >= c.hi) {
-        ++c.blk;
-        c.lo = c.hi;
-        c.hi = d.bs ? min(c.hi + d.bs, d.extent) : (int)d.splits[c.blk + 1];
-    }
-}
-
-// Where a tile's batch coordinates put it on one relation. Inside a block every index weighs the product of the lengths of the
-// indices after it. With f the earlier and s the later one of the relation's row and column index, fin / sin their positions
-// inside their intervals and fw / sw the intervals' lengths, a cell lies
-//     sw * (fin * cf + p0 * fw + p1) + sin * cs + p2
-// cells into its block; cf, cs, p0, p1, p2 hold the batch indices' share (before both, between, after both).
-struct BatchAt {
-    int64_t bytes;           // equal blocks: the batch indices' share of the byte offset
-    int flat;                // their share of the block number
-    int cf, cs, p0, p1, p2;
-};
-__device__ __forceinline__ BatchAt batch_at(const Rel& o, const int (&x)[MAX_BATCH]) {
-    BatchAt a = {0, 0, 1, 1, 0, 0, 0};
-    const int first = min(o.r.pos, o.k.pos), second = max(o.r.pos, o.k.pos);
-    int in[MAX_BATCH], w[MAX_BATCH];
-#pragma unroll
-    for (int i = 0; i < MAX_BATCH; ++i) {
-        in[i] = 0;
-        w[i] = 1;
-        if (o.b[i].pos < 0) continue;
-        const Cursor c = seek(o.b[i], x[i]);
-        in[i] = x[i] - c.lo;
-        w[i] = c.hi - c.lo;
-        a.flat += c.blk * o.b[i].nb_stride;
-        a.bytes += c.blk * o.b[i].blk_bytes + in[i] * o.b[i].cell_bytes;
-        if (o.b[i].pos > first) a.cf *= w[i];
-        if (o.b[i].pos > second) a.cs *= w[i];
-    }
-#pragma unroll
-    for (int i = 0; i < MAX_BATCH; ++i) {
-        const int pos = o.b[i].pos;
-        if (pos < 0) continue;
-        int v = in[i];
-#pragma unroll
-        for (int j = 0; j < MAX_BATCH; ++j)
-            if (j != i && o.b[j].pos > pos) v *= w[j];
-        if (pos < first) a.p0 += v;
-        else if (pos < second) a.p1 += v;
-        else a.p2 += v;
-    }
-    return a;
-}
 
 // Asynchronous copy of `bytes` (16, 8 or 4), zero-filled past src_bytes; nothing happens where `live` is 0 (a predicate, not a branch).
 __device__ __forceinline__ void cp_async(uint32_t dst, const char* src, int bytes, int src_bytes, uint32_t live) {
@@ -740,37 +649,6 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
 }
 
 // ---- host -----------------------------------------------------------------------------------------------------
-void set_dim(Dim* d, const ja_relation* r, const RelView& v, const std::string& term, char letter) {
-    memset(d, 0, sizeof *d);
-    const size_t p = letter ? term.find(letter) : std::string::npos;
-    d->pos = p == std::string::npos ? -1 : (int32_t)p;
-    if (d->pos < 0) return;
-    int64_t nb = 1, cells = 1;
-    for (int e = (int)p + 1; e < r->rank; ++e) {
-        nb *= r->nblk[e];
-        cells *= r->splits[e][1] - r->splits[e][0];
-    }
-    d->splits = v.splits[p];
-    d->bs = (int32_t)r->bs[p];
-    if (d->bs > 1) {   // magic = floor(2^(32 + s) / bs) + 1 with 2^s < bs <= 2^(s + 1): its error times x stays below 2^(32 + s) for x < 2^31
-        while ((2ll << d->shift) < d->bs) ++d->shift;
-        d->magic = (uint32_t)(((1ull << (32 + d->shift)) / (uint64_t)d->bs) + 1);
-    }
-    d->nblk = r->nblk[p];
-    d->extent = (int32_t)r->extent[p];
-    d->nb_stride = (int32_t)nb;
-    d->blk_bytes = nb * v.blk_stride;
-    d->cell_bytes = cells * r->esize;
-}
-
-// largest piece of 8, 4, 2 or 1 cells that never straddles a split point of the last index and is aligned wherever it starts
-int piece_cells(const ja_relation* r) {
-    int g = 8;
-    for (int64_t s : r->splits[r->rank - 1])
-        while (s % g) g /= 2;
-    return g;
-}
-
 template <int BN, bool RAW>
 ja_status_t launch(const Params& p, cudaStream_t st) {
     static bool configured[64] = {};
@@ -809,46 +687,11 @@ ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, co
                                 const ja_relation* C, std::shared_ptr<ContractTcPlan>* out, double* est_us) {
     out->reset();
     if (A->dtype == JA_F32 || B->dtype != A->dtype || (C->dtype != JA_F32 && C->dtype != A->dtype)) return JA_OK;
-    // ---- the indices' roles ----
-    char m = 0, n = 0, k = 0, batch[MAX_BATCH] = {0, 0};
-    int n_batch = 0;
-    std::string all = ta;
-    for (char c : tb)
-        if (all.find(c) == std::string::npos) all.push_back(c);
+    ProductRoles roles;
+    if (!product_roles(ta, tb, tc, &roles) || !fits_32_bits(A) || !fits_32_bits(B) || !fits_32_bits(C)) return JA_OK;
+    char m = roles.m, n = roles.n;
+    const char k = roles.k;
     auto has = [](const std::string& t, char c) { return t.find(c) != std::string::npos; };
-    for (char c : all)
-        if (!has(tc, c)) {
-            if (!has(ta, c) || !has(tb, c) || k) return JA_OK;   // one contracted index, in both operands
-            k = c;
-        }
-    if (!k) return JA_OK;
-    // m and n: each operand's contiguous index where it is not the contracted one, else the last index only it has
-    auto row_of = [&](const std::string& own, const std::string& other) -> char {
-        if (own.back() != k) return has(other, own.back()) || !has(tc, own.back()) ? 0 : own.back();
-        for (size_t i = own.size() - 1; i-- > 0;)
-            if (!has(other, own[i])) return own[i];
-        return 0;
-    };
-    m = row_of(ta, tb);
-    n = row_of(tb, ta);
-    if (!m || !n) return JA_OK;
-    for (char c : tc)
-        if (c != m && c != n) {
-            if (n_batch == MAX_BATCH) return JA_OK;
-            batch[n_batch++] = c;
-        }
-    for (const ja_relation* r : {A, B, C}) {
-        if (r->nblocks >= (1ll << 31)) return JA_OK;
-        int64_t cells = 1;   // of the largest block
-        for (int d = 0; d < r->rank; ++d) {
-            int64_t w = 0;
-            for (int i = 0; i < r->nblk[d]; ++i) w = std::max(w, r->splits[d][i + 1] - r->splits[d][i]);
-            cells *= w;
-        }
-        if (cells >= (1ll << 31)) return JA_OK;
-        for (int d = 0; d < r->rank; ++d)
-            if (r->extent[d] >= (1ll << 30)) return JA_OK;
-    }
     auto extent_of = [&](char c) { return c ? (has(ta, c) ? A->extent[ta.find(c)] : B->extent[tb.find(c)]) : (int64_t)1; };
     std::shared_ptr<ContractTcPlan> plan(new ContractTcPlan());
     Params& p = plan->p;
@@ -861,23 +704,11 @@ ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, co
     const ja_relation *rel_a = swap ? B : A, *rel_b = swap ? A : B;
     const std::string &t_a = swap ? tb : ta, &t_b = swap ? ta : tb;
     if (swap) { std::swap(m, n); std::swap(M, N); }
-    auto fill = [&](Rel* o, const ja_relation* r, const std::string& term, char cr, char ck) {
-        const RelView v = ja_view(r);
-        o->base = (char*)r->base;
-        o->blk_off = v.blk_off;
-        o->equal = r->equal_blocks ? 1 : 0;
-        o->g = piece_cells(r);
-        set_dim(&o->r, r, v, term, cr);
-        set_dim(&o->k, r, v, term, ck);
-        o->kc = o->k.pos > o->r.pos;
-        for (int i = 0; i < MAX_BATCH; ++i) set_dim(&o->b[i], r, v, term, batch[i]);
-        if (term.back() != cr && term.back() != ck) o->g = 1;   // (output only) a batch index is the contiguous one: cell by cell
-    };
-    fill(&p.A, rel_a, t_a, m, k);
-    fill(&p.B, rel_b, t_b, n, k);
-    fill(&p.C, C, tc, m, n);
+    fill_rel(&p.A, rel_a, t_a, m, k, roles.batch, 8);
+    fill_rel(&p.B, rel_b, t_b, n, k, roles.batch, 8);
+    fill_rel(&p.C, C, tc, m, n, roles.batch, 8);
     p.M = (int)M; p.N = (int)N; p.K = (int)K;
-    for (int i = 0; i < MAX_BATCH; ++i) p.batch[i] = (int)extent_of(batch[i]);
+    for (int i = 0; i < MAX_BATCH; ++i) p.batch[i] = (int)extent_of(roles.batch[i]);
     p.f16 = A->dtype == JA_F16;
     p.c_esize = C->esize;
     p.group_m = 8;
