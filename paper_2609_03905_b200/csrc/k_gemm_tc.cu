@@ -62,6 +62,7 @@ struct GemmParams {
     int32_t nbm, nbk, nbn;     // blocks along i, j, k
     int32_t M, N;              // tensor extents along i, k
     int32_t a_box_rows;        // rows per A box (= min(bm, 128))
+    int32_t a_boxes;           // A boxes per tile: 128 / bm where bm divides 128 (tiles cut from global rows), else 1
     int32_t m_tiles, n_tiles;  // tile grid (tiles are 128*CG rows x up to 256 columns)
     int32_t tiles_per_mblk;    // >= 1 when row tiles never leave a block, 0 when tiles are cut from global rows
     int32_t tiles_per_nblk;    // >= 1 when tiles stay inside one column block, 0 when tiles span blocks
@@ -120,10 +121,11 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmParams& p, int t, int 
     const int mt = band * p.group_m + tin % rows_in_band;
     int nt = tin / rows_in_band;
     if (p.heavy_first) nt = narrow ? nt * p.tiles_per_nblk + p.tiles_per_nblk - 1 : (nt / (p.tiles_per_nblk - 1)) * p.tiles_per_nblk + nt % (p.tiles_per_nblk - 1);
-    if (p.tiles_per_mblk > 0) {   // CG == 1 only: row tiles stay inside a block
-        tc.mb = mt / p.tiles_per_mblk;
-        tc.r0 = (mt % p.tiles_per_mblk) * BM;
-        tc.rows = min(BM, p.bm - tc.r0);
+    if (p.tiles_per_mblk > 0) {   // 128-row tiles stay inside a block; a pair of CTAs takes two consecutive ones
+        const int rt = mt * CG + cta_rank;
+        tc.mb = rt / p.tiles_per_mblk;
+        tc.r0 = (rt % p.tiles_per_mblk) * BM;
+        tc.rows = tc.mb < p.nbm ? min(BM, p.bm - tc.r0) : 0;   // an odd number of row tiles: the last pair's second one is all fill
         tc.row_g0 = tc.mb * p.bm + tc.r0;
     } else {                      // tiles cut from global rows (block height divides 128, or is a multiple of 128)
         tc.row_g0 = mt * (BM * CG) + cta_rank * BM;
@@ -228,7 +230,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const int my_cols = n_mma / CG;                    // B columns this CTA stages
                 const int my_c0 = cta_rank * my_cols;              // their offset inside the tile
                 const int nchunks = (my_cols + 63) / 64;
-                const uint32_t tx = (uint32_t)CG * (A_STAGE_BYTES + nchunks * B_CHUNK_BYTES);
+                const uint32_t tx = (uint32_t)CG * ((uint32_t)(p.a_boxes * p.a_box_rows) * (BK * 2) + nchunks * B_CHUNK_BYTES);
                 for (int jb = tc.jb0; jb < tc.jb1 && ok; ++jb) {    // the tuples of this output key, ascending j
                     for (int kc = 0; kc < kchunks; ++kc) {
                         if (!mbar_wait(empty_bar(stage), phase ^ 1, abort_flag, p.status)) { ok = false; break; }
@@ -238,7 +240,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         issued[stage] = true;
                         last_parity[stage] = phase;
                         // A: boxes of a_box_rows rows x 64 k, one set per 64-deep half of the stage
-                        const int nboxes = BM / p.a_box_rows;
+                        const int nboxes = p.a_boxes;
                         for (int kh = 0; kh < BK / 64; ++kh)
                             for (int bx = 0; bx < nboxes; ++bx)
                                 tma_load_4d<CG>(sA + stage * A_STAGE_BYTES + kh * A_HALF_BYTES + bx * p.a_box_rows * 128, &tmA, fb,
@@ -466,7 +468,8 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     const int64_t bm = A->bs[0], bk = A->bs[1], bn = B->bs[1];
     // TMA needs 16-byte row pitches; boxes are 64 elements wide; A boxes hold min(bm,128) rows
     if (bk % 8 || bn % 8 || bk < 64 || bn < 64) return JA_OK;
-    if (bm < 128 && (128 % bm != 0 || bm % 8 != 0)) return JA_OK;
+    const bool odd_rows = bm < 128 && (128 % bm != 0 || bm % 8 != 0);   // one block per row tile: plain products alone
+    if (odd_rows && (epi != EPI_NONE || C->esize != 2)) return JA_OK;
     if (A->extent[0] >= (1ll << 31) || B->extent[1] >= (1ll << 31)) return JA_OK;
     std::shared_ptr<GemmTcPlan> plan(new GemmTcPlan());
     GemmParams& p = plan->p;
@@ -477,6 +480,7 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     p.nbm = A->nblk[0]; p.nbk = A->nblk[1]; p.nbn = B->nblk[1];
     p.M = (int)A->extent[0]; p.N = (int)B->extent[1];
     p.a_box_rows = (int)std::min<int64_t>(bm, 128);
+    p.a_boxes = bm < 128 && !odd_rows ? (int)(128 / bm) : 1;
     p.epi = epi;
     p.bn_tile = bn_tile;
     p.n_copies = (ep && ep->partials) ? p.nbk : 1;
@@ -489,18 +493,20 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     p.rope_D = ep ? ep->rope_D : 2;
     if (bn % 64 == 0 && bn < bn_tile && p.nbn > 1) { p.tiles_per_nblk = 0; p.n_tiles = (p.N + bn_tile - 1) / bn_tile; }
     else { p.tiles_per_nblk = (int)((bn + bn_tile - 1) / bn_tile); p.n_tiles = p.tiles_per_nblk * p.nbn; }
-    // Two-CTA form: 256-row tiles cut from global rows; needs 128-row halves that never straddle a block and, when
+    // Two-CTA form: 256-row tiles cut from global rows where blocks are whole 128-row halves or divide them, else pairs of row tiles
+    // that each stay inside a block ([1260, 3840] x [3840, 10880] in one block: 145 us on single CTAs, 112 on pairs); when
     // tiles span column blocks, column tails whose halves still start on a 64-column box boundary.
     // narrow last tile in every column block (block width not a multiple of the tile width): schedule it after the full tiles
     const JaConfig& cfg = ja_config();
     p.heavy_first = (p.n_copies == 1 && p.tiles_per_nblk > 1 && bn % bn_tile != 0 && cfg.gemm_heavy_first != 0) ? 1 : 0;
     p.group_m = cfg.gemm_group_m >= 1 ? cfg.gemm_group_m : 8;
-    bool two = (bm % 128 == 0 || 128 % bm == 0) && p.M >= 256 && bk >= Cfg<2>::BK;
+    const bool by_block = odd_rows || (bm > 128 && bm % 128 != 0);
+    bool two = p.M >= 256 && bk >= Cfg<2>::BK;
     if (p.tiles_per_nblk == 0 && (p.N % bn_tile) % (bn_tile / 2) != 0) two = false;
     if (cfg.gemm_cta_group == 1) two = false;
     plan->cg = two ? 2 : 1;
-    if (two || bm < 128) { p.tiles_per_mblk = 0; p.m_tiles = (p.M + BM * plan->cg - 1) / (BM * plan->cg); }
-    else { p.tiles_per_mblk = (int)((bm + BM - 1) / BM); p.m_tiles = p.tiles_per_mblk * p.nbm; }
+    if (!by_block) { p.tiles_per_mblk = 0; p.m_tiles = (p.M + BM * plan->cg - 1) / (BM * plan->cg); }
+    else { p.tiles_per_mblk = (int)((bm + BM - 1) / BM); p.m_tiles = (p.tiles_per_mblk * p.nbm + plan->cg - 1) / plan->cg; }
     ja_status_t st;
     if ((st = encode_blocked_2d(A, 64, p.a_box_rows, &plan->tmA)) != JA_OK) return st;
     if ((st = encode_blocked_2d(B, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB)) != JA_OK) return st;
