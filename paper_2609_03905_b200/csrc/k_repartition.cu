@@ -1,7 +1,17 @@
 // ja_repartition data movement (Section 5.3): the overlay of the source and destination tilings gives
 // atoms; each atom is cut into 2-D slabs (rows x contiguous run) and copied from its source block to its
-// destination block -- "decompose" and "recompose" in one pass, no staging buffer. One CTA per slab,
-// 128-bit accesses when every offset, pitch and run length allows it. Pure byte movement: bit-exact.
+// destination block -- "decompose" and "recompose" in one pass, no staging buffer. One CTA per slab. Pure byte movement: bit-exact.
+//
+// Where every offset, pitch and run length is a multiple of 16 bytes a thread moves 16-byte words as they are (5.7 TB/s at 268 MB, of
+// 6.5). Long rows of any width are still written as whole aligned words, put together from the two aligned source words
+// around them, and only the ends of a row go cell by cell (12370 rows of 2919 bf16 cells: 81 -> 39 us); short ones go by the
+// widest access their alignment allows.
+//
+// The slabs travel in a table in device memory that the caller keeps, or -- up to JA_PARAM_SLABS of them -- in the kernel's
+// parameters, so that a relayout between relations that are used once (packing a dense tensor, unpacking a result) allocates
+// nothing on the device and copies nothing to it.
+#include <string.h>
+
 #include "ja_device.cuh"
 
 namespace {
@@ -23,18 +33,111 @@ __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict
     }
 }
 
+__device__ __forceinline__ uint4 shifted(const uint4& lo, const uint4& hi, int sh) {   // 16 bytes from byte sh (0..15, even) of lo:hi on
+    const bool s8 = sh & 8, s4 = sh & 4;
+    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
+    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
+    const int bits = (sh & 2) * 8;
+    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
+}
+
+// One slab at any even alignment. Word w of row r is the w-th aligned 16-byte word that the row touches in the destination. Only
+// source words that hold wanted bytes are read (payloads are 128-byte aligned and padded, so none leaves them).
+__device__ __forceinline__ void copy_slab_any(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+    const int words = (sl.row_bytes + 30) / 16;        // at most, whatever the alignment
+    const int total = words * sl.rows;
+    const int dr = 256 / words, dw = 256 - dr * words;
+    int r = (int)threadIdx.x / words, w = (int)threadIdx.x - r * words;
+    for (int i = threadIdx.x; i < total; i += 256) {
+        char* d = dp + (int64_t)r * sl.dst_pitch;
+        const char* s = sp + (int64_t)r * sl.src_pitch;
+        const int head = (int)(reinterpret_cast<uintptr_t>(d) & 15);
+        const int at = w * 16 - head;                   // byte of the row where this word starts
+        if (at < sl.row_bytes) {
+            const char* from = s + at;
+            const int sh = (int)(reinterpret_cast<uintptr_t>(from) & 15);
+            const uint4* q = reinterpret_cast<const uint4*>(from - sh);
+            const bool need_lo = at + 16 - sh > 0, need_hi = sh > 0 && at + 16 - sh < sl.row_bytes;   // the second word starts 16 - sh bytes in
+            uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
+            if (need_lo) lo = q[0];
+            if (need_hi) hi = q[1];
+            const uint4 v = shifted(lo, hi, sh);
+            if (at >= 0 && at + 16 <= sl.row_bytes) {
+                *reinterpret_cast<uint4*>(d + at) = v;
+            } else {
+                const uint32_t c[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int b = at + e * 2;
+                    if (b >= 0 && b < sl.row_bytes) *reinterpret_cast<uint16_t*>(d + b) = (uint16_t)(c[e >> 1] >> ((e & 1) * 16));
+                }
+            }
+        }
+        r += dr;
+        w += dw;
+        if (w >= words) { w -= words; ++r; }
+    }
+}
+__global__ void __launch_bounds__(256) repartition_any_kernel(const char* __restrict__ src, char* __restrict__ dst, const CopySlab* __restrict__ slabs,
+                                                              int64_t n_slabs) {
+    for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
+        const CopySlab sl = slabs[s];
+        copy_slab_any(src + sl.src_off, dst + sl.dst_off, sl);
+    }
+}
+
+template <int N> struct SlabParams {
+    CopySlab s[N];
+};
+template <int N, bool WORDS>
+__global__ void __launch_bounds__(256) repartition_param_kernel(const char* __restrict__ src, char* __restrict__ dst, const __grid_constant__ SlabParams<N> p) {
+    const CopySlab& sl = p.s[blockIdx.x];
+    const char* sp = src + sl.src_off;
+    char* dp = dst + sl.dst_off;
+    if (!WORDS) {
+        copy_slab_any(sp, dp, sl);
+        return;
+    }
+    const int vpr = sl.row_bytes / 16, total = vpr * sl.rows;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < total; i += 256) {
+        const int r = i / vpr, c = i - r * vpr;
+        *reinterpret_cast<uint4*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * 16) = *reinterpret_cast<const uint4*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * 16);
+    }
+}
+template <int N>
+void launch_param(const char* src, char* dst, const CopySlab* slabs, int n, bool words, cudaStream_t st) {
+    SlabParams<N> p;
+    memcpy(p.s, slabs, (size_t)n * sizeof(CopySlab));
+    if (words) repartition_param_kernel<N, true><<<n, 256, 0, st>>>(src, dst, p);
+    else repartition_param_kernel<N, false><<<n, 256, 0, st>>>(src, dst, p);
+}
+
 }  // namespace
 
-ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int vec_bytes,
+ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, cudaStream_t st) {
+    static_assert(JA_PARAM_SLABS == 960 && sizeof(CopySlab) == 32, "30 KiB of the 32764 bytes a kernel's parameters may hold");
+    if (n_slabs == 0) return JA_OK;
+    const bool words = vec_bytes == 16;
+    if (n_slabs <= 32) launch_param<32>(src, dst, slabs, n_slabs, words, st);
+    else if (n_slabs <= 256) launch_param<256>(src, dst, slabs, n_slabs, words, st);
+    else launch_param<JA_PARAM_SLABS>(src, dst, slabs, n_slabs, words, st);
+    ja_count_launch();
+    JA_CUDA(cudaGetLastError());
+    return JA_OK;
+}
+
+ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int vec_bytes, bool long_rows,
                                   cudaStream_t st) {
     if (n_slabs == 0) return JA_OK;
     unsigned grid = (unsigned)(n_slabs < (int64_t)148 * 64 ? n_slabs : (int64_t)148 * 64);
-    switch (vec_bytes) {
-        case 16: repartition_kernel<uint4><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs); break;
-        case 8: repartition_kernel<uint2><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs); break;
-        case 4: repartition_kernel<uint32_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs); break;
-        default: repartition_kernel<uint16_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs); break;
-    }
+    // words put together pay on rows long enough that their two ends do not matter, and not against 8-byte accesses (10901 x 1088 f32
+    // in 34-cell blocks 17 us, 26 as shifted words; 28480 x 916 f16 in 29-cell blocks 52 and 62; 12370 x 2919 bf16 81 and 39)
+    if (vec_bytes == 16) repartition_kernel<uint4><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    else if (vec_bytes == 8) repartition_kernel<uint2><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    else if (long_rows) repartition_any_kernel<<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    else if (vec_bytes == 4) repartition_kernel<uint32_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    else repartition_kernel<uint16_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
     return JA_OK;

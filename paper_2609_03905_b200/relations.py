@@ -110,16 +110,17 @@ def from_dense(dense: torch.Tensor, splits) -> Relation:
 
 
 def to_dense(rel: Relation) -> torch.Tensor:
-    """Recompose a relation into a dense row-major tensor: ja_repartition to the one-block tiling."""
-    one = Relation(rel.extents, [[0, e] for e in rel.extents], rel.dtype)
-    repartition(rel, one)
-    torch.cuda.current_stream().synchronize()
+    """Recompose a relation into a dense row-major tensor: ja_repartition to the one-block tiling. The tensor is that block."""
     n = 1
     for e in rel.extents:
         n *= e
-    out = one.payload[:n].reshape(rel.extents).clone()
+    pad = (-n * rel.dtype.itemsize) % 128
+    payload = torch.empty(n + pad // rel.dtype.itemsize, dtype=rel.dtype, device=rel.payload.device)
+    one = Relation(rel.extents, [[0, e] for e in rel.extents], rel.dtype, payload)
+    repartition(rel, one)
+    torch.cuda.current_stream().synchronize()
     one.close()
-    return out
+    return payload[:n].reshape(rel.extents)
 
 
 def _aligned_flat(t: torch.Tensor) -> torch.Tensor:

@@ -1,0 +1,58 @@
+"""ja_repartition at every alignment (whole words, shifted words, row ends) and with its slabs in the kernel's parameters or in a
+device table: bit-exact against the oracle's packing."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_03905_b200 as ja
+import synth_inputs as si
+from oracle import blocked
+
+from gpu_util import check_status, download_bits, empty_like_tiling, np_bits, upload
+
+pytestmark = pytest.mark.gpu
+ES = blocked.equal_splits
+BF, F32, F16 = torch.bfloat16, torch.float32, torch.float16
+
+
+@pytest.mark.parametrize("dtype", [BF, F32])
+@pytest.mark.parametrize("ext,src,dst", [
+    ([64, 1], [1, 1], [4, 1]), ([7, 3], [1, 1], [2, 3]), ([65, 129], [3, 2], [1, 5]), ([257, 1023], [4, 1], [1, 8]), ([300, 2049], [7, 3], [2, 1]),
+    ([128, 256], [2, 4], [4, 1]), ([1000, 37], [1, 1], [100, 1]), ([999, 515], [128, 2], [64, 32]),          # the last: a device table
+    ([5, 33, 17], [1, 2, 3], [5, 1, 2]), ([3, 4, 9, 11], [1, 2, 1, 3], [3, 1, 2, 1]), ([4096, 40], [1024, 1], [3, 1]),
+])
+def test_any_alignment(ext, src, dst, dtype):
+    s_sp, d_sp = [ES(e, g) for e, g in zip(ext, src)], [ES(e, g) for e, g in zip(ext, dst)]
+    x = si.normal(tuple(ext), 0.0, 1.0, dtype, 37, 1)
+    a, b, c = upload(x, s_sp), empty_like_tiling(ext, d_sp, dtype), empty_like_tiling(ext, s_sp, dtype)
+    ja.repartition(a, b)
+    assert np.array_equal(download_bits(b), blocked.pack(np_bits(x), d_sp))
+    ja.repartition(b, c)
+    assert np.array_equal(download_bits(c), blocked.pack(np_bits(x), s_sp))
+    check_status()          # guard zones around every payload
+
+
+@pytest.mark.parametrize("shape,cuts,dtype", [((97, 41), (4, 3), BF), ((1024, 512), (8, 4), F16), ((333,), (5,), F32)])
+def test_dense_round_trip(shape, cuts, dtype):
+    x = si.normal(shape, 0.0, 1.0, dtype, 37, 2)
+    rel = ja.from_dense(x.cuda(), [ES(e, g) for e, g in zip(shape, cuts)])
+    assert np.array_equal(np_bits(rel.payload.cpu()), blocked.pack(np_bits(x), rel.splits))
+    back = ja.to_dense(rel)
+    assert back.shape == x.shape and back.is_contiguous() and torch.equal(back.cpu(), x)
+
+
+def test_first_use_inside_a_capture_and_replay_after_the_plan_is_gone():
+    x = si.normal((130, 70), 0.0, 1.0, BF, 37, 3)
+    s_sp, d_sp = [ES(130, 2), ES(70, 1)], [ES(130, 1), ES(70, 4)]
+    a, b = upload(x, s_sp), empty_like_tiling([130, 70], d_sp, BF)
+    w1, w2 = upload(x, s_sp), empty_like_tiling([130, 70], d_sp, BF)
+    ja.repartition(w1, w2)                                   # the kernel's module is loaded
+    c = ja.Relation([130, 70], d_sp, BF, b.payload)          # another handle on the same payload
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ja.repartition(a, c)
+    c.close()                                                # drops the cached plan, not the captured launch
+    b.payload.zero_()
+    g.replay()
+    assert np.array_equal(download_bits(b), blocked.pack(np_bits(x), d_sp))
+    check_status()
