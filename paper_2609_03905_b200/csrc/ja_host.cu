@@ -1054,6 +1054,10 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
     const std::string R = lead_of(x);
     const bool x_ok = x.size() >= 2;
     auto stat_ok = [&](const ja_relation* r) { return r->dtype == JA_F32; };
+    {
+        const std::vector<int64_t>& sp = inputs[0]->splits[inputs[0]->rank - 1];
+        for (size_t i = 1; i < sp.size(); ++i) ra.widest = std::max(ra.widest, sp[i] - sp[i - 1]);
+    }
     if (x_ok && fn == JA_FN_SQUARE && agg == JA_AGG_SUM && n_in == 1 && o == R) {
         if (!stat_ok(out)) return ja_fail(JA_ERR_DTYPE, "statistics relations are f32");
         ra.x = ja_view(inputs[0]); ra.s0 = ja_view(out);

@@ -144,6 +144,7 @@ struct RowArgs {
     float theta;   // ROPE
     const float2* rope_table;  // device [extent(s)][d/2] (cos, sin)
     int rope_d;                // extent of the rotated index d (rows may hold several heads of d cells each)
+    int64_t widest;            // longest interval of x's last index
 };
 ja_status_t ja_launch_row(RowOp op, const RowArgs& a, ja_dtype_t dt, cudaStream_t st);
 // bulk-copy pipelined form for uniform tilings; *launched stays false when the shape does not fit it

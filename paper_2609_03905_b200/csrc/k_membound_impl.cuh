@@ -507,6 +507,179 @@ bool launch_fast_op(RowOp op, const RowArgs& a, const FastGeom& g, int64_t n_row
     return false;
 }
 
+// ---------------------------------------------------------------------------------------------------
+// any tiling, any width: rows as aligned 16-byte words. A row's cells are one run per column block, at any even byte offset. x and y
+// have one layout, so the words that a run touches in x are the words it touches in y: a thread loads the aligned words, ignores
+// the cells before the run's first and after its last, and stores whole words as such and only a run's two end words cell by
+// cell. (A cell at a time, each with its own block lookup, 4 x 1664 rows of 3239 bf16 cells took 195 us, 6449 rows of 7956
+// f32 cells in four column blocks 421; the copy rate gives 13 and 94.) Every run is given the same number of words, so a thread's
+// runs and words are the same for every row.
+// ---------------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint4 words_shifted(const uint4& lo, const uint4& hi, int sh) {   // 16 bytes from byte sh (0..15, even) of lo:hi on
+    const bool s8 = sh & 8, s4 = sh & 4;
+    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
+    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
+    const int bits = (sh & 2) * 8;
+    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
+}
+
+template <typename T, int VPT, int OP>
+__global__ void __launch_bounds__(256) row_word_kernel(RowArgs a, int64_t n_rows, int team, int words, int runs) {
+    __shared__ float red[64];
+    constexpr int CW = 16 / (int)sizeof(T);       // cells per word
+    constexpr bool HAS_STAT = (OP == ROW_SUMSQ || OP == ROW_MAX || OP == ROW_EXPSUM || OP == ROW_RMS_SCALE || OP == ROW_EXP_SUB_DIV);
+    constexpr bool HAS_G = (OP == ROW_RMS_SCALE || OP == ROW_RMSNORM);
+    const int rpc = 256 / team, row_in_cta = threadIdx.x / team, lane_t = threadIdx.x % team;
+    const int last = a.x.rank - 1;
+    const int64_t row = (int64_t)blockIdx.x * rpc + row_in_cta;
+    const bool live = row < n_rows;
+    const RowCtx ctx = row_ctx(a.x, a.s0, HAS_STAT, live ? row : 0);
+
+    union Word {
+        uint4 v;
+        T e[CW];
+        __device__ Word() {}
+    };
+    Word raw[VPT];
+    int64_t off[VPT];            // byte offset of the word in the payload of x and y
+    uint32_t mask[VPT];          // its cells that belong to the row
+    int g_run[HAS_G ? VPT : 1], g_cell[HAS_G ? VPT : 1];   // run, and position inside it of the word's first cell
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+        const int i = k * team + lane_t, run = i / words, w = i - run * words;
+        mask[k] = 0;
+        off[k] = 0;
+        if (HAS_G) g_run[k] = g_cell[k] = 0;
+        if (!live || run >= runs) continue;
+        int width;
+        if (a.x.bs[last]) width = min((int)a.x.bs[last], (int)a.x.extent[last] - run * (int)a.x.bs[last]);
+        else width = (int)(a.x.splits[last][run + 1] - a.x.splits[last][run]);
+        const int64_t at = blk_offset(a.x, ctx.lead_flat * runs + run) + ctx.lead_in * width * (int64_t)sizeof(T);
+        const int head = (int)(at & 15);
+        const int first = (16 * w - head) / (int)sizeof(T);          // cell of the run at the word's start (exact: both are whole cells)
+        const int lo = max(0, -first), hi = min(CW, width - first);
+        if (lo >= hi) continue;
+        off[k] = at - head + 16 * w;
+        mask[k] = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+        if (HAS_G) {
+            g_run[k] = run;
+            g_cell[k] = first;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < VPT; ++k)
+        if (mask[k]) raw[k].v = *reinterpret_cast<const uint4*>(a.x.base + off[k]);
+    auto for_each = [&](auto f) {
+#pragma unroll
+        for (int k = 0; k < VPT; ++k)
+#pragma unroll
+            for (int e = 0; e < CW; ++e)
+                if (mask[k] >> e & 1) f(ja_to_float(raw[k].e[e]));
+    };
+
+    float m = 0.f, l = 0.f, rstd = 0.f;
+    const int n = (int)a.x.extent[last];
+    if (OP == ROW_SUMSQ || OP == ROW_RMSNORM) {
+        float s = 0.f;
+        for_each([&](float f) { s = fmaf(f, f, s); });
+        s = team_reduce<false>(s, team, red, row_in_cta, lane_t);
+        if (OP == ROW_SUMSQ) {
+            if (live && lane_t == 0) *reinterpret_cast<float*>(a.s0.base + ctx.stat_off) = s;
+            return;
+        }
+        rstd = 1.0f / sqrtf(s / (float)n + a.eps);
+    }
+    if (OP == ROW_MAX || OP == ROW_SOFTMAX) {
+        float mx = -INFINITY;
+        for_each([&](float f) { mx = fmaxf(mx, f); });
+        m = team_reduce<true>(mx, team, red, row_in_cta, lane_t);
+        if (OP == ROW_MAX) {
+            if (live && lane_t == 0) *reinterpret_cast<float*>(a.s0.base + ctx.stat_off) = m;
+            return;
+        }
+    }
+    if (OP == ROW_EXPSUM || OP == ROW_EXP_SUB_DIV) m = live ? *reinterpret_cast<const float*>(a.s0.base + ctx.stat_off) : 0.f;
+    if (OP == ROW_EXPSUM || OP == ROW_SOFTMAX) {
+        float s = 0.f;
+        for_each([&](float f) { s += __expf(f - m); });
+        l = team_reduce<false>(s, team, red, row_in_cta, lane_t);
+        if (OP == ROW_EXPSUM) {
+            if (live && lane_t == 0) *reinterpret_cast<float*>(a.s1.base + ctx.stat_off) = l;
+            return;
+        }
+    }
+    if (OP == ROW_EXP_SUB_DIV) l = live ? *reinterpret_cast<const float*>(a.s1.base + ctx.stat_off) : 1.f;
+    if (OP == ROW_RMS_SCALE) {
+        const float ss = live ? *reinterpret_cast<const float*>(a.s0.base + ctx.stat_off) : 1.f;
+        rstd = 1.0f / sqrtf(ss / (float)n + a.eps);
+    }
+    const float inv_l = (OP == ROW_SOFTMAX || OP == ROW_EXP_SUB_DIV) ? 1.0f / l : 0.f;
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+        if (!mask[k]) continue;
+        Word o;
+        if (HAS_G) {   // the gain's cells of this word: its own alignment, so two aligned words shifted together
+            const int lo = __ffs(mask[k]) - 1, hi = 32 - __clz(mask[k]);
+            const int64_t gat = blk_offset(a.g, g_run[k]) + (int64_t)g_cell[k] * (int)sizeof(T);   // of the word's first cell, perhaps before the run
+            const int64_t g0 = gat & ~(int64_t)15;
+            const int sh = (int)(gat - g0);
+            Word gv;
+            uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+            if (sh + lo * (int)sizeof(T) < 16) x = *reinterpret_cast<const uint4*>(a.g.base + g0);          // only words that hold wanted cells
+            if (sh + hi * (int)sizeof(T) > 16) y = *reinterpret_cast<const uint4*>(a.g.base + g0 + 16);
+            gv.v = words_shifted(x, y, sh);
+#pragma unroll
+            for (int e = 0; e < CW; ++e) o.e[e] = ja_from_float<T>(ja_to_float(raw[k].e[e]) * rstd * ja_to_float(gv.e[e]));
+        } else {
+#pragma unroll
+            for (int e = 0; e < CW; ++e) o.e[e] = ja_from_float<T>(__expf(ja_to_float(raw[k].e[e]) - m) * inv_l);
+        }
+        char* dst = a.y.base + off[k];
+        if (mask[k] == (1u << CW) - 1u) {
+            *reinterpret_cast<uint4*>(dst) = o.v;
+        } else {
+#pragma unroll
+            for (int e = 0; e < CW; ++e)
+                if (mask[k] >> e & 1) reinterpret_cast<T*>(dst)[e] = o.e[e];
+        }
+    }
+}
+
+// false where a row has more words than a CTA holds in registers (the streaming form of row_kernel takes it)
+template <typename T, int OP>
+bool launch_row_words(const RowArgs& a, int64_t n_rows, cudaStream_t st) {
+    constexpr int CW = 16 / (int)sizeof(T);
+    const int runs = a.x.nblk[a.x.rank - 1];
+    const int64_t words = (a.widest + 2 * CW - 2) / CW, all = words * runs;    // a run of `widest` cells touches at most that many words
+    if (all > 256 * 16) return false;
+    // few words a thread (their loads are what is in flight), but no smaller teams than a warp
+    int team = 32;
+    while (team < 256 && all > (int64_t)team * 2) team *= 2;
+    const int vpt = (int)((all + team - 1) / team);
+    const unsigned grid = (unsigned)((n_rows + 256 / team - 1) / (256 / team));
+    if (vpt <= 1) row_word_kernel<T, 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    else if (vpt <= 2) row_word_kernel<T, 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    else if (vpt <= 4) row_word_kernel<T, 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    else if (vpt <= 8) row_word_kernel<T, 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    else row_word_kernel<T, 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    return true;
+}
+template <typename T>
+bool launch_row_words_op(RowOp op, const RowArgs& a, int64_t n_rows, cudaStream_t st) {
+    switch (op) {
+        case ROW_SUMSQ: return launch_row_words<T, ROW_SUMSQ>(a, n_rows, st);
+        case ROW_MAX: return launch_row_words<T, ROW_MAX>(a, n_rows, st);
+        case ROW_EXPSUM: return launch_row_words<T, ROW_EXPSUM>(a, n_rows, st);
+        case ROW_RMS_SCALE: return launch_row_words<T, ROW_RMS_SCALE>(a, n_rows, st);
+        case ROW_EXP_SUB_DIV: return launch_row_words<T, ROW_EXP_SUB_DIV>(a, n_rows, st);
+        case ROW_RMSNORM: return launch_row_words<T, ROW_RMSNORM>(a, n_rows, st);
+        case ROW_SOFTMAX: return launch_row_words<T, ROW_SOFTMAX>(a, n_rows, st);
+        case ROW_ROPE: return false;
+    }
+    return false;
+}
+
+// what the word form does not take: aligned rows in irregular blocks, rotations (a pair never straddles two vectors), and rows too long
 template <typename T, int VEC, int OP>
 ja_status_t launch_row_t(const RowArgs& a, int64_t n_rows, int64_t n, cudaStream_t st) {
     // team: the smallest power of two (32..256) that keeps at most 4 vectors per thread (few registers, many
@@ -516,11 +689,12 @@ ja_status_t launch_row_t(const RowArgs& a, int64_t n_rows, int64_t n, cudaStream
     int64_t vpt = (n + (int64_t)team * VEC - 1) / ((int64_t)team * VEC);
     const int rpc = 256 / team;
     unsigned grid = (unsigned)((n_rows + rpc - 1) / rpc);
-    if (vpt <= 1) row_kernel<T, VEC, 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 2) row_kernel<T, VEC, 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 4) row_kernel<T, VEC, 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 8) row_kernel<T, VEC, 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 16 && VEC > 1) row_kernel<T, VEC, 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    if (VEC == 1) row_kernel<T, VEC, 0, OP><<<grid, 256, 0, st>>>(a, n_rows, team);   // longer than the word form holds
+    else if (vpt <= 1) row_kernel<T, VEC, VEC == 1 ? 0 : 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 2) row_kernel<T, VEC, VEC == 1 ? 0 : 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 4) row_kernel<T, VEC, VEC == 1 ? 0 : 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 8) row_kernel<T, VEC, VEC == 1 ? 0 : 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 16 && VEC > 1) row_kernel<T, VEC, VEC == 1 ? 0 : 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
     else row_kernel<T, VEC, 0, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
@@ -531,7 +705,7 @@ template <typename T, int OP>
 ja_status_t launch_row_vec(const RowArgs& a, int vec, int64_t n_rows, int64_t n, cudaStream_t st) {
     constexpr int FULL = 16 / (int)sizeof(T);
     if (vec == FULL) return launch_row_t<T, FULL, OP>(a, n_rows, n, st);
-    if (vec == 2) return launch_row_t<T, 2, OP>(a, n_rows, n, st);
+    if (OP == ROW_ROPE) return launch_row_t<T, 2, OP>(a, n_rows, n, st);
     return launch_row_t<T, 1, OP>(a, n_rows, n, st);
 }
 
@@ -583,10 +757,17 @@ ja_status_t launch_row_typed(RowOp op, const RowArgs& a, cudaStream_t st) {
             return JA_OK;
         }
     }
-    // ---- generic path: any tiling, key tables read on the device ----------------------------------------------
+    // ---- any tiling, key tables read on the device ----------------------------------------------------------------
     int vec = 1;
     if (a.x.bs[last] != 0 && a.x.bs[last] % full == 0 && n % full == 0) vec = full;
     else if (op == ROW_ROPE) vec = 2;
+    // rows that are whole words anyway are better off with row_kernel's fewer, fuller threads (32 x 59 x 1792 f32: three calls 28 us, 36
+    // as masked words)
+    if (vec == 1 && launch_row_words_op<T>(op, a, n_rows, st)) {
+        ja_count_launch();
+        JA_CUDA(cudaGetLastError());
+        return JA_OK;
+    }
     return launch_row_op<T>(op, a, vec, n_rows, n, st);
 }
 
