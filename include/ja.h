@@ -320,6 +320,9 @@ ja_status_t ja_debug_wait_timeout(void* cuda_stream, int32_t* waiters_ok);
  * the time-out, clock at return. */
 ja_status_t ja_debug_bounded_wait_host(int64_t ready_at_poll, int64_t ns_per_poll, int64_t cap_ns, int64_t abort_at_poll,
                                        int64_t* polls, int32_t* succeeded, int32_t* recorded_timeout, int64_t* elapsed_ns);
+/* The tensor-memory attention kernels' addressing on the HOST (no CUDA call): *fits = whether they take a [b, s, h, d] relation of
+ * this tiling, and then cells[(b * S + s) * H + h] = the position of row (b, s, h, :) in the payload, in rows of extent(d) cells. */
+ja_status_t ja_debug_attention_rows(const ja_relation_t* rel, int32_t* fits, int64_t* cells);
 
 /* Number of kernels this library has launched since load (for launch accounting by callers). */
 int64_t ja_launch_count(void);

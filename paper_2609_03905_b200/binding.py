@@ -77,6 +77,7 @@ def _load() -> ctypes.CDLL:
         "ja_debug_set": [ctypes.c_char_p, i64],
         "ja_debug_wait_timeout": [vp, vp],
         "ja_debug_bounded_wait_host": [i64, i64, i64, i64, P(i64), P(i32), P(i32), P(i64)],
+        "ja_debug_attention_rows": [vp, P(i32), vp],
     }
     for name, argtypes in sigs.items():
         fn = getattr(lib, name)
@@ -344,3 +345,10 @@ def ja_debug_bounded_wait_host(ready_at_poll: int, ns_per_poll: int, cap_ns: int
     _check(LIB.ja_debug_bounded_wait_host(ready_at_poll, ns_per_poll, cap_ns, abort_at_poll, ctypes.byref(polls), ctypes.byref(ok),
                                           ctypes.byref(rec), ctypes.byref(ns)))
     return polls.value, bool(ok.value), bool(rec.value), ns.value
+
+
+def ja_debug_attention_rows(rel: int, extents):
+    """Where the tensor-memory attention kernels look for row (b, s, h, :) of a relation, in rows; None where they do not take it."""
+    cells, fits = np.empty(tuple(int(e) for e in extents[:3]), dtype=np.int64), ctypes.c_int32()
+    _check(LIB.ja_debug_attention_rows(ctypes.c_void_p(rel), ctypes.byref(fits), cells.ctypes.data_as(ctypes.c_void_p)))
+    return cells if fits.value else None

@@ -902,6 +902,16 @@ static bool bshd_rows_layout(const ja_relation* r) {
     return true;
 }
 
+// The tensor-memory attention kernels' addressing on the host (no CUDA call): *fits = whether they take a relation of this tiling;
+// where they do, cells[(b * S + s) * H + h] = the position of row (b, s, h, :) in its payload, in rows of extent(d) cells.
+extern "C" ja_status_t ja_debug_attention_rows(const ja_relation_t* rel, int32_t* fits, int64_t* cells) {
+    if (!rel || !fits || !cells) return ja_fail(JA_ERR_INVALID_ARG, "relation / fits / cells is NULL");
+    if (rel->rank != 4) return ja_fail(JA_ERR_SHAPE, "a [b, s, h, d] relation is expected");
+    const std::vector<int32_t> split(rel->splits[1].begin(), rel->splits[1].end());
+    *fits = bshd_rows_layout(rel) && ja_attention_tc_rows(ja_view(rel), split.data(), cells);
+    return JA_OK;
+}
+
 static ja_status_t check_tiling(const ja_spec* s, int operand, const ja_relation* r) {
     const std::string& term = spec_term(s, operand);
     if (!r) return ja_fail(JA_ERR_INVALID_ARG, "relation for operand %d is NULL", operand);

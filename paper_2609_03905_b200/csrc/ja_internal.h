@@ -220,6 +220,8 @@ struct AttnArgs {
 ja_status_t ja_launch_attention(const AttnArgs& a, cudaStream_t st);
 // tcgen05 / TMEM form; *launched stays false when the tiling does not fit it
 ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* launched);
+// where its row arithmetic puts every (b, s, h) of a relation (host; tests compare it with the key table)
+bool ja_attention_tc_rows(const RelView& v, const int32_t* host_split, int64_t* cells);
 // the online-softmax aggregation of m partial attention results (O_c, lse_c) into (O, lse); l may be nullptr
 ja_status_t ja_launch_attention_combine(const ja_relation* const* op, const ja_relation* const* lp, int m, const ja_relation* o,
                                         const ja_relation* l, cudaStream_t st);

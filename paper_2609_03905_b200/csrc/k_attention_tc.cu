@@ -49,7 +49,7 @@ constexpr int MAX_ORDER = 512;   // query tiles (pairs) whose launch order is he
 // Tiling of one "bshd" relation: uniform blocks along b and h, any split of s, d unsplit.
 struct SeqGeom {
     int32_t bblk, hblk, nhb;     // batch rows per block, heads per block, blocks along h
-    int32_t sblk;                // uniform rows per s block, or 0: split[] holds the nsb + 1 split points
+    int32_t sblk;                // rows per s block (the last one may hold fewer), or 0: split[] holds the nsb + 1 split points
     int32_t nsb;
     int32_t split[MAX_SB + 1];
 };
@@ -75,11 +75,11 @@ struct AttnTcParams {
 // Row coordinate of cell (b, s, h, :) in the rank-3 view (d, head in block, row). Block (bb, sb, hb) starts
 // 128 * hblk * [ (bb*bblk*S + bblk*start(sb)) * nhb + hb*bblk*rows(sb) ] elements into the payload (blocks are stored
 // in key order, each dense), and inside it the row is (b in block) * rows(sb) + (s - start(sb)).
-__device__ __forceinline__ int seq_row(const SeqGeom& g, int S, int b, int s, int h) {
+__host__ __device__ __forceinline__ int seq_row(const SeqGeom& g, int S, int b, int s, int h) {
     int start, rows;
     if (g.sblk) {
         start = (s / g.sblk) * g.sblk;
-        rows = g.sblk;
+        rows = S - start < g.sblk ? S - start : g.sblk;   // the last of equal blocks may be shorter
     } else {
         int sb = 0, hi = g.nsb - 1;
         while (sb < hi) {
@@ -1088,6 +1088,17 @@ bool fill_geom(const RelView& v, const int32_t* host_split, SeqGeom* g) {
 
 }  // namespace
 
+// The kernels' row arithmetic on the host, for every (b, s, h) of a "bshd" relation: cells[(b * S + s) * H + h] = the position of
+// cell (b, s, h, 0) in the payload, in runs of D cells. False where the relation's geometry does not fit the kernels' parameters.
+bool ja_attention_tc_rows(const RelView& v, const int32_t* host_split, int64_t* cells) {
+    SeqGeom g;
+    if (!fill_geom(v, host_split, &g)) return false;
+    const int B = (int)v.extent[0], S = (int)v.extent[1], H = (int)v.extent[2];
+    for (int b = 0; b < B; ++b)
+        for (int s = 0; s < S; ++s)
+            for (int h = 0; h < H; ++h) *cells++ = (int64_t)seq_row(g, S, b, s, h) * g.hblk + h % g.hblk;
+    return true;
+}
 
 // After a device-side failure (a bounded wait that expired) a persistent launch may have left its work counter non-zero:
 // put every counter pair of the current device back to zero. Called by ja_stream_status when it reports such a failure;

@@ -73,6 +73,17 @@ def test_packed_sequences(ends, causal, lse):
     _run(2, S, 8, 4, [0] + ends, [0] + ends, ends, causal, BF, lse=lse)
 
 
+# equal blocks with a shorter last one, several head blocks: the rows of a head block after the first start where the SHORT block
+# says (download() looks at the guard zones)
+@pytest.mark.parametrize("split,packed", [([0, 128, 256, 300], False), ([0, 300, 500], True), ([0, 777, 1291], True), ([0, 602, 668], True),
+                                          ([0, 256, 384], False), ([0, 512, 768], False), ([0, 256, 384], True)])
+@pytest.mark.parametrize("causal,lse", [(True, False), (False, True)])
+@pytest.mark.parametrize("dtype,b_blocks", [(BF, 2), (F16, 1)])
+def test_shorter_last_block(split, packed, causal, lse, dtype, b_blocks):
+    S = split[-1]
+    _run(2, S, 8, 4, split, split, split[1:] if packed else [], causal, dtype, lse=lse, b_blocks=b_blocks)
+
+
 def test_queries_and_keys_cut_differently():
     S = 600
     _run(1, S, 4, 2, [0, 130, 391, 600], ES(S, 3), [], True, BF)

@@ -331,3 +331,66 @@ def test_greedy_selector_against_the_oracle_and_the_optimizer():
     for op, J in zip(ops, plan):
         free = [None] * len(op["inputs"])
         assert optimizer.cost(op, J, free) == min(optimizer.cost(op, K, free) for K in optimizer.specs(op, 4))
+
+
+# ---------------------------------------------------------------------------------------------------
+# the tensor-memory attention kernels' row arithmetic against the key table (run before any GPU case: a wrong row is a wild store)
+# ---------------------------------------------------------------------------------------------------
+def _rows_by_key_table(extents, splits, rel):
+    """Position of every row (b, s, h, :) in the payload, in rows, from the relation's block offsets."""
+    coords, lower, upper, offs = ja.ja_relation_get_keys(rel)
+    want = np.full(extents[:3], -1, dtype=np.int64)
+    for lo, hi, off in zip(lower, upper, offs):
+        n = [int(h) - int(l) for l, h in zip(lo, hi)]
+        block = off // (extents[3] * 2) + np.arange(n[0] * n[1] * n[2]).reshape(n[:3])
+        want[tuple(slice(int(l), int(h)) for l, h in zip(lo[:3], hi[:3]))] = block
+    assert (want >= 0).all()
+    return want
+
+
+ROW_TILINGS = [   # (B, S, H), splits of b, s, h
+    ((1, 300, 2), [0, 1], [0, 128, 256, 300], [0, 1, 2]),          # equal sequence blocks with a shorter last one, one head per block
+    ((2, 500, 4), [0, 1, 2], [0, 300, 500], [0, 1, 2, 3, 4]),      # two packed sequences, the longer one first
+    ((2, 300, 2), [0, 2], [0, 128, 256, 300], [0, 2]),             # both batch rows in one block
+    ((1, 384, 2), [0, 1], [0, 256, 384], [0, 1, 2]),               # whole 128-row tiles
+    ((2, 668, 8), [0, 1, 2], [0, 602, 668], list(range(9))),
+    ((3, 130, 4), [0, 2, 3], [0, 130], [0, 4]),                    # a shorter last batch block
+    ((3, 130, 4), [0, 2, 3], [0, 65, 130], [0, 2, 4]),
+    ((2, 700, 2), [0, 1, 2], list(range(0, 700, 9)) + [700], [0, 1, 2]),   # more equal blocks than an irregular split may have
+]
+
+
+@pytest.mark.parametrize("case", range(len(ROW_TILINGS)))
+def test_attention_rows_match_the_key_table(case):
+    (B, S, H), b, s, h = ROW_TILINGS[case]
+    rel = _rel([B, S, H, 128], [b, s, h, [0, 128]])
+    got = ja.ja_debug_attention_rows(rel, (B, S, H))
+    if got is not None:
+        assert np.array_equal(got, _rows_by_key_table([B, S, H, 128], [b, s, h], rel))
+    if len(set(np.diff(h))) == 1 and len(set(np.diff(b))) == 1:   # equal batch and head blocks: taken under any split of the sequence
+        assert got is not None
+    ja.ja_relation_destroy(rel)
+
+
+def test_attention_rows_match_the_key_table_on_random_tilings():
+    taken = 0
+    for _ in range(300):
+        B, S, H = int(RNG.integers(1, 5)), int(RNG.integers(2, 90)), int(RNG.integers(1, 7))
+
+        def cut(e):
+            kind = RNG.integers(0, 3)
+            if kind == 0:                                            # equal blocks, the last one perhaps shorter
+                n = int(RNG.integers(1, e + 1))
+                return sorted(set(range(0, e, n)) | {e})
+            if kind == 1:
+                return [0, e]
+            return [0] + sorted(set(RNG.integers(1, e, int(RNG.integers(0, 4))).tolist()) if e > 1 else []) + [e]
+
+        b, s, h = cut(B), cut(S), list(range(H + 1)) if RNG.integers(0, 2) else [0, H]
+        rel = _rel([B, S, H, 128], [b, s, h, [0, 128]])
+        got = ja.ja_debug_attention_rows(rel, (B, S, H))
+        if got is not None:
+            taken += 1
+            assert np.array_equal(got, _rows_by_key_table([B, S, H, 128], [b, s, h], rel)), (b, s, h)
+        ja.ja_relation_destroy(rel)
+    assert taken > 60
