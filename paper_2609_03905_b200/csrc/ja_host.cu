@@ -884,11 +884,12 @@ struct ExecPlan {
     }
 };
 
-// True when a "bshd" relation has uniform blocks along b and h, an unsplit d, and every block starts where the closed
+// True when a "bshd" relation has uniform blocks along b, equal ones along h (a shorter last one would have shorter rows), an
+// unsplit d, and every block starts where the closed
 // form used by the tensor-memory attention kernel puts it: blocks in key order, each a dense run of rows of
 // hblk * extent(d) cells, so block (bb, sb, hb) starts (bb*bblk*S + bblk*start(sb)) * nhb + hb*bblk*rows(sb) rows in.
 static bool bshd_rows_layout(const ja_relation* r) {
-    if (r->rank != 4 || !r->bs[0] || !r->bs[2] || r->nblk[3] != 1) return false;
+    if (r->rank != 4 || !r->bs[0] || !r->bs[2] || r->extent[2] % r->bs[2] || r->nblk[3] != 1) return false;
     const int64_t S = r->extent[1], bblk = r->bs[0], hblk = r->bs[2], nhb = r->nblk[2];
     const int64_t row_bytes = hblk * r->extent[3] * r->esize;
     if (r->extent[0] * S * nhb >= ((int64_t)1 << 31)) return false;

@@ -19,10 +19,10 @@ ES = blocked.equal_splits
 BF, F32, F16 = torch.bfloat16, torch.float32, torch.float16
 
 
-def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_blocks=None):
+def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_blocks=None, g_split=None):
     grp = Hq // Hkv
     Q, K, V = (si.normal((B, S, h, 128), 0.0, 1.0, dtype, 4, 60 + n) for n, h in enumerate((Hq, Hkv, Hkv)))
-    b_sp, g_sp = ES(B, b_blocks or B), ES(Hkv, max(1, Hkv // 2))
+    b_sp, g_sp = ES(B, b_blocks or B), g_split or ES(Hkv, max(1, Hkv // 2))
     h_sp = [grp * v for v in g_sp]
     d = [0, 128]
     rq, rk, rv = upload(Q, [b_sp, q_split, h_sp, d]), upload(K, [b_sp, k_split, g_sp, d]), upload(V, [b_sp, k_split, g_sp, d])
@@ -82,6 +82,13 @@ def test_packed_sequences(ends, causal, lse):
 def test_shorter_last_block(split, packed, causal, lse, dtype, b_blocks):
     S = split[-1]
     _run(2, S, 8, 4, split, split, split[1:] if packed else [], causal, dtype, lse=lse, b_blocks=b_blocks)
+
+
+# a shorter last head block: its rows are shorter, so the kernels that hold rows of one length leave it to the mma.sync form
+@pytest.mark.parametrize("S", [300, 256])
+def test_shorter_last_head_block(S):
+    _run(1, S, 3, 3, [0, S], [0, S], [], True, BF, lse=True, g_split=[0, 2, 3])
+    _run(1, S, 6, 3, [0, S], [0, S], [], False, F16, g_split=[0, 2, 3])
 
 
 def test_queries_and_keys_cut_differently():

@@ -352,6 +352,8 @@ ROW_TILINGS = [   # (B, S, H), splits of b, s, h
     ((1, 300, 2), [0, 1], [0, 128, 256, 300], [0, 1, 2]),          # equal sequence blocks with a shorter last one, one head per block
     ((2, 500, 4), [0, 1, 2], [0, 300, 500], [0, 1, 2, 3, 4]),      # two packed sequences, the longer one first
     ((2, 300, 2), [0, 2], [0, 128, 256, 300], [0, 2]),             # both batch rows in one block
+    ((1, 300, 3), [0, 1], [0, 300], [0, 2, 3]),                    # a shorter last head block
+    ((1, 256, 3), [0, 1], [0, 256], [0, 2, 3]),
     ((1, 384, 2), [0, 1], [0, 256, 384], [0, 1, 2]),               # whole 128-row tiles
     ((2, 668, 8), [0, 1, 2], [0, 602, 668], list(range(9))),
     ((3, 130, 4), [0, 2, 3], [0, 130], [0, 4]),                    # a shorter last batch block
@@ -386,7 +388,7 @@ def test_attention_rows_match_the_key_table_on_random_tilings():
                 return [0, e]
             return [0] + sorted(set(RNG.integers(1, e, int(RNG.integers(0, 4))).tolist()) if e > 1 else []) + [e]
 
-        b, s, h = cut(B), cut(S), list(range(H + 1)) if RNG.integers(0, 2) else [0, H]
+        b, s, h = cut(B), cut(S), cut(H)
         rel = _rel([B, S, H, 128], [b, s, h, [0, 128]])
         got = ja.ja_debug_attention_rows(rel, (B, S, H))
         if got is not None:
