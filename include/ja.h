@@ -323,6 +323,9 @@ ja_status_t ja_debug_bounded_wait_host(int64_t ready_at_poll, int64_t ns_per_pol
 /* The tensor-memory attention kernels' addressing on the HOST (no CUDA call): *fits = whether they take a [b, s, h, d] relation of
  * this tiling, and then cells[(b * S + s) * H + h] = the position of row (b, s, h, :) in the payload, in rows of extent(d) cells. */
 ja_status_t ja_debug_attention_rows(const ja_relation_t* rel, int32_t* fits, int64_t* cells);
+/* The general join-agg's addressing on the HOST (no CUDA call): the byte offset in the payload at which its walk along dimension
+ * `moving` (-1: none moves) finds the cell with coordinates coord[0..rank). */
+ja_status_t ja_debug_cell_offset(const ja_relation_t* rel, int32_t moving, const int64_t* coord, int64_t* offset);
 
 /* Number of kernels this library has launched since load (for launch accounting by callers). */
 int64_t ja_launch_count(void);

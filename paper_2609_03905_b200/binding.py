@@ -78,6 +78,7 @@ def _load() -> ctypes.CDLL:
         "ja_debug_wait_timeout": [vp, vp],
         "ja_debug_bounded_wait_host": [i64, i64, i64, i64, P(i64), P(i32), P(i32), P(i64)],
         "ja_debug_attention_rows": [vp, P(i32), vp],
+        "ja_debug_cell_offset": [vp, i32, P(i64), P(i64)],
     }
     for name, argtypes in sigs.items():
         fn = getattr(lib, name)
@@ -352,3 +353,10 @@ def ja_debug_attention_rows(rel: int, extents):
     cells, fits = np.empty(tuple(int(e) for e in extents[:3]), dtype=np.int64), ctypes.c_int32()
     _check(LIB.ja_debug_attention_rows(ctypes.c_void_p(rel), ctypes.byref(fits), cells.ctypes.data_as(ctypes.c_void_p)))
     return cells if fits.value else None
+
+
+def ja_debug_cell_offset(rel: int, moving: int, coord) -> int:
+    """Byte offset at which the general join-agg's walk along dimension `moving` (-1: none) finds a cell."""
+    off = ctypes.c_int64()
+    _check(LIB.ja_debug_cell_offset(ctypes.c_void_p(rel), int(moving), (ctypes.c_int64 * len(coord))(*[int(x) for x in coord]), ctypes.byref(off)))
+    return off.value

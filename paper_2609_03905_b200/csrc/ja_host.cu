@@ -932,6 +932,16 @@ static ja_status_t check_tiling(const ja_spec* s, int operand, const ja_relation
     return JA_OK;
 }
 
+// The general join-agg's addressing on the host (no CUDA call)
+extern "C" ja_status_t ja_debug_cell_offset(const ja_relation_t* rel, int32_t moving, const int64_t* coord, int64_t* offset) {
+    if (!rel || !coord || !offset) return ja_fail(JA_ERR_INVALID_ARG, "relation / coord / offset is NULL");
+    if (moving < -1 || moving >= rel->rank) return ja_fail(JA_ERR_INVALID_ARG, "dimension %d out of range", moving);
+    for (int d = 0; d < rel->rank; ++d)
+        if (coord[d] < 0 || coord[d] >= rel->extent[d]) return ja_fail(JA_ERR_INVALID_ARG, "coordinate %d out of range", d);
+    *offset = ja_generic_cell_offset(rel, moving, coord);
+    return JA_OK;
+}
+
 // "Rj" style helpers: lead = all letters but the last
 static std::string lead_of(const std::string& t) { return t.substr(0, t.size() - 1); }
 

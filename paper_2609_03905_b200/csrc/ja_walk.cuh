@@ -37,10 +37,17 @@ struct Rel {
 struct Cursor {
     int blk, lo, hi;
 };
-__device__ __forceinline__ Cursor seek(const Dim& d, int x) {
+__host__ __device__ __forceinline__ uint32_t mul_hi(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)((uint64_t)a * b >> 32);
+#endif
+}
+__host__ __device__ __forceinline__ Cursor seek(const Dim& d, int x) {
     Cursor c;
     if (d.bs) {
-        c.blk = d.bs > 1 ? (int)(__umulhi((uint32_t)x, d.magic) >> d.shift) : x;
+        c.blk = d.bs > 1 ? (int)(mul_hi((uint32_t)x, d.magic) >> d.shift) : x;
         c.lo = c.blk * d.bs;
         c.hi = min(c.lo + d.bs, d.extent);
     } else {

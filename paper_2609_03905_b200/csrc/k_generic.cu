@@ -52,11 +52,11 @@ __device__ __forceinline__ float load_cell(const char* p, int dtype) {
 // One operand along the moving index with every other coordinate fixed: inside the interval [lo, hi) of x a cell lies
 // at + x * step bytes into the payload.
 struct Line {
-    int64_t at;
-    int64_t a, b;     // cells: ((a * w + x - lo) * post + b)
-    int post, flat, hi, step;
+    int64_t at, step;      // 64 bits: a block may hold 2^31 bytes and more after the moving index
+    int64_t a, b, post;    // cells: ((a * w + x - lo) * post + b)
+    int flat, hi;
 };
-__device__ __forceinline__ Line line_of(const Operand& o, const int* coord) {
+__host__ __device__ __forceinline__ Line line_of(const Operand& o, const int* coord) {
     Line l;
     l.a = l.b = 0;
     l.post = 1;
@@ -84,7 +84,7 @@ __device__ __forceinline__ Line line_of(const Operand& o, const int* coord) {
     }
     return l;
 }
-__device__ __forceinline__ void enter(const Operand& o, Line& l, int x) {   // the interval of x
+__host__ __device__ __forceinline__ void enter(const Operand& o, Line& l, int x) {   // the interval of x
     const Dim& d = o.dim[o.x];
     const Cursor c = seek(d, x);
     l.hi = c.hi;
@@ -179,11 +179,20 @@ __global__ void __launch_bounds__(WARPS * 32) generic_join_agg_kernel(const __gr
                         if (x >= l[k].hi) enter(p.in[k], l[k], x);
                         end = min(end, l[k].hi);
                     }
+                const char* cell_at[N];
+                int64_t ahead[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    cell_at[k] = p.in[k].base + (l[k].at + x * l[k].step);
+                    ahead[k] = x_step * l[k].step;
+                }
 #pragma unroll 4
                 for (; x < end; x += x_step) {
 #pragma unroll
-                    for (int k = 0; k < N; ++k)
-                        if (p.in[k].x >= 0) v[k] = load_cell(p.in[k].base + (l[k].at + (int64_t)x * l[k].step), p.in[k].dtype);
+                    for (int k = 0; k < N; ++k) {
+                        if (p.in[k].x >= 0) v[k] = load_cell(cell_at[k], p.in[k].dtype);
+                        cell_at[k] += ahead[k];
+                    }
                     acc = merged(p.agg, acc, joined<N>(p.fn, v));
                 }
             }
@@ -306,8 +315,36 @@ __global__ void __launch_bounds__(256) generic_join_agg_wide_kernel(const WidePa
     }
 }
 
+// One operand: `term` names its indices, `coords` the coordinate vector, xl the moving index (0: none)
+void fill_operand(Operand* o, const ja_relation* r, const RelView& v, const std::string& term, const std::string& coords, char xl) {
+    o->base = (char*)r->base;
+    o->blk_off = v.blk_off;
+    o->rank = r->rank;
+    o->dtype = (int)r->dtype;
+    o->x = -1;
+    for (int d = 0; d < r->rank; ++d) {
+        set_dim(&o->dim[d], r, v, term, term[d]);
+        o->coord[d] = (int)coords.find(term[d]);
+        if (term[d] == xl) o->x = d;
+    }
+}
 
 }  // namespace
+
+int64_t ja_generic_cell_offset(const ja_relation* r, int moving, const int64_t* coord) {
+    RelView v = ja_view(r);                     // the key table as it lies on the host
+    for (int d = 0; d < r->rank; ++d) v.splits[d] = r->splits[d].data();
+    v.blk_off = r->blk_off.data();
+    const std::string term = std::string("abcd").substr(0, r->rank);
+    Operand o;
+    fill_operand(&o, r, v, term, term, moving < 0 ? 0 : term[moving]);
+    int x[MAX_COORDS] = {};
+    for (int d = 0; d < r->rank; ++d) x[d] = (int)coord[d];
+    Line l = line_of(o, x);
+    if (moving < 0) return l.at;
+    enter(o, l, x[moving]);
+    return l.at + x[moving] * l.step;
+}
 
 // *launched stays false when the spec is outside this kernel's reach (more than four operands or summed indices, an
 // operator that is not a scalar function of the joined cells, NONE aggregation with summed indices).
@@ -371,21 +408,8 @@ ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inp
         return JA_OK;
     }
     p.x_ext = xl ? (int32_t)extent_of(xl) : 1;
-    auto fill = [&](Operand* o, const ja_relation* r, const std::string& term) {
-        const RelView v = ja_view(r);
-        o->base = (char*)r->base;
-        o->blk_off = v.blk_off;
-        o->rank = r->rank;
-        o->dtype = (int)r->dtype;
-        o->x = -1;
-        for (int d = 0; d < r->rank; ++d) {
-            set_dim(&o->dim[d], r, v, term, term[d]);
-            o->coord[d] = (int)coords.find(term[d]);
-            if (term[d] == xl) o->x = d;
-        }
-    };
-    for (int k = 0; k < n_in; ++k) fill(&p.in[k], inputs[k], spec->ins[k]);
-    fill(&p.out, out, spec->out);
+    for (int k = 0; k < n_in; ++k) fill_operand(&p.in[k], inputs[k], ja_view(inputs[k]), spec->ins[k], coords, xl);
+    fill_operand(&p.out, out, ja_view(out), spec->out, coords, xl);
     p.fn = (int)spec->fn;
     p.agg = (int)spec->agg;
     // Who shares a cell's tuples: warps first, then CTAs, until the chip has two CTAs an SM or a share is down to a few steps (a

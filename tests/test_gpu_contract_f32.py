@@ -94,3 +94,14 @@ def test_maximum_keeps_infinities():
     ja.Spec("ij->j", cuts, "ident", (), "max").execute([r], out)
     assert np.array_equal(download(out), x.max(0).values.double().numpy())
     check_status()
+
+
+def test_a_block_of_more_than_2_to_31_bytes_after_the_summed_index():
+    """Two slices of 2 GiB in one block: the step from a cell to the next one of the sum does not fit 32 bits. a + b is one rounding."""
+    n = 16384 * 32768
+    cuts = {"k": [0, 2], "i": [0, 16384], "j": [0, 32768]}
+    x = ja.Relation([2, 16384, 32768], [cuts[c] for c in "kij"], F32, torch.randn(2 * n, device="cuda"))
+    out = ja.Relation([16384, 32768], [cuts[c] for c in "ij"], F32, torch.full((n,), float("nan"), device="cuda"))
+    ja.Spec("kij->ij", cuts, "ident", (), "sum").execute([x], out)
+    assert torch.equal(out.payload, x.payload[:n] + x.payload[n:])
+    check_status()

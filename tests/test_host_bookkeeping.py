@@ -396,3 +396,26 @@ def test_attention_rows_match_the_key_table_on_random_tilings():
             assert np.array_equal(got, _rows_by_key_table([B, S, H, 128], [b, s, h], rel)), (b, s, h)
         ja.ja_relation_destroy(rel)
     assert taken > 60
+
+
+# ---------------------------------------------------------------------------------------------------
+# the general join-agg's addressing where a block holds 2^31 bytes and more
+# ---------------------------------------------------------------------------------------------------
+@pytest.mark.parametrize("extents,splits,dtype", [
+    ([2, 32768, 16384], [[0, 2], [0, 32768], [0, 16384]], ja.JA_F32),          # 2^29 f32 cells after the first index: a step of 2^31 bytes
+    ([3, 32768, 32768], [[0, 1, 3], [0, 32768], [0, 32768]], ja.JA_BF16),
+    ([5, 7, 1 << 29], [[0, 3, 5], [0, 7], [0, 1 << 28, 1 << 29]], ja.JA_F32),
+    ([40, 30, 20, 10], [[0, 40], [0, 13, 30], [0, 8, 16, 20], [0, 10]], ja.JA_BF16),
+])
+def test_general_join_agg_offsets(extents, splits, dtype):
+    rel, es = _rel(extents, splits, dtype), 4 if dtype == ja.JA_F32 else 2
+    _, lower, upper, offs = ja.ja_relation_get_keys(rel)
+    cells = [[0] * len(extents), [e - 1 for e in extents]] + [[int(RNG.integers(0, e)) for e in extents] for _ in range(60)]
+    for x in cells:
+        block = next(i for i, (lo, hi) in enumerate(zip(lower, upper)) if all(l <= c < h for l, c, h in zip(lo, x, hi)))
+        at = 0
+        for l, c, h in zip(lower[block], x, upper[block]):
+            at = at * (int(h) - int(l)) + c - int(l)
+        for moving in range(-1, len(extents)):
+            assert ja.ja_debug_cell_offset(rel, moving, x) == int(offs[block]) + at * es
+    ja.ja_relation_destroy(rel)
