@@ -326,6 +326,8 @@ ja_status_t ja_debug_attention_rows(const ja_relation_t* rel, int32_t* fits, int
 /* The general join-agg's addressing on the HOST (no CUDA call): the byte offset in the payload at which its walk along dimension
  * `moving` (-1: none moves) finds the cell with coordinates coord[0..rank). */
 ja_status_t ja_debug_cell_offset(const ja_relation_t* rel, int32_t moving, const int64_t* coord, int64_t* offset);
+/* Which form of the general join-agg a spec would run on (no CUDA call): 0 none, 1 32-bit coordinates and counts, 2 64-bit ones. */
+ja_status_t ja_debug_general_form(const ja_spec_t* spec, int32_t* form);
 
 /* Number of kernels this library has launched since load (for launch accounting by callers). */
 int64_t ja_launch_count(void);

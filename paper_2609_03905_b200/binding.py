@@ -79,6 +79,7 @@ def _load() -> ctypes.CDLL:
         "ja_debug_bounded_wait_host": [i64, i64, i64, i64, P(i64), P(i32), P(i32), P(i64)],
         "ja_debug_attention_rows": [vp, P(i32), vp],
         "ja_debug_cell_offset": [vp, i32, P(i64), P(i64)],
+        "ja_debug_general_form": [vp, P(i32)],
     }
     for name, argtypes in sigs.items():
         fn = getattr(lib, name)
@@ -360,3 +361,10 @@ def ja_debug_cell_offset(rel: int, moving: int, coord) -> int:
     off = ctypes.c_int64()
     _check(LIB.ja_debug_cell_offset(ctypes.c_void_p(rel), int(moving), (ctypes.c_int64 * len(coord))(*[int(x) for x in coord]), ctypes.byref(off)))
     return off.value
+
+
+def ja_debug_general_form(spec: int) -> int:
+    """The form of the general join-agg a spec would run on: 0 none, 1 32-bit coordinates and counts, 2 64-bit ones."""
+    form = ctypes.c_int32()
+    _check(LIB.ja_debug_general_form(ctypes.c_void_p(spec), ctypes.byref(form)))
+    return form.value

@@ -942,6 +942,12 @@ extern "C" ja_status_t ja_debug_cell_offset(const ja_relation_t* rel, int32_t mo
     return JA_OK;
 }
 
+extern "C" ja_status_t ja_debug_general_form(const ja_spec_t* spec, int32_t* form) {
+    if (!spec || !form) return ja_fail(JA_ERR_INVALID_ARG, "spec / form is NULL");
+    *form = ja_generic_form(spec);
+    return JA_OK;
+}
+
 // "Rj" style helpers: lead = all letters but the last
 static std::string lead_of(const std::string& t) { return t.substr(0, t.size() - 1); }
 

@@ -114,6 +114,7 @@ JaConfig& ja_config();
 // the definition in its relational form, cell by cell: any spec whose operator is a scalar function of the
 // joined cells (*launched stays false otherwise)
 ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inputs, const ja_relation* out, cudaStream_t st, bool* launched);
+int ja_generic_form(const ja_spec* spec);   // 0: not taken, 1: 32-bit coordinates, 2: the wide form
 // where its walk along dimension `moving` (-1: a fixed cell) finds a cell, in bytes into the payload (host; for tests)
 int64_t ja_generic_cell_offset(const ja_relation* r, int moving, const int64_t* coord);
 ja_status_t ja_launch_matmul_simt(const ja_relation* A, const ja_relation* B, const ja_relation* C, cudaStream_t st,

@@ -256,8 +256,8 @@ ja_status_t launch(const Params& p, int64_t groups, cudaStream_t st) {
     return JA_OK;
 }
 
-// Index extents, cell or tuple counts past 31 bits: one thread per output cell, every coordinate of every tuple resolved with
-// 64-bit arithmetic.
+// Index extents past 2^30, cell or tuple counts past 31 bits: one thread per output cell, every coordinate of every tuple resolved
+// with 64-bit arithmetic.
 struct WideParams {
     RelView in[MAX_OPERANDS];
     RelView out;
@@ -315,6 +315,46 @@ __global__ void __launch_bounds__(256) generic_join_agg_wide_kernel(const WidePa
     }
 }
 
+// What the kernels make of a spec: coordinates, the moving index, counts. False where the spec is outside their reach (more than four
+// operands or summed indices, an operator that is not a scalar function of the joined cells, NONE aggregation with summed indices).
+struct Shape {
+    std::string coords;          // output indices first, then the summed ones in order of first appearance
+    int n_out, n_sum, x;         // x: position of the moving index in coords, -1: nothing is summed
+    bool lanes, wide;
+    int64_t n_cells, n_tuples;   // output cells; tuples of the summed indices other than x (counted where wide is false)
+};
+bool shape_of(const ja_spec* spec, Shape* s) {
+    const int n_in = (int)spec->ins.size();
+    if (n_in < 1 || n_in > MAX_OPERANDS) return false;
+    switch (spec->fn) {
+        case JA_FN_MUL: case JA_FN_ADD: break;
+        case JA_FN_IDENT: case JA_FN_SQUARE: if (n_in != 1) return false; break;
+        case JA_FN_SILU_MUL: case JA_FN_EXP_SUB: if (n_in != 2) return false; break;
+        default: return false;
+    }
+    s->coords = spec->out;
+    for (char c : spec->letters)
+        if (s->coords.find(c) == std::string::npos) s->coords.push_back(c);
+    s->n_out = (int)spec->out.size();
+    s->n_sum = (int)s->coords.size() - s->n_out;
+    if (s->n_out < 1 || s->n_out > JA_MAX_RANK || s->n_sum > MAX_SUMMED) return false;
+    if (spec->agg != JA_AGG_SUM && spec->agg != JA_AGG_MAX && !(spec->agg == JA_AGG_NONE && s->n_sum == 0)) return false;
+    // the moving index
+    s->lanes = spec->out.find(spec->ins[0].back()) == std::string::npos;
+    const char xl = s->n_sum == 0 ? 0 : s->lanes ? spec->ins[0].back() : s->coords.back();
+    s->x = xl ? (int)s->coords.find(xl) : -1;
+    s->n_cells = s->n_tuples = 1;
+    s->wide = false;
+    for (int d = 0; d < (int)s->coords.size() && !s->wide; ++d) {
+        const int64_t e = spec->parts[spec->letters.find(s->coords[d])].back();
+        if (d < s->n_out) s->n_cells *= e;
+        else if (d != s->x) s->n_tuples *= e;
+        // 2^30: the end of an interval that starts at a coordinate, and the coordinate a walk steps to past the end, still fit an int
+        s->wide = e > (1ll << 30) || s->n_cells >= (1ll << 31) || s->n_tuples >= (1ll << 31);
+    }
+    return true;
+}
+
 // One operand: `term` names its indices, `coords` the coordinate vector, xl the moving index (0: none)
 void fill_operand(Operand* o, const ja_relation* r, const RelView& v, const std::string& term, const std::string& coords, char xl) {
     o->base = (char*)r->base;
@@ -346,48 +386,25 @@ int64_t ja_generic_cell_offset(const ja_relation* r, int moving, const int64_t* 
     return l.at + x[moving] * l.step;
 }
 
-// *launched stays false when the spec is outside this kernel's reach (more than four operands or summed indices, an
-// operator that is not a scalar function of the joined cells, NONE aggregation with summed indices).
+int ja_generic_form(const ja_spec* spec) {
+    Shape s;
+    return !shape_of(spec, &s) ? 0 : s.wide ? 2 : 1;
+}
+
+// *launched stays false when the spec is outside the kernels' reach (shape_of).
 ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inputs, const ja_relation* out, cudaStream_t st, bool* launched) {
     *launched = false;
+    Shape s;
+    if (!shape_of(spec, &s)) return JA_OK;
     const int n_in = (int)spec->ins.size();
-    if (n_in < 1 || n_in > MAX_OPERANDS) return JA_OK;
-    switch (spec->fn) {
-        case JA_FN_MUL: case JA_FN_ADD: break;
-        case JA_FN_IDENT: case JA_FN_SQUARE: if (n_in != 1) return JA_OK; break;
-        case JA_FN_SILU_MUL: case JA_FN_EXP_SUB: if (n_in != 2) return JA_OK; break;
-        default: return JA_OK;
-    }
-    Params p;
-    memset(&p, 0, sizeof p);
-    std::string coords = spec->out;             // output indices first, then the summed ones in order of first appearance
-    for (char c : spec->letters)
-        if (coords.find(c) == std::string::npos) coords.push_back(c);
-    p.n_out = (int)spec->out.size();
-    p.n_sum = (int)coords.size() - p.n_out;
-    if (p.n_out < 1 || p.n_out > JA_MAX_RANK || p.n_sum > MAX_SUMMED) return JA_OK;
-    if (spec->agg != JA_AGG_SUM && spec->agg != JA_AGG_MAX && !(spec->agg == JA_AGG_NONE && p.n_sum == 0)) return JA_OK;
+    const std::string& coords = s.coords;
     auto extent_of = [&](char c) { return spec->parts[spec->letters.find(c)].back(); };
-    // the moving index
-    const bool lanes = spec->out.find(spec->ins[0].back()) == std::string::npos;
-    const char xl = p.n_sum == 0 ? 0 : lanes ? spec->ins[0].back() : coords.back();
-    p.x = xl ? (int)coords.find(xl) : -1;
-    p.n_cells = p.n_tuples = 1;
-    bool wide = false;
-    for (size_t d = 0; d < coords.size(); ++d) {
-        const int64_t e = extent_of(coords[d]);
-        wide = wide || e >= (1ll << 31);
-        p.ext[d] = (int32_t)e;
-        if ((int)d < p.n_out) p.n_cells *= e;
-        else if ((int)d != p.x) p.n_tuples *= e;
-    }
-    wide = wide || p.n_cells >= (1ll << 31) || p.n_tuples >= (1ll << 31);
-    if (wide) {
+    if (s.wide) {
         WideParams w;
         memset(&w, 0, sizeof w);
         w.n_in = n_in;
-        w.n_out = p.n_out;
-        w.n_sum = p.n_sum;
+        w.n_out = s.n_out;
+        w.n_sum = s.n_sum;
         w.n_out_cells = w.n_sum_cells = 1;
         for (int d = 0; d < w.n_out; ++d) { w.out_ext[d] = extent_of(coords[d]); w.n_out_cells *= w.out_ext[d]; }
         for (int d = 0; d < w.n_sum; ++d) { w.sum_ext[d] = extent_of(coords[w.n_out + d]); w.n_sum_cells *= w.sum_ext[d]; }
@@ -407,6 +424,16 @@ ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inp
         *launched = true;
         return JA_OK;
     }
+    Params p;
+    memset(&p, 0, sizeof p);
+    p.n_out = s.n_out;
+    p.n_sum = s.n_sum;
+    p.x = s.x;
+    p.n_cells = s.n_cells;
+    p.n_tuples = s.n_tuples;
+    for (size_t d = 0; d < coords.size(); ++d) p.ext[d] = (int32_t)extent_of(coords[d]);
+    const bool lanes = s.lanes;
+    const char xl = s.x < 0 ? 0 : coords[s.x];
     p.x_ext = xl ? (int32_t)extent_of(xl) : 1;
     for (int k = 0; k < n_in; ++k) fill_operand(&p.in[k], inputs[k], ja_view(inputs[k]), spec->ins[k], coords, xl);
     fill_operand(&p.out, out, ja_view(out), spec->out, coords, xl);
@@ -433,10 +460,10 @@ ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inp
         while (p.cluster < 8 && groups * p.cluster < want && per_cta * p.cluster < shares && steps * p.n_tuples / (per_cta * p.cluster) >= 8) p.cluster *= 2;
         p.split_x = steps > p.n_tuples;
     }
-    ja_status_t s;
-    if (lanes && p.x >= 0) s = n_in == 1 ? launch<1, true>(p, groups, st) : n_in == 2 ? launch<2, true>(p, groups, st) : n_in == 3 ? launch<3, true>(p, groups, st) : launch<4, true>(p, groups, st);
-    else s = n_in == 1 ? launch<1, false>(p, groups, st) : n_in == 2 ? launch<2, false>(p, groups, st) : n_in == 3 ? launch<3, false>(p, groups, st) : launch<4, false>(p, groups, st);
-    if (s != JA_OK) return s;
+    ja_status_t status;
+    if (lanes && p.x >= 0) status = n_in == 1 ? launch<1, true>(p, groups, st) : n_in == 2 ? launch<2, true>(p, groups, st) : n_in == 3 ? launch<3, true>(p, groups, st) : launch<4, true>(p, groups, st);
+    else status = n_in == 1 ? launch<1, false>(p, groups, st) : n_in == 2 ? launch<2, false>(p, groups, st) : n_in == 3 ? launch<3, false>(p, groups, st) : launch<4, false>(p, groups, st);
+    if (status != JA_OK) return status;
     ja_count_launch();
     *launched = true;
     return JA_OK;

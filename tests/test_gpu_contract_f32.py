@@ -105,3 +105,17 @@ def test_a_block_of_more_than_2_to_31_bytes_after_the_summed_index():
     ja.Spec("kij->ij", cuts, "ident", (), "sum").execute([x], out)
     assert torch.equal(out.payload, x.payload[:n] + x.payload[n:])
     check_status()
+
+
+def test_an_index_of_more_than_2_to_30_cells():
+    """Equal intervals with a shorter last one on an index whose interval ends leave 31 bits: the form with 64-bit coordinates."""
+    n = (1 << 30) + 64
+    cuts = {"i": [0, 2], "j": [0, 1 << 30, n]}
+    x = ja.Relation([2, n], [cuts["i"], cuts["j"]], BF)
+    x.payload.normal_()
+    out = ja.Relation([n], [cuts["j"]], F32, torch.full((n,), float("nan"), device="cuda"))
+    ja.Spec("ij->j", cuts, "ident", (), "sum").execute([x], out)
+    check_status()
+    for lo, hi, at in ((0, 1 << 30, 0), (1 << 30, n, 2 << 30)):       # the two blocks: [2, 2^30] cells, then [2, 64]
+        w = hi - lo
+        assert torch.equal(out.payload[lo:hi], x.payload[at: at + w].float() + x.payload[at + w: at + 2 * w].float())

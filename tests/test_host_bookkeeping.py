@@ -419,3 +419,20 @@ def test_general_join_agg_offsets(extents, splits, dtype):
         for moving in range(-1, len(extents)):
             assert ja.ja_debug_cell_offset(rel, moving, x) == int(offs[block]) + at * es
     ja.ja_relation_destroy(rel)
+
+
+@pytest.mark.parametrize("einsum,fn,agg,ext,form", [
+    ("ij->j", "ident", "sum", {"i": 2, "j": 1 << 30}, 1),
+    ("ij->j", "ident", "sum", {"i": 2, "j": (1 << 30) + 1}, 2),       # an interval's end or a step past the end may leave 31 bits
+    ("ij->i", "ident", "max", {"i": 2, "j": (1 << 30) + 1}, 2),
+    ("ij->i", "ident", "max", {"i": 2, "j": 1 << 30}, 1),
+    ("ij->ji", "ident", "none", {"i": 1 << 16, "j": (1 << 15) - 1}, 1),
+    ("ij->ji", "ident", "none", {"i": 1 << 16, "j": 1 << 15}, 2),     # 2^31 output cells
+    ("ijk->i", "square", "sum", {"i": 4, "j": 1 << 30, "k": 8}, 1),    # 2^30 tuples beside the moving index
+    ("ijkl->i", "square", "sum", {"i": 4, "j": 1 << 30, "k": 2, "l": 8}, 2),
+    ("ij,jk->ik", "rmsnorm", "none", {"i": 4, "j": 4, "k": 4}, 0),
+])
+def test_general_join_agg_form_at_the_32_bit_edge(einsum, fn, agg, ext, form):
+    s = ja.ja_spec_create(einsum, {c: [0, e // 2, e] for c, e in ext.items()}, fn, (), agg)
+    assert ja.ja_debug_general_form(s) == form
+    ja.ja_spec_destroy(s)
