@@ -13,7 +13,7 @@
 //
 // This file holds the mma.sync form (m16n8k16, bf16 in, fp32 accumulate; operands staged in shared memory with
 // cp.async under an XOR swizzle and read with ldmatrix). It serves what the tensor-memory kernels cannot take (uneven blocks
-// along the batch or head index, blocks of a few rows) and sequences of one 64-row tile, where it has less to set up.
+// along the batch or head index, blocks of a few rows, scales that are not positive) and sequences of one 64-row tile, where it has less to set up.
 // RAGGED form of the same kernel: ANY split points of the sequence index, any sequence length and any sequence ends. Output
 // key tiles are then 64 consecutive positions wherever they fall: a tile may straddle blocks and packed sequences and run
 // past the end of the index, so every row is located on its own (block lookup per row), rows past the end are zero, and

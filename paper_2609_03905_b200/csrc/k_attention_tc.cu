@@ -1211,11 +1211,14 @@ bool list_ragged_tiles(const AttnArgs& a, RaggedTiles* rt) {
 
 // Returns JA_OK and sets *launched when a tensor-memory kernel took the job; leaves *launched false when the tiling does
 // not fit (blocks uniform along b and h, at most MAX_SB sequence blocks when they are irregular, tiles that are not mostly
-// empty). The four tensor maps are encoded once per (spec, relations) tuple and
+// empty, a positive scale). The four tensor maps are encoded once per (spec, relations) tuple and
 // kept in a.cache.
 ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* launched) {
     *launched = false;
     if (!a.rows_layout) return JA_OK;
+    // These kernels mask with -inf and take the maximum BEFORE they scale, which a scale of zero turns into NaN and a negative one
+    // into +inf and a minimum; the mma.sync form scales first.
+    if (!(a.scale > 0.f)) return JA_OK;
     AttnTcParams p;
     memset(&p, 0, sizeof p);
     if (!fill_geom(a.q, a.q_split, &p.q) || !fill_geom(a.k, a.k_split, &p.k)) return JA_OK;

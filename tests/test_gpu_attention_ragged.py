@@ -19,7 +19,7 @@ ES = blocked.equal_splits
 BF, F32, F16 = torch.bfloat16, torch.float32, torch.float16
 
 
-def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_blocks=None, g_split=None):
+def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_blocks=None, g_split=None, scale=1.0 / math.sqrt(128)):
     grp = Hq // Hkv
     Q, K, V = (si.normal((B, S, h, 128), 0.0, 1.0, dtype, 4, 60 + n) for n, h in enumerate((Hq, Hkv, Hkv)))
     b_sp, g_sp = ES(B, b_blocks or B), g_split or ES(Hkv, max(1, Hkv // 2))
@@ -28,7 +28,6 @@ def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_bloc
     rq, rk, rv = upload(Q, [b_sp, q_split, h_sp, d]), upload(K, [b_sp, k_split, g_sp, d]), upload(V, [b_sp, k_split, g_sp, d])
     ro = empty_like_tiling([B, S, Hq, 128], [b_sp, q_split, h_sp, d], dtype, fill=float("nan"))
     rl = empty_like_tiling([B, S, Hq], [b_sp, q_split, h_sp], F32, fill=float("nan")) if lse else None
-    scale = 1.0 / math.sqrt(128)
     parts = {"b": b_sp, "q": q_split, "h": h_sp, "d": d, "k": k_split}
     if grp > 1:
         parts["g"] = g_sp
@@ -36,7 +35,7 @@ def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_bloc
                    (scale, 1.0 if causal else 0.0) + tuple(float(e) for e in ends), "online_softmax")
     spec.execute([rq, rk, rv], [ro, rl] if lse else ro)
     got = download(ro)
-    ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), grp, ends or None, causal, {BF: "bf16", F16: "f16"}[dtype])
+    ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), grp, ends or None, causal, {BF: "bf16", F16: "f16"}[dtype], scale)
     assert relfro(got, ref) <= TOL[dtype]
     # no row is worse than the whole: a row that lost or gained a key would be
     err = np.linalg.norm(got - ref, axis=-1) / np.maximum(np.linalg.norm(ref, axis=-1), 1e-3)
@@ -89,6 +88,13 @@ def test_shorter_last_block(split, packed, causal, lse, dtype, b_blocks):
 def test_shorter_last_head_block(S):
     _run(1, S, 3, 3, [0, S], [0, S], [], True, BF, lse=True, g_split=[0, 2, 3])
     _run(1, S, 6, 3, [0, S], [0, S], [], False, F16, g_split=[0, 2, 3])
+
+
+# any scale: 0 (every key counts alike), a negative one (the most negative product wins)
+@pytest.mark.parametrize("scale", [0.0, -1.0 / math.sqrt(128)])
+@pytest.mark.parametrize("S,causal", [(300, True), (145, False), (512, True), (256, False)])
+def test_scales_that_are_not_positive(S, causal, scale):
+    _run(2, S, 4, 2, [0, S], [0, S], [], causal, BF if S % 2 else F16, lse=True, scale=scale)
 
 
 def test_queries_and_keys_cut_differently():
