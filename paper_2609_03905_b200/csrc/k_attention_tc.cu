@@ -921,11 +921,12 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                         if (i > kmax) v[i] = 0xff800000u;
                 }
                 const float mx = row_max128(v);
-                const float m_new = mx * p.scale_log2e;        // finite: the first key of a sequence is never masked
-                // lazy rescale: raise the offset only when the row maximum outgrew it by more than 2^8
+                const float m_new = mx * p.scale_log2e;
+                // lazy rescale: raise the offset only when the row maximum outgrew it by more than 2^8. A row whose scores have all been
+                // -inf so far has no offset yet and nothing to rescale; it exponentiates against 0 until a maximum comes.
                 float alpha = 1.f;
                 bool need = false;
-                if (j == 0) m_used = m_new;
+                if (m_used == -INFINITY) m_used = m_new;
                 else if (m_new > m_used + 8.f) { alpha = ex2(m_used - m_new); m_used = m_new; need = true; }
                 const bool rescale = __any_sync(0xffffffffu, need);
                 // Two things have to hold before P of this step may be stored: the P V of the tile's previous key step has
@@ -955,7 +956,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                     l_run *= alpha;
                 }
                 uint32_t pk[64];
-                l_run += row_exp_pack128<POLY, F16>(v, p.scale_log2e, m_used, pk);
+                l_run += row_exp_pack128<POLY, F16>(v, p.scale_log2e, m_used == -INFINITY ? 0.f : m_used, pk);
                 if (!(WAIT_FIRST || rescale)) {
                     if (!wait_p_tile()) { ok = false; break; }
                 }
@@ -972,7 +973,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
             // TMA stores -- 16-byte stores from 32 lanes to 32 different rows would write half-filled sectors
             if (!mbar_wait(bar(O_FULL + t), (uint32_t)(cs + n_t - 1) & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
-            const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+            const float inv = l_run > 0.f && m_used != -INFINITY ? 1.f / l_run : 0.f;   // no key but ones that score -inf: 0
             if (RAGGED) {
                 if (rt->lse.base && r < q_rows) {
                     const int64_t x[3] = {it.b, qrow, it.h};

@@ -97,6 +97,31 @@ def test_scales_that_are_not_positive(S, causal, scale):
     _run(2, S, 4, 2, [0, S], [0, S], [], causal, BF if S % 2 else F16, lse=True, scale=scale)
 
 
+@pytest.mark.parametrize("S", [131, 145, 300, 512, 768])        # ragged lengths and whole pairs of tiles
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_scores_of_minus_infinity(S, causal, dtype):
+    """The first 130 keys score -inf with every query (more than a key tile): a row's weights are those of its other keys, whose scores
+    lie far below 0 here, and a row without any has O = 0 and lse = -inf."""
+    H, n = 2, 130
+    Q, K, V = (si.normal((1, S, H, 128), 0.0, 1.0, dtype, 4, 90 + i) for i in range(3))
+    Q[..., 0] = 1.0
+    K[:, n:, :, 0] = -300.0
+    ref = operators.attention(si.to_f64(Q)[:, n:], si.to_f64(K)[:, n:], si.to_f64(V)[:, n:], causal, {BF: "bf16", F16: "f16"}[dtype])
+    ref_l = operators.attention_lse(si.to_f64(Q)[:, n:], si.to_f64(K)[:, n:], causal)
+    K[:, :n, :, 0] = float("-inf")
+    sp = [[0, 1], [0, S], ES(H, 2), [0, 128]]
+    ro, rl = empty_like_tiling([1, S, H, 128], sp, dtype, fill=float("nan")), empty_like_tiling([1, S, H], sp[:3], F32, fill=float("nan"))
+    ja.Spec("bqhd,bkhd,bkhd->bqhd", {"b": sp[0], "q": sp[1], "h": sp[2], "d": sp[3], "k": sp[1]}, "attention",
+            (1.0 / math.sqrt(128), 1.0 if causal else 0.0), "online_softmax").execute([upload(Q, sp), upload(K, sp), upload(V, sp)], [ro, rl])
+    got, lse = download(ro), download(rl)
+    check_status()
+    assert relfro(got[:, n:], ref) <= TOL[dtype]
+    assert np.abs(lse[:, n:] - ref_l).max() <= 1e-3
+    if causal:
+        assert (got[:, :n] == 0).all() and np.isneginf(lse[:, :n]).all()
+
+
 def test_queries_and_keys_cut_differently():
     S = 600
     _run(1, S, 4, 2, [0, 130, 391, 600], ES(S, 3), [], True, BF)
