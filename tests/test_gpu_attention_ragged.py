@@ -1,7 +1,8 @@
 """Attention over sequences and blocks that are no whole pairs of 128-row tiles, on the tensor-memory kernel (its ragged form)
 against the oracle. Lengths sit at the edges of tiles (128 rows), of pairs, of the 16-key groups of the P V product and of the
-pieces a tile is made of. Tolerances: those of the other attention tests (ten half-ulps of the stored type; lse 1e-3 absolute:
-2^-9 of scores of order one plus the f32 logarithm)."""
+pieces a tile is made of. Tolerances: those of the other attention tests (ten half-ulps of the stored type). lse is held in f32:
+scores of order five to 2^-21, exponentials to 2^-22, sums and a logarithm in f32 stay below 1e-5; where lengths are whole pairs of tiles
+and blocks whole tiles a quarter of the exponentials are a cubic (7.5e-5 relative, so at most as much in a logarithm): 1e-4."""
 import math
 
 import numpy as np
@@ -41,12 +42,13 @@ def _run(B, S, Hq, Hkv, q_split, k_split, ends, causal, dtype, lse=False, b_bloc
     err = np.linalg.norm(got - ref, axis=-1) / np.maximum(np.linalg.norm(ref, axis=-1), 1e-3)
     assert err.max() <= 4 * TOL[dtype]
     if lse:
+        whole = all(e % 256 == 0 for e in ends or [S]) and all(x % 128 == 0 for x in q_split + k_split)
         s0 = 0
         L = download(rl)
         for s1 in ends or [S]:
             K2 = np.repeat(si.to_f64(K)[:, s0:s1], grp, axis=2)
             want = operators.attention_lse(si.to_f64(Q)[:, s0:s1], K2, causal, scale)
-            assert np.abs(L[:, s0:s1] - want).max() <= 1e-3
+            assert np.abs(L[:, s0:s1] - want).max() <= (1e-4 if whole and scale > 0 else 1e-5)
             s0 = s1
     check_status()
 
@@ -117,7 +119,7 @@ def test_scores_of_minus_infinity(S, causal, dtype):
     got, lse = download(ro), download(rl)
     check_status()
     assert relfro(got[:, n:], ref) <= TOL[dtype]
-    assert np.abs(lse[:, n:] - ref_l).max() <= 1e-3
+    assert np.abs(lse[:, n:] - ref_l).max() <= 1e-4     # logarithms of order 30
     if causal:
         assert (got[:, :n] == 0).all() and np.isneginf(lse[:, :n]).all()
 
