@@ -131,6 +131,17 @@ __device__ __forceinline__ void umma_ss_w(uint32_t d_tmem, uint64_t a_desc, uint
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(pred)
         : "memory");
 }
+// the same on every lane of D whose bit in `off` is clear; the others keep what they hold
+__device__ __forceinline__ void umma_ss_lanes_w(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate, const uint32_t (&off)[4],
+                                                uint32_t pred) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%6, %7, %8, %9}, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(pred), "r"(off[0]), "r"(off[1]), "r"(off[2]), "r"(off[3])
+        : "memory");
+}
 // D[tmem] (+)= A[tmem] * B[smem desc]
 __device__ __forceinline__ void umma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate, uint32_t pred) {
     asm volatile(
@@ -779,20 +790,30 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
             }
             commit1_w(bar(S_FULL + t), leader);
         };
-        auto issue_pv = [&](int t, int sl, bool first, int keys) {   // O~_t (+)= P_t V, P in shared memory (K-major), V in slot sl (MN-major)
+        // RAGGED: keys = the tile's keys; rows = the query rows that join it; a row below `before` + k joins none of its keys from k on
+        // (causal; without: before is far below 0)
+        auto issue_pv = [&](int t, int sl, bool first, int keys, int rows, int before) {   // O~_t (+)= P_t V, P in shared memory (K-major), V in slot sl (MN-major)
             const uint32_t vaddr = sKV + sl * TILE_BYTES, paddr = sP + t * TILE_BYTES;
-            if (!RAGGED || keys == KT) {
+            if (!RAGGED || (keys == KT && before + KT <= 16)) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
                     const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
                     umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + off, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
                               (!first || kk > 0) ? 1u : 0u, leader);
                 }
-            } else {      // a short key tile: only the groups of 16 keys that exist
-                for (int kk = 0; kk * 16 < keys; ++kk) {
-                    const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
-                    umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + off, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
-                              (!first || kk > 0) ? 1u : 0u, leader);
+            } else {
+                // A short or diagonal key tile: only the groups of 16 keys that exist and that some row joins, and of a group only the rows
+                // that join its first key: P is 0 elsewhere, but 0 times an infinite or NaN V row of a later key would not be.
+                for (int kk = 0; kk * 16 < keys && before + kk * 16 < rows; ++kk) {
+                    const uint32_t at = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
+                    uint32_t off[4];
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) {
+                        const int n = before + kk * 16 - w * 32;   // lanes [0, n) of this word are off
+                        off[w] = n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u;
+                    }
+                    umma_ss_lanes_w(tmem_base + 256 + t * 128, desc_sw128(paddr + at, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
+                                    (!first || kk > 0) ? 1u : 0u, off, leader);
                 }
             }
             commit1_w(bar(P_EMPTY + t), leader);
@@ -858,7 +879,12 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                         // the first P V of an item overwrites O~: the row threads must have read the previous item's
                         if (j == 0 && done[t] > 0 && !mbar_wait(bar(O_READ + t), (uint32_t)(done[t] - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        issue_pv(t, sl, j == 0, keys);
+                        int rows = QT, before = -KT;
+                        if constexpr (RAGGED) {
+                            rows = tile_rows(rt->q[it.qt + t]);
+                            if (p.causal) before = tile_start(rt->k[it.kt + j]) - tile_start(rt->q[it.qt + t]);
+                        }
+                        issue_pv(t, sl, j == 0, keys, rows, before);
                     }
                 }
                 if (!ok) break;
