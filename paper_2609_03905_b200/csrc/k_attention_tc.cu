@@ -22,6 +22,7 @@
 // Grouped-query attention: query head h joins key/value head h / group. Packed sequences (Example 3.10): an output
 // key tile joins only the key/value tiles of its own sequence [s0, s1), so the walk starts at s0.
 // Every mbarrier wait is bounded; on expiry the CTA records JA_ERR_TIMEOUT and leaves through the normal exit.
+#include <float.h>
 #include <stdlib.h>
 
 #include <atomic>
@@ -948,11 +949,12 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                 }
                 const float mx = row_max128(v);
                 const float m_new = mx * p.scale_log2e;
-                // lazy rescale: raise the offset only when the row maximum outgrew it by more than 2^8. A row whose scores have all been
-                // -inf so far has no offset yet and nothing to rescale; it exponentiates against 0 until a maximum comes.
+                // lazy rescale: raise the offset only when the row maximum outgrew it by more than 2^8. The offset is finite also where all
+                // scores so far are -inf: they exponentiate to 0, and the first maximum that comes outgrows it. (A test for -inf at every
+                // key step and an offset selected by it cost 1 % of B4 S2048.)
                 float alpha = 1.f;
                 bool need = false;
-                if (m_used == -INFINITY) m_used = m_new;
+                if (j == 0) m_used = fmaxf(m_new, -FLT_MAX);
                 else if (m_new > m_used + 8.f) { alpha = ex2(m_used - m_new); m_used = m_new; need = true; }
                 const bool rescale = __any_sync(0xffffffffu, need);
                 // Two things have to hold before P of this step may be stored: the P V of the tile's previous key step has
@@ -982,7 +984,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                     l_run *= alpha;
                 }
                 uint32_t pk[64];
-                l_run += row_exp_pack128<POLY, F16>(v, p.scale_log2e, m_used == -INFINITY ? 0.f : m_used, pk);
+                l_run += row_exp_pack128<POLY, F16>(v, p.scale_log2e, m_used, pk);
                 if (!(WAIT_FIRST || rescale)) {
                     if (!wait_p_tile()) { ok = false; break; }
                 }
@@ -999,7 +1001,8 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
             // TMA stores -- 16-byte stores from 32 lanes to 32 different rows would write half-filled sectors
             if (!mbar_wait(bar(O_FULL + t), (uint32_t)(cs + n_t - 1) & 1, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
-            const float inv = l_run > 0.f && m_used != -INFINITY ? 1.f / l_run : 0.f;   // no key but ones that score -inf: 0
+            if (m_used == -FLT_MAX && l_run < 1e-30f) l_run = 0.f;   // no key but ones that score -inf (the cubic's least value is 2^-126)
+            const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             if (RAGGED) {
                 if (rt->lse.base && r < q_rows) {
                     const int64_t x[3] = {it.b, qrow, it.h};
