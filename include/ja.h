@@ -188,8 +188,13 @@ ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* const* inputs
 /* ---- repartition (Section 5.3: overlay -> atoms, decompose + recompose) ---------------------------
  * Copies the tensor held by `src` into the tiling of `dst` (same rank, extents, dtype): every atom of the
  * overlay of the two tilings moves from its source block to its destination block.  Bit-exact, no
- * aggregation.  Asynchronous on `cuda_stream`. */
+ * aggregation.  Asynchronous on `cuda_stream`. The first call for a pair of relations plans the copy on the host and, where the
+ * overlay is cut into more than 960 slabs (of up to 64 KiB), puts the plan into a device table (a synchronous cudaMalloc and
+ * cudaMemcpy, about 0.4 ms); later calls only launch. A first call inside a stream capture makes no table (up to 7680 slabs). */
 ja_status_t ja_repartition(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream);
+/* The same for two relations that meet once: nothing is kept and, up to 7680 slabs, nothing is allocated on the device (one launch
+ * per 960 slabs). */
+ja_status_t ja_repartition_once(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream);
 /* Overlay introspection (host, no CUDA): number of atoms, then per atom lower[rank], upper[rank],
  * flat source block, flat destination block.  Pass NULL arrays to query the count only. */
 ja_status_t ja_overlay_atoms(const ja_relation_t* src, const ja_relation_t* dst, int64_t* n_atoms, int64_t* lower,

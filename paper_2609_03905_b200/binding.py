@@ -64,6 +64,7 @@ def _load() -> ctypes.CDLL:
         "ja_relation_get_keys": [vp, vp, vp, vp, vp],
         "ja_execute": [vp, P(vp), i32, P(vp), i32, vp],
         "ja_repartition": [vp, vp, vp],
+        "ja_repartition_once": [vp, vp, vp],
         "ja_execute_join": [vp, P(vp), i32, vp, vp],
         "ja_plan_optimize": [P(ja_plan_node_t), i32, i32, P(i32), P(i64)],
         "ja_plan_cost": [P(ja_plan_node_t), i32, P(i32), P(i64)],
@@ -213,6 +214,11 @@ def ja_execute(spec: int, inputs, outputs, stream: int = 0):
 
 def ja_repartition(src: int, dst: int, stream: int = 0):
     _check(LIB.ja_repartition(src, dst, ctypes.c_void_p(stream)))
+
+
+def ja_repartition_once(src: int, dst: int, stream: int = 0):
+    """ja_repartition between two relations that meet once: nothing is kept, nothing allocated (up to 7680 slabs)."""
+    _check(LIB.ja_repartition_once(ctypes.c_void_p(src), ctypes.c_void_p(dst), ctypes.c_void_p(stream)))
 
 
 def ja_execute_join(spec: int, inputs, partials: int, stream: int = 0):

@@ -656,8 +656,8 @@ extern "C" ja_status_t ja_overlay_atoms(const ja_relation_t* src, const ja_relat
 }
 
 struct RepartPlan {
-    CopySlab* d_slabs = nullptr;         // device table; ja_repartition makes it at the second call only, where
-    std::vector<CopySlab> slabs;         // these are few enough to travel in the parameters of a few launches
+    std::vector<CopySlab> slabs;         // until d_slabs holds them
+    CopySlab* d_slabs = nullptr;         // device table of more than JA_PARAM_SLABS slabs
     bool long_rows = false;              // rows of 256 bytes and more
     int64_t n_slabs = 0;
     int vec_bytes = 16;
@@ -726,68 +726,90 @@ static void plan_slabs(const ja_relation* src, const ja_relation* dst, std::vect
     }
 }
 
-extern "C" ja_status_t ja_repartition(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream) {
-    ja_status_t st = check_same_tensor(src, dst);
+static std::shared_ptr<RepartPlan> plan_repartition(const ja_relation* src, const ja_relation* dst) {
+    std::shared_ptr<RepartPlan> plan(new RepartPlan());
+    int64_t src_or = 0, dst_or = 0;
+    plan_slabs(src, dst, &plan->slabs, &src_or, &dst_or);
+    const int64_t all_or = src_or | dst_or;
+    while (plan->vec_bytes > src->esize && (all_or % plan->vec_bytes) != 0) plan->vec_bytes /= 2;
+    plan->n_slabs = (int64_t)plan->slabs.size();
+    int64_t bytes = 0, rows = 0;
+    for (const CopySlab& c : plan->slabs) {
+        bytes += (int64_t)c.rows * c.row_bytes;
+        rows += c.rows;
+    }
+    plan->long_rows = bytes >= 256 * rows;
+    return plan;
+}
+static ja_status_t launch_slabs_by_parameters(const RepartPlan& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t st) {
+    for (int64_t at = 0; at < plan.n_slabs; at += JA_PARAM_SLABS) {
+        const ja_status_t s = ja_launch_repartition_param((const char*)src->base, (char*)dst->base, plan.slabs.data() + at,
+                                                          (int)std::min<int64_t>(JA_PARAM_SLABS, plan.n_slabs - at), plan.vec_bytes, plan.long_rows, st);
+        if (s != JA_OK) return s;
+    }
+    return JA_OK;
+}
+static ja_status_t check_repartition(const ja_relation* src, const ja_relation* dst) {
+    const ja_status_t st = check_same_tensor(src, dst);
     if (st != JA_OK) return st;
-    if (src->base == dst->base) return ja_fail(JA_ERR_INVALID_ARG, "repartition in place is not supported");
-    std::shared_ptr<RepartPlan> plan;
-    auto launch_by_parameters = [&]() -> ja_status_t {
-        for (int64_t at = 0; at < plan->n_slabs; at += JA_PARAM_SLABS) {
-            const ja_status_t s = ja_launch_repartition_param((const char*)src->base, (char*)dst->base, plan->slabs.data() + at,
-                                                              (int)std::min<int64_t>(JA_PARAM_SLABS, plan->n_slabs - at), plan->vec_bytes,
-                                                              (cudaStream_t)cuda_stream);
-            if (s != JA_OK) return s;
+    return src->base == dst->base ? ja_fail(JA_ERR_INVALID_ARG, "repartition in place is not supported") : JA_OK;
+}
+constexpr int64_t SLABS_OF_A_FEW_LAUNCHES = 8 * JA_PARAM_SLABS;
+
+// the plan that the pair keeps: the one given, or another thread's where that was first
+static std::shared_ptr<RepartPlan> keep_repartition(const ja_relation* src, const ja_relation* dst, const std::shared_ptr<RepartPlan>& plan) {
+    std::lock_guard<std::mutex> lk(g_repart_mu);
+    return g_repart_plans.emplace(std::make_pair(src->id, dst->id), plan).first->second;
+}
+static ja_status_t run_repartition(const std::shared_ptr<RepartPlan>& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t stream) {
+    // One launch whose parameters hold the slabs is as fast as a table (33 MB in 512 slabs: 10.3 us either way) and needs no memory;
+    // more slabs are read from a table that the pair's FIRST call makes, so that every later one, captured or not, only launches.
+    if (plan->n_slabs <= JA_PARAM_SLABS) return launch_slabs_by_parameters(*plan, src, dst, stream);
+    {
+        std::lock_guard<std::mutex> lk(g_repart_mu);
+        if (!plan->d_slabs) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusNone;
+            if (cap != cudaStreamCaptureStatusNone && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES)
+                return launch_slabs_by_parameters(*plan, src, dst, stream);   // a capture allows no allocation
+            CopySlab* table = nullptr;
+            cudaError_t e = cudaMalloc((void**)&table, plan->slabs.size() * sizeof(CopySlab));
+            if (e == cudaErrorMemoryAllocation && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES) {
+                cudaGetLastError();   // no memory left for a table: slower, but it runs
+                return launch_slabs_by_parameters(*plan, src, dst, stream);
+            }
+            if (e != cudaSuccess) return ja_cuda_fail(e, "cudaMalloc(copy slabs)");
+            e = cudaMemcpy(table, plan->slabs.data(), plan->slabs.size() * sizeof(CopySlab), cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                cudaFree(table);
+                return ja_cuda_fail(e, "cudaMemcpy(copy slabs)");
+            }
+            plan->d_slabs = table;
+            std::vector<CopySlab>().swap(plan->slabs);
         }
-        return JA_OK;
-    };
+    }
+    return ja_launch_repartition((const char*)src->base, (char*)dst->base, plan->d_slabs, plan->n_slabs, plan->vec_bytes, plan->long_rows, stream);
+}
+
+extern "C" ja_status_t ja_repartition(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream) {
+    const ja_status_t st = check_repartition(src, dst);
+    if (st != JA_OK) return st;
+    std::shared_ptr<RepartPlan> plan;
     {
         std::lock_guard<std::mutex> lk(g_repart_mu);
         auto it = g_repart_plans.find({src->id, dst->id});
         if (it != g_repart_plans.end()) plan = it->second;
     }
-    if (!plan) {
-        const int es = src->esize;
-        std::vector<CopySlab> slabs;
-        int64_t src_or = 0, dst_or = 0;
-        plan_slabs(src, dst, &slabs, &src_or, &dst_or);
-        const int64_t all_or = src_or | dst_or;
-        plan.reset(new RepartPlan());
-        plan->vec_bytes = 16;
-        while (plan->vec_bytes > es && (all_or % plan->vec_bytes) != 0) plan->vec_bytes /= 2;
-        plan->n_slabs = (int64_t)slabs.size();
-        int64_t bytes = 0, rows = 0;
-        for (const CopySlab& c : slabs) {
-            bytes += (int64_t)c.rows * c.row_bytes;
-            rows += c.rows;
-        }
-        plan->long_rows = bytes >= 256 * rows;
-        plan->slabs.swap(slabs);
-        {
-            std::lock_guard<std::mutex> lk(g_repart_mu);
-            g_repart_plans[{src->id, dst->id}] = plan;
-        }
-        // Relations that meet once (a dense tensor packed, a result unpacked) allocate nothing on the device: 1.3 to 1.5 ms of
-        // allocation, copy and release a round trip. Where a table is kept the launch is up to 9 us shorter, so the pair's second
-        // call makes one.
-        if (plan->n_slabs <= 8 * JA_PARAM_SLABS) return launch_by_parameters();
-    }
-    {
-        std::lock_guard<std::mutex> lk(g_repart_mu);
-        if (!plan->d_slabs) {
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing((cudaStream_t)cuda_stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusNone;
-            if (cap != cudaStreamCaptureStatusNone && plan->n_slabs <= 8 * JA_PARAM_SLABS) return launch_by_parameters();   // a capture allows no allocation
-            JA_CUDA(cudaMalloc((void**)&plan->d_slabs, plan->slabs.size() * sizeof(CopySlab)));
-            const cudaError_t e = cudaMemcpy(plan->d_slabs, plan->slabs.data(), plan->slabs.size() * sizeof(CopySlab), cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) {
-                cudaFree(plan->d_slabs);
-                plan->d_slabs = nullptr;
-                return ja_cuda_fail(e, "cudaMemcpy(copy slabs)");
-            }
-        }
-    }
-    return ja_launch_repartition((const char*)src->base, (char*)dst->base, plan->d_slabs, plan->n_slabs, plan->vec_bytes, plan->long_rows,
-                                 (cudaStream_t)cuda_stream);
+    if (!plan) plan = keep_repartition(src, dst, plan_repartition(src, dst));
+    return run_repartition(plan, src, dst, (cudaStream_t)cuda_stream);
+}
+
+extern "C" ja_status_t ja_repartition_once(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream) {
+    const ja_status_t st = check_repartition(src, dst);
+    if (st != JA_OK) return st;
+    const std::shared_ptr<RepartPlan> plan = plan_repartition(src, dst);
+    if (plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES) return launch_slabs_by_parameters(*plan, src, dst, (cudaStream_t)cuda_stream);
+    return run_repartition(keep_repartition(src, dst, plan), src, dst, (cudaStream_t)cuda_stream);   // the table lives as long as the relations
 }
 
 // ---------------------------------------------------------------------------------------------------

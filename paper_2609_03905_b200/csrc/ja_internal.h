@@ -167,7 +167,8 @@ ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_
                                   cudaStream_t st);
 // the same with the slabs in the kernel's parameters: n_slabs <= JA_PARAM_SLABS, host pointer, read before the call returns
 #define JA_PARAM_SLABS 960
-ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, cudaStream_t st);
+ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, bool long_rows,
+                                        cudaStream_t st);
 // Aggregating relayout: every slab is read from n_copies copies of the source, copy_stride bytes apart, (+)-combined
 // in ascending copy order in f32 and stored once. Slab sizes are in SOURCE bytes; destination offsets / pitches in
 // destination bytes. vec = cells per access (8 / 4 for 16-byte accesses of bf16 / f32 sources, or 1).

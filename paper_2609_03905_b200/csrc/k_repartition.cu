@@ -7,9 +7,11 @@
 // around them, and only the ends of a row go cell by cell (12370 rows of 2919 bf16 cells: 81 -> 39 us); short ones go by the
 // widest access their alignment allows.
 //
-// The slabs travel in a table in device memory that the caller keeps, or -- up to JA_PARAM_SLABS of them -- in the kernel's
-// parameters, so that a relayout between relations that are used once (packing a dense tensor, unpacking a result) allocates
-// nothing on the device and copies nothing to it.
+// The slabs travel in the kernel's parameters where JA_PARAM_SLABS hold them -- nothing is allocated or copied for a pair of
+// relations, on its first call or any other -- else in a table in device memory that the caller keeps, or, for relations that meet
+// once (packing a dense tensor, unpacking a result), in the parameters of several launches: 0.4 ms less than a table's allocation
+// and copy, but 20 to 30 % slower per call than one launch with a table (134 MB: 59 against 47 us, the ends of three launches).
+// Both move a slab by the same rule (copy_of).
 #include <string.h>
 
 #include "ja_device.cuh"
@@ -17,19 +19,14 @@
 namespace {
 
 template <typename V>
-__global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict__ src, char* __restrict__ dst,
-                                                          const CopySlab* __restrict__ slabs, int64_t n_slabs) {
-    for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
-        const CopySlab sl = slabs[s];
-        const int vpr = sl.row_bytes / (int)sizeof(V);  // vectors per row
-        const int total = vpr * sl.rows;
-        const char* sp = src + sl.src_off;
-        char* dp = dst + sl.dst_off;
-        for (int i = threadIdx.x; i < total; i += 256) {
-            int r = i / vpr, c = i - r * vpr;
-            V v = *reinterpret_cast<const V*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * sizeof(V));
-            *reinterpret_cast<V*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * sizeof(V)) = v;
-        }
+__device__ __forceinline__ void copy_slab(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+    const int vpr = sl.row_bytes / (int)sizeof(V);  // vectors per row
+    const int total = vpr * sl.rows;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < total; i += 256) {
+        const int r = i / vpr, c = i - r * vpr;
+        const V v = *reinterpret_cast<const V*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * sizeof(V));
+        *reinterpret_cast<V*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * sizeof(V)) = v;
     }
 }
 
@@ -78,50 +75,68 @@ __device__ __forceinline__ void copy_slab_any(const char* __restrict__ sp, char*
         if (w >= words) { w -= words; ++r; }
     }
 }
-__global__ void __launch_bounds__(256) repartition_any_kernel(const char* __restrict__ src, char* __restrict__ dst, const CopySlab* __restrict__ slabs,
-                                                              int64_t n_slabs) {
+// How the slabs of a pair are copied. vec_bytes: the widest access that divides every offset, pitch and run length. Words put together
+// pay on rows long enough that their two ends do not matter, and not against 8-byte accesses (10901 x 1088 f32 in 34-cell blocks
+// 17 us, 26 as shifted words; 28480 x 916 f16 in 29-cell blocks 52 and 62; 12370 x 2919 bf16 81 and 39).
+enum Copy { COPY_16, COPY_8, COPY_4, COPY_2, COPY_ANY };
+Copy copy_of(int vec_bytes, bool long_rows) {
+    return vec_bytes == 16 ? COPY_16 : vec_bytes == 8 ? COPY_8 : long_rows ? COPY_ANY : vec_bytes == 4 ? COPY_4 : COPY_2;
+}
+template <int HOW>
+__device__ __forceinline__ void copy_slab_by(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+    if (HOW == COPY_16) copy_slab<uint4>(sp, dp, sl);
+    else if (HOW == COPY_8) copy_slab<uint2>(sp, dp, sl);
+    else if (HOW == COPY_4) copy_slab<uint32_t>(sp, dp, sl);
+    else if (HOW == COPY_2) copy_slab<uint16_t>(sp, dp, sl);
+    else copy_slab_any(sp, dp, sl);
+}
+
+template <int HOW>
+__global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict__ src, char* __restrict__ dst, const CopySlab* __restrict__ slabs,
+                                                          int64_t n_slabs) {
     for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
         const CopySlab sl = slabs[s];
-        copy_slab_any(src + sl.src_off, dst + sl.dst_off, sl);
+        copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
     }
 }
 
 template <int N> struct SlabParams {
     CopySlab s[N];
 };
-template <int N, bool WORDS>
+template <int N, int HOW>
 __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __restrict__ src, char* __restrict__ dst, const __grid_constant__ SlabParams<N> p) {
     const CopySlab& sl = p.s[blockIdx.x];
-    const char* sp = src + sl.src_off;
-    char* dp = dst + sl.dst_off;
-    if (!WORDS) {
-        copy_slab_any(sp, dp, sl);
-        return;
-    }
-    const int vpr = sl.row_bytes / 16, total = vpr * sl.rows;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < total; i += 256) {
-        const int r = i / vpr, c = i - r * vpr;
-        *reinterpret_cast<uint4*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * 16) = *reinterpret_cast<const uint4*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * 16);
-    }
+    copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
 }
-template <int N>
-void launch_param(const char* src, char* dst, const CopySlab* slabs, int n, bool words, cudaStream_t st) {
-    SlabParams<N> p;
-    memcpy(p.s, slabs, (size_t)n * sizeof(CopySlab));
-    if (words) repartition_param_kernel<N, true><<<n, 256, 0, st>>>(src, dst, p);
-    else repartition_param_kernel<N, false><<<n, 256, 0, st>>>(src, dst, p);
+template <int HOW>
+void launch_param(const char* src, char* dst, const CopySlab* slabs, int n, cudaStream_t st) {
+    auto go = [&](auto p) {
+        constexpr int N = (int)(sizeof p.s / sizeof p.s[0]);
+        memcpy(p.s, slabs, (size_t)n * sizeof(CopySlab));
+        repartition_param_kernel<N, HOW><<<n, 256, 0, st>>>(src, dst, p);
+    };
+    if (n <= 32) go(SlabParams<32>());
+    else if (n <= 256) go(SlabParams<256>());
+    else go(SlabParams<JA_PARAM_SLABS>());
+}
+template <int HOW>
+void launch_table(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, cudaStream_t st) {
+    const unsigned grid = (unsigned)(n_slabs < (int64_t)148 * 64 ? n_slabs : (int64_t)148 * 64);
+    repartition_kernel<HOW><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
 }
 
 }  // namespace
 
-ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, cudaStream_t st) {
+ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, bool long_rows, cudaStream_t st) {
     static_assert(JA_PARAM_SLABS == 960 && sizeof(CopySlab) == 32, "30 KiB of the 32764 bytes a kernel's parameters may hold");
     if (n_slabs == 0) return JA_OK;
-    const bool words = vec_bytes == 16;
-    if (n_slabs <= 32) launch_param<32>(src, dst, slabs, n_slabs, words, st);
-    else if (n_slabs <= 256) launch_param<256>(src, dst, slabs, n_slabs, words, st);
-    else launch_param<JA_PARAM_SLABS>(src, dst, slabs, n_slabs, words, st);
+    switch (copy_of(vec_bytes, long_rows)) {
+        case COPY_16: launch_param<COPY_16>(src, dst, slabs, n_slabs, st); break;
+        case COPY_8: launch_param<COPY_8>(src, dst, slabs, n_slabs, st); break;
+        case COPY_4: launch_param<COPY_4>(src, dst, slabs, n_slabs, st); break;
+        case COPY_2: launch_param<COPY_2>(src, dst, slabs, n_slabs, st); break;
+        case COPY_ANY: launch_param<COPY_ANY>(src, dst, slabs, n_slabs, st); break;
+    }
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
     return JA_OK;
@@ -130,14 +145,13 @@ ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySl
 ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int vec_bytes, bool long_rows,
                                   cudaStream_t st) {
     if (n_slabs == 0) return JA_OK;
-    unsigned grid = (unsigned)(n_slabs < (int64_t)148 * 64 ? n_slabs : (int64_t)148 * 64);
-    // words put together pay on rows long enough that their two ends do not matter, and not against 8-byte accesses (10901 x 1088 f32
-    // in 34-cell blocks 17 us, 26 as shifted words; 28480 x 916 f16 in 29-cell blocks 52 and 62; 12370 x 2919 bf16 81 and 39)
-    if (vec_bytes == 16) repartition_kernel<uint4><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
-    else if (vec_bytes == 8) repartition_kernel<uint2><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
-    else if (long_rows) repartition_any_kernel<<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
-    else if (vec_bytes == 4) repartition_kernel<uint32_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
-    else repartition_kernel<uint16_t><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    switch (copy_of(vec_bytes, long_rows)) {
+        case COPY_16: launch_table<COPY_16>(src, dst, d_slabs, n_slabs, st); break;
+        case COPY_8: launch_table<COPY_8>(src, dst, d_slabs, n_slabs, st); break;
+        case COPY_4: launch_table<COPY_4>(src, dst, d_slabs, n_slabs, st); break;
+        case COPY_2: launch_table<COPY_2>(src, dst, d_slabs, n_slabs, st); break;
+        case COPY_ANY: launch_table<COPY_ANY>(src, dst, d_slabs, n_slabs, st); break;
+    }
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
     return JA_OK;

@@ -103,7 +103,7 @@ def from_dense(dense: torch.Tensor, splits) -> Relation:
     dense = dense.contiguous()
     one = Relation(list(dense.shape), [[0, e] for e in dense.shape], dense.dtype, _aligned_flat(dense))
     dst = Relation(list(dense.shape), splits, dense.dtype)
-    repartition(one, dst)
+    B.ja_repartition_once(one.handle, dst.handle, current_stream())
     torch.cuda.current_stream().synchronize()
     one.close()
     return dst
@@ -117,7 +117,7 @@ def to_dense(rel: Relation) -> torch.Tensor:
     pad = (-n * rel.dtype.itemsize) % 128
     payload = torch.empty(n + pad // rel.dtype.itemsize, dtype=rel.dtype, device=rel.payload.device)
     one = Relation(rel.extents, [[0, e] for e in rel.extents], rel.dtype, payload)
-    repartition(rel, one)
+    B.ja_repartition_once(rel.handle, one.handle, current_stream())
     torch.cuda.current_stream().synchronize()
     one.close()
     return payload[:n].reshape(rel.extents)

@@ -21,13 +21,19 @@ BF, F32, F16 = torch.bfloat16, torch.float32, torch.float16
     ([128, 256], [2, 4], [4, 1]), ([1000, 37], [1, 1], [100, 1]), ([999, 515], [128, 2], [64, 32]),          # the last: a device table
     ([5, 33, 17], [1, 2, 3], [5, 1, 2]), ([3, 4, 9, 11], [1, 2, 1, 3], [3, 1, 2, 1]), ([4096, 40], [1024, 1], [3, 1]),
 ])
-def test_any_alignment(ext, src, dst, dtype):
+@pytest.mark.parametrize("once", [False, True])
+def test_any_alignment(ext, src, dst, dtype, once):
+    def move(x, y):
+        if once:
+            ja.ja_repartition_once(x.handle, y.handle, torch.cuda.current_stream().cuda_stream)
+        else:
+            ja.repartition(x, y)
     s_sp, d_sp = [ES(e, g) for e, g in zip(ext, src)], [ES(e, g) for e, g in zip(ext, dst)]
     x = si.normal(tuple(ext), 0.0, 1.0, dtype, 37, 1)
     a, b, c = upload(x, s_sp), empty_like_tiling(ext, d_sp, dtype), empty_like_tiling(ext, s_sp, dtype)
-    ja.repartition(a, b)
+    move(a, b)
     assert np.array_equal(download_bits(b), blocked.pack(np_bits(x), d_sp))
-    ja.repartition(b, c)
+    move(b, c)
     assert np.array_equal(download_bits(c), blocked.pack(np_bits(x), s_sp))
     check_status()          # guard zones around every payload
 
@@ -55,4 +61,31 @@ def test_first_use_inside_a_capture_and_replay_after_the_plan_is_gone():
     b.payload.zero_()
     g.replay()
     assert np.array_equal(download_bits(b), blocked.pack(np_bits(x), d_sp))
+    check_status()
+
+
+def test_every_call_of_a_pair_costs_the_same():
+    """4096 slabs: the first call makes the table that every later one reads, captured or not (one launch each); relations that meet
+    once make none (a launch per 960 slabs)."""
+    ext, s_sp, d_sp = [999, 515], [ES(999, 128), ES(515, 2)], [ES(999, 64), ES(515, 32)]
+    x = si.normal(tuple(ext), 0.0, 1.0, BF, 37, 4)
+    a, b = upload(x, s_sp), empty_like_tiling(ext, d_sp, BF)
+
+    def launches(call):
+        before = ja.ja_launch_count()
+        call()
+        return ja.ja_launch_count() - before
+
+    stream = torch.cuda.current_stream().cuda_stream
+    assert launches(lambda: ja.ja_repartition_once(a.handle, b.handle, stream)) == 5
+    assert [launches(lambda: ja.repartition(a, b)) for _ in range(3)] == [1, 1, 1]
+    g = torch.cuda.CUDAGraph()
+    c = empty_like_tiling(ext, d_sp, BF)
+    ja.repartition(a, c)
+    with torch.cuda.graph(g):                                  # after ONE call of the pair
+        assert launches(lambda: ja.repartition(a, c)) == 1
+    c.payload.zero_()
+    g.replay()
+    want = blocked.pack(np_bits(x), d_sp)
+    assert np.array_equal(download_bits(b), want) and np.array_equal(download_bits(c), want)
     check_status()
