@@ -36,6 +36,15 @@ __device__ __forceinline__ int64_t ja_elem_off(const RelView& v, const int64_t* 
     return v.blk_off[flat] + off * v.esize;
 }
 
+// the 16 bytes from byte sh (0..15, even) of lo:hi on
+__device__ __forceinline__ uint4 ja_shift16(const uint4& lo, const uint4& hi, int sh) {
+    const bool s8 = sh & 8, s4 = sh & 4;
+    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
+    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
+    const int bits = (sh & 2) * 8;
+    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
+}
+
 __device__ __forceinline__ float ja_to_float(float x) { return x; }
 __device__ __forceinline__ float ja_to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float ja_to_float(__half x) { return __half2float(x); }

@@ -515,13 +515,6 @@ bool launch_fast_op(RowOp op, const RowArgs& a, const FastGeom& g, int64_t n_row
 // f32 cells in four column blocks 421; the copy rate gives 13 and 94.) Every run is given the same number of words, so a thread's
 // runs and words are the same for every row.
 // ---------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint4 words_shifted(const uint4& lo, const uint4& hi, int sh) {   // 16 bytes from byte sh (0..15, even) of lo:hi on
-    const bool s8 = sh & 8, s4 = sh & 4;
-    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
-    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
-    const int bits = (sh & 2) * 8;
-    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
-}
 
 template <typename T, int VPT, int OP>
 __global__ void __launch_bounds__(256) row_word_kernel(RowArgs a, int64_t n_rows, int team, int words, int runs) {
@@ -627,7 +620,7 @@ __global__ void __launch_bounds__(256) row_word_kernel(RowArgs a, int64_t n_rows
             uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
             if (sh + lo * (int)sizeof(T) < 16) x = *reinterpret_cast<const uint4*>(a.g.base + g0);          // only words that hold wanted cells
             if (sh + hi * (int)sizeof(T) > 16) y = *reinterpret_cast<const uint4*>(a.g.base + g0 + 16);
-            gv.v = words_shifted(x, y, sh);
+            gv.v = ja_shift16(x, y, sh);
 #pragma unroll
             for (int e = 0; e < CW; ++e) o.e[e] = ja_from_float<T>(ja_to_float(raw[k].e[e]) * rstd * ja_to_float(gv.e[e]));
         } else {
@@ -645,13 +638,20 @@ __global__ void __launch_bounds__(256) row_word_kernel(RowArgs a, int64_t n_rows
     }
 }
 
-// false where a row has more words than a CTA holds in registers (the streaming form of row_kernel takes it)
+// false where a row has more words than a CTA holds in registers, or words that hold too little: row_kernel takes it
 template <typename T, int OP>
 bool launch_row_words(const RowArgs& a, int64_t n_rows, cudaStream_t st) {
     constexpr int CW = 16 / (int)sizeof(T);
     const int runs = a.x.nblk[a.x.rank - 1];
     const int64_t words = (a.widest + 2 * CW - 2) / CW, all = words * runs;    // a run of `widest` cells touches at most that many words
     if (all > 256 * 16) return false;
+    // Short runs are words that are mostly mask, each with a run of its own to find, and where a few runs are much wider than the rest
+    // most words are empty (every run is given the widest one's): row_kernel's cells are cheaper there. Swept over runs of 1 to 50
+    // cells and one wide run before narrow ones, 150 to 7000 cells, against row_kernel: 16-bit softmax and RMSNorm 0.34 of its rate at
+    // two cells a run, 0.9 at nine, 1.1 to 2.5 above; 0.23 where words outnumber cells twice; statistics and f32 turn earlier.
+    const int64_t n = a.x.extent[a.x.rank - 1];
+    constexpr bool DEAR = sizeof(T) == 2 && !(OP == ROW_SUMSQ || OP == ROW_MAX || OP == ROW_EXPSUM);   // eight cells to convert, twice
+    if (2 * n < (DEAR ? 16 : 7) * (int64_t)runs || 10 * all > (DEAR && n <= 2048 ? 6 : 9) * n) return false;
     // few words a thread (their loads are what is in flight), but no smaller teams than a warp
     int team = 32;
     while (team < 256 && all > (int64_t)team * 2) team *= 2;
@@ -679,7 +679,8 @@ bool launch_row_words_op(RowOp op, const RowArgs& a, int64_t n_rows, cudaStream_
     return false;
 }
 
-// what the word form does not take: aligned rows in irregular blocks, rotations (a pair never straddles two vectors), and rows too long
+// What the word form does not take: uniform blocks of whole words, rotations (a pair never straddles two vectors), rows of more
+// words than it holds, of short runs or of runs of very different widths.
 template <typename T, int VEC, int OP>
 ja_status_t launch_row_t(const RowArgs& a, int64_t n_rows, int64_t n, cudaStream_t st) {
     // team: the smallest power of two (32..256) that keeps at most 4 vectors per thread (few registers, many
@@ -689,12 +690,11 @@ ja_status_t launch_row_t(const RowArgs& a, int64_t n_rows, int64_t n, cudaStream
     int64_t vpt = (n + (int64_t)team * VEC - 1) / ((int64_t)team * VEC);
     const int rpc = 256 / team;
     unsigned grid = (unsigned)((n_rows + rpc - 1) / rpc);
-    if (VEC == 1) row_kernel<T, VEC, 0, OP><<<grid, 256, 0, st>>>(a, n_rows, team);   // longer than the word form holds
-    else if (vpt <= 1) row_kernel<T, VEC, VEC == 1 ? 0 : 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 2) row_kernel<T, VEC, VEC == 1 ? 0 : 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 4) row_kernel<T, VEC, VEC == 1 ? 0 : 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 8) row_kernel<T, VEC, VEC == 1 ? 0 : 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 16 && VEC > 1) row_kernel<T, VEC, VEC == 1 ? 0 : 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    if (vpt <= 1) row_kernel<T, VEC, 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 2) row_kernel<T, VEC, 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 4) row_kernel<T, VEC, 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 8) row_kernel<T, VEC, 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    else if (vpt <= 16 && VEC > 1) row_kernel<T, VEC, 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
     else row_kernel<T, VEC, 0, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
@@ -761,8 +761,8 @@ ja_status_t launch_row_typed(RowOp op, const RowArgs& a, cudaStream_t st) {
     int vec = 1;
     if (a.x.bs[last] != 0 && a.x.bs[last] % full == 0 && n % full == 0) vec = full;
     else if (op == ROW_ROPE) vec = 2;
-    // rows that are whole words anyway are better off with row_kernel's fewer, fuller threads (32 x 59 x 1792 f32: three calls 28 us, 36
-    // as masked words)
+    // rows of uniform blocks of whole words are better off with row_kernel's fewer, fuller threads (32 x 59 x 1792 f32: three calls
+    // 28 us, 36 as masked words)
     if (vec == 1 && launch_row_words_op<T>(op, a, n_rows, st)) {
         ja_count_launch();
         JA_CUDA(cudaGetLastError());

@@ -19,7 +19,9 @@ EPS = 1e-5
 
 CASES = [((5, 1), ES(5, 1), ES(1, 1)), ((9, 7), ES(9, 2), ES(7, 3)), ((33, 139), ES(33, 4), ES(139, 4)), ((40, 903), ES(40, 3), [0, 1, 500, 903]),
          ((17, 13676), ES(17, 1), ES(13676, 1)), ((6, 16001), ES(6, 2), ES(16001, 8)), ((64, 3239), ES(64, 2), ES(3239, 1)),
-         ((12, 96), [0, 5, 12], ES(96, 1)), ((50, 260), ES(50, 1), list(range(0, 261, 20))), ((3, 33001), ES(3, 1), ES(33001, 2))]
+         ((12, 96), [0, 5, 12], ES(96, 1)), ((50, 260), ES(50, 1), list(range(0, 261, 20))), ((3, 33001), ES(3, 1), ES(33001, 2)),
+         ((21, 2000), ES(21, 2), [0, 1000, *range(1010, 2001, 10)]),       # more words than a CTA holds, counted by the widest run
+         ((9, 800), ES(9, 1), [*range(0, 800, 3), 800]), ((9, 800), ES(9, 2), list(range(0, 801, 8))), ((9, 660), ES(9, 1), [0, 300, *range(309, 661, 9)])]
 
 
 @pytest.mark.parametrize("shape,si_,sj", CASES)
