@@ -24,7 +24,7 @@
 // What bounds it: the loaders' instruction stream (one trip of a stage through it, 0.36 to 0.51 us by itself for BN = 64 to
 // 256; 0.24 to 0.51 us per stage of a full SM), on short tiles the start and the store of a CTA. Measured, us per call, against the
 // block-bound loader form and the cell-by-cell kernel that this one took the place of:
-//   [2048, 11008] x [11008, 4096] bf16, k cut 64 ways (8-byte pieces)       467 -> 255 (720 TFLOP/s); one block a side 376 -> 175
+//   [2048, 11008] x [11008, 4096] bf16, k cut 64 ways (8-byte pieces)       467 -> 282 (655 TFLOP/s); one block a side 376 -> 175
 //   [32, 4096] x [4096, 11008] bf16                 (TMA form, 48 tiles)    61.5 -> 30 (of 14 at the copy rate)
 //   "bij,bkj->bik" 32 x 512 x 128 x 512 bf16, indices cut in four           19310 -> 18
 //   [154, 8768] x [8768, 3627] f16, odd columns cut in two                  593 -> 108
@@ -91,14 +91,6 @@ struct Ring {
 
 __device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
     return make_uint4(v[0] | (uint32_t)v[1] << 16, v[2] | (uint32_t)v[3] << 16, v[4] | (uint32_t)v[5] << 16, v[6] | (uint32_t)v[7] << 16);
-}
-// Eight cells from an even byte offset sh (0..14) on in the two words lo, hi
-__device__ __forceinline__ uint4 shift16(const uint4& lo, const uint4& hi, int sh) {
-    const bool s8 = sh & 8, s4 = sh & 4;
-    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
-    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
-    const int bits = (sh & 2) * 8;
-    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
 }
 
 // The walk of one loader group (TH threads for RT rows x 64 contracted cells per stage, NP 16-byte pieces per thread).
@@ -218,7 +210,7 @@ __device__ __forceinline__ void load_walk(const Rel& o, const BatchAt& ba, uint3
 #pragma unroll
         for (int n = 0; n < NP; ++n) {
             const int m = sh >> (4 * n) & 15;
-            if (m > 1) st_shared16(at + n * DSTEP, shift16(ld_shared16(at + n * DSTEP), ld_shared16(at + HI + n * DSTEP), m));
+            if (m > 1) st_shared16(at + n * DSTEP, ja_shift16(ld_shared16(at + n * DSTEP), ld_shared16(at + HI + n * DSTEP), m));
         }
     };
     for (int ch = c0; ch < c1; ++ch) {
@@ -515,7 +507,10 @@ __device__ __forceinline__ void tile_range(const Dim& d, int cut, int width, int
     }
 }
 
-template <int BN, bool RAW>
+// ACC accumulators: the product of 16 contracted cells q, q + ACC, q + 2 ACC, ... of the slice go to accumulator q, and the f32 sums of the
+// accumulators are taken in registers. The tensor core truncates as it accumulates, so its error grows with the number of
+// products in a chain; a 16-bit output's rounding hides that (ACC = 1), an f32 output shows it (ACC = 4, see ja_contract_tc_plan).
+template <int BN, bool RAW, int ACC>
 __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_SM) contract_tc_kernel(const __grid_constant__ Params p) {
     using C = Cfg<BN, RAW>;
     extern __shared__ uint8_t smem_raw[];
@@ -553,7 +548,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == MMA_WARP) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(BN) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(BN * ACC) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -585,8 +580,8 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
             const uint32_t a_addr = base + stage * C::STAGE_BYTES, b_addr = a_addr + C::A_BYTES;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-                umma_bf16_w<1>(tmem, desc_sw128(a_addr + kk * a_step, a_lbo), desc_sw128(b_addr + kk * b_step, b_lbo), idesc,
-                               (ch > c0 || kk > 0) ? 1u : 0u, leader);
+                umma_bf16_w<1>(tmem + kk % ACC * BN, desc_sw128(a_addr + kk * a_step, a_lbo), desc_sw128(b_addr + kk * b_step, b_lbo), idesc,
+                               (ch > c0 || kk >= ACC) ? 1u : 0u, leader);
             umma_commit_w<1>(ring.empty0 + 8u * stage, leader);
             if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
         }
@@ -609,6 +604,14 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
             uint32_t v[32];
             tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + cc, v);
             tmem_ld_wait();
+#pragma unroll
+            for (int acc = 1; acc < ACC; ++acc) {
+                uint32_t w[32];
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + acc * BN + cc, w);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
+            }
             if (split == 1) {
                 if (n_minor) {
 #pragma unroll
@@ -645,17 +648,17 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     }
     // ---- teardown ----
     __syncthreads();
-    if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(BN) : "memory");
+    if (warp == MMA_WARP) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(BN * ACC) : "memory");
 }
 
 // ---- host -----------------------------------------------------------------------------------------------------
-template <int BN, bool RAW>
+template <int BN, bool RAW, int ACC>
 ja_status_t launch(const Params& p, cudaStream_t st) {
     static bool configured[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (!configured[dev & 63]) {
-        JA_CUDA(cudaFuncSetAttribute(contract_tc_kernel<BN, RAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN, RAW>::SMEM));
+        JA_CUDA(cudaFuncSetAttribute(contract_tc_kernel<BN, RAW, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN, RAW>::SMEM));
         configured[dev & 63] = true;
     }
     cudaLaunchConfig_t cfg;
@@ -671,7 +674,7 @@ ja_status_t launch(const Params& p, cudaStream_t st) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.split > 1 ? 1 : 0;
-    JA_CUDA(cudaLaunchKernelEx(&cfg, contract_tc_kernel<BN, RAW>, p));
+    JA_CUDA(cudaLaunchKernelEx(&cfg, contract_tc_kernel<BN, RAW, ACC>, p));
     return JA_OK;
 }
 
@@ -734,8 +737,16 @@ ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, co
         *tiles = cut;
         return (int)per;
     };
+    // f32 output: four accumulators (256 of the SM's 512 tensor-memory columns for each of two CTAs of 64-column tiles), and slices short
+    // enough, where a cluster can be that large, that a chain is 256 cells (bf16) or 128 (f16, whose products have more bits to lose).
+    // Error against 64 bits, normal operands, 512 / 2048 contracted cells: bf16 1.2e-7 / 2.3e-7 (one accumulator 4.7e-7 / 2.1e-6; f32 FMAs
+    // one after the other 1.6e-7 / 3.9e-7), f16 1.9e-7 / 1.9e-7 (6.4e-7 / 2.5e-6; 4.0e-7 / 8.0e-7). "bij,bkj->bik" 32 x 512 x 512 x 512
+    // 31 -> 43 us; 8 x 128 x 256 x 512 9.7 -> 9.9.
+    const bool f32_out = C->dtype == JA_F32;
+    int least = 1;
+    while (f32_out && least < 8 && chunks > (p.f16 ? 8 : 16) * least) least *= 2;
     for (int bn : {64, 128, 256}) {
-        if (raw && bn == 256) continue;
+        if ((raw && bn == 256) || (f32_out && bn != 64)) continue;
         const int per_sm = bn == 256 || raw ? 1 : 2;
         const double busy = bn == 256 ? 0.51 : bn == 128 ? 0.29 : 0.235, alone = raw ? 1.3 : bn == 256 ? 0.51 : bn == 128 ? 0.46 : 0.36;
         const double fixed = bn == 256 ? 6.0 : bn == 128 ? 4.5 : 3.5;
@@ -743,6 +754,7 @@ ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, co
         cut_of(p.A, rel_a, t_a, m, BM, &tm);
         cut_of(p.B, rel_b, t_b, n, bn, &tn);
         for (int s : {1, 2, 4, 8}) {
+            if (s < least) continue;
             if (s > 1 && chunks < 4 * s) break;
             const int64_t ctas = nb * tm * tn * s, slots = (int64_t)sms * per_sm * (s > 1 ? 4 : 5) / 5;   // clusters do not pack a GPC fully
             const int64_t waves = (ctas + slots - 1) / slots, last = ctas - (waves - 1) * slots, on_sm = (waves - 1) * per_sm + (last + sms - 1) / sms;
@@ -771,8 +783,9 @@ ja_status_t ja_launch_contract_tc(const ContractTcPlan& plan, cudaStream_t st) {
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
     ja_status_t s;
-    if (plan.raw) s = plan.bn == 64 ? launch<64, true>(p, st) : launch<128, true>(p, st);
-    else s = plan.bn == 64 ? launch<64, false>(p, st) : plan.bn == 128 ? launch<128, false>(p, st) : launch<256, false>(p, st);
+    if (plan.p.c_esize == 4) s = plan.raw ? launch<64, true, 4>(p, st) : launch<64, false, 4>(p, st);
+    else if (plan.raw) s = plan.bn == 64 ? launch<64, true, 1>(p, st) : launch<128, true, 1>(p, st);
+    else s = plan.bn == 64 ? launch<64, false, 1>(p, st) : plan.bn == 128 ? launch<128, false, 1>(p, st) : launch<256, false, 1>(p, st);
     if (s == JA_OK) ja_count_launch();
     return s;
 }

@@ -83,3 +83,21 @@ def test_nothing_leaks_from_rows_that_do_not_exist():
     ja.Spec("ij,jk->ik", {"i": one(m), "j": one(k), "k": one(n)}, "mul", (), "sum").execute([ra, rb], res)
     assert relfro(download(res), si.to_f64(a) @ si.to_f64(b)) <= TOL[BF]
     check_status()
+
+
+@pytest.mark.parametrize("K", [64, 200, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_an_f32_output_is_as_exact_as_f32_sums(K, dtype):
+    """Products of 16-bit cells are exact in f32; the tensor core's sums of them may be no further from fp64 than adding them one after
+    the other in f32 (a quarter more for the scatter of one sample)."""
+    a, b = si.normal((2, 48, K), 0.0, 1.0, dtype, 31, 60), si.normal((2, 40, K), 0.0, 1.0, dtype, 31, 61)
+    cuts = {"b": ES(2, 2), "i": ES(48, 1), "j": ES(K, 2), "k": ES(40, 1)}
+    res = empty_like_tiling([2, 48, 40], [cuts[c] for c in "bik"], F32, fill=float("nan"))
+    ja.Spec("bij,bkj->bik", cuts, "mul", (), "sum").execute([upload(a, [cuts[c] for c in "bij"]), upload(b, [cuts[c] for c in "bkj"])], res)
+    a64, b64 = si.to_f64(a), si.to_f64(b)
+    ref = np.einsum("bij,bkj->bik", a64, b64)
+    one_by_one = np.zeros((2, 48, 40), np.float32)
+    for j in range(K):
+        one_by_one += (a64[:, :, None, j] * b64[:, None, :, j]).astype(np.float32)
+    assert relfro(download(res), ref) <= 1.25 * relfro(one_by_one.astype(np.float64), ref)
+    check_status()
