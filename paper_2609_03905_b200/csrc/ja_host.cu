@@ -656,7 +656,7 @@ extern "C" ja_status_t ja_overlay_atoms(const ja_relation_t* src, const ja_relat
 }
 
 struct RepartPlan {
-    std::vector<CopySlab> slabs;         // until d_slabs holds them
+    std::vector<CopySlab> slabs;         // n_slabs of them, and as many more as a launch by parameters may read; until d_slabs holds them
     CopySlab* d_slabs = nullptr;         // device table of more than JA_PARAM_SLABS slabs
     bool long_rows = false;              // rows of 256 bytes and more
     int64_t n_slabs = 0;
@@ -739,6 +739,8 @@ static std::shared_ptr<RepartPlan> plan_repartition(const ja_relation* src, cons
         rows += c.rows;
     }
     plan->long_rows = bytes >= 256 * rows;
+    const int last = (int)(plan->n_slabs % JA_PARAM_SLABS);
+    plan->slabs.resize((size_t)(plan->n_slabs - last + (last ? ja_param_capacity(last) : 0)), CopySlab{});
     return plan;
 }
 static ja_status_t launch_slabs_by_parameters(const RepartPlan& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t st) {
@@ -773,13 +775,13 @@ static ja_status_t run_repartition(const std::shared_ptr<RepartPlan>& plan, cons
             if (cap != cudaStreamCaptureStatusNone && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES)
                 return launch_slabs_by_parameters(*plan, src, dst, stream);   // a capture allows no allocation
             CopySlab* table = nullptr;
-            cudaError_t e = cudaMalloc((void**)&table, plan->slabs.size() * sizeof(CopySlab));
+            cudaError_t e = cudaMalloc((void**)&table, plan->n_slabs * sizeof(CopySlab));
             if (e == cudaErrorMemoryAllocation && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES) {
                 cudaGetLastError();   // no memory left for a table: slower, but it runs
                 return launch_slabs_by_parameters(*plan, src, dst, stream);
             }
             if (e != cudaSuccess) return ja_cuda_fail(e, "cudaMalloc(copy slabs)");
-            e = cudaMemcpy(table, plan->slabs.data(), plan->slabs.size() * sizeof(CopySlab), cudaMemcpyHostToDevice);
+            e = cudaMemcpy(table, plan->slabs.data(), plan->n_slabs * sizeof(CopySlab), cudaMemcpyHostToDevice);
             if (e != cudaSuccess) {
                 cudaFree(table);
                 return ja_cuda_fail(e, "cudaMemcpy(copy slabs)");

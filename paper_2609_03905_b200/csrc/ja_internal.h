@@ -165,8 +165,10 @@ struct CopySlab {
 };
 ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int vec_bytes, bool long_rows,
                                   cudaStream_t st);
-// the same with the slabs in the kernel's parameters: n_slabs <= JA_PARAM_SLABS, host pointer, read before the call returns
+// the same with the slabs in the kernel's parameters: n_slabs <= JA_PARAM_SLABS, host pointer to ja_param_capacity(n_slabs) readable
+// slabs, read before the call returns
 #define JA_PARAM_SLABS 960
+inline int ja_param_capacity(int n_slabs) { return n_slabs <= 16 ? 16 : n_slabs <= 64 ? 64 : n_slabs <= 192 ? 192 : n_slabs <= 448 ? 448 : JA_PARAM_SLABS; }
 ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, bool long_rows,
                                         cudaStream_t st);
 // Aggregating relayout: every slab is read from n_copies copies of the source, copy_stride bytes apart, (+)-combined

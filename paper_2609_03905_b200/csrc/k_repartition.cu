@@ -12,7 +12,6 @@
 // once (packing a dense tensor, unpacking a result), in the parameters of several launches: 0.4 ms less than a table's allocation
 // and copy, but 20 to 30 % slower per call than one launch with a table (134 MB: 59 against 47 us, the ends of three launches).
 // Both move a slab by the same rule (copy_of).
-#include <string.h>
 
 #include "ja_device.cuh"
 
@@ -28,14 +27,6 @@ __device__ __forceinline__ void copy_slab(const char* __restrict__ sp, char* __r
         const V v = *reinterpret_cast<const V*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * sizeof(V));
         *reinterpret_cast<V*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * sizeof(V)) = v;
     }
-}
-
-__device__ __forceinline__ uint4 shifted(const uint4& lo, const uint4& hi, int sh) {   // 16 bytes from byte sh (0..15, even) of lo:hi on
-    const bool s8 = sh & 8, s4 = sh & 4;
-    const uint32_t a0 = s8 ? lo.z : lo.x, a1 = s8 ? lo.w : lo.y, a2 = s8 ? hi.x : lo.z, a3 = s8 ? hi.y : lo.w, a4 = s8 ? hi.z : hi.x, a5 = s8 ? hi.w : hi.y;
-    const uint32_t b0 = s4 ? a1 : a0, b1 = s4 ? a2 : a1, b2 = s4 ? a3 : a2, b3 = s4 ? a4 : a3, b4 = s4 ? a5 : a4;
-    const int bits = (sh & 2) * 8;
-    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits), __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
 }
 
 // One slab at any even alignment. Word w of row r is the w-th aligned 16-byte word that the row touches in the destination. Only
@@ -58,7 +49,7 @@ __device__ __forceinline__ void copy_slab_any(const char* __restrict__ sp, char*
             uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
             if (need_lo) lo = q[0];
             if (need_hi) hi = q[1];
-            const uint4 v = shifted(lo, hi, sh);
+            const uint4 v = ja_shift16(lo, hi, sh);
             if (at >= 0 && at + 16 <= sl.row_bytes) {
                 *reinterpret_cast<uint4*>(d + at) = v;
             } else {
@@ -108,16 +99,21 @@ __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __re
     const CopySlab& sl = p.s[blockIdx.x];
     copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
 }
+// The launch reads the parameters where they lie (a struct by value is copied twice before the driver copies it: 1.0 to 1.6 us of a call).
+template <int HOW, int N>
+void launch_param_n(const char* src, char* dst, const CopySlab* slabs, int n, cudaStream_t st) {
+    void* args[] = {&src, &dst, const_cast<CopySlab*>(slabs)};
+    cudaLaunchKernel(reinterpret_cast<const void*>(repartition_param_kernel<N, HOW>), dim3((unsigned)n), dim3(256), args, 0, st);
+}
 template <int HOW>
 void launch_param(const char* src, char* dst, const CopySlab* slabs, int n, cudaStream_t st) {
-    auto go = [&](auto p) {
-        constexpr int N = (int)(sizeof p.s / sizeof p.s[0]);
-        memcpy(p.s, slabs, (size_t)n * sizeof(CopySlab));
-        repartition_param_kernel<N, HOW><<<n, 256, 0, st>>>(src, dst, p);
-    };
-    if (n <= 32) go(SlabParams<32>());
-    else if (n <= 256) go(SlabParams<256>());
-    else go(SlabParams<JA_PARAM_SLABS>());
+    switch (ja_param_capacity(n)) {
+        case 16: launch_param_n<HOW, 16>(src, dst, slabs, n, st); break;
+        case 64: launch_param_n<HOW, 64>(src, dst, slabs, n, st); break;
+        case 192: launch_param_n<HOW, 192>(src, dst, slabs, n, st); break;
+        case 448: launch_param_n<HOW, 448>(src, dst, slabs, n, st); break;
+        default: launch_param_n<HOW, JA_PARAM_SLABS>(src, dst, slabs, n, st); break;
+    }
 }
 template <int HOW>
 void launch_table(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, cudaStream_t st) {
