@@ -452,7 +452,7 @@ __device__ __forceinline__ float row_max128(const uint32_t (&v)[128]) {
 }
 
 // 2^x for a pair of exponents on the FMA pipe (no special-function unit): x = n + f with n = round(x), f in [-1/2, 1/2];
-// 2^f by a cubic fitted to a relative error of 7.5e-5 (bf16 keeps 8 bits of P); n is added to the exponent field. x is
+// 2^f by a cubic fitted to a relative error of 7.5e-5 (P is rounded to 2^-9 in bf16, 2^-11 in f16); n is added to the exponent field. x is
 // clamped at -126 so that the exponent field cannot wrap; scores above the offset by more than 2^8 never reach here (lazy
 // rescale keeps x <= 8).
 __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, float& p0, float& p1) {
@@ -476,7 +476,7 @@ __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, float& p0, float& p1
 }
 
 // One row of P = 2^(S * scale - m) for 128 keys as 64 packed bf16 (or f16) pairs in registers; returns the row sum (f32, of the
-// unrounded values); a score of -inf (a masked key) gives exactly 0. POLY: which pairs of every group of eight keys take the
+// unrounded values); a score of -inf (a masked key) gives 0, or 2^-126 by the cubic (its clamp). POLY: which pairs of every group of eight keys take the
 // FMA-pipe exponential instead of ex2 -- 0 none, 1 one of four, 2 two of four, 3 one of eight -- interleaved so that both
 // pipes stay busy.
 template <int POLY, bool F16>
@@ -532,7 +532,7 @@ __device__ __forceinline__ float row_exp_pack128(const uint32_t (&v)[128], float
 // VAR selects row-thread variants ("attn_variant"; all verified against the oracle): bits 0-1 = POLY of row_exp_pack128, bit 2 =
 //   exponentiate into registers first and wait for the P tile only before storing. Default 1: a quarter of the exponentials
 //   on the FMA pipe (B4 S2048 H32 causal, same run: POLY 0 0.1430 ms, one of eight 0.1405, one of four 0.1403, two of four
-//   0.1509; exponentials first 0.1542).
+//   0.1509; exponentials first 0.1542). The ragged form has POLY 0 fixed (its five packed sequences: 109.6 us, POLY 1 111.1).
 // Timing-only ablations of this kernel before the masked loops were merged (B4 S2048 H32 causal, 0.163 ms on the box of
 //   that run): no P stores -6 %, no exponentials -7 %, QK^T or P V reduced to one instruction of eight -6 % / 0 %, no K / V
 //   loads -10 %, no output stage -3 %; all of them together still left 0.067 ms: the row threads' own instruction stream (two
@@ -581,7 +581,7 @@ __device__ int32_t g_attn_queues[2 * ATTN_QUEUES];
 // start anywhere; what a box brings past a tile's rows is masked (scores), not multiplied (whole 16-key groups of V), zeroed in
 // shared memory (the rest of the last group) or not stored. The cost against whole tiles is the masks and the empty parts of the
 // last tiles. Measured, us, against the mma.sync kernel it took these from (48 to 60 TFLOP/s there, 600 to 980 here):
-//   five packed f16 sequences, 6001 rows, 32 / 8 heads     1413 -> 101      2 x 6080 rows in 64-row blocks, 8 heads   1525 -> 310
+//   five packed f16 sequences, 6001 rows, 32 / 8 heads     1413 -> 110      2 x 6080 rows in 64-row blocks, 8 heads   1525 -> 310
 //   one sequence of 684 rows, 4 heads                        97 -> 18       2 x 3473 rows, 8 heads                     855 -> 61
 // and against the one-tile kernel where blocks are whole tiles: 4 x 896 rows, 32 heads 101 -> 48, 16 x 128 rows 31.6 -> 22.8,
 // 1 x 128 rows, 16 heads 8.4 -> 8.1.
@@ -938,7 +938,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(S_FREE + t));   // S_t is in registers: the next Q K^T of this tile may run
-                if (diag) {   // Keys after the query row score -inf: they lose every maximum and exponentiate to exactly 0, so ONE copy of
+                if (diag) {   // Keys after the query row score -inf: they lose every maximum and exponentiate to 0 (or 2^-126), so ONE copy of
                               // the maximum / exponential code serves masked and unmasked tiles. (A masked variant of both loops --
                               // a select per score inside them, the maximum as one chain of 128 dependent selects -- cost 12 % of
                               // the kernel on B4 S2048: the chain sits on every item's critical path, and the second copy of the
@@ -1083,7 +1083,7 @@ __global__ void __launch_bounds__(NUM_THREADS2, 1)
 attention_ragged_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                         const __grid_constant__ AttnTcParams p, const __grid_constant__ RaggedTiles rt) {
-    // every exponential by ex2 (2^-22): the cubic of the other forms (7.5e-5) is coarser than f16's half ulp of P and shows in lse
+    // every exponential by ex2 (2^-22), as the mma.sync form has them: the cubic of the other forms (7.5e-5) shows in lse, which is f32
     attention_tc2<true, 0, F16, true>(tmQ, tmK, tmV, tmO, p, &rt);
 }
 
@@ -1215,17 +1215,18 @@ bool list_ragged_tiles(const AttnArgs& a, RaggedTiles* rt) {
     rt->lse = a.lse;
     struct Item { int q, k, n_a, n_b; };
     std::vector<Item> items;
-    for (size_t i = 0; i < ends.size(); ++i)
+    for (size_t i = 0; i < ends.size(); ++i) {
+        int n_keys = 0;
         for (int q = q_first[i]; q < q_first[i + 1]; q += 2) {
-            auto joined = [&](int t) {       // key tiles of this sequence that start no later than the tile's last row
-                if (!a.causal) return k_first[i + 1] - k_first[i];
-                const int last = (int)(rt->q[t] & 0xffffffu) + (int)(rt->q[t] >> 24);
-                int n = 0;
-                while (k_first[i] + n < k_first[i + 1] && (int)(rt->k[k_first[i] + n] & 0xffffffu) <= last) ++n;
-                return n;
+            auto joined = [&](int t) {       // key tiles of this sequence that start no later than the tile's last row; t only grows
+                const int last = (int)(rt->q[t] & 0xffffffu) + (int)(rt->q[t] >> 24), all = k_first[i + 1] - k_first[i];
+                while (n_keys < all && (!a.causal || (int)(rt->k[k_first[i] + n_keys] & 0xffffffu) <= last)) ++n_keys;
+                return n_keys;
             };
-            items.push_back({q, k_first[i], joined(q), q + 1 < q_first[i + 1] ? joined(q + 1) : 0});
+            const int n_a = joined(q), n_b = q + 1 < q_first[i + 1] ? joined(q + 1) : 0;
+            items.push_back({q, k_first[i], n_a, n_b});
         }
+    }
     if ((int)items.size() > MAX_ITEMS) return false;
     std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.n_a + x.n_b > y.n_a + y.n_b; });
     for (size_t i = 0; i < items.size(); ++i) {
