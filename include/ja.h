@@ -175,8 +175,9 @@ ja_status_t ja_relation_get_keys(const ja_relation_t* rel, int32_t* coords, int6
  *                                                          Q, K, V, O of one 16-bit dtype (bf16 or f16; the probabilities
  *                                                          enter the second product rounded to that dtype)
  *   any other einsum       MUL | ADD | IDENT | SQUARE | SILU_MUL | EXP_SUB with SUM | MAX | NONE: up to four operands
- *                          and four summed indices, any tilings and dtypes -- Definition 3.7 executed cell by cell (one
- *                          thread per output cell walks its joined tuples in ascending order): complete, not fast
+ *                          and four summed indices, any tilings and dtypes. Products (MUL / SUM) of two relations of one
+ *                          dtype with one contracted index, batched or transposed, run on contraction kernels; everything
+ *                          else is Definition 3.7 executed cell by cell, a cell's joined tuples shared by lanes, warps and CTAs
  * n_outputs is 1, except for ATTENTION where it may be 2: outputs[1] then receives lse[b, q, h] = log of the softmax
  * denominator of every query row (f32, tiled like the first three indices of outputs[0]) -- with it two results over
  * disjoint key ranges combine by the online-softmax aggregation: O = w1 O1 + w2 O2, w_i = exp(lse_i - lse).
@@ -188,12 +189,13 @@ ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* const* inputs
 /* ---- repartition (Section 5.3: overlay -> atoms, decompose + recompose) ---------------------------
  * Copies the tensor held by `src` into the tiling of `dst` (same rank, extents, dtype): every atom of the
  * overlay of the two tilings moves from its source block to its destination block.  Bit-exact, no
- * aggregation.  Asynchronous on `cuda_stream`. The first call for a pair of relations plans the copy on the host and, where the
- * overlay is cut into more than 960 slabs (of up to 64 KiB), puts the plan into a device table (a synchronous cudaMalloc and
- * cudaMemcpy, about 0.4 ms); later calls only launch. A first call inside a stream capture makes no table (up to 7680 slabs). */
+ * aggregation.  Asynchronous on `cuda_stream`. The first call for a pair of relations plans the copy on the host. Where one launch
+ * can carry the plan in its parameters (up to 960 slabs of up to 64 KiB of the overlay) it does, and the second call copies a
+ * table for its stream without waiting; otherwise the first call makes a table (a synchronous cudaMalloc and cudaMemcpy, about
+ * 0.4 ms; inside a stream capture, and where no memory is left: up to eight launches by parameters instead). Later calls only launch. */
 ja_status_t ja_repartition(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream);
-/* The same for two relations that meet once: nothing is kept and, up to 7680 slabs, nothing is allocated on the device (one launch
- * per 960 slabs). */
+/* The same for two relations that meet once: nothing is kept and, up to 7680 slabs, nothing is allocated on the device (a launch per
+ * 960 slabs). */
 ja_status_t ja_repartition_once(const ja_relation_t* src, ja_relation_t* dst, void* cuda_stream);
 /* Overlay introspection (host, no CUDA): number of atoms, then per atom lower[rank], upper[rank],
  * flat source block, flat destination block.  Pass NULL arrays to query the count only. */

@@ -1681,13 +1681,14 @@ extern "C" ja_status_t ja_exchange_combine(const void* const* parts, int32_t n_p
     return ja_launch_exchange_combine(parts, n_parts, out, bytes, dtype, agg, (cudaStream_t)cuda_stream);
 }
 
-// Scratch of ja_exchange_execute: a stream-ordered pool of the library's own per device that keeps what it has been given
+// Scratch of ja_exchange_execute and small tables of relayouts: a stream-ordered pool of the library's own per device that keeps what it has been given
 // (the default pool hands memory back to the driver at every synchronisation, and getting a gigabyte again costs milliseconds);
 // ja_exchange_trim returns it.
 namespace {
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
-ja_status_t exchange_pool(cudaMemPool_t* out) {
+}  // namespace
+ja_status_t ja_library_pool(cudaMemPool_t* out) {
     int dev = 0;
     JA_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1708,7 +1709,6 @@ ja_status_t exchange_pool(cudaMemPool_t* out) {
     *out = it->second;
     return JA_OK;
 }
-}  // namespace
 
 extern "C" ja_status_t ja_exchange_trim(void) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -1952,7 +1952,7 @@ extern "C" ja_status_t ja_exchange_execute(const ja_exprog_t* prog, const ja_rel
     }
     char* pool = nullptr;
     cudaMemPool_t mp = nullptr;
-    if ((st = exchange_pool(&mp)) != JA_OK) return st;
+    if ((st = ja_library_pool(&mp)) != JA_OK) return st;
     JA_CUDA(cudaMallocFromPoolAsync((void**)&pool, (size_t)B.scratch, mp, stream));
     ja_status_t rc = JA_OK;
     do {

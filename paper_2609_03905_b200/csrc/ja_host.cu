@@ -656,13 +656,18 @@ extern "C" ja_status_t ja_overlay_atoms(const ja_relation_t* src, const ja_relat
 }
 
 struct RepartPlan {
-    std::vector<CopySlab> slabs;         // n_slabs of them, and as many more as a launch by parameters may read; until d_slabs holds them
-    CopySlab* d_slabs = nullptr;         // device table of more than JA_PARAM_SLABS slabs
+    std::unique_ptr<SlabChunk> chunk;    // all slabs, where the parameters of one launch hold them
+    std::vector<CopySlab> slabs;         // until d_slabs holds them
+    CopySlab* d_slabs = nullptr;         // device table: of more slabs than that on any stream, else on stream `home` alone
+    unsigned long long home = 0;         // the stream (id) that d_slabs was copied on, where there is a chunk
+    bool seen = false, no_table = false; // (with a chunk) launched before; a table could not be had
     bool long_rows = false;              // rows of 256 bytes and more
     int64_t n_slabs = 0;
     int vec_bytes = 16;
     ~RepartPlan() {
-        if (d_slabs) cudaFree(d_slabs);
+        if (!d_slabs) return;
+        if (chunk) cudaDeviceSynchronize();   // pooled memory is handed out again at once
+        cudaFree(d_slabs);
     }
 };
 static std::mutex g_repart_mu;
@@ -726,6 +731,26 @@ static void plan_slabs(const ja_relation* src, const ja_relation* dst, std::vect
     }
 }
 
+// Slabs from *at on, as many as the parameters of one launch hold; false where one does not fit them at all.
+static bool fill_chunk(const std::vector<CopySlab>& slabs, size_t* at, SlabChunk* c) {
+    int n_shapes = 0;
+    c->n = 0;
+    for (; *at < slabs.size() && c->n < JA_PARAM_SLABS; ++*at) {
+        const CopySlab& s = slabs[*at];
+        const int64_t most = 2ll * UINT32_MAX;
+        if (s.src_off > most || s.dst_off > most || ((s.src_off | s.dst_off) & 1) || s.rows > UINT16_MAX) return false;
+        int shape = n_shapes - 1;   // neighbours are alike
+        auto is = [&](const SlabShape& h) { return h.row_bytes == s.row_bytes && h.src_pitch == s.src_pitch && h.dst_pitch == s.dst_pitch; };
+        while (shape >= 0 && !is(c->p.shapes[shape])) --shape;
+        if (shape < 0) {
+            if (n_shapes == JA_PARAM_SHAPES) return true;
+            shape = n_shapes++;
+            c->p.shapes[shape] = {s.row_bytes, s.src_pitch, s.dst_pitch};
+        }
+        c->p.s[c->n++] = {(uint32_t)(s.src_off / 2), (uint32_t)(s.dst_off / 2), (uint16_t)s.rows, (uint16_t)shape};
+    }
+    return true;
+}
 static std::shared_ptr<RepartPlan> plan_repartition(const ja_relation* src, const ja_relation* dst) {
     std::shared_ptr<RepartPlan> plan(new RepartPlan());
     int64_t src_or = 0, dst_or = 0;
@@ -739,14 +764,29 @@ static std::shared_ptr<RepartPlan> plan_repartition(const ja_relation* src, cons
         rows += c.rows;
     }
     plan->long_rows = bytes >= 256 * rows;
-    const int last = (int)(plan->n_slabs % JA_PARAM_SLABS);
-    plan->slabs.resize((size_t)(plan->n_slabs - last + (last ? ja_param_capacity(last) : 0)), CopySlab{});
+    if (plan->n_slabs <= JA_PARAM_SLABS) {
+        plan->chunk.reset(new SlabChunk);   // (not cleared: 12 KiB)
+        size_t at = 0;
+        if (!fill_chunk(plan->slabs, &at, plan->chunk.get()) || at < plan->slabs.size()) plan->chunk.reset();
+    }
     return plan;
 }
-static ja_status_t launch_slabs_by_parameters(const RepartPlan& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t st) {
-    for (int64_t at = 0; at < plan.n_slabs; at += JA_PARAM_SLABS) {
-        const ja_status_t s = ja_launch_repartition_param((const char*)src->base, (char*)dst->base, plan.slabs.data() + at,
-                                                          (int)std::min<int64_t>(JA_PARAM_SLABS, plan.n_slabs - at), plan.vec_bytes, plan.long_rows, st);
+constexpr int PARAM_LAUNCHES = 8;
+// By parameters: one launch, or a few of them that are filled here. *fits = false (and nothing launched) where a few are not enough.
+static ja_status_t launch_by_parameters(const RepartPlan& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t st, bool* fits) {
+    *fits = true;
+    auto launch = [&](const SlabChunk& c) {
+        return ja_launch_repartition_param((const char*)src->base, (char*)dst->base, c, plan.vec_bytes, plan.long_rows, st);
+    };
+    if (plan.chunk) return launch(*plan.chunk);
+    std::vector<std::unique_ptr<SlabChunk>> chunks;
+    for (size_t at = 0; at < plan.slabs.size();) {
+        if (chunks.size() == PARAM_LAUNCHES) { *fits = false; return JA_OK; }
+        chunks.emplace_back(new SlabChunk);
+        if (!fill_chunk(plan.slabs, &at, chunks.back().get())) { *fits = false; return JA_OK; }
+    }
+    for (const auto& c : chunks) {
+        const ja_status_t s = launch(*c);
         if (s != JA_OK) return s;
     }
     return JA_OK;
@@ -756,29 +796,66 @@ static ja_status_t check_repartition(const ja_relation* src, const ja_relation* 
     if (st != JA_OK) return st;
     return src->base == dst->base ? ja_fail(JA_ERR_INVALID_ARG, "repartition in place is not supported") : JA_OK;
 }
-constexpr int64_t SLABS_OF_A_FEW_LAUNCHES = 8 * JA_PARAM_SLABS;
-
 // the plan that the pair keeps: the one given, or another thread's where that was first
 static std::shared_ptr<RepartPlan> keep_repartition(const ja_relation* src, const ja_relation* dst, const std::shared_ptr<RepartPlan>& plan) {
     std::lock_guard<std::mutex> lk(g_repart_mu);
     return g_repart_plans.emplace(std::make_pair(src->id, dst->id), plan).first->second;
 }
+// A pair whose slabs fit one launch's parameters: its first call goes by them and allocates nothing. On the GPU both forms take the
+// same time, but the parameters cost the host 0.5 to 3 us a launch, so the second call copies a table on its stream (from the library's
+// pool, without waiting), and calls on that stream read it. Calls on other streams, which nothing orders after the copy, and calls
+// that a capture records, whose replays nothing does, keep to the parameters.
+static ja_status_t run_small_repartition(RepartPlan* plan, const ja_relation* src, const ja_relation* dst, cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    const CopySlab* table = nullptr;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || (cap == cudaStreamCaptureStatusNone && cudaStreamGetId(stream, &id) != cudaSuccess)) {
+        cudaGetLastError();   // the question's own error; the launch will tell
+    } else if (cap == cudaStreamCaptureStatusNone) {
+        std::lock_guard<std::mutex> lk(g_repart_mu);
+        if (plan->seen && !plan->d_slabs && !plan->no_table) {
+            cudaMemPool_t pool = nullptr;
+            void* t = nullptr;
+            const size_t bytes = plan->n_slabs * sizeof(CopySlab);
+            if (ja_library_pool(&pool) == JA_OK && cudaMallocFromPoolAsync(&t, bytes, pool, stream) == cudaSuccess) {
+                if (cudaMemcpyAsync(t, plan->slabs.data(), bytes, cudaMemcpyHostToDevice, stream) == cudaSuccess) {
+                    plan->d_slabs = (CopySlab*)t;
+                    plan->home = id;
+                } else {
+                    cudaFreeAsync(t, stream);
+                }
+            }
+            if (!plan->d_slabs) {
+                plan->no_table = true;
+                cudaGetLastError();
+            }
+            std::vector<CopySlab>().swap(plan->slabs);   // the copy has staged them
+        }
+        plan->seen = true;
+        if (plan->d_slabs && plan->home == id) table = plan->d_slabs;
+    }
+    if (!table) return ja_launch_repartition_param((const char*)src->base, (char*)dst->base, *plan->chunk, plan->vec_bytes, plan->long_rows, stream);
+    return ja_launch_repartition((const char*)src->base, (char*)dst->base, table, plan->n_slabs, plan->vec_bytes, plan->long_rows, stream);
+}
 static ja_status_t run_repartition(const std::shared_ptr<RepartPlan>& plan, const ja_relation* src, const ja_relation* dst, cudaStream_t stream) {
-    // One launch whose parameters hold the slabs is as fast as a table (33 MB in 512 slabs: 10.3 us either way) and needs no memory;
-    // more slabs are read from a table that the pair's FIRST call makes, so that every later one, captured or not, only launches.
-    if (plan->n_slabs <= JA_PARAM_SLABS) return launch_slabs_by_parameters(*plan, src, dst, stream);
+    if (plan->chunk) return run_small_repartition(plan.get(), src, dst, stream);
+    // more slabs are read from a table that the pair's FIRST call makes, so that every later one, captured or not, only launches
+    bool done;
     {
         std::lock_guard<std::mutex> lk(g_repart_mu);
         if (!plan->d_slabs) {
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
             if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusNone;
-            if (cap != cudaStreamCaptureStatusNone && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES)
-                return launch_slabs_by_parameters(*plan, src, dst, stream);   // a capture allows no allocation
+            if (cap != cudaStreamCaptureStatusNone) {   // a capture allows no allocation
+                const ja_status_t s = launch_by_parameters(*plan, src, dst, stream, &done);
+                if (s != JA_OK || done) return s;
+            }
             CopySlab* table = nullptr;
             cudaError_t e = cudaMalloc((void**)&table, plan->n_slabs * sizeof(CopySlab));
-            if (e == cudaErrorMemoryAllocation && plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES) {
-                cudaGetLastError();   // no memory left for a table: slower, but it runs
-                return launch_slabs_by_parameters(*plan, src, dst, stream);
+            if (e == cudaErrorMemoryAllocation) {   // no memory left for a table: slower, but it runs
+                cudaGetLastError();
+                const ja_status_t s = launch_by_parameters(*plan, src, dst, stream, &done);
+                if (s != JA_OK || done) return s;
             }
             if (e != cudaSuccess) return ja_cuda_fail(e, "cudaMalloc(copy slabs)");
             e = cudaMemcpy(table, plan->slabs.data(), plan->n_slabs * sizeof(CopySlab), cudaMemcpyHostToDevice);
@@ -810,7 +887,11 @@ extern "C" ja_status_t ja_repartition_once(const ja_relation_t* src, ja_relation
     const ja_status_t st = check_repartition(src, dst);
     if (st != JA_OK) return st;
     const std::shared_ptr<RepartPlan> plan = plan_repartition(src, dst);
-    if (plan->n_slabs <= SLABS_OF_A_FEW_LAUNCHES) return launch_slabs_by_parameters(*plan, src, dst, (cudaStream_t)cuda_stream);
+    if (plan->n_slabs <= (int64_t)PARAM_LAUNCHES * JA_PARAM_SLABS) {
+        bool done;
+        const ja_status_t s = launch_by_parameters(*plan, src, dst, (cudaStream_t)cuda_stream, &done);
+        if (s != JA_OK || done) return s;
+    }
     return run_repartition(keep_repartition(src, dst, plan), src, dst, (cudaStream_t)cuda_stream);   // the table lives as long as the relations
 }
 

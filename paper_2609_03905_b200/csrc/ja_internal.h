@@ -80,6 +80,7 @@ RelView ja_view(const ja_relation* r);
 // later streams of a device share the last word). nullptr when the table's address cannot be resolved.
 int* ja_device_status_word(cudaStream_t st);
 void ja_count_launch(int n = 1);
+ja_status_t ja_library_pool(cudaMemPool_t* pool);   // stream-ordered memory of the current device that stays with the library until ja_exchange_trim
 int ja_sm_count();   // multiprocessors of the current device (cached per device)
 
 // Switches that force a kernel form or a schedule. Read ONCE from the environment (JA_* variables) when the library is
@@ -165,12 +166,26 @@ struct CopySlab {
 };
 ja_status_t ja_launch_repartition(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int vec_bytes, bool long_rows,
                                   cudaStream_t st);
-// the same with the slabs in the kernel's parameters: n_slabs <= JA_PARAM_SLABS, host pointer to ja_param_capacity(n_slabs) readable
-// slabs, read before the call returns
+// The same with the slabs in the kernel's parameters. A launch with 30 KiB of them costs the host 3.6 us more than one with a table, one
+// with 6 KiB 0.5, so they travel in 12 bytes: offsets in units of two bytes, and what many slabs share in a table of shapes.
 #define JA_PARAM_SLABS 960
-inline int ja_param_capacity(int n_slabs) { return n_slabs <= 16 ? 16 : n_slabs <= 64 ? 64 : n_slabs <= 192 ? 192 : n_slabs <= 448 ? 448 : JA_PARAM_SLABS; }
-ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, bool long_rows,
-                                        cudaStream_t st);
+#define JA_PARAM_SHAPES 64
+struct SlabShape {
+    int32_t row_bytes, src_pitch, dst_pitch;
+};
+struct ParamSlab {
+    uint32_t src, dst;
+    uint16_t rows, shape;
+};
+template <int N> struct SlabParams {
+    SlabShape shapes[JA_PARAM_SHAPES];
+    ParamSlab s[N];
+};
+struct SlabChunk {                       // the slabs of one launch; a launch of fewer reads the front of it
+    SlabParams<JA_PARAM_SLABS> p;
+    int32_t n;
+};
+ja_status_t ja_launch_repartition_param(const char* src, char* dst, const SlabChunk& chunk, int vec_bytes, bool long_rows, cudaStream_t st);
 // Aggregating relayout: every slab is read from n_copies copies of the source, copy_stride bytes apart, (+)-combined
 // in ascending copy order in f32 and stored once. Slab sizes are in SOURCE bytes; destination offsets / pitches in
 // destination bytes. vec = cells per access (8 / 4 for 16-byte accesses of bf16 / f32 sources, or 1).

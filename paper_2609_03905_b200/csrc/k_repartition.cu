@@ -7,7 +7,7 @@
 // around them, and only the ends of a row go cell by cell (12370 rows of 2919 bf16 cells: 81 -> 39 us); short ones go by the
 // widest access their alignment allows.
 //
-// The slabs travel in the kernel's parameters where JA_PARAM_SLABS hold them -- nothing is allocated or copied for a pair of
+// The slabs travel in the kernel's parameters where one launch holds them -- nothing is allocated or copied for a pair of
 // relations, on its first call or any other -- else in a table in device memory that the caller keeps, or, for relations that meet
 // once (packing a dense tensor, unpacking a result), in the parameters of several launches: 0.4 ms less than a table's allocation
 // and copy, but 20 to 30 % slower per call than one launch with a table (134 MB: 59 against 47 us, the ends of three launches).
@@ -91,29 +91,25 @@ __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict
     }
 }
 
-template <int N> struct SlabParams {
-    CopySlab s[N];
-};
 template <int N, int HOW>
 __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __restrict__ src, char* __restrict__ dst, const __grid_constant__ SlabParams<N> p) {
-    const CopySlab& sl = p.s[blockIdx.x];
-    copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
+    const ParamSlab ps = p.s[blockIdx.x];
+    const SlabShape sh = p.shapes[ps.shape];
+    const CopySlab sl = {0, 0, ps.rows, sh.row_bytes, sh.src_pitch, sh.dst_pitch};
+    copy_slab_by<HOW>(src + 2 * (int64_t)ps.src, dst + 2 * (int64_t)ps.dst, sl);
 }
-// The launch reads the parameters where they lie (a struct by value is copied twice before the driver copies it: 1.0 to 1.6 us of a call).
+// The launch reads the parameters where they lie (a struct by value is copied twice before the driver copies it).
 template <int HOW, int N>
-void launch_param_n(const char* src, char* dst, const CopySlab* slabs, int n, cudaStream_t st) {
-    void* args[] = {&src, &dst, const_cast<CopySlab*>(slabs)};
-    cudaLaunchKernel(reinterpret_cast<const void*>(repartition_param_kernel<N, HOW>), dim3((unsigned)n), dim3(256), args, 0, st);
+void launch_param_n(const char* src, char* dst, const SlabChunk& c, cudaStream_t st) {
+    void* args[] = {&src, &dst, const_cast<SlabParams<JA_PARAM_SLABS>*>(&c.p)};
+    cudaLaunchKernel(reinterpret_cast<const void*>(repartition_param_kernel<N, HOW>), dim3((unsigned)c.n), dim3(256), args, 0, st);
 }
 template <int HOW>
-void launch_param(const char* src, char* dst, const CopySlab* slabs, int n, cudaStream_t st) {
-    switch (ja_param_capacity(n)) {
-        case 16: launch_param_n<HOW, 16>(src, dst, slabs, n, st); break;
-        case 64: launch_param_n<HOW, 64>(src, dst, slabs, n, st); break;
-        case 192: launch_param_n<HOW, 192>(src, dst, slabs, n, st); break;
-        case 448: launch_param_n<HOW, 448>(src, dst, slabs, n, st); break;
-        default: launch_param_n<HOW, JA_PARAM_SLABS>(src, dst, slabs, n, st); break;
-    }
+void launch_param(const char* src, char* dst, const SlabChunk& c, cudaStream_t st) {
+    if (c.n <= 64) launch_param_n<HOW, 64>(src, dst, c, st);
+    else if (c.n <= 256) launch_param_n<HOW, 256>(src, dst, c, st);
+    else if (c.n <= 512) launch_param_n<HOW, 512>(src, dst, c, st);
+    else launch_param_n<HOW, JA_PARAM_SLABS>(src, dst, c, st);
 }
 template <int HOW>
 void launch_table(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, cudaStream_t st) {
@@ -123,15 +119,15 @@ void launch_table(const char* src, char* dst, const CopySlab* d_slabs, int64_t n
 
 }  // namespace
 
-ja_status_t ja_launch_repartition_param(const char* src, char* dst, const CopySlab* slabs, int n_slabs, int vec_bytes, bool long_rows, cudaStream_t st) {
-    static_assert(JA_PARAM_SLABS == 960 && sizeof(CopySlab) == 32, "30 KiB of the 32764 bytes a kernel's parameters may hold");
-    if (n_slabs == 0) return JA_OK;
+ja_status_t ja_launch_repartition_param(const char* src, char* dst, const SlabChunk& chunk, int vec_bytes, bool long_rows, cudaStream_t st) {
+    static_assert(sizeof(ParamSlab) == 12 && sizeof(SlabParams<JA_PARAM_SLABS>) <= 32000, "a kernel's parameters hold 32764 bytes");
+    if (chunk.n == 0) return JA_OK;
     switch (copy_of(vec_bytes, long_rows)) {
-        case COPY_16: launch_param<COPY_16>(src, dst, slabs, n_slabs, st); break;
-        case COPY_8: launch_param<COPY_8>(src, dst, slabs, n_slabs, st); break;
-        case COPY_4: launch_param<COPY_4>(src, dst, slabs, n_slabs, st); break;
-        case COPY_2: launch_param<COPY_2>(src, dst, slabs, n_slabs, st); break;
-        case COPY_ANY: launch_param<COPY_ANY>(src, dst, slabs, n_slabs, st); break;
+        case COPY_16: launch_param<COPY_16>(src, dst, chunk, st); break;
+        case COPY_8: launch_param<COPY_8>(src, dst, chunk, st); break;
+        case COPY_4: launch_param<COPY_4>(src, dst, chunk, st); break;
+        case COPY_2: launch_param<COPY_2>(src, dst, chunk, st); break;
+        case COPY_ANY: launch_param<COPY_ANY>(src, dst, chunk, st); break;
     }
     ja_count_launch();
     JA_CUDA(cudaGetLastError());

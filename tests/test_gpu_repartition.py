@@ -38,6 +38,21 @@ def test_any_alignment(ext, src, dst, dtype, once):
     check_status()          # guard zones around every payload
 
 
+@pytest.mark.parametrize("dtype", [BF, F32])
+@pytest.mark.parametrize("n,cuts", [(200, 13), (200, 24), (900, 60)])   # more shapes of slabs than a launch holds; more slabs; more than a few launches hold
+def test_many_shapes(n, cuts, dtype):
+    rng = np.random.default_rng(5)
+    s_sp, d_sp = ([[0] + sorted(rng.choice(np.arange(1, n), cuts - 1, replace=False).tolist()) + [n] for _ in range(2)] for _ in range(2))
+    x = si.normal((n, n), 0.0, 1.0, dtype, 37, 5)
+    a, b, c = upload(x, s_sp), empty_like_tiling([n, n], d_sp, dtype), empty_like_tiling([n, n], d_sp, dtype)
+    for _ in range(2):
+        ja.repartition(a, b)
+    ja.ja_repartition_once(a.handle, c.handle, torch.cuda.current_stream().cuda_stream)
+    want = blocked.pack(np_bits(x), d_sp)
+    assert np.array_equal(download_bits(b), want) and np.array_equal(download_bits(c), want)
+    check_status()
+
+
 @pytest.mark.parametrize("shape,cuts,dtype", [((97, 41), (4, 3), BF), ((1024, 512), (8, 4), F16), ((333,), (5,), F32)])
 def test_dense_round_trip(shape, cuts, dtype):
     x = si.normal(shape, 0.0, 1.0, dtype, 37, 2)
@@ -88,4 +103,32 @@ def test_every_call_of_a_pair_costs_the_same():
     g.replay()
     want = blocked.pack(np_bits(x), d_sp)
     assert np.array_equal(download_bits(b), want) and np.array_equal(download_bits(c), want)
+    check_status()
+
+
+def test_a_small_pair_on_several_streams_and_in_a_graph():
+    """Few slabs: the second call copies a table that only its stream reads; other streams, captures and a second pair in the memory of a
+    closed one carry the slabs in parameters or in tables of their own."""
+    ext, s_sp, d_sp = [300, 260], [ES(300, 3), ES(260, 2)], [ES(300, 2), ES(260, 5)]
+    want = None
+    for trial in range(3):
+        x = si.normal(tuple(ext), 0.0, 1.0, BF, 37, 6 + trial)
+        a, b = upload(x, s_sp), empty_like_tiling(ext, d_sp, BF)
+        want = blocked.pack(np_bits(x), d_sp)
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        torch.cuda.synchronize()
+        for st in [streams[0], streams[0], streams[1], streams[0], streams[2], streams[1]]:
+            b.payload.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(st):
+                ja.repartition(a, b)
+            torch.cuda.synchronize()
+            assert np.array_equal(download_bits(b), want)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[0]):
+            ja.repartition(a, b)
+        b.payload.zero_()
+        g.replay()
+        assert np.array_equal(download_bits(b), want)
+        a.close(), b.close()
     check_status()
