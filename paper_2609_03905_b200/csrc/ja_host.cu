@@ -1102,6 +1102,19 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 if (!ok) plan->gemm.reset();
                 if ((st = ja_contract_tc_plan(in[0], in[1], o, A, B, out, &plan->contract, &us)) != JA_OK) return st;
                 plan->contract_first = plan->contract && (!plan->gemm || us < 0.9 * ja_gemm_tc_estimate_us(*plan->gemm));
+                // A small product that TMA cannot address, in odd intervals: the plain-ALU kernel where its 32 x 32 tiles fit the chip twice
+                // over (64 x 314 x 320 in 2 x 8 x 4: 19 us against 46, 250 x 314 x 333 in 2 x 2 x 4: 15 against 27; 64 x 3001 x 320 in 8 x 64
+                // x 4 is 123 against 60 and stays). Its time: a start, and so much a cell and an interval of the contracted index.
+                if (plan->contract && !plan->gemm && loader != 1) {
+                    auto tiles = [](const ja_relation* r, int d) {
+                        int64_t n = 0;
+                        for (int i = 0; i < r->nblk[d]; ++i) n += (r->splits[d][i + 1] - r->splits[d][i] + 31) / 32;
+                        return n;
+                    };
+                    const int64_t t = tiles(A, 0) * tiles(B, 1), sms = ja_sm_count();
+                    const double simt_us = (3.0 + 0.0295 * (double)A->extent[1] + 0.85 * A->nblk[1]) * (t <= sms ? 1.0 : 1.4);
+                    if (t <= 2 * sms && simt_us < 1.1 * us) plan->contract.reset();
+                }
                 plan->contract_checked = true;
             }
             if (plan->gemm && loader != 1 && (loader == 0 || !plan->contract_first)) return ja_launch_gemm_tc(*plan->gemm, stream);

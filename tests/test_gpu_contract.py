@@ -101,3 +101,11 @@ def test_an_f32_output_is_as_exact_as_f32_sums(K, dtype):
         one_by_one += (a64[:, :, None, j] * b64[:, None, :, j]).astype(np.float32)
     assert relfro(download(res), ref) <= 1.25 * relfro(one_by_one.astype(np.float64), ref)
     check_status()
+
+
+# two-index products that TMA cannot address, on both sides of the line between the plain-ALU kernel and this one
+@pytest.mark.parametrize("m,gi,k,gj,n,gk", [(64, 2, 314, 8, 320, 4), (250, 2, 313, 1, 333, 4), (16, 1, 700, 8, 320, 1), (64, 8, 1501, 64, 320, 4),
+                                            (500, 2, 314, 8, 1007, 8), (33, 3, 70, 2, 75, 5)])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_products_in_odd_intervals(m, gi, k, gj, n, gk, dtype):
+    _run("ij,jk->ik", {"i": ES(m, gi), "j": ES(k, gj), "k": ES(n, gk)}, dtype, dtype)
