@@ -795,7 +795,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
         // (causal; without: before is far below 0)
         auto issue_pv = [&](int t, int sl, bool first, int keys, int rows, int before) {   // O~_t (+)= P_t V, P in shared memory (K-major), V in slot sl (MN-major)
             const uint32_t vaddr = sKV + sl * TILE_BYTES, paddr = sP + t * TILE_BYTES;
-            if (!RAGGED || (keys == KT && before + KT <= 16)) {
+            if (!RAGGED || (keys == KT && before + KT / 2 <= 0)) {
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
                     const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
@@ -803,18 +803,50 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                               (!first || kk > 0) ? 1u : 0u, leader);
                 }
             } else {
-                // A short or diagonal key tile: only the groups of 16 keys that exist and that some row joins, and of a group only the rows
-                // that join its first key: P is 0 elsewhere, but 0 times an infinite or NaN V row of a later key would not be.
-                for (int kk = 0; kk * 16 < keys && before + kk * 16 < rows; ++kk) {
-                    const uint32_t at = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
-                    uint32_t off[4];
+                // A short or diagonal key tile, as two halves of 64 keys: only the groups of 16 keys that exist, and of a half only the rows
+                // that join its first key: P is 0 elsewhere, but 0 times an infinite or NaN V row of a later key would not be. (Masks for
+                // every 16 keys, in a loop: up to 2 us more on an attention of 12, whose tiles are all diagonal.) The mask of a tile
+                // on the diagonal itself is a constant.
+                auto plain = [&](int kk) {
+                    umma_ss_w(tmem_base + 256 + t * 128, desc_sw128(paddr + (kk >> 2) * HALF_BYTES + (kk & 3) * 32, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
+                              (!first || kk > 0) ? 1u : 0u, kk * 16 < keys ? leader : 0u);
+                };
+                auto masked = [&](int kk, const uint32_t (&lanes_off)[4]) {
+                    umma_ss_lanes_w(tmem_base + 256 + t * 128, desc_sw128(paddr + (kk >> 2) * HALF_BYTES + (kk & 3) * 32, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES),
+                                    idesc_pv, (!first || kk > 0) ? 1u : 0u, lanes_off, kk * 16 < keys ? leader : 0u);
+                };
+                auto lanes_before = [&](int n0, uint32_t (&lanes_off)[4]) {   // lanes [0, n0)
 #pragma unroll
                     for (int w = 0; w < 4; ++w) {
-                        const int n = before + kk * 16 - w * 32;   // lanes [0, n) of this word are off
-                        off[w] = n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u;
+                        const int n = n0 - w * 32;
+                        lanes_off[w] = n <= 0 ? 0u : n >= 32 ? 0xffffffffu : (1u << n) - 1u;
                     }
-                    umma_ss_lanes_w(tmem_base + 256 + t * 128, desc_sw128(paddr + at, 16), desc_sw128(vaddr + kk * 2048, HALF_BYTES), idesc_pv,
-                                    (!first || kk > 0) ? 1u : 0u, off, leader);
+                };
+                if (before <= 0) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) plain(kk);
+                    if (keys <= 64 || before + 64 >= rows) {          // no second half
+                    } else if (before == 0) {
+                        const uint32_t lanes_off[4] = {0xffffffffu, 0xffffffffu, 0u, 0u};
+#pragma unroll
+                        for (int kk = 4; kk < 8; ++kk) masked(kk, lanes_off);
+                    } else if (before + 64 <= 0) {
+#pragma unroll
+                        for (int kk = 4; kk < 8; ++kk) plain(kk);
+                    } else {
+                        uint32_t lanes_off[4];
+                        lanes_before(before + 64, lanes_off);
+#pragma unroll 1
+                        for (int kk = 4; kk < 8; ++kk) masked(kk, lanes_off);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int half = 0; half < 2 && before + half * 64 < rows; ++half) {
+                        uint32_t lanes_off[4];
+                        lanes_before(before + half * 64, lanes_off);
+#pragma unroll 1
+                        for (int kk = half * 4; kk < half * 4 + 4; ++kk) masked(kk, lanes_off);
+                    }
                 }
             }
             commit1_w(bar(P_EMPTY + t), leader);
@@ -827,6 +859,13 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
         AttnItem it;
         for (int item = 0; ok && next_item(item, &it); ++item) {
             const int n_of[2] = {it.n_a, it.n_b};
+            int rows[2] = {QT, QT}, q_start[2] = {0, 0};   // RAGGED: read once an item, not between a wait and the products
+            if constexpr (RAGGED) {
+                for (int t = 0; t < (it.n_b ? 2 : 1); ++t) {
+                    rows[t] = tile_rows(rt->q[it.qt + t]);
+                    q_start[t] = tile_start(rt->q[it.qt + t]);
+                }
+            }
             ok = mbar_wait(bar(Q_FULL), (uint32_t)item & 1, abort_flag, p.status);
             {
                 const int sl = li % 3;
@@ -862,9 +901,10 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                 }
                 const int sl = li % 3;
                 if (!mbar_wait(bar(KV_FULL + sl), (uint32_t)(li / 3) & 1, abort_flag, p.status)) { ok = false; break; }
-                int keys = KT;
+                int keys = KT, k_start = 0;
                 if constexpr (RAGGED) {
                     keys = tile_rows(rt->k[it.kt + j]);
+                    k_start = tile_start(rt->k[it.kt + j]);
                     if (keys & 15) {   // the last group's missing keys have P = 0: their V rows (other cells of the relation) must not be NaN
                         uint8_t* v = smem + (2 + sl) * TILE_BYTES;
                         const int gap = 16 - (keys & 15);
@@ -880,12 +920,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                         // the first P V of an item overwrites O~: the row threads must have read the previous item's
                         if (j == 0 && done[t] > 0 && !mbar_wait(bar(O_READ + t), (uint32_t)(done[t] - 1) & 1, abort_flag, p.status)) { ok = false; break; }
                         tc_fence_after();
-                        int rows = QT, before = -KT;
-                        if constexpr (RAGGED) {
-                            rows = tile_rows(rt->q[it.qt + t]);
-                            if (p.causal) before = tile_start(rt->k[it.kt + j]) - tile_start(rt->q[it.qt + t]);
-                        }
-                        issue_pv(t, sl, j == 0, keys, rows, before);
+                        issue_pv(t, sl, j == 0, keys, rows[t], p.causal ? k_start - q_start[t] : -KT);
                     }
                 }
                 if (!ok) break;

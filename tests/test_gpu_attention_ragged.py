@@ -102,21 +102,21 @@ def test_scales_that_are_not_positive(S, causal, scale):
 @pytest.mark.parametrize("split", [[0, 300], [0, 37, 101, 200, 333], [0, 200, 400]])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 def test_later_values_that_are_not_finite(split, bad):
-    """V is NaN or infinite from some key on: no query more than a 16-key group before it notices (causal)."""
+    """V is NaN or infinite from some key on: no query more than 63 positions before it notices (causal; half a key tile)."""
     S, H = split[-1], 2
     Q, K, V = (si.normal((1, S, H, 128), 0.0, 1.0, BF, 4, 100 + n) for n in range(3))
     ref = operators.attention_gqa_packed(si.to_f64(Q), si.to_f64(K), si.to_f64(V), 1, None, True, "bf16")
     sp = [[0, 1], split, [0, H], [0, 128]]
     spec = ja.Spec("bqhd,bkhd,bkhd->bqhd", {"b": sp[0], "q": sp[1], "h": sp[2], "d": sp[3], "k": sp[1]}, "attention", (1.0 / math.sqrt(128), 1.0),
                    "online_softmax")
-    for first_bad in (100, 190, 127, 250, S - 1):
+    for first_bad in (100, 190, 127, 128, 250, S - 1):
         V2 = V.clone()
         V2[:, first_bad:] = bad
         ro = empty_like_tiling([1, S, H, 128], sp, BF, fill=float("nan"))
         spec.execute([upload(Q, sp), upload(K, sp), upload(V2, sp)], ro)
         got = download(ro)
         check_status()
-        n = first_bad - 15
+        n = first_bad - 63
         assert relfro(got[:, :n], ref[:, :n]) <= TOL[BF]
         assert not np.isfinite(got[:, first_bad:]).any()
 
