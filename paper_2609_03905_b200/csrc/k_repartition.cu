@@ -7,11 +7,11 @@
 // around them, and only the ends of a row go cell by cell (12370 rows of 2919 bf16 cells: 81 -> 39 us); short ones go by the
 // widest access their alignment allows.
 //
-// The slabs travel in the kernel's parameters where one launch holds them -- nothing is allocated or copied for a pair of
-// relations, on its first call or any other -- else in a table in device memory that the caller keeps, or, for relations that meet
-// once (packing a dense tensor, unpacking a result), in the parameters of several launches: 0.4 ms less than a table's allocation
-// and copy, but 20 to 30 % slower per call than one launch with a table (134 MB: 59 against 47 us, the ends of three launches).
-// Both move a slab by the same rule (copy_of).
+// The slabs travel in the kernel's parameters (12 bytes each, up to 960 a launch) where nothing is to be allocated or nothing orders
+// the launch after a table's copy, else in a table in device memory that the caller keeps. On the GPU both take the same time; the
+// parameters cost the host 0.5 to 1.8 us a launch. For relations that meet once a table's allocation and copy (0.4 ms) cost more than the
+// several launches by parameters that many slabs take (134 MB: 59 us against 47 for one launch with a table). Both move a slab by
+// the same rule (copy_of).
 
 #include "ja_device.cuh"
 
