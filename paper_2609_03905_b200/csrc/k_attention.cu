@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -90,6 +91,8 @@ __global__ void __launch_bounds__(QT * 2, 1) attention_kernel(AttnArgs a) {
     uint8_t* sQ = smem;                          // QT x 128 (reused to stage O)
     uint8_t* sK = smem + QT * ROW_BYTES;         // 2 x KT x 128
     uint8_t* sV = sK + 2 * KT * ROW_BYTES;       // 2 x KT x 128
+    ja_wait_for_stream();
+    ja_let_next_start();
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int g = lane / 4, t4 = lane % 4;
 
@@ -322,7 +325,7 @@ ja_status_t ja_launch_attention(const AttnArgs& a, cudaStream_t st) {
 #define JA_ATTN_SYNC(Q, F, R)                                                                                          \
     do {                                                                                                              \
         JA_CUDA(cudaFuncSetAttribute(attention_kernel<Q, F, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)); \
-        attention_kernel<Q, F, R><<<grid, 2 * Q, smem, st>>>(a2);                                                    \
+        JA_CUDA(ja_launch_kernel(attention_kernel<Q, F, R>, grid, 2 * Q, smem, 1, st, a2));                           \
     } while (0)
     if (ragged) {
         if (a.f16) JA_ATTN_SYNC(64, true, true);

@@ -13,6 +13,7 @@
 #include <string.h>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -58,6 +59,8 @@ template <> __device__ __forceinline__ uint4 pack_vec<__half>(const float (&f)[8
 template <typename T, bool FAST, int MC>
 __global__ void __launch_bounds__(256) attention_combine_kernel(const CombineParams p) {
     constexpr int R = (MAX_COPIES / MC + 1) / 2, CELLS = Vec16<T>::CELLS, LPR = 128 / CELLS, RPL = 32 / LPR, ROWS = R * RPL;
+    ja_wait_for_stream();
+    ja_let_next_start();
     const int lane = threadIdx.x & 31, sub = lane / LPR, col = (lane % LPR) * 16;      // col: byte offset of the lane's vector in its row
     const uint32_t warps = gridDim.x * 8u, n_rows = (uint32_t)(p.B * p.S * p.H);   // the host keeps the row count below 2^31
     for (uint32_t row0 = (blockIdx.x * 8u + (threadIdx.x >> 5)) * ROWS; row0 < n_rows; row0 += warps * ROWS) {
@@ -171,8 +174,7 @@ ja_status_t ja_launch_attention_combine(const ja_relation* const* op, const ja_r
     const unsigned grid = (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
 #define JA_COMBINE_MC(T, MC)                                                          \
     do {                                                                              \
-        if (fast) attention_combine_kernel<T, true, MC><<<grid, 256, 0, st>>>(p);    \
-        else attention_combine_kernel<T, false, MC><<<grid, 256, 0, st>>>(p);        \
+        JA_CUDA(ja_launch_kernel(fast ? attention_combine_kernel<T, true, MC> : attention_combine_kernel<T, false, MC>, dim3(grid), 256, 0, 1, st, p)); \
     } while (0)
 #define JA_COMBINE(T)                                                                 \
     do {                                                                              \

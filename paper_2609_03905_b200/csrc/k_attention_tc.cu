@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 
 namespace {
@@ -228,6 +229,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    ja_wait_for_stream();
+    ja_let_next_start();
     const uint32_t tS[2] = {tmem_base, tmem_base + 128};
     const uint32_t tO[2] = {tmem_base + 256, tmem_base + 384};
 
@@ -689,6 +692,8 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    ja_wait_for_stream();
+    ja_let_next_start();
 
     if (warp == 0) {
         // ================= TMA producer =================
@@ -1181,13 +1186,13 @@ ja_status_t launch_two_tiles(int variant, bool f16, dim3 grid, cudaStream_t st, 
                              const CUtensorMap& tv, const CUtensorMap& to, const AttnTcParams& p) {
     if (f16) {   // f16 cells: the default row-thread variant only
         JA_CUDA(cudaFuncSetAttribute(attention_tc2_kernel<PERSIST, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-        attention_tc2_kernel<PERSIST, 1, true><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p);
+        JA_CUDA(ja_launch_kernel(attention_tc2_kernel<PERSIST, 1, true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));
         return JA_OK;
     }
 #define JA_ATTN_LAUNCH(V)                                                                                                          \
     case V: {                                                                                                                      \
         JA_CUDA(cudaFuncSetAttribute(attention_tc2_kernel<PERSIST, V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2)); \
-        attention_tc2_kernel<PERSIST, V, false><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p);                      \
+        JA_CUDA(ja_launch_kernel(attention_tc2_kernel<PERSIST, V, false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));                      \
         return JA_OK;                                                                                                              \
     }
     switch (variant) {
@@ -1355,10 +1360,10 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         const dim3 grid((unsigned)std::min<int64_t>(items, sms), 1, 1);
         if (a.f16) {
             JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-            attention_ragged_kernel<true><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p, rt);
+            JA_CUDA(ja_launch_kernel(attention_ragged_kernel<true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
         } else {
             JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-            attention_ragged_kernel<false><<<grid, NUM_THREADS2, SMEM_BYTES2, st>>>(tq, tk, tv, to, p, rt);
+            JA_CUDA(ja_launch_kernel(attention_ragged_kernel<false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
         }
         ja_count_launch();
         JA_CUDA(cudaGetLastError());
@@ -1411,10 +1416,10 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         dim3 grid((unsigned)((int64_t)a.H * a.B * (a.S / QT)), 1, 1);
         if (a.f16) {
             JA_CUDA(cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-            attention_tc_kernel<true><<<grid, NUM_THREADS, SMEM_BYTES, st>>>(tq, tk, tv, p);
+            JA_CUDA(ja_launch_kernel(attention_tc_kernel<true>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
         } else {
             JA_CUDA(cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-            attention_tc_kernel<false><<<grid, NUM_THREADS, SMEM_BYTES, st>>>(tq, tk, tv, p);
+            JA_CUDA(ja_launch_kernel(attention_tc_kernel<false>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
         }
     }
     ja_count_launch();

@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 #include "ja_walk.cuh"
 
@@ -170,6 +171,8 @@ __global__ void __launch_bounds__(NT) contract_f32_kernel(const __grid_constant_
     Walk<T, KCB, WB, EQ> wb;
     wa.init(p.A, batch_at(p.A, bx), tid, m0, c0 * TK);
     wb.init(p.B, batch_at(p.B, bx), tid, n0, c0 * TK);
+    ja_wait_for_stream();
+    ja_let_next_start();
     uint64_t acc2[U][U / 2];                    // pairs of neighbouring columns
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -323,20 +326,8 @@ ja_status_t launch(const Params& p, cudaStream_t st) {
         JA_CUDA(cudaFuncSetAttribute(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<T>::SMEM));
         configured[dev & 63] = true;
     }
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]);
-    cfg.blockDim = dim3(NT, 1, 1);
-    cfg.dynamicSmemBytes = Cfg<T>::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)p.split;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = p.split > 1 ? 1 : 0;
-    JA_CUDA(cudaLaunchKernelEx(&cfg, contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, p));
+    JA_CUDA(ja_launch_kernel(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, dim3((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]), NT,
+                             Cfg<T>::SMEM, (unsigned)p.split, st, p));
     return JA_OK;
 }
 template <int T, bool KCA, int WA, bool KCB, int WB>

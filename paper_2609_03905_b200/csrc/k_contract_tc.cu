@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 #include "ja_walk.cuh"
 
@@ -555,6 +556,10 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    if (p.split == 1) {   // launched to start inside the kernel before it
+        ja_wait_for_stream();
+        ja_let_next_start();
+    }
 
     const int chunks = (p.K + BK - 1) / BK;
     const int c0 = (int)((int64_t)chunks * rank / split), c1 = (int)((int64_t)chunks * (rank + 1) / split);
@@ -661,20 +666,10 @@ ja_status_t launch(const Params& p, cudaStream_t st) {
         JA_CUDA(cudaFuncSetAttribute(contract_tc_kernel<BN, RAW, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN, RAW>::SMEM));
         configured[dev & 63] = true;
     }
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]);
-    cfg.blockDim = dim3(Cfg<BN, RAW>::THREADS, 1, 1);
-    cfg.dynamicSmemBytes = Cfg<BN, RAW>::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)p.split;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = p.split > 1 ? 1 : 0;
-    JA_CUDA(cudaLaunchKernelEx(&cfg, contract_tc_kernel<BN, RAW, ACC>, p));
+    const dim3 grid((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]);
+    // clusters wait for the launch before them: [32, 4096] x [4096, 11008] 30.6 us, 32.8 when they start inside it
+    if (p.split > 1) JA_CUDA(ja_launch_kernel_after(contract_tc_kernel<BN, RAW, ACC>, grid, Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::SMEM, (unsigned)p.split, st, p));
+    else JA_CUDA(ja_launch_kernel(contract_tc_kernel<BN, RAW, ACC>, grid, Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::SMEM, 1, st, p));
     return JA_OK;
 }
 

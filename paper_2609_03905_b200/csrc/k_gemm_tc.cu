@@ -27,6 +27,7 @@
 #include <string.h>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 
 namespace {
@@ -207,6 +208,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (CG == 2) cluster_sync_all();   // the peer's barriers exist before anything remote touches them
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    ja_wait_for_stream();
+    ja_let_next_start();
 
     const int total_tiles = p.m_tiles * p.n_tiles * p.n_copies;
     const int kchunks = (p.bk + Cfg<CG>::BK - 1) / Cfg<CG>::BK;
@@ -545,27 +548,11 @@ ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st) {
     p.status = ja_device_status_word(st);
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
-    if (plan.cg == 2) {
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof cfg);
-        cfg.gridDim = dim3((unsigned)plan.grid, 1, 1);
-        cfg.blockDim = dim3(NUM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = Cfg<2>::SMEM_BYTES;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (p.f16) JA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<2, true>, plan.tmA, plan.tmB, plan.tmB2, p));
-        else JA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<2, false>, plan.tmA, plan.tmB, plan.tmB2, p));
-    } else {
-        if (p.f16) gemm_tc_kernel<1, true><<<plan.grid, NUM_THREADS, Cfg<1>::SMEM_BYTES, st>>>(plan.tmA, plan.tmB, plan.tmB2, p);
-        else gemm_tc_kernel<1, false><<<plan.grid, NUM_THREADS, Cfg<1>::SMEM_BYTES, st>>>(plan.tmA, plan.tmB, plan.tmB2, p);
-        JA_CUDA(cudaGetLastError());
-    }
+    const dim3 grid((unsigned)plan.grid, 1, 1);
+    if (plan.cg == 2)
+        JA_CUDA(ja_launch_kernel(p.f16 ? gemm_tc_kernel<2, true> : gemm_tc_kernel<2, false>, grid, NUM_THREADS, Cfg<2>::SMEM_BYTES, 2, st, plan.tmA, plan.tmB, plan.tmB2, p));
+    else
+        JA_CUDA(ja_launch_kernel(p.f16 ? gemm_tc_kernel<1, true> : gemm_tc_kernel<1, false>, grid, NUM_THREADS, Cfg<1>::SMEM_BYTES, 1, st, plan.tmA, plan.tmB, plan.tmB2, p));
     ja_count_launch();
     return JA_OK;
 }

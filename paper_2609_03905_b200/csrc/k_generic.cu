@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 #include "ja_walk.cuh"
 
@@ -117,6 +118,8 @@ __device__ __forceinline__ float merged(int agg, float a, float b) { return agg 
 template <int N, bool LANES>
 __global__ void __launch_bounds__(WARPS * 32) generic_join_agg_kernel(const __grid_constant__ Params p) {
     __shared__ float part[WARPS][32];
+    ja_wait_for_stream();
+    ja_let_next_start();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int rank = (int)blockIdx.x % p.cluster;
     const int64_t group = blockIdx.x / p.cluster;
@@ -240,19 +243,7 @@ __global__ void __launch_bounds__(WARPS * 32) generic_join_agg_kernel(const __gr
 
 template <int N, bool LANES>
 ja_status_t launch(const Params& p, int64_t groups, cudaStream_t st) {
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)(groups * p.cluster), 1, 1);
-    cfg.blockDim = dim3(WARPS * 32, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)p.cluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = p.cluster > 1 ? 1 : 0;
-    JA_CUDA(cudaLaunchKernelEx(&cfg, generic_join_agg_kernel<N, LANES>, p));
+    JA_CUDA(ja_launch_kernel(generic_join_agg_kernel<N, LANES>, dim3((unsigned)(groups * p.cluster)), WARPS * 32, 0, (unsigned)p.cluster, st, p));
     return JA_OK;
 }
 
@@ -277,6 +268,8 @@ __device__ __forceinline__ float load_wide(const RelView& v, int dtype, const in
 }
 
 __global__ void __launch_bounds__(256) generic_join_agg_wide_kernel(const WideParams p) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     for (int64_t cell = (int64_t)blockIdx.x * 256 + threadIdx.x; cell < p.n_out_cells; cell += (int64_t)gridDim.x * 256) {
         int64_t coord[JA_MAX_RANK + MAX_SUMMED];
         int64_t rem = cell;
@@ -418,7 +411,7 @@ ja_status_t ja_launch_generic(const ja_spec* spec, const ja_relation* const* inp
         w.fn = (int)spec->fn;
         w.agg = (int)spec->agg;
         const int64_t blocks = std::max<int64_t>(1, (w.n_out_cells + 255) / 256), cap = (int64_t)ja_sm_count() * 32;
-        generic_join_agg_wide_kernel<<<(unsigned)std::min(blocks, cap), 256, 0, st>>>(w);
+        JA_CUDA(ja_launch_kernel(generic_join_agg_wide_kernel, dim3((unsigned)std::min(blocks, cap)), 256, 0, 1, st, w));
         ja_count_launch();
         JA_CUDA(cudaGetLastError());
         *launched = true;

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -70,6 +71,8 @@ __global__ void __launch_bounds__(NT) matmul_simt_kernel(const SimtParams p) {
     constexpr int NB = VECTOR ? (TK * TN / W + NT - 1) / NT : TK * TN / NT;
     __shared__ __align__(16) float As[TK][TM + 4];
     __shared__ __align__(16) float Bs[TK][TN + 4];
+    ja_wait_for_stream();
+    ja_let_next_start();
     const RelView &A = p.A, &B = p.B, &C = p.C;
     const int tid = threadIdx.x;
     const int kb = blockIdx.x / p.tiles_k, tk = blockIdx.x % p.tiles_k;
@@ -224,8 +227,7 @@ __global__ void __launch_bounds__(NT) matmul_simt_kernel(const SimtParams p) {
 
 template <typename T, int TM, int TN>
 void launch(const SimtParams& p, dim3 grid, bool vec, cudaStream_t st) {
-    if (vec) matmul_simt_kernel<T, TM, TN, true><<<grid, NT, 0, st>>>(p);
-    else matmul_simt_kernel<T, TM, TN, false><<<grid, NT, 0, st>>>(p);
+    ja_launch_kernel(vec ? matmul_simt_kernel<T, TM, TN, true> : matmul_simt_kernel<T, TM, TN, false>, grid, NT, 0, 1, st, p);
 }
 
 }  // namespace

@@ -12,14 +12,14 @@ ja_status_t ja_launch_flat(ja_fn_t fn, const void* a, const void* b, void* out, 
     int64_t want = (n_vec + 255) / 256;
     unsigned grid = (unsigned)(want < (int64_t)148 * 32 ? (want > 0 ? want : 1) : (int64_t)148 * 32);
     if (dt == JA_BF16) {
-        if (fn == JA_FN_ADD) flat_16bit_kernel<JA_FN_ADD, false><<<grid, 256, 0, st>>>((const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
-        else flat_16bit_kernel<JA_FN_SILU_MUL, false><<<grid, 256, 0, st>>>((const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
+        if (fn == JA_FN_ADD) ja_launch_kernel(flat_16bit_kernel<JA_FN_ADD, false>, dim3(grid), 256, 0, 1, st, (const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
+        else ja_launch_kernel(flat_16bit_kernel<JA_FN_SILU_MUL, false>, dim3(grid), 256, 0, 1, st, (const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
     } else if (dt == JA_F16) {
-        if (fn == JA_FN_ADD) flat_16bit_kernel<JA_FN_ADD, true><<<grid, 256, 0, st>>>((const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
-        else flat_16bit_kernel<JA_FN_SILU_MUL, true><<<grid, 256, 0, st>>>((const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
+        if (fn == JA_FN_ADD) ja_launch_kernel(flat_16bit_kernel<JA_FN_ADD, true>, dim3(grid), 256, 0, 1, st, (const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
+        else ja_launch_kernel(flat_16bit_kernel<JA_FN_SILU_MUL, true>, dim3(grid), 256, 0, 1, st, (const uint4*)a, (const uint4*)b, (uint4*)out, n_vec);
     } else {
-        if (fn == JA_FN_ADD) flat_f32_kernel<JA_FN_ADD><<<grid, 256, 0, st>>>((const float4*)a, (const float4*)b, (float4*)out, n_vec);
-        else flat_f32_kernel<JA_FN_SILU_MUL><<<grid, 256, 0, st>>>((const float4*)a, (const float4*)b, (float4*)out, n_vec);
+        if (fn == JA_FN_ADD) ja_launch_kernel(flat_f32_kernel<JA_FN_ADD>, dim3(grid), 256, 0, 1, st, (const float4*)a, (const float4*)b, (float4*)out, n_vec);
+        else ja_launch_kernel(flat_f32_kernel<JA_FN_SILU_MUL>, dim3(grid), 256, 0, 1, st, (const float4*)a, (const float4*)b, (float4*)out, n_vec);
     }
     ja_count_launch();
     JA_CUDA(cudaGetLastError());

@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -31,6 +32,8 @@ __device__ __forceinline__ float flat_fn(float a, float b) {
 template <int FN, bool F16>
 __global__ void __launch_bounds__(256) flat_16bit_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b,
                                                          uint4* __restrict__ out, int64_t n_vec) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * 256) {
         uint4 va = a[i], vb = b[i], vo;
         const uint32_t* pa = reinterpret_cast<const uint32_t*>(&va);
@@ -48,6 +51,8 @@ __global__ void __launch_bounds__(256) flat_16bit_kernel(const uint4* __restrict
 template <int FN>
 __global__ void __launch_bounds__(256) flat_f32_kernel(const float4* __restrict__ a, const float4* __restrict__ b,
                                                        float4* __restrict__ out, int64_t n_vec) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * 256) {
         float4 va = a[i], vb = b[i], vo;
         vo.x = flat_fn<FN>(va.x, vb.x); vo.y = flat_fn<FN>(va.y, vb.y);
@@ -158,6 +163,8 @@ __device__ __forceinline__ float team_reduce(float v, int team, float* smem, int
 template <typename T, int VEC, int VPT, int OP>
 __global__ void __launch_bounds__(256) row_kernel(RowArgs a, int64_t n_rows, int team) {
     __shared__ float red[64];
+    ja_wait_for_stream();
+    ja_let_next_start();
     constexpr bool RES = VPT > 0;
     constexpr int NV = RES ? VPT : 1;
     using V = Vec<T, VEC>;
@@ -288,6 +295,8 @@ struct FastGeom {
 template <typename T, int VEC, int VPT, int OP>
 __global__ void __launch_bounds__(256, (VPT <= 2 ? 4 : (VPT <= 4 ? 3 : 1))) row_fast_kernel(RowArgs a, FastGeom g, int64_t n_rows, int team) {
     __shared__ float red[64];
+    ja_wait_for_stream();
+    ja_let_next_start();
     using V = Vec<T, VEC>;
     const int rpc = blockDim.x / team;
     const int row_in_cta = threadIdx.x / team, lane_t = threadIdx.x % team;
@@ -468,7 +477,7 @@ void launch_fast_v(const RowArgs& a, const FastGeom& g, int64_t n_rows, int team
         resident = per_sm * ja_sm_count();
     }
     unsigned grid = (unsigned)(want < resident ? want : resident);
-    row_fast_kernel<T, VEC, VPT, OP><<<grid, block, 0, st>>>(a, g, n_rows, team);
+    ja_launch_kernel(row_fast_kernel<T, VEC, VPT, OP>, dim3(grid), (unsigned)block, 0, 1, st, a, g, n_rows, team);
 }
 
 // returns false if the shape does not fit the fast path (caller falls back to the generic kernel)
@@ -519,6 +528,8 @@ bool launch_fast_op(RowOp op, const RowArgs& a, const FastGeom& g, int64_t n_row
 template <typename T, int VPT, int OP>
 __global__ void __launch_bounds__(256) row_word_kernel(RowArgs a, int64_t n_rows, int team, int words, int runs) {
     __shared__ float red[64];
+    ja_wait_for_stream();
+    ja_let_next_start();
     constexpr int CW = 16 / (int)sizeof(T);       // cells per word
     constexpr bool HAS_STAT = (OP == ROW_SUMSQ || OP == ROW_MAX || OP == ROW_EXPSUM || OP == ROW_RMS_SCALE || OP == ROW_EXP_SUB_DIV);
     constexpr bool HAS_G = (OP == ROW_RMS_SCALE || OP == ROW_RMSNORM);
@@ -657,11 +668,11 @@ bool launch_row_words(const RowArgs& a, int64_t n_rows, cudaStream_t st) {
     while (team < 256 && all > (int64_t)team * 2) team *= 2;
     const int vpt = (int)((all + team - 1) / team);
     const unsigned grid = (unsigned)((n_rows + 256 / team - 1) / (256 / team));
-    if (vpt <= 1) row_word_kernel<T, 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
-    else if (vpt <= 2) row_word_kernel<T, 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
-    else if (vpt <= 4) row_word_kernel<T, 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
-    else if (vpt <= 8) row_word_kernel<T, 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
-    else row_word_kernel<T, 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team, (int)words, runs);
+    if (vpt <= 1) ja_launch_kernel(row_word_kernel<T, 1, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team, (int)words, runs);
+    else if (vpt <= 2) ja_launch_kernel(row_word_kernel<T, 2, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team, (int)words, runs);
+    else if (vpt <= 4) ja_launch_kernel(row_word_kernel<T, 4, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team, (int)words, runs);
+    else if (vpt <= 8) ja_launch_kernel(row_word_kernel<T, 8, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team, (int)words, runs);
+    else ja_launch_kernel(row_word_kernel<T, 16, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team, (int)words, runs);
     return true;
 }
 template <typename T>
@@ -690,12 +701,12 @@ ja_status_t launch_row_t(const RowArgs& a, int64_t n_rows, int64_t n, cudaStream
     int64_t vpt = (n + (int64_t)team * VEC - 1) / ((int64_t)team * VEC);
     const int rpc = 256 / team;
     unsigned grid = (unsigned)((n_rows + rpc - 1) / rpc);
-    if (vpt <= 1) row_kernel<T, VEC, 1, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 2) row_kernel<T, VEC, 2, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 4) row_kernel<T, VEC, 4, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 8) row_kernel<T, VEC, 8, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else if (vpt <= 16 && VEC > 1) row_kernel<T, VEC, 16, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
-    else row_kernel<T, VEC, 0, OP><<<grid, 256, 0, st>>>(a, n_rows, team);
+    if (vpt <= 1) ja_launch_kernel(row_kernel<T, VEC, 1, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
+    else if (vpt <= 2) ja_launch_kernel(row_kernel<T, VEC, 2, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
+    else if (vpt <= 4) ja_launch_kernel(row_kernel<T, VEC, 4, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
+    else if (vpt <= 8) ja_launch_kernel(row_kernel<T, VEC, 8, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
+    else if (vpt <= 16 && VEC > 1) ja_launch_kernel(row_kernel<T, VEC, 16, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
+    else ja_launch_kernel(row_kernel<T, VEC, 0, OP>, dim3(grid), 256, 0, 1, st, a, n_rows, team);
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
     return JA_OK;

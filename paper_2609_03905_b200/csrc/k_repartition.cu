@@ -14,6 +14,7 @@
 // the same rule (copy_of).
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -85,6 +86,8 @@ __device__ __forceinline__ void copy_slab_by(const char* __restrict__ sp, char* 
 template <int HOW>
 __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict__ src, char* __restrict__ dst, const CopySlab* __restrict__ slabs,
                                                           int64_t n_slabs) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
         const CopySlab sl = slabs[s];
         copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
@@ -93,6 +96,8 @@ __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict
 
 template <int N, int HOW>
 __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __restrict__ src, char* __restrict__ dst, const __grid_constant__ SlabParams<N> p) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     const ParamSlab ps = p.s[blockIdx.x];
     const SlabShape sh = p.shapes[ps.shape];
     const CopySlab sl = {0, 0, ps.rows, sh.row_bytes, sh.src_pitch, sh.dst_pitch};
@@ -102,7 +107,7 @@ __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __re
 template <int HOW, int N>
 void launch_param_n(const char* src, char* dst, const SlabChunk& c, cudaStream_t st) {
     void* args[] = {&src, &dst, const_cast<SlabParams<JA_PARAM_SLABS>*>(&c.p)};
-    cudaLaunchKernel(reinterpret_cast<const void*>(repartition_param_kernel<N, HOW>), dim3((unsigned)c.n), dim3(256), args, 0, st);
+    ja_launch_kernel_args(reinterpret_cast<const void*>(repartition_param_kernel<N, HOW>), dim3((unsigned)c.n), 256, 0, 1, st, args);
 }
 template <int HOW>
 void launch_param(const char* src, char* dst, const SlabChunk& c, cudaStream_t st) {
@@ -114,7 +119,7 @@ void launch_param(const char* src, char* dst, const SlabChunk& c, cudaStream_t s
 template <int HOW>
 void launch_table(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, cudaStream_t st) {
     const unsigned grid = (unsigned)(n_slabs < (int64_t)148 * 64 ? n_slabs : (int64_t)148 * 64);
-    repartition_kernel<HOW><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs);
+    ja_launch_kernel(repartition_kernel<HOW>, dim3(grid), 256, 0, 1, st, src, dst, d_slabs, n_slabs);
 }
 
 }  // namespace

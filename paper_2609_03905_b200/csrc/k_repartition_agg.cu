@@ -5,6 +5,7 @@
 // once, rounded once, at the cell's place in the consumer's block ("recompose"). One pass, no staging buffer.
 // HBM-bound: m source cells read and one destination cell written per cell.
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -66,6 +67,8 @@ template <typename TS, typename TD, int VEC, bool IS_MAX, bool FEW>
 __global__ void __launch_bounds__(256) repartition_agg_kernel(const char* __restrict__ src, char* __restrict__ dst,
                                                               const CopySlab* __restrict__ slabs, int64_t n_slabs, int n_copies,
                                                               int64_t copy_stride) {
+    ja_wait_for_stream();
+    ja_let_next_start();
     for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
         const CopySlab sl = slabs[s];
         const int vpr = sl.row_bytes / (int)(VEC * sizeof(TS));  // accesses per row
@@ -135,7 +138,7 @@ template <typename TS, typename TD>
 void launch(const char* src, char* dst, const CopySlab* d_slabs, int64_t n_slabs, int n_copies, int64_t copy_stride, bool is_max,
             bool vec, unsigned grid, cudaStream_t st) {
     constexpr int V = VecOf<TS>::N;
-#define JA_AGG_LAUNCH(VV, MAXF, FEWF) repartition_agg_kernel<TS, TD, VV, MAXF, FEWF><<<grid, 256, 0, st>>>(src, dst, d_slabs, n_slabs, n_copies, copy_stride)
+#define JA_AGG_LAUNCH(VV, MAXF, FEWF) ja_launch_kernel(repartition_agg_kernel<TS, TD, VV, MAXF, FEWF>, dim3(grid), 256, 0, 1, st, src, dst, d_slabs, n_slabs, n_copies, copy_stride)
     const bool few = vec && n_copies <= 4;
     if (vec) {
         if (few) {

@@ -22,6 +22,7 @@
 #include <string.h>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 
 namespace {
 
@@ -77,6 +78,8 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const char* __restrict_
     constexpr int VEC = Cells<T>::VEC;
     constexpr bool IS_MAX = OP == ROW_MAX;
     constexpr int UNROLL = 8;                                // 16-byte loads in flight per lane
+    ja_wait_for_stream();
+    ja_let_next_start();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nvec = g.n / VEC;                              // 16-byte vectors per row
@@ -164,7 +167,7 @@ ja_status_t launch_reduce(const RowArgs& a, const ReduceGeom& g, cudaStream_t st
     const unsigned grid = (unsigned)(want < resident ? want : resident);
     const char* s_in = OP == ROW_EXPSUM ? a.s0.base : nullptr;
     char* s_out = OP == ROW_EXPSUM ? a.s1.base : a.s0.base;
-    row_reduce_kernel<T, OP><<<grid, 256, 0, st>>>(a.x.base, s_in, s_out, g);
+    JA_CUDA(ja_launch_kernel(row_reduce_kernel<T, OP>, dim3(grid), 256, 0, 1, st, (const char*)a.x.base, s_in, s_out, g));
     ja_count_launch();
     JA_CUDA(cudaGetLastError());
     return JA_OK;

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "ja_device.cuh"
+#include "ja_launch.cuh"
 #include "ja_ptx.cuh"
 
 namespace {
@@ -383,6 +384,8 @@ __global__ void __launch_bounds__(NUM_THREADS, (ctas_per_sm<T, OP, VPL>())) row_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    ja_wait_for_stream();
+    ja_let_next_start();
     if (HAS_G && warp < CONSUMER_WARPS) {   // the gain vector, dense, once per CTA; the loader is already fetching rows meanwhile
         for (int v = threadIdx.x; v * VEC < g.n; v += CONSUMER_WARPS * 32) {
             const int col = v * VEC, cb = col / g.bsc, ci = col - cb * g.bsc;
@@ -546,7 +549,7 @@ ja_status_t launch_v(const RowMaps& tm, const RowArgs& a, RowTmaGeom g, int g_by
     }
     const int smem_bytes = g.stages * g.stage_bytes + g_bytes + (3 * MAX_STAGES + CONSUMER_WARPS + 2) * 8 + CONSUMER_WARPS * 16 * 4 + 128;
     const unsigned grid = (unsigned)std::min<int64_t>(g.n_units, (int64_t)sms * CTAS);
-    row_tma_kernel<T, OP, VPL><<<grid, NUM_THREADS, smem_bytes, st>>>(tm.x, tm.y, a, g, status);
+    JA_CUDA(ja_launch_kernel(row_tma_kernel<T, OP, VPL>, dim3(grid), NUM_THREADS, smem_bytes, 1, st, tm.x, tm.y, a, g, status));
     return JA_OK;
 }
 
