@@ -82,6 +82,13 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void st_cluster16(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t cluster_addr, uint32_t a) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_addr), "r"(a) : "memory");
+}
+
 // TMA tile load; `bar` is a shared::cta address (CG 1) or a shared::cluster address that may name the peer CTA's
 // barrier (CG 2). No multicast: every CTA fetches its own boxes.
 template <int CG>
@@ -144,14 +151,14 @@ __device__ __forceinline__ void umma_bf16_w(uint32_t d_tmem, uint64_t a_desc, ui
     }
 }
 template <int CG>
-__device__ __forceinline__ void umma_commit_w(uint32_t bar, uint32_t pred) {
+__device__ __forceinline__ void umma_commit_w(uint32_t bar, uint32_t pred, uint32_t pair0 = 0) {   // pair0: rank of the pair's leader in its cluster
     if (CG == 1) {
         asm volatile(
             "{\n\t.reg .pred q;\n\t"
             "setp.ne.b32 q, %1, 0;\n\t"
             "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(pred) : "memory");
     } else {
-        const uint16_t mask = 3;
+        const uint16_t mask = (uint16_t)(3u << pair0);
         asm volatile(
             "{\n\t.reg .pred q;\n\t"
             "setp.ne.b32 q, %2, 0;\n\t"
@@ -222,3 +229,6 @@ inline EncodeTiledFn get_encode() {
 }
 
 }  // namespace ja_ptx
+
+// Tensor map of a relation [R, C] of equal 16-bit blocks, boxes of box_inner cells of box_rows rows of a block (k_gemm_tc.cu)
+ja_status_t ja_encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows, CUtensorMap* tm);

@@ -388,13 +388,6 @@ __device__ __forceinline__ void load_walk_any(const Rel& o, const BatchAt& ba, u
     }
 }
 
-__device__ __forceinline__ void st_cluster16(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void st_cluster4(uint32_t cluster_addr, uint32_t a) {
-    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_addr), "r"(a) : "memory");
-}
-
 // One thread's share of the finished tile: the 8-cell piece at column c of every STEP-th line from l on, summed over the
 // cluster's slices, rounded once, stored in granules of G cells. Short tiles (a batch of small products) spend as long here as
 // in their main loop, so the loop holds little beyond the loads and stores: along one interval the address moves by a constant.

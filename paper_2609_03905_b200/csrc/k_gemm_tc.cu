@@ -26,6 +26,9 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+#include <atomic>
+
 #include "ja_device.cuh"
 #include "ja_launch.cuh"
 #include "ja_ptx.cuh"
@@ -72,6 +75,8 @@ struct GemmParams {
     // fused epilogue (a join-agg chain executed in one pass, the intermediate never stored)
     int32_t epi;               // EPI_*
     int32_t bn_tile;           // output columns per tile: 256, or 128 for EPI_SWIGLU (two 128-column products per tile)
+    int32_t tile0, tile_end;   // the tiles of this launch
+    int32_t split;             // SPLIT: slices of the contracted index = CTA pairs per cluster
     int32_t n_copies;          // 1: SUM over all contracted blocks (aggregated output). nbk: join only -- tile (c, ., .) covers the
                                // single contracted block c and is stored to copy c of a partial relation [c, i, k]
     int32_t c_esize;           // bytes per output cell: 2 (bf16 / f16) or 4 (f32, partial relations only)
@@ -158,7 +163,7 @@ __device__ __forceinline__ int tile_of_iter(const GemmParams& p, int i, int firs
 
 // F16: cell type of the operands and of a 2-byte output -- bf16 or f16 (a compile-time choice: a select between the two
 // conversions in the epilogue cost the plain contraction a tenth of its rate)
-template <int CG, bool F16>
+template <int CG, bool F16, bool SPLIT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmB2, const GemmParams p) {
@@ -181,7 +186,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;   // warp-uniform by construction
-    const int cta_rank = CG == 2 ? (int)cluster_ctarank() : 0;   // 0 = leader of the pair
+    const int cl_rank = CG == 2 ? (int)cluster_ctarank() : 0;
+    const int cta_rank = SPLIT ? cl_rank & 1 : cl_rank;           // 0 = leader of the pair
+    const uint32_t pair0 = SPLIT ? (uint32_t)(cl_rank & ~1) : 0;  // the leader's rank in the cluster
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar(s), 1);    // CG 2: only the leader's is used; both CTAs' copies complete_tx on it
@@ -211,9 +218,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     ja_wait_for_stream();
     ja_let_next_start();
 
-    const int total_tiles = p.m_tiles * p.n_tiles * p.n_copies;
     const int kchunks = (p.bk + Cfg<CG>::BK - 1) / Cfg<CG>::BK;
-    const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
+    const int total_tiles = p.tile_end;
+    const int first_tile = SPLIT ? p.tile0 + (int)blockIdx.x / (2 * p.split) : (int)blockIdx.x / CG, tile_step = SPLIT ? p.tile_end : (int)gridDim.x / CG;
+    // the stages [ch0, ch1) of a tile that this CTA group accumulates: all of its contracted blocks', or (SPLIT) one slice of them
+    auto stages_of = [&](const TileCoord& tc, int* ch0, int* ch1) {
+        *ch0 = tc.jb0 * kchunks;
+        *ch1 = tc.jb1 * kchunks;
+        if (SPLIT) {
+            const int64_t n = *ch1;
+            *ch0 = (int)(n * (cl_rank >> 1) / p.split);
+            *ch1 = (int)(n * ((cl_rank >> 1) + 1) / p.split);
+        }
+    };
 
     if (warp == 0) {
         // ================= TMA producer (one per CTA) =================
@@ -234,11 +251,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 const int my_c0 = cta_rank * my_cols;              // their offset inside the tile
                 const int nchunks = (my_cols + 63) / 64;
                 const uint32_t tx = (uint32_t)CG * ((uint32_t)(p.a_boxes * p.a_box_rows) * (BK * 2) + nchunks * B_CHUNK_BYTES);
-                for (int jb = tc.jb0; jb < tc.jb1 && ok; ++jb) {    // the tuples of this output key, ascending j
-                    for (int kc = 0; kc < kchunks; ++kc) {
-                        if (!mbar_wait(empty_bar(stage), phase ^ 1, abort_flag, p.status)) { ok = false; break; }
+                int ch, ch1;
+                stages_of(tc, &ch, &ch1);
+                for (int jb = ch / kchunks, kc = ch - jb * kchunks; ch < ch1; ++jb, kc = 0) {    // the tuples of this output key, ascending j
+                    for (; kc < kchunks && ch < ch1; ++kc, ++ch) {
+                        if (!mbar_wait(empty_bar(stage), phase ^ 1, abort_flag, p.status)) { ok = false; ch = ch1; break; }
                         uint32_t fb = full_bar(stage);
-                        if (CG == 2) fb = mapa_cluster(fb, 0);      // completion is counted on the leader's barrier
+                        if (CG == 2) fb = mapa_cluster(fb, pair0);  // completion is counted on the leader's barrier
                         if (cta_rank == 0) mbar_expect_tx(full_bar(stage), tx);
                         issued[stage] = true;
                         last_parity[stage] = phase;
@@ -273,6 +292,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             (void)issued; (void)last_parity;
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ================= MMA issuer (leader CTA only): the whole warp runs the loop, one elected lane issues =================
         if (cta_rank == 0) {
@@ -296,9 +316,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 uint32_t accumulate = 0;
-                for (int jb = tc.jb0; jb < tc.jb1 && ok; ++jb) {
-                    for (int kc = 0; kc < kchunks; ++kc) {
-                        if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) { ok = false; break; }
+                int ch, ch1;
+                stages_of(tc, &ch, &ch1);
+                for (int kc = ch % kchunks; ch < ch1; kc = 0) {
+                    for (; kc < kchunks && ch < ch1; ++kc, ++ch) {
+                        if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) { ok = false; ch = ch1; break; }
                         tc_fence_after();
                         const int kvalid = min(BK, p.bk - kc * BK);
                         const int k16 = (kvalid + 15) / 16;
@@ -321,14 +343,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             }
                         }
                         accumulate = 1;
-                        umma_commit_w<CG>(empty_bar(stage), leader);  // frees the smem stage (in both CTAs) once these MMAs have read it
+                        umma_commit_w<CG>(empty_bar(stage), leader, pair0);  // frees the smem stage (in both CTAs) once these MMAs have read it
                         if (++stage == STAGES) { stage = 0; phase ^= 1; }
                     }
                 }
-                if (ok) umma_commit_w<CG>(tfull_bar(acc), leader);    // accumulator complete -> epilogue(s)
+                if (ok) umma_commit_w<CG>(tfull_bar(acc), leader, pair0);    // accumulator complete -> epilogue(s)
             }
         }
-    } else {
+    } else if (!SPLIT) {
         // ================= epilogue (warps 2..5 of every CTA) =================
         const int q = warp & 3;  // TMEM lane group this warp may access
         uint32_t acc_phase[2] = {0, 0};
@@ -420,6 +442,80 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
         }
     }
+    if constexpr (SPLIT) {
+        // ================= the slices' sum: every row goes to one CTA of the cluster, [slice][row][column] f32 over the stages =================
+        const TileCoord tc = tile_coord<CG>(p, first_tile, cta_rank);
+        const bool ok = mbar_wait(tfull_bar(0), 0, abort_flag, p.status);
+        tc_fence_after();
+        __syncwarp();
+        cluster_sync_all();   // every product of the cluster has read its stages
+        constexpr int PITCH = BN + 4;
+        const int mine = BM / p.split, slice = cl_rank >> 1;
+        if (ok && warp >= 2) {
+            const int q = warp & 3, r = q * 32 + lane;
+            const uint32_t at = mapa_cluster(base + (uint32_t)((slice * mine + r % mine) * PITCH) * 4u, (uint32_t)(r / mine * 2 + cta_rank));
+            const int cols = p.epi == EPI_SWIGLU ? BN : tc.width;
+            for (int ch = 0; ch * 32 < cols; ++ch) {
+                uint32_t v[32];
+                tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + ch * 32, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) st_cluster16(at + ch * 128 + e * 4, v[e], v[e + 1], v[e + 2], v[e + 3]);
+            }
+        }
+        tc_fence_before();
+        __syncwarp();
+        cluster_sync_all();
+        if (*abort_flag == 0) {
+            const int ppr = (tc.width + 7) / 8;      // 8-column pieces of a row
+            for (int i = threadIdx.x; i < mine * ppr; i += NUM_THREADS) {
+                const int own = i / ppr, c = (i - own * ppr) * 8, r = slice * mine + own;
+                if (r >= tc.rows) break;             // rows only grow
+                const float* src = reinterpret_cast<const float*>(smem) + own * PITCH + c;
+                auto sum8 = [&](const float* s, float (&f)[8]) {   // slices in ascending order
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) f[e] = 0.f;
+                    for (int k = 0; k < p.split; ++k, s += mine * PITCH) {
+                        const float4 u = *reinterpret_cast<const float4*>(s), w = *reinterpret_cast<const float4*>(s + 4);
+                        f[0] += u.x; f[1] += u.y; f[2] += u.z; f[3] += u.w; f[4] += w.x; f[5] += w.y; f[6] += w.z; f[7] += w.w;
+                    }
+                };
+                float f[8];
+                sum8(src, f);
+                const int grow = tc.row_g0 + r, gcol = tc.n_g0 + c, kb = gcol / p.bn, cin = gcol - kb * p.bn, ib = grow / p.bm, iin = grow - ib * p.bm;
+                const int64_t off = p.c_blk_off[(int64_t)ib * p.nbn + kb] + ((int64_t)iin * p.bn + cin) * 2;
+                if (p.epi == EPI_SWIGLU) {
+                    float g[8];
+                    sum8(src + p.bn_tile, g);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) f[e] = f[e] / (1.f + __expf(-f[e])) * g[e];
+                } else if (p.epi == EPI_ROPE) {
+                    const float2* tab = p.rope_table + ((int64_t)(grow % p.rope_S) * p.rope_D + gcol % p.rope_D) / 2;
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        const float2 cs = tab[e / 2];
+                        const float x0 = f[e], x1 = f[e + 1];
+                        f[e] = x0 * cs.x - x1 * cs.y;
+                        f[e + 1] = x0 * cs.y + x1 * cs.x;
+                    }
+                } else if (p.epi == EPI_ADD) {
+                    const uint4 rv = *reinterpret_cast<const uint4*>(p.r_base + off);
+                    const uint32_t* pr = reinterpret_cast<const uint32_t*>(&rv);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 rf = ja_unpack16<F16>(pr[e]);
+                        f[2 * e] += rf.x;
+                        f[2 * e + 1] += rf.y;
+                    }
+                }
+                uint4 o;
+                uint32_t* po = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) po[e] = ja_pack16<F16>(f[2 * e], f[2 * e + 1]);
+                *reinterpret_cast<uint4*>(p.c_base + off) = o;
+            }
+        }
+    }
     // ---- teardown ---------------------------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
@@ -431,9 +527,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
+}  // namespace
+
 // ---- host: tensor maps -------------------------------------------------------------------------------------
 // A relation [R, C] with equal blocks br x bc is the rank-4 tensor (c in block, r in block, col-block, row-block).
-ja_status_t encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows, CUtensorMap* tm) {
+ja_status_t ja_encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows, CUtensorMap* tm) {
     if (box_rows > 256) return ja_fail(JA_ERR_INVALID_ARG, "TMA box too tall");
     EncodeTiledFn enc = get_encode();
     if (!enc) return ja_fail(JA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
@@ -450,14 +548,82 @@ ja_status_t encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows,
     return JA_OK;
 }
 
-}  // namespace
-
 struct GemmTcPlan {
     CUtensorMap tmA, tmB, tmB2;
     GemmParams p;
-    int grid;
-    int cg;   // CTAs per tile: 1 or 2
+    int cg;      // CTAs per tile: 1 or 2
+    int tiles;   // of the whole launch; the last `tail` of them go to a launch of their own, each split along the contracted index
+    int tail, split;
+    double us;   // what the launches are expected to take
 };
+
+namespace {
+
+template <bool F16>
+cudaError_t configure() {
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<1, F16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES);
+    return e;
+}
+
+// clusters of `split` CTA pairs that the device holds at once
+int clusters_at_once(int split) {
+    static std::atomic<int> known[64][3];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::atomic<int>& n = known[dev & 63][split == 2 ? 0 : 1];
+    if (n.load() == 0) {
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof cfg);
+        cfg.gridDim = dim3((unsigned)(2 * split), 1, 1);
+        cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+        cfg.dynamicSmemBytes = Cfg<2>::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        memset(attr, 0, sizeof attr);
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)(2 * split);
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc_kernel<2, false, true>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            c = 0;
+        }
+        n.store(c > 0 ? c : -1);
+    }
+    return std::max(n.load(), 0);
+}
+
+// Whether the tiles of the last, partly empty round over the pairs of SMs are each split along the contracted index over a
+// cluster of pairs. A 128-deep stage of a 256-row tile takes 0.96 us (1.3 PFLOP/s over the chip); the clusters' sums and their own
+// start and end take 10 us ([1024, 4096] x [4096, 1024] 26 us with four slices a tile, 35 whole), and 2 more where a launch of whole tiles runs
+// before them.
+void choose_tail(GemmTcPlan* plan) {
+    const GemmParams& p = plan->p;
+    const int stages = (p.bk + Cfg<2>::BK - 1) / Cfg<2>::BK * p.nbk, pairs = ja_sm_count() / 2;
+    const int whole = plan->tiles / pairs, rest = plan->tiles % pairs;
+    plan->tail = 0;
+    plan->split = 1;
+    double best = (double)(whole + (rest > 0)) * stages * 0.96;
+    // (tiles sorted by weight fill the last round with narrow ones: [2048, 4096] x [4096, 11008] in 1376-wide blocks 147 us, 150 with its last 14 split)
+    if (p.n_copies == 1 && rest > 0 && !p.heavy_first && ja_config().gemm_split != 0) {
+        for (int s : {2, 4}) {
+            const int at_once = clusters_at_once(s);
+            if (stages < 2 * s || at_once == 0) continue;
+            const double t = (double)whole * stages * 0.96 + (double)((rest + at_once - 1) / at_once) * ((stages + s - 1) / s) * 0.96 + (whole ? 12.0 : 10.0);
+            if (t < best) {
+                best = t;
+                plan->tail = rest;
+                plan->split = s;
+            }
+        }
+    }
+    plan->us = best + 8.0;
+}
+
+}  // namespace
 
 ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, const GemmEpilogue* ep,
                             std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
@@ -504,7 +670,7 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     p.heavy_first = (p.n_copies == 1 && p.tiles_per_nblk > 1 && bn % bn_tile != 0 && cfg.gemm_heavy_first != 0) ? 1 : 0;
     p.group_m = cfg.gemm_group_m >= 1 ? cfg.gemm_group_m : 8;
     const bool by_block = odd_rows || (bm > 128 && bm % 128 != 0);
-    bool two = p.M >= 256 && bk >= Cfg<2>::BK;
+    bool two = p.M > BM && bk >= Cfg<2>::BK;
     // join-only tiles of short blocks are mostly store, and pairs of row tiles hand out half as many: [8048, 576] x [576, 320] in blocks of
     // 4024 x 144 x 80 22.8 us single, 27.9 on pairs; 1.23 times as fast on pairs at 1000 contracted cells
     if (by_block && p.n_copies > 1 && bk < 512) two = false;
@@ -514,33 +680,51 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     if (!by_block) { p.tiles_per_mblk = 0; p.m_tiles = (p.M + BM * plan->cg - 1) / (BM * plan->cg); }
     else { p.tiles_per_mblk = (int)((bm + BM - 1) / BM); p.m_tiles = (p.tiles_per_mblk * p.nbm + plan->cg - 1) / plan->cg; }
     ja_status_t st;
-    if ((st = encode_blocked_2d(A, 64, p.a_box_rows, &plan->tmA)) != JA_OK) return st;
-    if ((st = encode_blocked_2d(B, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB)) != JA_OK) return st;
+    if ((st = ja_encode_blocked_2d(A, 64, p.a_box_rows, &plan->tmA)) != JA_OK) return st;
+    if ((st = ja_encode_blocked_2d(B, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB)) != JA_OK) return st;
     plan->tmB2 = plan->tmB;
-    if (epi == EPI_SWIGLU && (st = encode_blocked_2d(ep->B2, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB2)) != JA_OK) return st;
-    const int sms = ja_sm_count();
-    const int tiles = p.m_tiles * p.n_tiles * p.n_copies;
-    plan->grid = two ? 2 * std::min(sms / 2, tiles) : std::min(sms, tiles);
-    cudaError_t e;
-    if (p.f16)
-        e = two ? cudaFuncSetAttribute(gemm_tc_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES)
-                : cudaFuncSetAttribute(gemm_tc_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES);
-    else
-        e = two ? cudaFuncSetAttribute(gemm_tc_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES)
-                : cudaFuncSetAttribute(gemm_tc_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES);
+    if (epi == EPI_SWIGLU && (st = ja_encode_blocked_2d(ep->B2, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB2)) != JA_OK) return st;
+    cudaError_t e = p.f16 ? configure<true>() : configure<false>();
     if (e != cudaSuccess) return ja_cuda_fail(e, "cudaFuncSetAttribute(gemm_tc_kernel)");
+    plan->tiles = p.m_tiles * p.n_tiles * p.n_copies;
+    plan->tail = 0;
+    plan->split = 1;
+    if (two) choose_tail(plan.get());
+    else plan->us = (double)((plan->tiles + ja_sm_count() - 1) / ja_sm_count()) * ((p.bk + 63) / 64) * (p.n_copies > 1 ? 1 : p.nbk) * 0.70 + 8.0;
     *out = plan;
     *eligible = true;
     return JA_OK;
 }
 
-// What the launch is expected to take: rounds of tiles over the CTA groups, 0.48 us per 64 contracted cells of a 256-row tile on
-// a pair of SMs (1.3 PFLOP/s over the chip), 0.70 of a 128-row tile on one, and a start and an end.
-double ja_gemm_tc_estimate_us(const GemmTcPlan& plan) {
-    const GemmParams& p = plan.p;
-    const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles * p.n_copies, groups = plan.grid / plan.cg;
-    const double stages = (double)((p.bk + 63) / 64) * (p.n_copies > 1 ? 1 : p.nbk);
-    return (double)((tiles + groups - 1) / groups) * stages * (plan.cg == 2 ? 0.48 : 0.70) + 8.0;
+// What the launches are expected to take: rounds of tiles over the CTA groups, 0.96 us per 128 contracted cells of a 256-row tile on
+// a pair of SMs, 0.70 per 64 of a 128-row tile on one, and a start and an end.
+double ja_gemm_tc_estimate_us(const GemmTcPlan& plan) { return plan.us; }
+
+template <bool F16>
+static ja_status_t launch_gemm(const GemmTcPlan& plan, GemmParams& p, cudaStream_t st) {
+    const int sms = ja_sm_count();
+    p.tile0 = 0;
+    p.tile_end = plan.tiles - plan.tail;
+    if (plan.cg == 1) {
+        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<1, F16, false>, dim3((unsigned)std::min(sms, p.tile_end), 1, 1), NUM_THREADS, Cfg<1>::SMEM_BYTES, 1, st, plan.tmA,
+                                 plan.tmB, plan.tmB2, p));
+        ja_count_launch();
+        return JA_OK;
+    }
+    if (p.tile_end > 0) {
+        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<2, F16, false>, dim3((unsigned)(2 * std::min(sms / 2, p.tile_end)), 1, 1), NUM_THREADS, Cfg<2>::SMEM_BYTES, 2, st,
+                                 plan.tmA, plan.tmB, plan.tmB2, p));
+        ja_count_launch();
+    }
+    if (plan.tail > 0) {
+        p.tile0 = p.tile_end;
+        p.tile_end = plan.tiles;
+        p.split = plan.split;
+        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<2, F16, true>, dim3((unsigned)(plan.tail * 2 * plan.split), 1, 1), NUM_THREADS, Cfg<2>::SMEM_BYTES,
+                                 (unsigned)(2 * plan.split), st, plan.tmA, plan.tmB, plan.tmB2, p));
+        ja_count_launch();
+    }
+    return JA_OK;
 }
 
 ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st) {
@@ -548,11 +732,5 @@ ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st) {
     p.status = ja_device_status_word(st);
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
-    const dim3 grid((unsigned)plan.grid, 1, 1);
-    if (plan.cg == 2)
-        JA_CUDA(ja_launch_kernel(p.f16 ? gemm_tc_kernel<2, true> : gemm_tc_kernel<2, false>, grid, NUM_THREADS, Cfg<2>::SMEM_BYTES, 2, st, plan.tmA, plan.tmB, plan.tmB2, p));
-    else
-        JA_CUDA(ja_launch_kernel(p.f16 ? gemm_tc_kernel<1, true> : gemm_tc_kernel<1, false>, grid, NUM_THREADS, Cfg<1>::SMEM_BYTES, 1, st, plan.tmA, plan.tmB, plan.tmB2, p));
-    ja_count_launch();
-    return JA_OK;
+    return p.f16 ? launch_gemm<true>(plan, p, st) : launch_gemm<false>(plan, p, st);
 }

@@ -1,0 +1,67 @@
+"""Products that leave most of the chip idle as whole tiles: few tiles, or a few in the last round,
+split along the contracted index over clusters (k_gemm_tc.cu), against an fp64 product of the same 16-bit inputs.
+Tolerance: gpu_util.TOL, ten half-ulps of the stored type."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_03905_b200 as ja
+import synth_inputs as si
+from oracle import blocked
+
+from gpu_util import TOL, check_status, download, empty_like_tiling, relfro, upload
+
+pytestmark = pytest.mark.gpu
+ES = blocked.equal_splits
+BF, F16 = torch.bfloat16, torch.float16
+
+
+def _problem(ti, tj, tk, dtype):
+    m, k, n = ti[-1], tj[-1], tk[-1]
+    a, b = si.normal((m, k), 0.0, 1.0, dtype, 37, 40), si.normal((k, n), 0.0, 1.0, dtype, 37, 41)
+    res = empty_like_tiling([m, n], [ti, tk], dtype, fill=float("nan"))
+    return a, b, upload(a, [ti, tj]), upload(b, [tj, tk]), res, ja.Spec("ij,jk->ik", {"i": ti, "j": tj, "k": tk})
+
+
+def _check(res, a, b, dtype):
+    got, ref = download(res), si.to_f64(a) @ si.to_f64(b)
+    check_status()
+    assert relfro(got, ref) <= TOL[dtype]
+    ulp = 2.0 ** (-7 if dtype == BF else -10)      # of the largest value: a misplaced cell is far outside it
+    assert np.abs(got - ref).max() <= ulp * np.abs(ref).max()
+
+
+# whole tiles, split tiles, and both: few tiles (clusters of two and of four pairs), one more than a round, blocks whose ends are inside a slice
+@pytest.mark.parametrize("m,gi,k,gj,n,gk", [(512, 4, 4096, 8, 1024, 8), (1024, 8, 4096, 8, 2048, 4), (256, 2, 2048, 2, 4096, 8), (1280, 1, 1024, 1, 3840, 1),
+                                            (600, 1, 1376, 8, 512, 1), (2560, 10, 512, 1, 1920, 1)])
+@pytest.mark.parametrize("fn", ["mul", "matmul_add", "swiglu_up", "matmul_rope"])
+def test_split_tiles(m, gi, k, gj, n, gk, fn):
+    ti, tj, tk = ES(m, gi), ES(k, gj), ES(n, gk)
+    if fn != "mul" and ((n // gk) % 128 or (k // gj) % 8):
+        pytest.skip("the fused forms take whole 128-column blocks and rows of whole 16 bytes")
+    a, b, ra, rb, res, spec = _problem(ti, tj, tk, BF)
+    parts, scale = {"i": ti, "j": tj, "k": tk}, k ** -0.5
+    b = (b.float() * scale).to(BF)
+    rb = upload(b, [tj, tk])
+    ref = si.to_f64(a) @ si.to_f64(b)
+    if fn == "mul":
+        spec.execute([ra, rb], res)
+    elif fn == "matmul_add":
+        x = si.normal((m, n), 0.0, 1.0, BF, 37, 42)
+        ref = ref + si.to_f64(x)
+        ja.Spec("ij,jk,ik->ik", parts, fn).execute([ra, rb, upload(x, [ti, tk])], res)
+    elif fn == "swiglu_up":
+        b2 = (si.normal((k, n), 0.0, 1.0, BF, 37, 43).float() * scale).to(BF)
+        ref = ref / (1.0 + np.exp(-ref)) * (si.to_f64(a) @ si.to_f64(b2))
+        ja.Spec("ij,jk,jk->ik", parts, fn).execute([ra, rb, upload(b2, [tj, tk])], res)
+    else:
+        s_len, d = m // 2, 128
+        ang = np.arange(s_len)[:, None] * 10000.0 ** (-2.0 * np.arange(d // 2) / d)[None, :]
+        c, s = np.tile(np.cos(ang), (2, n // d)), np.tile(np.sin(ang), (2, n // d))
+        x0, x1 = ref[:, 0::2].copy(), ref[:, 1::2].copy()
+        ref[:, 0::2], ref[:, 1::2] = x0 * c - x1 * s, x0 * s + x1 * c
+        ja.Spec("ij,jk->ik", parts, fn, (10000.0, float(s_len), float(d))).execute([ra, rb], res)
+    got = download(res)
+    check_status()
+    assert relfro(got, ref) <= TOL[BF]
+    assert np.abs(got - ref).max() <= 2.0 ** -6 * np.abs(ref).max()
