@@ -976,6 +976,7 @@ extern "C" ja_status_t ja_repartition_agg(const ja_relation_t* partials, ja_agg_
 // ---------------------------------------------------------------------------------------------------
 struct ExecPlan {
     std::shared_ptr<GemmTcPlan> gemm;
+    std::shared_ptr<StreamTcPlan> stream;   // kept where it is expected to be faster than the other two forms
     bool gemm_checked = false;
     std::shared_ptr<ContractTcPlan> contract;
     std::shared_ptr<ContractF32Plan> contract_f32;
@@ -1102,6 +1103,10 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 if (!ok) plan->gemm.reset();
                 if ((st = ja_contract_tc_plan(in[0], in[1], o, A, B, out, &plan->contract, &us)) != JA_OK) return st;
                 plan->contract_first = plan->contract && (!plan->gemm || us < 0.9 * ja_gemm_tc_estimate_us(*plan->gemm));
+                double stream_us = 0;
+                if ((st = ja_stream_tc_plan(A, B, out, &plan->stream, &stream_us)) != JA_OK) return st;
+                if (plan->stream && (loader >= 0 || (plan->gemm && stream_us > ja_gemm_tc_estimate_us(*plan->gemm)) || (plan->contract && stream_us > us)))
+                    plan->stream.reset();
                 // A small product that TMA cannot address, in odd intervals: the plain-ALU kernel where its 32 x 32 tiles fit the chip twice
                 // over (64 x 314 x 320 in 2 x 8 x 4: 19 us against 46, 250 x 314 x 333 in 2 x 2 x 4: 15 against 27; 64 x 3001 x 320 in 8 x 64
                 // x 4 is 123 against 60 and stays). Its time: a start, and so much a cell and an interval of the contracted index.
@@ -1117,6 +1122,7 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 }
                 plan->contract_checked = true;
             }
+            if (plan->stream) return ja_launch_stream_tc(*plan->stream, stream);
             if (plan->gemm && loader != 1 && (loader == 0 || !plan->contract_first)) return ja_launch_gemm_tc(*plan->gemm, stream);
             if (plan->contract && loader != 0) return ja_launch_contract_tc(*plan->contract, stream);
         } else {

@@ -211,6 +211,11 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
 ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st);
 double ja_gemm_tc_estimate_us(const GemmTcPlan& plan);
 
+// Few rows against a large second operand: a TMA stream over it (k_stream_tc.cu). *out stays empty where the relations do not fit.
+struct StreamTcPlan;
+ja_status_t ja_stream_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us);
+ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st);
+
 // Attention join-agg (QK^T join, online-softmax aggregation, PV).
 // the four tensor maps (Q, K, V, O) of the tensor-memory kernels, encoded once per (spec, relations) tuple
 struct AttnTcCache {

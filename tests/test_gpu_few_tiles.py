@@ -1,5 +1,5 @@
-"""Products that leave most of the chip idle as whole tiles: few tiles, or a few in the last round,
-split along the contracted index over clusters (k_gemm_tc.cu), against an fp64 product of the same 16-bit inputs.
+"""Products that leave most of the chip idle as whole tiles: few rows against a large second operand (k_stream_tc.cu), and few tiles, or a few
+in the last round, split along the contracted index over clusters (k_gemm_tc.cu), against an fp64 product of the same 16-bit inputs.
 Tolerance: gpu_util.TOL, ten half-ulps of the stored type."""
 import numpy as np
 import pytest
@@ -29,6 +29,16 @@ def _check(res, a, b, dtype):
     assert relfro(got, ref) <= TOL[dtype]
     ulp = 2.0 ** (-7 if dtype == BF else -10)      # of the largest value: a misplaced cell is far outside it
     assert np.abs(got - ref).max() <= ulp * np.abs(ref).max()
+
+
+# few rows that need no copy: row blocks of any height, column tiles inside blocks and across them, every number of slices
+@pytest.mark.parametrize("m,gi,k,gj,n,gk", [(32, 1, 4096, 8, 11008, 8), (8, 1, 512, 1, 256, 1), (1, 1, 2048, 2, 4096, 4), (100, 1, 1024, 4, 1000, 1), (128, 4, 2048, 1, 640, 5),
+                                            (36, 3, 1024, 1, 768, 1), (64, 1, 64, 1, 8192, 1), (16, 2, 4096, 1, 1504, 1)])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_few_rows(m, gi, k, gj, n, gk, dtype):
+    a, b, ra, rb, res, spec = _problem(ES(m, gi), ES(k, gj), ES(n, gk), dtype)
+    spec.execute([ra, rb], res)
+    _check(res, a, b, dtype)
 
 
 # whole tiles, split tiles, and both: few tiles (clusters of two and of four pairs), one more than a round, blocks whose ends are inside a slice
