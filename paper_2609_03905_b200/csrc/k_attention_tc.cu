@@ -532,6 +532,13 @@ __device__ __forceinline__ float row_exp_pack128(const uint32_t (&v)[128], float
 //   two-entry queue in shared memory, and runs ahead into the next item as soon as the Q buffers are free, so the next
 //   item's Q and first K tile load, and its first Q K^T run, while the row threads finish this item. Barrier phases follow
 //   running counters (items; key steps per tile). Otherwise one CTA per item, handed out by the hardware in grid order.
+//   What lies between two items of a row warp was 6400 cycles (a key step is 3400): the TMA stores of the output are now waited for
+//   where their tile is written again, the producer hands out items worked out, and a CTA's first item is its own number.
+//   B4 S2048 171.0 -> 169.5 us, five packed sequences 111.8 -> 110.0 (a loop of calls, at the power limit's clock).
+//   Traces of the row warps at that point: per key step 220 cycles to the scores, 240 for the load, 500 for the maximum, 280 for the P
+//   tile, 1530 for the exponentials and the store of P. Tiles taking turns at the exponentials (+3 %: by itself a warp's take as long),
+//   and P in tensor memory with one S tile that passes between the two (+4 %, packed +11 %: each waits for the other's load) were built,
+//   verified and taken back.
 // VAR selects row-thread variants ("attn_variant"; all verified against the oracle): bits 0-1 = POLY of row_exp_pack128, bit 2 =
 //   exponentiate into registers first and wait for the P tile only before storing. Default 1: a quarter of the exponentials
 //   on the FMA pipe (B4 S2048 H32 causal, same run: POLY 0 0.1430 ms, one of eight 0.1405, one of four 0.1403, two of four
@@ -571,7 +578,7 @@ __device__ __forceinline__ float row_exp_pack128(const uint32_t (&v)[128], float
 //   add half as much again: the shared-memory port, not a pipe, bounds long sequences (tensor-core reads 53 % + stores
 //   19 % of its cycles over a whole launch of B4 S2048).
 constexpr int NUM_THREADS2 = 320;
-constexpr int SMEM_BYTES2 = 7 * TILE_BYTES + 1024 + 256;
+constexpr int SMEM_BYTES2 = 7 * TILE_BYTES + 1024 + 512;
 
 // {next item, CTAs finished} pairs for launches of the persistent form: a launch takes the next pair of the ring, and its
 // last CTA zeroes the pair again, so a pair is ready for reuse (also by a replay of a captured launch) as soon as its kernel
@@ -660,7 +667,9 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
     auto bar = [&](int i) { return bar0 + 8u * i; };
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);   // two words: abort flag, wait limit
-    volatile int* item_rank = reinterpret_cast<volatile int*>(tmem_slot + 3);    // [2]: the item numbers in flight
+    // the items in flight, as the producer has worked them out: a row warp that did the divisions itself spent 1200 cycles an item on them
+    AttnItem* item_at = reinterpret_cast<AttnItem*>(bars + NBAR + 2);            // [2]
+    static_assert((NBAR + 2) * 8 + 2 * sizeof(AttnItem) <= 512, "barriers and items behind the tiles");
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     // consumers of the item queue (MMA warp, row warps): wait for entry k, read it, release it
@@ -668,11 +677,10 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
         if (!PERSIST) return k == 0 && attn_item(p, (int)blockIdx.x, it);
         const int e = k & 1;
         if (!mbar_wait(bar(ITEM_FULL + e), (uint32_t)(k >> 1) & 1, abort_flag, p.status)) return false;
-        const int rank = item_rank[e];
+        *it = item_at[e];
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + e));
-        if constexpr (RAGGED) return attn_item(p, *rt, rank, it);
-        else return attn_item(p, rank, it);
+        return it->n > 0;
     };
 
     if (threadIdx.x == 0) {
@@ -703,23 +711,21 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
             AttnItem it;
             for (int item = 0; ok; ++item) {
                 int rank;
+                // the first item of a CTA is its own number, the counter hands out the ones after those (its trip to memory is 2500 cycles)
+                if (!PERSIST && item > 0) break;
+                rank = item == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(p.queue, 1);
+                bool more;
+                if constexpr (RAGGED) more = attn_item(p, *rt, rank, &it);
+                else more = attn_item(p, rank, &it);
                 if (PERSIST) {
-                    // claim the next item and publish its number (entry item & 1 of the queue, free once all nine consumer
-                    // warps have read what it held two items ago)
+                    // publish the item (entry item & 1 of the queue, free once all nine consumer warps have read what it held two items ago)
                     const int e = item & 1;
                     if (item >= 2 && !mbar_wait(bar(ITEM_EMPTY + e), (uint32_t)((item >> 1) - 1) & 1, abort_flag, p.status)) break;
-                    rank = atomicAdd(p.queue, 1);
-                    item_rank[e] = rank;
+                    if (!more) it.n = 0;
+                    item_at[e] = it;
                     mbar_arrive(bar(ITEM_FULL + e));
-                } else {
-                    if (item > 0) break;
-                    rank = (int)blockIdx.x;
                 }
-                if constexpr (RAGGED) {
-                    if (!attn_item(p, *rt, rank, &it)) break;
-                } else {
-                    if (!attn_item(p, rank, &it)) break;
-                }
+                if (!more) break;
                 const int hk = it.h / p.group;
                 // the Q buffers are free once the previous item's last Q K^T has read them
                 if (item > 0 && !mbar_wait(bar(Q_EMPTY), (uint32_t)(item - 1) & 1, abort_flag, p.status)) break;
@@ -1001,6 +1007,10 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                 // read the P tile (P_EMPTY; O~ then also holds every product so far), and at the first step of an item the
                 // TMA stores of the previous item's output, which was staged in the P tile, have read it (P_STORED).
                 auto wait_p_tile = [&]() -> bool {
+                    if (j == 0 && done > 0 && q == 0 && lane == 0) {   // the thread that issued those stores
+                        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        mbar_arrive(bar(P_STORED + t));
+                    }
                     if (c > 0 && !mbar_wait(bar(P_EMPTY + t), (uint32_t)(c - 1) & 1, abort_flag, p.status)) return false;
                     if (j == 0 && done > 0 && !mbar_wait(bar(P_STORED + t), (uint32_t)(done - 1) & 1, abort_flag, p.status)) return false;
                     return true;
@@ -1093,15 +1103,15 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
                                 tma_store_3d(&tmO, sP + t * TILE_BYTES + half * HALF_BYTES + i * 128, half * 64, it.h % p.q.hblk, orow);
                         }
                     }
+                    // waited for where the P tile is written again: waiting here held the warp for 1300 cycles an item
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory may be reused after this
-                    mbar_arrive(bar(P_STORED + t));  // the P tile may be written again
                 }
             }
             ok = __all_sync(0xffffffffu, ok);
             cs += n_t;
             ++done;
         }
+        if (q == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // shared memory goes with the CTA
     }
     tc_fence_before();
     __syncthreads();
