@@ -72,6 +72,29 @@ template <bool F16> __device__ __forceinline__ float2 ja_unpack16(uint32_t w) {
     return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
 }
 
+// the interval [lo, hi) of dimension d that holds x: the tables are read only where the intervals differ (a trip to memory a lookup)
+__device__ __forceinline__ int ja_interval(const RelView& v, int d, int x, int* lo, int* hi) {
+    if (v.nblk[d] == 1) {
+        *lo = 0;
+        *hi = (int)v.extent[d];
+        return 0;
+    }
+    if (v.bs[d]) {
+        const int bs = (int)v.bs[d], b = x / bs;
+        *lo = b * bs;
+        *hi = min(*lo + bs, (int)v.extent[d]);
+        return b;
+    }
+    const int b = ja_find_blk(v, d, x);
+    *lo = (int)v.splits[d][b];
+    *hi = (int)v.splits[d][b + 1];
+    return b;
+}
+// byte offset of block (rb, cb) of a two-index relation
+__device__ __forceinline__ int64_t ja_block_at(const RelView& v, int rb, int cb) {
+    const int64_t flat = (int64_t)rb * v.nblk[1] + cb;
+    return v.blk_stride ? flat * v.blk_stride : v.blk_off[flat];
+}
 // Launch order of the attention CTAs (CTAs are handed to SMs in order of blockIdx.x). One CTA = one query tile (or pair
 // of tiles) of one (batch, head). (batch, head) pairs are taken in sections of `sect` consecutive pairs and inside a
 // section all pairs run their heaviest tile first, then the next one, and so on. One section holding every pair is

@@ -977,6 +977,7 @@ extern "C" ja_status_t ja_repartition_agg(const ja_relation_t* partials, ja_agg_
 struct ExecPlan {
     std::shared_ptr<GemmTcPlan> gemm;
     std::shared_ptr<StreamTcPlan> stream;   // kept where it is expected to be faster than the other two forms
+    std::shared_ptr<StagedPlan> staged;     // likewise
     bool gemm_checked = false;
     std::shared_ptr<ContractTcPlan> contract;
     std::shared_ptr<ContractF32Plan> contract_f32;
@@ -1110,6 +1111,7 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 // A small product that TMA cannot address, in odd intervals: the plain-ALU kernel where its 32 x 32 tiles fit the chip twice
                 // over (64 x 314 x 320 in 2 x 8 x 4: 19 us against 46, 250 x 314 x 333 in 2 x 2 x 4: 15 against 27; 64 x 3001 x 320 in 8 x 64
                 // x 4 is 123 against 60 and stays). Its time: a start, and so much a cell and an interval of the contracted index.
+                double now = plan->contract ? us * ja_contract_tc_pieces(*plan->contract) : 1e30;
                 if (plan->contract && !plan->gemm && loader != 1) {
                     auto tiles = [](const ja_relation* r, int d) {
                         int64_t n = 0;
@@ -1118,9 +1120,21 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                     };
                     const int64_t t = tiles(A, 0) * tiles(B, 1), sms = ja_sm_count();
                     const double simt_us = (3.0 + 0.0295 * (double)A->extent[1] + 0.85 * A->nblk[1]) * (t <= sms ? 1.0 : 1.4);
-                    if (t <= 2 * sms && simt_us < 1.1 * us) plan->contract.reset();
+                    if (t <= 2 * sms && simt_us < 1.1 * us) {
+                        plan->contract.reset();
+                        now = simt_us;
+                    }
+                }
+                if (!plan->gemm && !plan->stream && loader < 0) {
+                    double staged_us = 0;
+                    if ((st = ja_staged_plan(A, B, out, &plan->staged, &staged_us)) != JA_OK) return st;
+                    if (plan->staged && staged_us > 0.9 * now) plan->staged.reset();
                 }
                 plan->contract_checked = true;
+            }
+            if (plan->staged) {
+                bool launched = false;
+                if ((st = ja_launch_staged(plan->staged.get(), stream, &launched)) != JA_OK || launched) return st;
             }
             if (plan->stream) return ja_launch_stream_tc(*plan->stream, stream);
             if (plan->gemm && loader != 1 && (loader == 0 || !plan->contract_first)) return ja_launch_gemm_tc(*plan->gemm, stream);

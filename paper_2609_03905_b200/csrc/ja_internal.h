@@ -128,6 +128,7 @@ struct ContractTcPlan;
 ja_status_t ja_contract_tc_plan(const std::string& ta, const std::string& tb, const std::string& tc, const ja_relation* A, const ja_relation* B,
                                 const ja_relation* C, std::shared_ptr<ContractTcPlan>* out, double* est_us);
 ja_status_t ja_launch_contract_tc(const ContractTcPlan& plan, cudaStream_t st);
+double ja_contract_tc_pieces(const ContractTcPlan& plan);   // how many times its estimate a launch with pieces of 4 or 2 cells takes
 // the same products of f32 relations on the FMA pipe (k_contract_f32.cu)
 struct ContractF32Plan;
 ja_status_t ja_contract_f32_plan(const std::string& ta, const std::string& tb, const std::string& tc, const ja_relation* A, const ja_relation* B,
@@ -215,6 +216,17 @@ double ja_gemm_tc_estimate_us(const GemmTcPlan& plan);
 struct StreamTcPlan;
 ja_status_t ja_stream_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us);
 ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st);
+// Products of relations that TMA cannot address, on copies that it can (k_stage.cu). *out stays empty where that is not possible or the
+// relations need no copy; *launched stays false where this call cannot have its scratch (a capture, no memory). Key tables must be on the device.
+struct StagedPlan;
+struct TmaOperand;
+ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StagedPlan>* out, double* est_us);
+ja_status_t ja_launch_staged(StagedPlan* plan, cudaStream_t st, bool* launched);
+// what it runs on: plans for operands whose bases are set before every launch
+ja_status_t ja_gemm_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<GemmTcPlan>* out, bool* eligible);
+ja_status_t ja_gemm_tc_set_bases(GemmTcPlan* plan, char* a, char* b);
+ja_status_t ja_stream_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us);
+ja_status_t ja_stream_tc_set_bases(StreamTcPlan* plan, char* a, char* b);
 
 // Attention join-agg (QK^T join, online-softmax aggregation, PV).
 // the four tensor maps (Q, K, V, O) of the tensor-memory kernels, encoded once per (spec, relations) tuple

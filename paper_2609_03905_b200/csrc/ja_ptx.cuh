@@ -230,5 +230,14 @@ inline EncodeTiledFn get_encode() {
 
 }  // namespace ja_ptx
 
-// Tensor map of a relation [R, C] of equal 16-bit blocks, boxes of box_inner cells of box_rows rows of a block (k_gemm_tc.cu)
-ja_status_t ja_encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows, CUtensorMap* tm);
+// One operand of a two-index product as TMA sees it: nrb x ncb blocks of rows x cols 16-bit cells
+struct TmaOperand {
+    char* base;
+    ja_dtype_t dtype;
+    int64_t rows, cols;                      // of a block
+    int32_t nrb, ncb;
+    int64_t pitch, col_stride, row_stride;   // bytes from row to row of a block, and to the next block along the columns / the rows
+};
+TmaOperand ja_tma_operand(const ja_relation* r);   // of a relation of equal blocks
+// its rank-4 tensor map, boxes of box_inner cells of box_rows rows of a block (k_gemm_tc.cu)
+ja_status_t ja_encode_blocked_2d(const TmaOperand& o, int box_inner, int box_rows, CUtensorMap* tm);

@@ -55,6 +55,8 @@ template <int CG> struct Cfg {
     static constexpr int B_CHUNK_BYTES = BK * 64 * 2;                // one box: BK k-rows x 64 columns
     static constexpr int B_STAGE_BYTES = B_CHUNK_BYTES * (BN / CG / 64);
     static constexpr int SMEM_BYTES = STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + 1024 /*align*/ + 256 /*barriers*/;
+    // ANYC: 32 rows x 32 columns of every epilogue warp on their way to stores along the rows (rows of 34 cells: no bank conflicts)
+    static constexpr int SMEM_BYTES_ANYC = SMEM_BYTES + 4 * 32 * 34 * 2;
 };
 
 struct GemmParams {
@@ -64,6 +66,7 @@ struct GemmParams {
     uint32_t wait_cap_us;      // limit of every bounded wait (set at launch)
     int32_t bm, bk, bn;        // block extents along i, j, k
     int32_t nbm, nbk, nbn;     // blocks along i, j, k
+    int32_t c_bm, c_bn, c_nbn; // block extents of the output, and its blocks along k (other than the operands' where those were copied)
     int32_t M, N;              // tensor extents along i, k
     int32_t a_box_rows;        // rows per A box (= min(bm, 128))
     int32_t a_boxes;           // A boxes per tile: 128 / bm where bm divides 128 (tiles cut from global rows), else 1
@@ -83,6 +86,7 @@ struct GemmParams {
     int32_t f16;               // cell type of the operands (and of a 2-byte output): 0 = bf16, 1 = f16
     const char* r_base;        // EPI_ADD: payload of the relation added to the product (tiled exactly like the output)
     const float2* rope_table;  // EPI_ROPE: (cos, sin)[position][pair]
+    RelView c;                 // ANYC: the output, whose blocks may have any shapes
     int32_t rope_S, rope_D;    // EPI_ROPE: positions per sequence (row % rope_S), rotated extent (column % rope_D)
 };
 enum { EPI_NONE = 0, EPI_ADD = 1, EPI_ROPE = 2, EPI_SWIGLU = 3 };
@@ -163,7 +167,9 @@ __device__ __forceinline__ int tile_of_iter(const GemmParams& p, int i, int firs
 
 // F16: cell type of the operands and of a 2-byte output -- bf16 or f16 (a compile-time choice: a select between the two
 // conversions in the epilogue cost the plain contraction a tenth of its rate)
-template <int CG, bool F16, bool SPLIT>
+// ANYC: the output's tiling is not the one that TMA sees of the operands (operands staged by k_stage.cu, rows of no whole 16 bytes): every
+// cell is located through its key table and stored by itself, 32 columns of a row at a time
+template <int CG, bool F16, bool SPLIT, bool ANYC>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmB2, const GemmParams p) {
@@ -368,8 +374,52 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int r = q * 32 + lane;                     // row of this CTA's 128 rows held by this thread
             const int grow = tc.row_g0 + r;                  // global row
             const bool row_ok = r < tc.rows;
+            if constexpr (ANYC) {
+                int rb = 0, rin = 0;
+                if (row_ok) {
+                    int lo, hi;
+                    rb = ja_interval(p.c, 0, grow, &lo, &hi);
+                    rin = grow - lo;
+                }
+                uint16_t* cells = reinterpret_cast<uint16_t*>(smem + STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + 256) + q * 32 * 34;
+                const int n_rows = min(32, tc.rows - q * 32);
+                for (int ch = 0; ch * 32 < tc.width; ++ch) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + ch * 32, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        *reinterpret_cast<uint32_t*>(cells + lane * 34 + 2 * e) = ja_pack16<F16>(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+                    __syncwarp();
+                    const bool col_ok = ch * 32 + lane < tc.width;
+                    const int col = tc.n_g0 + ch * 32 + lane;
+                    int cb = 0, cin = 0;
+                    int64_t pitch = 0;
+                    if (col_ok) {
+                        int lo, hi;
+                        cb = ja_interval(p.c, 1, col, &lo, &hi);
+                        pitch = (int64_t)(hi - lo) * 2;
+                        cin = col - lo;
+                    }
+                    // the warp's rows in one block: row after row. (With every row's block looked up by shuffles a tile took 17 us to store.)
+                    const int b0 = __shfl_sync(0xffffffffu, rb, 0), in0 = __shfl_sync(0xffffffffu, rin, 0);
+                    if (n_rows > 0 && __shfl_sync(0xffffffffu, rb, n_rows - 1) == b0) {
+                        if (col_ok) {
+                            char* at = p.c.base + ja_block_at(p.c, b0, cb) + cin * 2 + in0 * pitch;
+#pragma unroll 8
+                            for (int rr = 0; rr < n_rows; ++rr, at += pitch) *reinterpret_cast<uint16_t*>(at) = cells[rr * 34 + lane];
+                        }
+                    } else {
+                        for (int rr = 0; rr < n_rows; ++rr) {
+                            const int b = __shfl_sync(0xffffffffu, rb, rr), in = __shfl_sync(0xffffffffu, rin, rr);
+                            if (col_ok) *reinterpret_cast<uint16_t*>(p.c.base + ja_block_at(p.c, b, cb) + cin * 2 + in * pitch) = cells[rr * 34 + lane];
+                        }
+                    }
+                    __syncwarp();
+                }
+            } else {
             int ib = 0, iin = 0;
-            if (row_ok) { ib = grow / p.bm; iin = grow % p.bm; }
+            if (row_ok) { ib = grow / p.c_bm; iin = grow % p.c_bm; }
             for (int ch = 0; ch * 32 < tc.width; ++ch) {
                 uint32_t v[32];
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + ch * 32, v);
@@ -387,8 +437,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
                 if (row_ok) {
                     const int gcol = tc.n_g0 + ch * 32;
-                    const int kb = gcol / p.bn, cin = gcol % p.bn;
-                    const int64_t off = p.c_blk_off[((int64_t)tc.copy * p.nbm + ib) * p.nbn + kb] + ((int64_t)iin * p.bn + cin) * p.c_esize;
+                    const int kb = gcol / p.c_bn, cin = gcol % p.c_bn;
+                    const int64_t off = p.c_blk_off[((int64_t)tc.copy * p.nbm + ib) * p.c_nbn + kb] + ((int64_t)iin * p.c_bn + cin) * p.c_esize;
                     char* dst = p.c_base + off;
                     const int valid = min(32, tc.width - ch * 32);  // multiple of 8
                     if (p.c_esize == 4) {   // partial relation kept in f32: the accumulator is stored as it is
@@ -434,6 +484,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     }
                 }
             }
+            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -466,7 +517,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         tc_fence_before();
         __syncwarp();
         cluster_sync_all();
-        if (*abort_flag == 0) {
+        if (ANYC) {
+            // lanes along the columns: 64 contiguous bytes a store wherever a row's blocks start
+            for (int c = lane; c < tc.width && *abort_flag == 0; c += 32) {
+                int lo, hi, rlo, rhi;
+                const int cb = ja_interval(p.c, 1, tc.n_g0 + c, &lo, &hi);
+                for (int own = warp; own < mine && slice * mine + own < tc.rows; own += NUM_THREADS / 32) {
+                    const float* src = reinterpret_cast<const float*>(smem) + own * PITCH + c;
+                    float f = 0.f;
+                    for (int k = 0; k < p.split; ++k) f += src[k * mine * PITCH];   // slices in ascending order
+                    const int row = tc.row_g0 + slice * mine + own, rb = ja_interval(p.c, 0, row, &rlo, &rhi);
+                    *reinterpret_cast<uint16_t*>(p.c.base + ja_block_at(p.c, rb, cb) + ((int64_t)(row - rlo) * (hi - lo) + (tc.n_g0 + c - lo)) * 2) =
+                        (uint16_t)ja_pack16<F16>(f, 0.f);
+                }
+            }
+        } else if (*abort_flag == 0) {
             const int ppr = (tc.width + 7) / 8;      // 8-column pieces of a row
             for (int i = threadIdx.x; i < mine * ppr; i += NUM_THREADS) {
                 const int own = i / ppr, c = (i - own * ppr) * 8, r = slice * mine + own;
@@ -482,8 +547,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 };
                 float f[8];
                 sum8(src, f);
-                const int grow = tc.row_g0 + r, gcol = tc.n_g0 + c, kb = gcol / p.bn, cin = gcol - kb * p.bn, ib = grow / p.bm, iin = grow - ib * p.bm;
-                const int64_t off = p.c_blk_off[(int64_t)ib * p.nbn + kb] + ((int64_t)iin * p.bn + cin) * 2;
+                const int grow = tc.row_g0 + r, gcol = tc.n_g0 + c, kb = gcol / p.c_bn, cin = gcol - kb * p.c_bn, ib = grow / p.c_bm, iin = grow - ib * p.c_bm;
+                const int64_t off = p.c_blk_off[(int64_t)ib * p.c_nbn + kb] + ((int64_t)iin * p.c_bn + cin) * 2;
                 if (p.epi == EPI_SWIGLU) {
                     float g[8];
                     sum8(src + p.bn_tile, g);
@@ -530,19 +595,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }  // namespace
 
 // ---- host: tensor maps -------------------------------------------------------------------------------------
+TmaOperand ja_tma_operand(const ja_relation* r) {
+    const int64_t blk_stride = r->nblocks > 1 ? r->blk_off[1] - r->blk_off[0] : (int64_t)r->bytes;
+    return {(char*)r->base, r->dtype, r->bs[0], r->bs[1], r->nblk[0], r->nblk[1], r->bs[1] * 2, blk_stride, blk_stride * r->nblk[1]};
+}
+
 // A relation [R, C] with equal blocks br x bc is the rank-4 tensor (c in block, r in block, col-block, row-block).
-ja_status_t ja_encode_blocked_2d(const ja_relation* r, int box_inner, int box_rows, CUtensorMap* tm) {
+ja_status_t ja_encode_blocked_2d(const TmaOperand& o, int box_inner, int box_rows, CUtensorMap* tm) {
     if (box_rows > 256) return ja_fail(JA_ERR_INVALID_ARG, "TMA box too tall");
     EncodeTiledFn enc = get_encode();
     if (!enc) return ja_fail(JA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    const int64_t br = r->bs[0], bc = r->bs[1];
-    const int64_t blk_stride = r->nblocks > 1 ? r->blk_off[1] - r->blk_off[0] : (int64_t)r->bytes;
-    cuuint64_t dims[4] = {(cuuint64_t)bc, (cuuint64_t)br, (cuuint64_t)r->nblk[1], (cuuint64_t)r->nblk[0]};
-    cuuint64_t strides[3] = {(cuuint64_t)(bc * 2), (cuuint64_t)blk_stride, (cuuint64_t)(blk_stride * r->nblk[1])};
+    cuuint64_t dims[4] = {(cuuint64_t)o.cols, (cuuint64_t)o.rows, (cuuint64_t)o.ncb, (cuuint64_t)o.nrb};
+    cuuint64_t strides[3] = {(cuuint64_t)o.pitch, (cuuint64_t)o.col_stride, (cuuint64_t)o.row_stride};
     cuuint32_t box[4] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows, 1, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
-    const CUtensorMapDataType cell = r->dtype == JA_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    CUresult res = enc(tm, cell, 4, r->base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    const CUtensorMapDataType cell = o.dtype == JA_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    CUresult res = enc(tm, cell, 4, o.base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (res != CUDA_SUCCESS) return ja_fail(JA_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)res);
     return JA_OK;
@@ -554,16 +622,20 @@ struct GemmTcPlan {
     int cg;      // CTAs per tile: 1 or 2
     int tiles;   // of the whole launch; the last `tail` of them go to a launch of their own, each split along the contracted index
     int tail, split;
+    bool any_c;
+    bool staged = false;   // on copies: launched behind the whole launch before it (k_stage.cu)
+    TmaOperand a, b;
     double us;   // what the launches are expected to take
 };
 
 namespace {
 
-template <bool F16>
+template <bool F16, bool ANYC>
 cudaError_t configure() {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<1, F16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES);
+    constexpr int S1 = ANYC ? Cfg<1>::SMEM_BYTES_ANYC : Cfg<1>::SMEM_BYTES, S2 = ANYC ? Cfg<2>::SMEM_BYTES_ANYC : Cfg<2>::SMEM_BYTES;
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<1, F16, false, ANYC>, cudaFuncAttributeMaxDynamicSharedMemorySize, S1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, false, ANYC>, cudaFuncAttributeMaxDynamicSharedMemorySize, S2);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<2, F16, true, ANYC>, cudaFuncAttributeMaxDynamicSharedMemorySize, S2);
     return e;
 }
 
@@ -587,7 +659,7 @@ int clusters_at_once(int split) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc_kernel<2, false, true>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc_kernel<2, false, true, false>, &cfg) != cudaSuccess) {
             cudaGetLastError();
             c = 0;
         }
@@ -625,36 +697,39 @@ void choose_tail(GemmTcPlan* plan) {
 
 }  // namespace
 
-ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, const GemmEpilogue* ep,
-                            std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
-    *eligible = false;
-    if (!A->equal_blocks || !B->equal_blocks || !C->equal_blocks) return JA_OK;
-    if (A->dtype == JA_F32 || B->dtype != A->dtype || (C->esize == 2 && C->dtype != A->dtype)) return JA_OK;
+static ja_status_t encode_operands(GemmTcPlan* plan) {
+    const int b_rows = plan->cg == 2 ? Cfg<2>::BK : Cfg<1>::BK;
+    ja_status_t st = ja_encode_blocked_2d(plan->a, 64, plan->p.a_box_rows, &plan->tmA);
+    if (st == JA_OK) st = ja_encode_blocked_2d(plan->b, 64, b_rows, &plan->tmB);
+    return st;
+}
+
+// a, b: the operands' blocks, of one contracted extent. any_c: C has its own tiling of the same index ranges. Operands without a base get
+// one by ja_gemm_tc_set_bases before every launch.
+static ja_status_t plan_gemm(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, const GemmEpilogue* ep, bool any_c,
+                             std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
     const int epi = ep ? ep->epi : 0;
     const int bn_tile = epi == EPI_SWIGLU ? 128 : BN;
-    if (epi == EPI_SWIGLU && (B->bs[1] % 128 != 0 || !ep->B2 || !ep->B2->equal_blocks)) return JA_OK;
-    if (epi == EPI_ROPE && (ep->rope_D % 32 != 0 || B->bs[1] % 32 != 0)) return JA_OK;
-    const int64_t bm = A->bs[0], bk = A->bs[1], bn = B->bs[1];
-    // TMA needs 16-byte row pitches; boxes are 64 elements wide; A boxes hold min(bm,128) rows
-    if (bk % 8 || bn % 8 || bk < 64 || bn < 64) return JA_OK;
+    const int64_t bm = a.rows, bk = a.cols, bn = b.cols;
     const bool odd_rows = bm < 128 && (128 % bm != 0 || bm % 8 != 0);   // one block per row tile: plain products alone
     if (odd_rows && (epi != EPI_NONE || C->esize != 2)) return JA_OK;
-    if (A->extent[0] >= (1ll << 31) || B->extent[1] >= (1ll << 31)) return JA_OK;
     std::shared_ptr<GemmTcPlan> plan(new GemmTcPlan());
     GemmParams& p = plan->p;
     p.c_base = (char*)C->base;
-    p.c_blk_off = ja_view(C).blk_off;
+    p.c = ja_view(C);
+    p.c_blk_off = p.c.blk_off;
     p.status = nullptr;
     p.bm = (int)bm; p.bk = (int)bk; p.bn = (int)bn;
-    p.nbm = A->nblk[0]; p.nbk = A->nblk[1]; p.nbn = B->nblk[1];
-    p.M = (int)A->extent[0]; p.N = (int)B->extent[1];
+    p.nbm = a.nrb; p.nbk = a.ncb; p.nbn = b.ncb;
+    p.M = (int)C->extent[C->rank - 2]; p.N = (int)C->extent[C->rank - 1];
+    p.c_bm = (int)C->bs[C->rank - 2]; p.c_bn = (int)C->bs[C->rank - 1]; p.c_nbn = C->nblk[C->rank - 1];
     p.a_box_rows = (int)std::min<int64_t>(bm, 128);
     p.a_boxes = bm < 128 && !odd_rows ? (int)(128 / bm) : 1;
     p.epi = epi;
     p.bn_tile = bn_tile;
     p.n_copies = (ep && ep->partials) ? p.nbk : 1;
     p.c_esize = C->esize;
-    p.f16 = A->dtype == JA_F16;
+    p.f16 = a.dtype == JA_F16;
     if (p.c_esize == 4 && !(ep && ep->partials)) return JA_OK;
     p.r_base = (epi == EPI_ADD) ? (const char*)ep->addend->base : nullptr;
     p.rope_table = (epi == EPI_ROPE) ? ep->rope_table : nullptr;
@@ -679,12 +754,14 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     plan->cg = two ? 2 : 1;
     if (!by_block) { p.tiles_per_mblk = 0; p.m_tiles = (p.M + BM * plan->cg - 1) / (BM * plan->cg); }
     else { p.tiles_per_mblk = (int)((bm + BM - 1) / BM); p.m_tiles = (p.tiles_per_mblk * p.nbm + plan->cg - 1) / plan->cg; }
+    plan->a = a;
+    plan->b = b;
+    plan->any_c = any_c;
     ja_status_t st;
-    if ((st = ja_encode_blocked_2d(A, 64, p.a_box_rows, &plan->tmA)) != JA_OK) return st;
-    if ((st = ja_encode_blocked_2d(B, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB)) != JA_OK) return st;
-    plan->tmB2 = plan->tmB;
-    if (epi == EPI_SWIGLU && (st = ja_encode_blocked_2d(ep->B2, 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB2)) != JA_OK) return st;
-    cudaError_t e = p.f16 ? configure<true>() : configure<false>();
+    if (a.base && b.base && (st = encode_operands(plan.get())) != JA_OK) return st;
+    if (epi == EPI_SWIGLU && (st = ja_encode_blocked_2d(ja_tma_operand(ep->B2), 64, two ? Cfg<2>::BK : Cfg<1>::BK, &plan->tmB2)) != JA_OK) return st;
+    if (epi != EPI_SWIGLU) plan->tmB2 = plan->tmB;
+    cudaError_t e = any_c ? (p.f16 ? configure<true, true>() : configure<false, true>()) : (p.f16 ? configure<true, false>() : configure<false, false>());
     if (e != cudaSuccess) return ja_cuda_fail(e, "cudaFuncSetAttribute(gemm_tc_kernel)");
     plan->tiles = p.m_tiles * p.n_tiles * p.n_copies;
     plan->tail = 0;
@@ -696,35 +773,62 @@ ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja
     return JA_OK;
 }
 
+ja_status_t ja_gemm_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, const GemmEpilogue* ep,
+                            std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
+    *eligible = false;
+    if (!A->equal_blocks || !B->equal_blocks || !C->equal_blocks) return JA_OK;
+    if (A->dtype == JA_F32 || B->dtype != A->dtype || (C->esize == 2 && C->dtype != A->dtype)) return JA_OK;
+    const int epi = ep ? ep->epi : 0;
+    if (epi == EPI_SWIGLU && (B->bs[1] % 128 != 0 || !ep->B2 || !ep->B2->equal_blocks)) return JA_OK;
+    if (epi == EPI_ROPE && (ep->rope_D % 32 != 0 || B->bs[1] % 32 != 0)) return JA_OK;
+    const int64_t bk = A->bs[1], bn = B->bs[1];
+    // TMA needs 16-byte row pitches; boxes are 64 elements wide; A boxes hold min(bm,128) rows
+    if (bk % 8 || bn % 8 || bk < 64 || bn < 64) return JA_OK;
+    if (A->extent[0] >= (1ll << 31) || B->extent[1] >= (1ll << 31)) return JA_OK;
+    return plan_gemm(ja_tma_operand(A), ja_tma_operand(B), C, ep, false, out, eligible);
+}
+
+ja_status_t ja_gemm_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
+    *eligible = false;
+    if (a.cols < 64 || b.cols < 64) return JA_OK;
+    // 32 columns at a time lie in one block of the output, in rows of whole 16 bytes: stored as ever
+    const bool any_c = !(C->equal_blocks && C->bs[1] % 8 == 0 && (C->bs[1] == b.cols || C->bs[1] % 32 == 0));
+    ja_status_t st = plan_gemm(a, b, C, nullptr, any_c, out, eligible);
+    if (*out) (*out)->staged = true;
+    return st;
+}
+
+ja_status_t ja_gemm_tc_set_bases(GemmTcPlan* plan, char* a, char* b) {
+    if (plan->a.base == a && plan->b.base == b) return JA_OK;
+    plan->a.base = a;
+    plan->b.base = b;
+    return encode_operands(plan);
+}
+
 // What the launches are expected to take: rounds of tiles over the CTA groups, 0.96 us per 128 contracted cells of a 256-row tile on
 // a pair of SMs, 0.70 per 64 of a 128-row tile on one, and a start and an end.
 double ja_gemm_tc_estimate_us(const GemmTcPlan& plan) { return plan.us; }
 
-template <bool F16>
+template <bool F16, bool ANYC>
 static ja_status_t launch_gemm(const GemmTcPlan& plan, GemmParams& p, cudaStream_t st) {
+    constexpr int S1 = ANYC ? Cfg<1>::SMEM_BYTES_ANYC : Cfg<1>::SMEM_BYTES, S2 = ANYC ? Cfg<2>::SMEM_BYTES_ANYC : Cfg<2>::SMEM_BYTES;
     const int sms = ja_sm_count();
-    p.tile0 = 0;
-    p.tile_end = plan.tiles - plan.tail;
-    if (plan.cg == 1) {
-        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<1, F16, false>, dim3((unsigned)std::min(sms, p.tile_end), 1, 1), NUM_THREADS, Cfg<1>::SMEM_BYTES, 1, st, plan.tmA,
-                                 plan.tmB, plan.tmB2, p));
+    auto launch = [&](auto kernel, int grid, int smem, int cluster) -> ja_status_t {
+        if (plan.staged) JA_CUDA(ja_launch_kernel_after(kernel, dim3((unsigned)grid, 1, 1), NUM_THREADS, smem, (unsigned)cluster, st, plan.tmA, plan.tmB, plan.tmB2, p));
+        else JA_CUDA(ja_launch_kernel(kernel, dim3((unsigned)grid, 1, 1), NUM_THREADS, smem, (unsigned)cluster, st, plan.tmA, plan.tmB, plan.tmB2, p));
         ja_count_launch();
         return JA_OK;
-    }
-    if (p.tile_end > 0) {
-        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<2, F16, false>, dim3((unsigned)(2 * std::min(sms / 2, p.tile_end)), 1, 1), NUM_THREADS, Cfg<2>::SMEM_BYTES, 2, st,
-                                 plan.tmA, plan.tmB, plan.tmB2, p));
-        ja_count_launch();
-    }
-    if (plan.tail > 0) {
-        p.tile0 = p.tile_end;
-        p.tile_end = plan.tiles;
-        p.split = plan.split;
-        JA_CUDA(ja_launch_kernel(gemm_tc_kernel<2, F16, true>, dim3((unsigned)(plan.tail * 2 * plan.split), 1, 1), NUM_THREADS, Cfg<2>::SMEM_BYTES,
-                                 (unsigned)(2 * plan.split), st, plan.tmA, plan.tmB, plan.tmB2, p));
-        ja_count_launch();
-    }
-    return JA_OK;
+    };
+    p.tile0 = 0;
+    p.tile_end = plan.tiles - plan.tail;
+    if (plan.cg == 1) return launch(gemm_tc_kernel<1, F16, false, ANYC>, std::min(sms, p.tile_end), S1, 1);
+    ja_status_t s = JA_OK;
+    if (p.tile_end > 0) s = launch(gemm_tc_kernel<2, F16, false, ANYC>, 2 * std::min(sms / 2, p.tile_end), S2, 2);
+    if (s != JA_OK || plan.tail == 0) return s;
+    p.tile0 = p.tile_end;
+    p.tile_end = plan.tiles;
+    p.split = plan.split;
+    return launch(gemm_tc_kernel<2, F16, true, ANYC>, plan.tail * 2 * plan.split, S2, 2 * plan.split);
 }
 
 ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st) {
@@ -732,5 +836,6 @@ ja_status_t ja_launch_gemm_tc(const GemmTcPlan& plan, cudaStream_t st) {
     p.status = ja_device_status_word(st);
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
-    return p.f16 ? launch_gemm<true>(plan, p, st) : launch_gemm<false>(plan, p, st);
+    if (plan.any_c) return p.f16 ? launch_gemm<true, true>(plan, p, st) : launch_gemm<false, true>(plan, p, st);
+    return p.f16 ? launch_gemm<true, false>(plan, p, st) : launch_gemm<false, false>(plan, p, st);
 }

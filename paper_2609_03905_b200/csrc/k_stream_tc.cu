@@ -10,7 +10,7 @@
 //   warps 2..5  the partial tile from tensor memory to its owners
 // Every mbarrier wait is bounded; on expiry the CTA records JA_ERR_TIMEOUT, drains its copies and leaves through the normal exit.
 //
-// What bounds it: the stream of B out of HBM. Two or three CTAs of 3 stages share an SM, 100 to 150 KiB of copies in flight per SM.
+// What bounds it: the stream of B out of HBM; on small products the trips of a CTA's stages, so up to eight are in flight.
 #include <cuda.h>
 #include <string.h>
 
@@ -24,13 +24,11 @@ namespace {
 
 using namespace ja_ptx;
 
-constexpr int BM = 128, BK = 64, STAGES = 3, NUM_THREADS = 192;
+constexpr int BM = 128, BK = 64, MAX_STAGES = 8, NUM_THREADS = 192;
 constexpr int W_BYTES = BM * BK * 2, W_BOX = W_BYTES / 2;
 constexpr int MAX_TOKENS = 128;
 
 struct Params {
-    char* c_base;
-    const int64_t* c_blk_off;
     int32_t* status;
     uint32_t wait_cap_us;
     int32_t bm, nbm, pad;      // rows per row block, row blocks, rows a block takes in the tile (a multiple of 8: swizzle atoms)
@@ -39,8 +37,10 @@ struct Params {
     int32_t bk, nbk, per_blk;  // contracted cells per block, blocks, stages per block
     int32_t bn, nbn, N;
     int32_t tiles_per_nblk;    // 0: tiles are cut from the whole column index
-    int32_t split;
+    int32_t split, stages;
     int32_t f16;
+    int32_t any_c;             // the output has its own tiling: cells stored one by one through its key table
+    RelView c;
 };
 
 __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -50,17 +50,18 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     const uint32_t base = (raw + 1023u) & ~1023u;   // swizzle atoms need 1024-byte alignment
     uint8_t* smem = smem_raw + (base - raw);
     const uint32_t stage_bytes = W_BYTES + (uint32_t)p.n_mma * (BK * 2);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * stage_bytes);
+    const int stages = p.stages;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes);
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
-    const uint32_t done_bar = bar0 + 8u * (2 * STAGES);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+    const uint32_t done_bar = bar0 + 8u * (2 * MAX_STAGES);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 1);
     volatile int* ctl = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(full_bar(s), 1);
             mbar_init(empty_bar(s), 1);
         }
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
                 for (int c = 0; c < boxes; ++c) tma_load_4d<1>(w + c * W_BOX, &tmB, fb, cin[c], kc * BK, nb[c], jb);
                 for (int b = 0; b < p.nbm; ++b) tma_load_4d<1>(x + b * p.pad * (BK * 2), &tmA, fb, kc * BK, 0, jb, b);
                 if (++kc == p.per_blk) { kc = 0; ++jb; }
-                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+                if (++stage == stages) { stage = 0; phase ^= 1; }
             }
         }
         __syncwarp();
@@ -131,15 +132,15 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
             for (int kk = 0; kk < BK / 16; ++kk)   // cells past a block's end are zero in both operands
                 umma_bf16_w<1>(tmem, desc_sw128(w + kk * 2048, W_BOX), desc_sw128(x + kk * 32, 16), idesc, (ch > ch0 || kk > 0) ? 1u : 0u, leader);
             umma_commit_w<1>(empty_bar(stage), leader);
-            if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            if (++stage == stages) { stage = 0; phase ^= 1; }
         }
         if (ok) umma_commit_w<1>(done_bar, leader);
     }
     const bool ok = mbar_wait(done_bar, 0, ctl, p.status);
     tc_fence_after();
     if (!ok && warp == 0 && lane == 0) {   // gave up: wait (bounded) for the copies in flight before the shared memory goes
-        for (int s = 0; s < STAGES && ch0 + s < ch1; ++s) {
-            const uint32_t last = (uint32_t)((ch1 - 1 - ch0 - s) / STAGES) & 1;
+        for (int s = 0; s < stages && ch0 + s < ch1; ++s) {
+            const uint32_t last = (uint32_t)((ch1 - 1 - ch0 - s) / stages) & 1;
             const uint64_t t0 = global_ns();
             while (!mbar_try_wait(full_bar(s), last) && global_ns() - t0 < 200000000ull) {}
         }
@@ -173,20 +174,37 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     if (split > 1) cluster_sync_all();     // the slices have arrived
     // ---- one rounding, 16-byte stores ----
     if (ctl[0] == 0) {
-        for (int i = threadIdx.x; i < mine * (BM / 8); i += NUM_THREADS) {
-            const int own = i / (BM / 8), n = i % (BM / 8) * 8, slot = rank * mine + own, b = slot / p.pad, r = slot % p.pad;
-            if (r >= p.bm || n >= width) continue;
-            const float* src = reinterpret_cast<const float*>(smem) + own * BM + n;
-            float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            for (int s = 0; s < split; ++s) {   // slices in ascending order
-                const float4 u = *reinterpret_cast<const float4*>(src + s * mine * BM), v = *reinterpret_cast<const float4*>(src + s * mine * BM + 4);
-                f[0] += u.x; f[1] += u.y; f[2] += u.z; f[3] += u.w; f[4] += v.x; f[5] += v.y; f[6] += v.z; f[7] += v.w;
+        if (p.any_c) {   // lanes along the columns, a cell a store
+            for (int c = lane; c < width; c += 32) {
+                int lo, hi, rlo, rhi;
+                const int cb = ja_interval(p.c, 1, n0 + c, &lo, &hi);
+                for (int own = warp; own < mine; own += NUM_THREADS / 32) {
+                    const int slot = rank * mine + own, b = slot / p.pad, r = slot % p.pad;
+                    if (r >= p.bm) continue;
+                    float f = 0.f;
+                    for (int s = 0; s < split; ++s) f += reinterpret_cast<const float*>(smem)[(s * mine + own) * BM + c];   // slices in ascending order
+                    const int row = b * p.bm + r, rb = ja_interval(p.c, 0, row, &rlo, &rhi);
+                    *reinterpret_cast<uint16_t*>(p.c.base + ja_block_at(p.c, rb, cb) + ((int64_t)(row - rlo) * (hi - lo) + (n0 + c - lo)) * 2) =
+                        (uint16_t)(p.f16 ? ja_pack16<true>(f, 0.f) : ja_pack16<false>(f, 0.f));
+                }
             }
-            const int g = n0 + n, kb = g / p.bn, cin = g - kb * p.bn;
-            uint4 o;
-            if (p.f16) o = make_uint4(ja_pack16<true>(f[0], f[1]), ja_pack16<true>(f[2], f[3]), ja_pack16<true>(f[4], f[5]), ja_pack16<true>(f[6], f[7]));
-            else o = make_uint4(ja_pack16<false>(f[0], f[1]), ja_pack16<false>(f[2], f[3]), ja_pack16<false>(f[4], f[5]), ja_pack16<false>(f[6], f[7]));
-            *reinterpret_cast<uint4*>(p.c_base + p.c_blk_off[(int64_t)b * p.nbn + kb] + ((int64_t)r * p.bn + cin) * 2) = o;
+        } else {
+            for (int i = threadIdx.x; i < mine * (BM / 8); i += NUM_THREADS) {
+                const int own = i / (BM / 8), n = i % (BM / 8) * 8, slot = rank * mine + own, b = slot / p.pad, r = slot % p.pad;
+                if (r >= p.bm || n >= width) continue;
+                const float* src = reinterpret_cast<const float*>(smem) + own * BM + n;
+                float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int s = 0; s < split; ++s) {   // slices in ascending order
+                    const float4 u = *reinterpret_cast<const float4*>(src + s * mine * BM), v = *reinterpret_cast<const float4*>(src + s * mine * BM + 4);
+                    f[0] += u.x; f[1] += u.y; f[2] += u.z; f[3] += u.w; f[4] += v.x; f[5] += v.y; f[6] += v.z; f[7] += v.w;
+                }
+                const int g = n0 + n, cbn = (int)p.c.bs[1], kb = g / cbn, cin = g - kb * cbn;
+                const int row = b * p.bm + r, cbm = (int)p.c.bs[0], ib = row / cbm, iin = row - ib * cbm;
+                uint4 o;
+                if (p.f16) o = make_uint4(ja_pack16<true>(f[0], f[1]), ja_pack16<true>(f[2], f[3]), ja_pack16<true>(f[4], f[5]), ja_pack16<true>(f[6], f[7]));
+                else o = make_uint4(ja_pack16<false>(f[0], f[1]), ja_pack16<false>(f[2], f[3]), ja_pack16<false>(f[4], f[5]), ja_pack16<false>(f[6], f[7]));
+                *reinterpret_cast<uint4*>(p.c.base + ja_block_at(p.c, ib, kb) + ((int64_t)iin * cbn + cin) * 2) = o;
+            }
         }
     }
     __syncthreads();
@@ -199,50 +217,84 @@ struct StreamTcPlan {
     CUtensorMap tmA, tmB;
     Params p;
     int grid, smem;
+    TmaOperand a, b;
+    bool staged = false;   // on copies: launched behind the whole launch before it (k_stage.cu)
 };
+
+static ja_status_t encode_operands(StreamTcPlan* plan) {
+    ja_status_t st = ja_encode_blocked_2d(plan->a, BK, plan->p.bm, &plan->tmA);
+    if (st == JA_OK) st = ja_encode_blocked_2d(plan->b, 64, BK, &plan->tmB);
+    return st;
+}
+
+static ja_status_t plan_stream(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, bool any_c, std::shared_ptr<StreamTcPlan>* out, double* est_us) {
+    const int64_t bm = a.rows, bk = a.cols, bn = b.cols, N = C->extent[1], K = bk * a.ncb;
+    // TMA boxes are 64 cells wide, and narrower blocks would leave most of a box empty
+    if (bk < 64 || bn < 64 || K >= (1ll << 31) || N >= (1ll << 31)) return JA_OK;
+    const int64_t pad = (bm + 7) / 8 * 8, slots = a.nrb * pad;
+    if (slots > MAX_TOKENS) return JA_OK;
+    std::shared_ptr<StreamTcPlan> plan(new StreamTcPlan());
+    Params& p = plan->p;
+    memset(&p, 0, sizeof p);
+    p.c = ja_view(C);
+    p.any_c = any_c;
+    p.bm = (int)bm; p.nbm = a.nrb; p.pad = (int)pad;
+    p.n_mma = (int)((slots + 15) / 16 * 16);
+    p.tmem_cols = 32;
+    while (p.tmem_cols < p.n_mma) p.tmem_cols *= 2;
+    p.bk = (int)bk; p.nbk = a.ncb; p.per_blk = (int)((bk + BK - 1) / BK);
+    p.bn = (int)bn; p.nbn = b.ncb; p.N = (int)N;
+    p.tiles_per_nblk = bn % 64 == 0 ? 0 : (int)((bn + BM - 1) / BM);
+    p.f16 = a.dtype == JA_F16;
+    const int64_t tiles = p.tiles_per_nblk ? (int64_t)p.tiles_per_nblk * p.nbn : (N + BM - 1) / BM, chunks = (int64_t)p.nbk * p.per_blk;
+    // as many slices as leave the CTAs resident at once at three stages each ([100, 3001] x [3001, 5001] in 320 CTAs, 296 of which fit: two
+    // rounds), and then as many stages as the CTAs of an SM have room for
+    const int sms = ja_sm_count(), stage_bytes = W_BYTES + p.n_mma * BK * 2;
+    auto smem_of = [&](int stages) { return stages * stage_bytes + 1024 + 256; };
+    const int room = 227 * 1024, fit = std::max(1, std::min(3, room / (smem_of(3) + 1024)));
+    int split = 1;
+    while (split < 8 && tiles * split * 2 <= (int64_t)sms * fit && chunks >= 8 * split) split *= 2;
+    p.split = split;
+    if (tiles * split >= (1ll << 31)) return JA_OK;
+    plan->grid = (int)(tiles * split);
+    const int per_sm = std::min(fit, (plan->grid + sms - 1) / sms);
+    p.stages = 3;
+    while (p.stages < MAX_STAGES && p.stages < (chunks + split - 1) / split && per_sm * (smem_of(p.stages + 1) + 1024) <= room) ++p.stages;
+    plan->smem = smem_of(p.stages);
+    plan->a = a;
+    plan->b = b;
+    ja_status_t st;
+    if (a.base && b.base && (st = encode_operands(plan.get())) != JA_OK) return st;
+    JA_CUDA(cudaFuncSetAttribute(stream_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room));
+    // The stream at 6 TB/s and the tokens' stages from L2 at 9, or, where that leaves a CTA's stages in a row, 0.25 us each; a start, and an end in which every
+    // token's sums cross the cluster.
+    const double stream = (double)(K * N * 2) / 6.0e6 + (double)(tiles * chunks) * p.n_mma * BK * 2 / 9.0e6;
+    const double rounds = (double)((plan->grid + sms * per_sm - 1) / (sms * per_sm)) * (double)((chunks + split - 1) / split) * 0.25;
+    *est_us = std::max(stream, rounds) + 7.0 + 0.05 * (double)slots;
+    *out = plan;
+    return JA_OK;
+}
 
 ja_status_t ja_stream_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us) {
     out->reset();
     if (!A->equal_blocks || !B->equal_blocks || !C->equal_blocks) return JA_OK;
     if (A->dtype == JA_F32 || B->dtype != A->dtype || C->dtype != A->dtype) return JA_OK;
-    const int64_t bm = A->bs[0], bk = A->bs[1], bn = B->bs[1], M = A->extent[0], K = A->extent[1], N = B->extent[1];
-    // TMA needs 16-byte row pitches; boxes are 64 cells wide, and narrower blocks would leave most of a box empty
-    if (bk % 8 || bn % 8 || bk < 64 || bn < 64 || K >= (1ll << 31) || N >= (1ll << 31)) return JA_OK;
-    const int64_t pad = (bm + 7) / 8 * 8, slots = A->nblk[0] * pad;
-    if (slots > MAX_TOKENS) return JA_OK;
-    std::shared_ptr<StreamTcPlan> plan(new StreamTcPlan());
-    Params& p = plan->p;
-    memset(&p, 0, sizeof p);
-    p.c_base = (char*)C->base;
-    p.c_blk_off = ja_view(C).blk_off;
-    p.bm = (int)bm; p.nbm = A->nblk[0]; p.pad = (int)pad;
-    p.n_mma = (int)((slots + 15) / 16 * 16);
-    p.tmem_cols = 32;
-    while (p.tmem_cols < p.n_mma) p.tmem_cols *= 2;
-    p.bk = (int)bk; p.nbk = A->nblk[1]; p.per_blk = (int)((bk + BK - 1) / BK);
-    p.bn = (int)bn; p.nbn = B->nblk[1]; p.N = (int)N;
-    p.tiles_per_nblk = bn % 64 == 0 ? 0 : (int)((bn + BM - 1) / BM);
-    p.f16 = A->dtype == JA_F16;
-    const int64_t tiles = p.tiles_per_nblk ? (int64_t)p.tiles_per_nblk * p.nbn : (N + BM - 1) / BM, chunks = (int64_t)p.nbk * p.per_blk;
-    // enough slices that every SM has two CTAs, each with more stages than are in flight
-    const int sms = ja_sm_count();
-    int split = 1;
-    while (split < 8 && tiles * split < 2 * sms && chunks >= 8 * split) split *= 2;
-    p.split = split;
-    if (tiles * split >= (1ll << 31)) return JA_OK;
-    plan->grid = (int)(tiles * split);
-    plan->smem = STAGES * (W_BYTES + p.n_mma * BK * 2) + 1024 + 256;
-    ja_status_t st;
-    if ((st = ja_encode_blocked_2d(A, BK, (int)bm, &plan->tmA)) != JA_OK) return st;
-    if ((st = ja_encode_blocked_2d(B, 64, BK, &plan->tmB)) != JA_OK) return st;
-    JA_CUDA(cudaFuncSetAttribute(stream_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGES * (W_BYTES + MAX_TOKENS * BK * 2) + 1024 + 256));
-    // The stream at 6 TB/s and the tokens' stages from L2 at 9, or, where that leaves a CTA's stages in a row, 0.25 us each; a start and an end.
-    const double stream = (double)(K * N * 2) / 6.0e6 + (double)(tiles * chunks) * p.n_mma * BK * 2 / 9.0e6;
-    const int per_sm = std::max(1, std::min(3, (227 * 1024) / plan->smem));
-    const double rounds = (double)((plan->grid + sms * per_sm - 1) / (sms * per_sm)) * (double)((chunks + split - 1) / split) * 0.25;
-    *est_us = std::max(stream, rounds) + 7.0;
-    *out = plan;
-    return JA_OK;
+    if (A->bs[1] % 8 || B->bs[1] % 8) return JA_OK;   // TMA needs 16-byte row pitches
+    return plan_stream(ja_tma_operand(A), ja_tma_operand(B), C, false, out, est_us);
+}
+
+ja_status_t ja_stream_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us) {
+    out->reset();
+    ja_status_t st = plan_stream(a, b, C, !(C->equal_blocks && C->bs[1] % 8 == 0), out, est_us);
+    if (*out) (*out)->staged = true;
+    return st;
+}
+
+ja_status_t ja_stream_tc_set_bases(StreamTcPlan* plan, char* a, char* b) {
+    if (plan->a.base == a && plan->b.base == b) return JA_OK;
+    plan->a.base = a;
+    plan->b.base = b;
+    return encode_operands(plan);
 }
 
 ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st) {
@@ -250,7 +302,9 @@ ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st) {
     p.status = ja_device_status_word(st);
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
-    JA_CUDA(ja_launch_kernel(stream_tc_kernel, dim3((unsigned)plan.grid, 1, 1), NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
+    const dim3 grid((unsigned)plan.grid, 1, 1);
+    if (plan.staged) JA_CUDA(ja_launch_kernel_after(stream_tc_kernel, grid, NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
+    else JA_CUDA(ja_launch_kernel(stream_tc_kernel, grid, NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
     ja_count_launch();
     return JA_OK;
 }

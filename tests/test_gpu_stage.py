@@ -1,0 +1,102 @@
+"""Products of 16-bit relations that TMA cannot address as they lie, on copies that it can (k_stage.cu), and the stores that go with them, against
+an fp64 product of the same 16-bit inputs. Tolerance: gpu_util.TOL, ten half-ulps of the stored type; f32 accumulation does not show
+beside it."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_03905_b200 as ja
+import synth_inputs as si
+from oracle import blocked
+
+from gpu_util import TOL, check_status, download, empty_like_tiling, relfro, upload
+
+pytestmark = pytest.mark.gpu
+ES = blocked.equal_splits
+BF, F16 = torch.bfloat16, torch.float16
+
+
+def _problem(ti, tj, tk, dtype):
+    m, k, n = ti[-1], tj[-1], tk[-1]
+    a, b = si.normal((m, k), 0.0, 1.0, dtype, 37, 40), si.normal((k, n), 0.0, 1.0, dtype, 37, 41)
+    res = empty_like_tiling([m, n], [ti, tk], dtype, fill=float("nan"))
+    return a, b, upload(a, [ti, tj]), upload(b, [tj, tk]), res, ja.Spec("ij,jk->ik", {"i": ti, "j": tj, "k": tk})
+
+
+def _check(res, a, b, dtype):
+    got, ref = download(res), si.to_f64(a) @ si.to_f64(b)
+    check_status()
+    assert relfro(got, ref) <= TOL[dtype]
+    ulp = 2.0 ** (-7 if dtype == BF else -10)      # of the largest value: a misplaced cell is far outside it
+    assert np.abs(got - ref).max() <= ulp * np.abs(ref).max()
+
+
+# which operand is copied (odd columns of either or both, rows in unequal blocks), remainders of tiles, stages and 16-byte words, words that
+# cross split points, blocks narrower than a word, one and two CTAs a tile, the last tiles split, few rows
+@pytest.mark.parametrize("ti,tj,tk", [
+    (ES(1000, 1), ES(2001, 1), ES(1504, 1)),                 # A alone has odd rows
+    (ES(1000, 1), ES(2000, 1), ES(1501, 1)),                 # B alone
+    (ES(1025, 1), ES(2001, 1), ES(1281, 1)),                 # both, one past a tile
+    (ES(1500, 2), ES(2503, 2), ES(2001, 2)),                 # odd halves
+    (ES(4001, 4), ES(3000, 1), ES(2504, 1)),                 # unequal row blocks only
+    ([0, 100, 1301], [0, 130, 1931], [0, 135, 271, 1400]),   # ragged
+    (ES(1640, 3), list(range(0, 1407, 7)), ES(1520, 2)),     # contracted intervals shorter than a 16-byte word
+    (ES(1640, 3), ES(1699, 1), list(range(0, 1407, 7))),     # and columns
+    (ES(1024, 1), ES(2200, 8), ES(1024, 4)),                 # contracted blocks of 275 rows in four columns of blocks: B is copied as well
+    (ES(1024, 1), ES(2200, 8), ES(1024, 1)),                 # in one: B stays, as one block
+    (ES(1280, 10), ES(4416, 4), ES(1511, 1)),                # A stays, B copied with A's contracted blocks
+    (ES(4097, 7), ES(4416, 4), ES(3072, 4)),                 # B stays in its blocks, A copied with them
+    (ES(4097, 1), ES(321, 1), ES(4351, 1)),                  # more tiles than pairs of SMs, and a short contracted index
+    (ES(30, 1), ES(4001, 1), ES(3501, 1)),                   # few rows
+    (ES(1, 1), ES(5001, 1), ES(3999, 3)),
+    (ES(65, 5), ES(3999, 1), ES(3000, 5)),                   # few rows in several blocks
+])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_copied_operands(ti, tj, tk, dtype):
+    a, b, ra, rb, res, spec = _problem(ti, tj, tk, dtype)
+    before = ja.ja_launch_count()
+    spec.execute([ra, rb], res)
+    assert ja.ja_launch_count() - before >= 2               # a copy and a product
+    _check(res, a, b, dtype)
+
+
+def test_captures():
+    """A capture cannot take the scratch of the copies: before any other call it records the form without them, afterwards the copies."""
+    a, b, ra, rb, res, first = _problem(ES(1000, 1), ES(2001, 1), ES(1501, 1), BF)
+    first.execute([ra, rb], res)                 # puts the relations' key tables on the device, which a capture cannot either
+    torch.cuda.current_stream().synchronize()
+    spec = ja.Spec("ij,jk->ik", {"i": ES(1000, 1), "j": ES(2001, 1), "k": ES(1501, 1)}, "mul", (), "sum")
+    st = torch.cuda.Stream()
+    for launches in (1, 2):
+        with torch.cuda.stream(st):
+            g = torch.cuda.CUDAGraph()
+            before = ja.ja_launch_count()
+            with torch.cuda.graph(g, stream=st):
+                spec.execute([ra, rb], res)
+            assert ja.ja_launch_count() - before == launches
+            res.payload.fill_(float("nan"))
+            g.replay()
+            st.synchronize()
+            _check(res, a, b, BF)
+            res.payload.fill_(float("nan"))
+            spec.execute([ra, rb], res)
+            st.synchronize()
+            _check(res, a, b, BF)
+
+
+def test_one_plan_on_two_streams_and_many_calls_in_a_row():
+    """Scratch taken on one stream serves another one behind it, and a queue of calls of several plans gives each its own result."""
+    sets = [_problem(ES(1300, 2), ES(1501, 1), ES(1401, 3), BF) for _ in range(2)]
+    other = torch.cuda.Stream()
+    for k in range(20):
+        _, _, ra, rb, res, spec = sets[k % 2]
+        spec.execute([ra, rb], res)
+    torch.cuda.current_stream().synchronize()
+    for a, b, ra, rb, res, spec in sets:
+        _check(res, a, b, BF)
+        res.payload.fill_(float("nan"))
+        torch.cuda.current_stream().synchronize()
+        with torch.cuda.stream(other):
+            spec.execute([ra, rb], res)
+            other.synchronize()
+        _check(res, a, b, BF)
