@@ -16,6 +16,12 @@
 #include <string.h>
 
 __device__ __forceinline__ void ja_wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer that is known only after the wait: what a kernel reads through it is not fetched before, nor by the path for data that no
+// kernel writes meanwhile (a const __restrict__ parameter invites both).
+template <typename T> __device__ __forceinline__ T* ja_after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 __device__ __forceinline__ void ja_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 struct JaLaunch {

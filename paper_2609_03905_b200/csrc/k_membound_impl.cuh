@@ -34,8 +34,10 @@ __global__ void __launch_bounds__(256) flat_16bit_kernel(const uint4* __restrict
                                                          uint4* __restrict__ out, int64_t n_vec) {
     ja_wait_for_stream();
     ja_let_next_start();
+    a = ja_after_wait(a);
+    b = ja_after_wait(b);
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * 256) {
-        uint4 va = a[i], vb = b[i], vo;
+        uint4 va = __ldcs(a + i), vb = __ldcs(b + i), vo;   // read once
         const uint32_t* pa = reinterpret_cast<const uint32_t*>(&va);
         const uint32_t* pb = reinterpret_cast<const uint32_t*>(&vb);
         uint32_t* po = reinterpret_cast<uint32_t*>(&vo);
@@ -53,8 +55,10 @@ __global__ void __launch_bounds__(256) flat_f32_kernel(const float4* __restrict_
                                                        float4* __restrict__ out, int64_t n_vec) {
     ja_wait_for_stream();
     ja_let_next_start();
+    a = ja_after_wait(a);
+    b = ja_after_wait(b);
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * 256) {
-        float4 va = a[i], vb = b[i], vo;
+        float4 va = __ldcs(a + i), vb = __ldcs(b + i), vo;
         vo.x = flat_fn<FN>(va.x, vb.x); vo.y = flat_fn<FN>(va.y, vb.y);
         vo.z = flat_fn<FN>(va.z, vb.z); vo.w = flat_fn<FN>(va.w, vb.w);
         out[i] = vo;

@@ -18,21 +18,34 @@
 
 namespace {
 
+// Four accesses of a thread at a time, all loads before the first store: nothing tells the compiler that source and destination differ,
+// and one access at a time took 48.0 us on 16384 x 4096 instead of 42.1.
 template <typename V>
-__device__ __forceinline__ void copy_slab(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+__device__ __forceinline__ void copy_slab(const char* sp, char* dp, const CopySlab& sl) {
     const int vpr = sl.row_bytes / (int)sizeof(V);  // vectors per row
     const int total = vpr * sl.rows;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < total; i += 256) {
-        const int r = i / vpr, c = i - r * vpr;
-        const V v = *reinterpret_cast<const V*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * sizeof(V));
-        *reinterpret_cast<V*>(dp + (int64_t)r * sl.dst_pitch + (int64_t)c * sizeof(V)) = v;
+    for (int i = threadIdx.x; i < total; i += 4 * 256) {
+        V v[4];
+        int64_t to[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = i + u * 256;
+            if (k >= total) break;
+            const int r = k / vpr, c = k - r * vpr;
+            v[u] = *reinterpret_cast<const V*>(sp + (int64_t)r * sl.src_pitch + (int64_t)c * sizeof(V));
+            to[u] = (int64_t)r * sl.dst_pitch + (int64_t)c * sizeof(V);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i + u * 256 >= total) break;
+            *reinterpret_cast<V*>(dp + to[u]) = v[u];
+        }
     }
 }
 
 // One slab at any even alignment. Word w of row r is the w-th aligned 16-byte word that the row touches in the destination. Only
 // source words that hold wanted bytes are read (payloads are 128-byte aligned and padded, so none leaves them).
-__device__ __forceinline__ void copy_slab_any(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+__device__ __forceinline__ void copy_slab_any(const char* sp, char* dp, const CopySlab& sl) {
     const int words = (sl.row_bytes + 30) / 16;        // at most, whatever the alignment
     const int total = words * sl.rows;
     const int dr = 256 / words, dw = 256 - dr * words;
@@ -75,7 +88,7 @@ Copy copy_of(int vec_bytes, bool long_rows) {
     return vec_bytes == 16 ? COPY_16 : vec_bytes == 8 ? COPY_8 : long_rows ? COPY_ANY : vec_bytes == 4 ? COPY_4 : COPY_2;
 }
 template <int HOW>
-__device__ __forceinline__ void copy_slab_by(const char* __restrict__ sp, char* __restrict__ dp, const CopySlab& sl) {
+__device__ __forceinline__ void copy_slab_by(const char* sp, char* dp, const CopySlab& sl) {
     if (HOW == COPY_16) copy_slab<uint4>(sp, dp, sl);
     else if (HOW == COPY_8) copy_slab<uint2>(sp, dp, sl);
     else if (HOW == COPY_4) copy_slab<uint32_t>(sp, dp, sl);
@@ -86,8 +99,10 @@ __device__ __forceinline__ void copy_slab_by(const char* __restrict__ sp, char* 
 template <int HOW>
 __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict__ src, char* __restrict__ dst, const CopySlab* __restrict__ slabs,
                                                           int64_t n_slabs) {
+    // The next launch starts as the last slabs finish: the slabs are one round of several CTAs an SM, and a launch that is let in earlier
+    // takes the room that is left, unevenly (10901 x 1088 f32 in 34-cell blocks 22.0 us, 20.7 without; 3000 x 700 f16 20.4, 19.2).
     ja_wait_for_stream();
-    ja_let_next_start();
+    src = ja_after_wait(src);
     for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
         const CopySlab sl = slabs[s];
         copy_slab_by<HOW>(src + sl.src_off, dst + sl.dst_off, sl);
@@ -97,7 +112,7 @@ __global__ void __launch_bounds__(256) repartition_kernel(const char* __restrict
 template <int N, int HOW>
 __global__ void __launch_bounds__(256) repartition_param_kernel(const char* __restrict__ src, char* __restrict__ dst, const __grid_constant__ SlabParams<N> p) {
     ja_wait_for_stream();
-    ja_let_next_start();
+    src = ja_after_wait(src);
     const ParamSlab ps = p.s[blockIdx.x];
     const SlabShape sh = p.shapes[ps.shape];
     const CopySlab sl = {0, 0, ps.rows, sh.row_bytes, sh.src_pitch, sh.dst_pitch};

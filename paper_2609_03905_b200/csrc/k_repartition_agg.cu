@@ -30,12 +30,12 @@ template <typename TS> __device__ __forceinline__ void unpack_cells(const uint4&
         }
     }
 }
-// p points into GLOBAL memory (the read-only path is used)
+// p points into GLOBAL memory. Copies are read once: they leave the cache first, so that the copies the producer wrote last are still there
 template <typename TS, int VEC> __device__ __forceinline__ void load_cells(const char* p, float* f) {
     if (VEC == 1) {
         f[0] = ja_to_float(*reinterpret_cast<const TS*>(p));
     } else {
-        unpack_cells<TS>(__ldg(reinterpret_cast<const uint4*>(p)), f);
+        unpack_cells<TS>(__ldcs(reinterpret_cast<const uint4*>(p)), f);
     }
 }
 
@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(256) repartition_agg_kernel(const char* __rest
                                                               int64_t copy_stride) {
     ja_wait_for_stream();
     ja_let_next_start();
+    src = ja_after_wait(src);
     for (int64_t s = blockIdx.x; s < n_slabs; s += gridDim.x) {
         const CopySlab sl = slabs[s];
         const int vpr = sl.row_bytes / (int)(VEC * sizeof(TS));  // accesses per row
@@ -85,8 +86,8 @@ __global__ void __launch_bounds__(256) repartition_agg_kernel(const char* __rest
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
                     if (c < n_copies) {
-                        raw0[c] = __ldg(reinterpret_cast<const uint4*>(sp0 + (int64_t)c * copy_stride));
-                        raw1[c] = __ldg(reinterpret_cast<const uint4*>(sp1 + (int64_t)c * copy_stride));
+                        raw0[c] = __ldcs(reinterpret_cast<const uint4*>(sp0 + (int64_t)c * copy_stride));
+                        raw1[c] = __ldcs(reinterpret_cast<const uint4*>(sp1 + (int64_t)c * copy_stride));
                     }
                 float a0[VEC], a1[VEC];
                 unpack_cells<TS>(raw0[0], a0);

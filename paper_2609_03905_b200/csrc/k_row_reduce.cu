@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const char* __restrict_
     constexpr int UNROLL = 8;                                // 16-byte loads in flight per lane
     ja_wait_for_stream();
     ja_let_next_start();
+    x = ja_after_wait(x);
+    s_in = ja_after_wait(s_in);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int nvec = g.n / VEC;                              // 16-byte vectors per row
@@ -120,7 +122,7 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const char* __restrict_
             uint4 buf[UNROLL];
 #pragma unroll
             for (int u = 0; u < UNROLL; ++u) {
-                if (v0 + 32 * u < nvec) buf[u] = __ldg(reinterpret_cast<const uint4*>(xrow + (int64_t)cb * g.blk_elems + ci));
+                if (v0 + 32 * u < nvec) buf[u] = *reinterpret_cast<const uint4*>(xrow + (int64_t)cb * g.blk_elems + ci);
                 ci += 32 * VEC;
                 while (ci >= g.bsc) { ci -= g.bsc; ++cb; }
             }
