@@ -167,6 +167,8 @@ __device__ __forceinline__ int tile_of_iter(const GemmParams& p, int i, int firs
 
 // F16: cell type of the operands and of a 2-byte output -- bf16 or f16 (a compile-time choice: a select between the two
 // conversions in the epilogue cost the plain contraction a tenth of its rate)
+// SPLIT: a tile's contracted index over a cluster of CTA pairs, one tile a cluster, the slices' f32 sums taken through distributed shared
+// memory. What bounds it is the sum and the cluster's start and end, 10 us of [512, 4096] x [4096, 4096]'s 27.1 (33.9 as whole tiles).
 // ANYC: the output's tiling is not the one that TMA sees of the operands (operands staged by k_stage.cu, rows of no whole 16 bytes): every
 // cell is located through its key table and stored by itself, 32 columns of a row at a time
 template <int CG, bool F16, bool SPLIT, bool ANYC>

