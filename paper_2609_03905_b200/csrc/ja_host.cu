@@ -1111,7 +1111,7 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 // A small product that TMA cannot address, in odd intervals: the plain-ALU kernel where its 32 x 32 tiles fit the chip twice
                 // over (64 x 314 x 320 in 2 x 8 x 4: 19 us against 46, 250 x 314 x 333 in 2 x 2 x 4: 15 against 27; 64 x 3001 x 320 in 8 x 64
                 // x 4 is 123 against 60 and stays). Its time: a start, and so much a cell and an interval of the contracted index.
-                double now = plan->contract ? us * ja_contract_tc_pieces(*plan->contract) : 1e30;
+                double now = plan->contract ? us + (ja_contract_tc_pieces(*plan->contract) - 1.0) * std::max(us - 8.0, 0.0) : 1e30;   // (a start and an end know no pieces)
                 if (plan->contract && !plan->gemm && loader != 1) {
                     auto tiles = [](const ja_relation* r, int d) {
                         int64_t n = 0;
@@ -1128,7 +1128,8 @@ extern "C" ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* co
                 if (!plan->gemm && !plan->stream && loader < 0) {
                     double staged_us = 0;
                     if ((st = ja_staged_plan(A, B, out, &plan->staged, &staged_us)) != JA_OK) return st;
-                    if (plan->staged && staged_us > 0.9 * now) plan->staged.reset();
+                    // (small ones are mostly starts and ends, which the estimates know to a few us: 534 x 1498 x 320 in eight row blocks 31 us, 34 on copies)
+                    if (plan->staged && staged_us > 0.9 * now - 4.0) plan->staged.reset();
                 }
                 plan->contract_checked = true;
             }

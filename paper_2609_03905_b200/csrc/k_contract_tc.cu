@@ -790,5 +790,5 @@ ja_status_t ja_launch_contract_tc(const ContractTcPlan& plan, cudaStream_t st) {
 // are part of the estimate.
 double ja_contract_tc_pieces(const ContractTcPlan& plan) {
     const int g = std::min(plan.p.A.g, plan.p.B.g);
-    return (g == 4 ? 1.45 : g == 2 ? 3.4 : 1.0) * (g > 1 && !(plan.p.A.equal && plan.p.B.equal) ? 1.4 : 1.0);
+    return std::max(g == 4 ? 1.45 : g == 2 ? 3.4 : 1.0, g > 1 && !(plan.p.A.equal && plan.p.B.equal) ? 1.4 : 1.0);
 }
