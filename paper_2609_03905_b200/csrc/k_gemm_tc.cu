@@ -682,7 +682,8 @@ void choose_tail(GemmTcPlan* plan) {
     plan->split = 1;
     double best = (double)(whole + (rest > 0)) * stages * 0.96;
     // (tiles sorted by weight fill the last round with narrow ones: [2048, 4096] x [4096, 11008] in 1376-wide blocks 147 us, 150 with its last 14 split)
-    if (p.n_copies == 1 && rest > 0 && !p.heavy_first && ja_config().gemm_split != 0) {
+    // The slices' sums are stored in 16 bits: a join-only product of one copy into an f32 partial relation keeps whole tiles.
+    if (p.n_copies == 1 && p.c_esize == 2 && rest > 0 && !p.heavy_first && ja_config().gemm_split != 0) {
         for (int s : {2, 4}) {
             const int at_once = clusters_at_once(s);
             if (stages < 2 * s || at_once == 0) continue;

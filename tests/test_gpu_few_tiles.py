@@ -75,3 +75,17 @@ def test_split_tiles(m, gi, k, gj, n, gk, fn):
     check_status()
     assert relfro(got, ref) <= TOL[BF]
     assert np.abs(got - ref).max() <= 2.0 ** -6 * np.abs(ref).max()
+
+
+# the join alone over ONE contracted block: few tiles, which as an aggregated product would be split, in partial relations of both cell sizes
+@pytest.mark.parametrize("m,gi,k,n,gk", [(256, 1, 4096, 4096, 1), (512, 4, 4096, 1024, 2), (384, 3, 2048, 768, 3)])
+@pytest.mark.parametrize("dtype,pdtype", [(BF, torch.float32), (F16, torch.float32), (BF, BF), (F16, F16)])
+def test_join_only_one_copy(m, gi, k, n, gk, dtype, pdtype):
+    ti, tj, tk = ES(m, gi), ES(k, 1), ES(n, gk)
+    a, b, ra, rb, _, spec = _problem(ti, tj, tk, dtype)
+    part = empty_like_tiling([1, m, n], [[0, 1], ti, tk], pdtype, fill=float("nan"))
+    spec.execute_join([ra, rb], part)
+    got, ref = download(part)[0], si.to_f64(a) @ si.to_f64(b)
+    check_status()
+    # in f32 the tensor core's truncated sums show: one unit of 2^-23 of the running sum for each of k / 16 additions, at most
+    assert relfro(got, ref) <= (k / 16 * 2.0 ** -23 if pdtype == torch.float32 else TOL[dtype])
