@@ -641,9 +641,10 @@ cudaError_t configure() {
     return e;
 }
 
-// clusters of `split` CTA pairs that the device holds at once
+// clusters of `split` CTA pairs of this instantiation (whose shared memory configure() has set) that the device holds at once
+template <bool F16, bool ANYC>
 int clusters_at_once(int split) {
-    static std::atomic<int> known[64][3];
+    static std::atomic<int> known[64][2];
     int dev = 0;
     cudaGetDevice(&dev);
     std::atomic<int>& n = known[dev & 63][split == 2 ? 0 : 1];
@@ -652,7 +653,7 @@ int clusters_at_once(int split) {
         memset(&cfg, 0, sizeof cfg);
         cfg.gridDim = dim3((unsigned)(2 * split), 1, 1);
         cfg.blockDim = dim3(NUM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = Cfg<2>::SMEM_BYTES;
+        cfg.dynamicSmemBytes = ANYC ? Cfg<2>::SMEM_BYTES_ANYC : Cfg<2>::SMEM_BYTES;
         cudaLaunchAttribute attr[1];
         memset(attr, 0, sizeof attr);
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -661,9 +662,9 @@ int clusters_at_once(int split) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc_kernel<2, false, true, false>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc_kernel<2, F16, true, ANYC>, &cfg) != cudaSuccess) {
             cudaGetLastError();
-            c = 0;
+            return 0;      // not kept: the next plan asks again
         }
         n.store(c > 0 ? c : -1);
     }
@@ -685,7 +686,8 @@ void choose_tail(GemmTcPlan* plan) {
     // The slices' sums are stored in 16 bits: a join-only product of one copy into an f32 partial relation keeps whole tiles.
     if (p.n_copies == 1 && p.c_esize == 2 && rest > 0 && !p.heavy_first && ja_config().gemm_split != 0) {
         for (int s : {2, 4}) {
-            const int at_once = clusters_at_once(s);
+            const int at_once = plan->any_c ? (p.f16 ? clusters_at_once<true, true>(s) : clusters_at_once<false, true>(s))
+                                            : (p.f16 ? clusters_at_once<true, false>(s) : clusters_at_once<false, false>(s));
             if (stages < 2 * s || at_once == 0) continue;
             const double t = (double)whole * stages * 0.96 + (double)((rest + at_once - 1) / at_once) * ((stages + s - 1) / s) * 0.96 + (whole ? 12.0 : 10.0);
             if (t < best) {

@@ -1,6 +1,10 @@
 """Products that leave most of the chip idle as whole tiles: few rows against a large second operand (k_stream_tc.cu), and few tiles, or a few
 in the last round, split along the contracted index over clusters (k_gemm_tc.cu), against an fp64 product of the same 16-bit inputs.
 Tolerance: gpu_util.TOL, ten half-ulps of the stored type."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -89,3 +93,29 @@ def test_join_only_one_copy(m, gi, k, n, gk, dtype, pdtype):
     check_status()
     # in f32 the tensor core's truncated sums show: one unit of 2^-23 of the running sum for each of k / 16 additions, at most
     assert relfro(got, ref) <= (k / 16 * 2.0 ** -23 if pdtype == torch.float32 else TOL[dtype])
+
+
+FIRST_PLANS = """
+import sys
+import torch
+import paper_2609_03905_b200 as ja
+from oracle import blocked
+ES = blocked.equal_splits
+for name in sys.argv[1:]:
+    dt, ti = {"f16": (torch.float16, ES(2560, 1)), "bf16": (torch.bfloat16, ES(2560, 1)), "copies": (torch.bfloat16, [0, 100, 2560])}[name]
+    tj, tk = ES(4096, 1), ES(2048, 1)
+    a, b, c = ja.Relation([2560, 4096], [ti, tj], dt), ja.Relation([4096, 2048], [tj, tk], dt), ja.Relation([2560, 2048], [ti, tk], dt)
+    before = ja.ja_launch_count()
+    ja.Spec("ij,jk->ik", {"i": ti, "j": tj, "k": tk}).execute([a, b], c)
+    torch.cuda.synchronize()
+    print(ja.ja_launch_count() - before)
+"""
+
+
+# 80 tiles over 74 pairs of SMs: a launch of whole tiles and one of split ones, whichever product the process plans first
+@pytest.mark.parametrize("order", [("f16", "bf16"), ("bf16", "f16"), ("copies", "f16", "bf16")])
+def test_split_whatever_was_planned_first(order):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", FIRST_PLANS, *order], cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    assert out.stdout.split() == ["3" if name == "copies" else "2" for name in order]
