@@ -62,6 +62,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, ctl, status);
 }
+// The same for a whole warp, converged again behind it and of one mind: a limit can run out for some lanes and not for others, and
+// what follows is for whole warps (cluster barriers, tensor memory).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* ctl, int32_t* status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctl, status));
+}
 // what a CTA's first thread writes into the two control words before any wait
 __device__ __forceinline__ void wait_ctl_init(volatile int* ctl, uint32_t cap_us) {
     ctl[0] = 0;

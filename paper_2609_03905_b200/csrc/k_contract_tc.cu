@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     // contiguous index, so that stores are coalesced whatever the block widths are and a cluster can sum its slices ----
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
-    const bool ok = mbar_wait(done_bar, 0, ctl, p.status);
+    const bool ok = mbar_wait_warp(done_bar, 0, ctl, p.status);
     tc_fence_after();
     const bool n_minor = p.C.kc != 0;
     const int pitch = (n_minor ? BN : BM) + 4, lines = n_minor ? BM : BN, mine = lines / split;   // the lines each CTA of the cluster stores

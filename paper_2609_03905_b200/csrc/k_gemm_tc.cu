@@ -498,9 +498,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if constexpr (SPLIT) {
         // ================= the slices' sum: every row goes to one CTA of the cluster, [slice][row][column] f32 over the stages =================
         const TileCoord tc = tile_coord<CG>(p, first_tile, cta_rank);
-        const bool ok = mbar_wait(tfull_bar(0), 0, abort_flag, p.status);
+        const bool ok = mbar_wait_warp(tfull_bar(0), 0, abort_flag, p.status);
         tc_fence_after();
-        __syncwarp();
         cluster_sync_all();   // every product of the cluster has read its stages
         constexpr int PITCH = BN + 4;
         const int mine = BM / p.split, slice = cl_rank >> 1;

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
         }
         if (ok) umma_commit_w<1>(done_bar, leader);
     }
-    const bool ok = mbar_wait(done_bar, 0, ctl, p.status);
+    const bool ok = mbar_wait_warp(done_bar, 0, ctl, p.status);
     tc_fence_after();
     if (!ok && warp == 0 && lane == 0) {   // gave up: wait (bounded) for the copies in flight before the shared memory goes
         for (int s = 0; s < stages && ch0 + s < ch1; ++s) {
@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
             while (!mbar_try_wait(full_bar(s), last) && global_ns() - t0 < 200000000ull) {}
         }
     }
+    __syncwarp();
     // ---- every token's partial sums go to the CTA of the cluster that owns the token: [slice][own token][128 columns] f32 over the
     // stages, which every product has read ----
     const int slots = p.nbm * p.pad, mine = slots / split;
