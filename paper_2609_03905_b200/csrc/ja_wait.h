@@ -32,3 +32,7 @@ JA_HD bool ja_bounded_wait(TryWait try_wait, Clock now_ns, Aborted aborted, Fail
         }
     }
 }
+
+// A ring of `stages` buffers has been filled `issued` times, buffer after buffer: the parity of the phase that the last fill of buffer s
+// completes, or -1 where it was never filled. Who leaves early waits for these before its shared memory goes.
+JA_HD int ja_last_fill_parity(int issued, int stages, int s) { return s < issued ? (issued - 1 - s) / stages & 1 : -1; }

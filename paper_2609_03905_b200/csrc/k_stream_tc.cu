@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     const int chunks = p.nbk * p.per_blk;
     const int ch0 = (int)((int64_t)chunks * rank / split), ch1 = (int)((int64_t)chunks * (rank + 1) / split);
 
+    int issued = 0;            // stages that this thread has started to fill
     if (warp == 0) {
         if (lane == 0) {
             const int boxes = width > 64 ? 2 : 1;
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
                 mbar_expect_tx(fb, tx);
                 for (int c = 0; c < boxes; ++c) tma_load_4d<1>(w + c * W_BOX, &tmB, fb, cin[c], kc * BK, nb[c], jb);
                 for (int b = 0; b < p.nbm; ++b) tma_load_4d<1>(x + b * p.pad * (BK * 2), &tmA, fb, kc * BK, 0, jb, b);
+                ++issued;
                 if (++kc == p.per_blk) { kc = 0; ++jb; }
                 if (++stage == stages) { stage = 0; phase ^= 1; }
             }
@@ -140,10 +142,9 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     const bool ok = mbar_wait_warp(done_bar, 0, ctl, p.status);
     tc_fence_after();
     if (!ok && warp == 0 && lane == 0) {   // gave up: wait (bounded) for the copies in flight before the shared memory goes
-        for (int s = 0; s < stages && ch0 + s < ch1; ++s) {
-            const uint32_t last = (uint32_t)((ch1 - 1 - ch0 - s) / stages) & 1;
+        for (int s = 0; s < stages && s < issued; ++s) {
             const uint64_t t0 = global_ns();
-            while (!mbar_try_wait(full_bar(s), last) && global_ns() - t0 < 200000000ull) {}
+            while (!mbar_try_wait(full_bar(s), (uint32_t)ja_last_fill_parity(issued, stages, s)) && global_ns() - t0 < 200000000ull) {}
         }
     }
     __syncwarp();

@@ -6,6 +6,10 @@ compiled for the host, against a scripted barrier and clock. The GPU test launch
 nobody arrives at, with a 1 ms limit: the kernel must return normally, the stream's status word must read JA_ERR_TIMEOUT
 once and be clear afterwards, and ordinary launches (the persistent attention kernel, whose work counters the status
 call resets) must then pass parity as if nothing had happened. No product kernel is made to stall."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -52,6 +56,22 @@ def test_wait_follows_the_abort_flag_without_recording_a_second_error():
     polls, ok, recorded, ns = ja.ja_debug_bounded_wait_host(0, 100, 10**12, abort_at_poll=500)
     assert not ok and not recorded
     assert 500 <= polls <= 500 + 64
+
+
+def test_who_leaves_early_waits_for_the_fills_it_has_issued(tmp_path):
+    """csrc/ja_wait.h compiled for the host: a producer that gives up after any number of fills waits for the phase of the last one of
+    every buffer of its ring, and for no phase that nothing will complete."""
+    csrc = os.path.join(os.path.dirname(ja.__file__), "csrc")
+    src, lib = tmp_path / "fills.cpp", tmp_path / "fills.so"
+    src.write_text('#include "ja_wait.h"\nextern "C" int parity(int issued, int stages, int s) { return ja_last_fill_parity(issued, stages, s); }\n')
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", csrc, "-o", str(lib), str(src)], check=True)
+    parity = ctypes.CDLL(str(lib)).parity
+    for stages in range(1, 9):
+        fills = [0] * stages                      # of each buffer
+        for issued in range(40):
+            for s in range(stages):
+                assert parity(issued, stages, s) == ((fills[s] - 1) & 1 if fills[s] else -1), (stages, issued, s)
+            fills[issued % stages] += 1
 
 
 def test_switches_reject_unknown_names_and_bad_limits():
