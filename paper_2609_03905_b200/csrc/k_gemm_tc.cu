@@ -709,7 +709,7 @@ static ja_status_t encode_operands(GemmTcPlan* plan) {
 }
 
 // a, b: the operands' blocks, of one contracted extent. any_c: C has its own tiling of the same index ranges. Operands without a base get
-// one by ja_gemm_tc_set_bases before every launch.
+// one by ja_gemm_tc_set_bases before the first launch.
 static ja_status_t plan_gemm(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, const GemmEpilogue* ep, bool any_c,
                              std::shared_ptr<GemmTcPlan>* out, bool* eligible) {
     const int epi = ep ? ep->epi : 0;
@@ -803,7 +803,6 @@ ja_status_t ja_gemm_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, con
 }
 
 ja_status_t ja_gemm_tc_set_bases(GemmTcPlan* plan, char* a, char* b) {
-    if (plan->a.base == a && plan->b.base == b) return JA_OK;
     plan->a.base = a;
     plan->b.base = b;
     return encode_operands(plan);

@@ -242,18 +242,24 @@ ja_status_t ja_launch_staged(StagedPlan* plan, cudaStream_t st, bool* launched) 
             const int64_t bytes = (int64_t)(plan->a_bytes + plan->b_bytes);
             cudaMemPool_t pool;
             if ((s = ja_library_pool(&pool)) != JA_OK) return s;
-            if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES || cudaMallocFromPoolAsync((void**)&plan->scratch, (size_t)bytes, pool, st) != cudaSuccess) {
+            char* taken = nullptr;
+            if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES || cudaMallocFromPoolAsync((void**)&taken, (size_t)bytes, pool, st) != cudaSuccess) {
                 cudaGetLastError();    // no memory for it: the other form
-                plan->scratch = nullptr;
                 g_staged_bytes -= bytes;
                 return JA_OK;
             }
+            char *a = plan->a_bytes ? taken : plan->a_base, *b = plan->b_bytes ? taken + plan->a_bytes : plan->b_base;
+            if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) {
+                cudaFreeAsync(taken, st);
+                g_staged_bytes -= bytes;
+                return s;
+            }
+            // kept only now: a plan that has scratch has maps of it
             cudaGetDevice(&plan->device);
+            plan->scratch = taken;
             plan->home = st;
-            char *a = plan->a_bytes ? plan->scratch : plan->a_base, *b = plan->b_bytes ? plan->scratch + plan->a_bytes : plan->b_base;
             plan->copies.c[0].dst = a;
             plan->copies.c[1].dst = b;
-            if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) return s;
         }
     }
     const Copies& c = plan->copies;

@@ -294,7 +294,6 @@ ja_status_t ja_stream_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, c
 }
 
 ja_status_t ja_stream_tc_set_bases(StreamTcPlan* plan, char* a, char* b) {
-    if (plan->a.base == a && plan->b.base == b) return JA_OK;
     plan->a.base = a;
     plan->b.base = b;
     return encode_operands(plan);
