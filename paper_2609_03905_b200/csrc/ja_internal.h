@@ -217,7 +217,7 @@ struct StreamTcPlan;
 ja_status_t ja_stream_tc_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us);
 ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st);
 // Products of relations that TMA cannot address, on copies that it can (k_stage.cu). *out stays empty where that is not possible or the
-// relations need no copy; *launched stays false where this call cannot have its scratch (a capture, no memory). Key tables must be on the device.
+// relations need no copy; *launched stays false where there is no scratch (no memory, or no call yet but ones that a capture records). Key tables must be on the device.
 struct StagedPlan;
 struct TmaOperand;
 ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StagedPlan>* out, double* est_us);

@@ -15,6 +15,8 @@
 
 #include <algorithm>
 #include <atomic>
+#include <map>
+#include <mutex>
 
 #include "ja_device.cuh"
 #include "ja_launch.cuh"
@@ -148,8 +150,6 @@ struct StagedPlan {
     std::shared_ptr<StreamTcPlan> stream;
     char* scratch = nullptr;
     int device = 0;
-    cudaStream_t home = nullptr;    // the stream that the scratch was taken on
-    bool everywhere = false;        // other streams may use it
     ~StagedPlan() {
         if (!scratch) return;
         int now = 0;
@@ -228,39 +228,64 @@ ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_
     return JA_OK;
 }
 
+namespace {
+
+// Calls that a capture of any thread may forbid, made while this lives: on streams of the library's own and on memory that no capture knows
+struct OutsideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Memory of the library's pool that is good for every stream, and for captures, when this returns. It is taken on a stream of the
+// library's own: nothing runs there, so the wait for it is no wait for any caller's work.
+bool take_scratch(int64_t bytes, char** out) {
+    static std::mutex mu;
+    static std::map<int, cudaStream_t> own;
+    const OutsideCaptures relaxed;
+    int dev = 0;
+    cudaMemPool_t pool;
+    if (cudaGetDevice(&dev) != cudaSuccess || ja_library_pool(&pool) != JA_OK) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    cudaStream_t& st = own[dev];
+    if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+        st = nullptr;
+        return false;
+    }
+    char* p = nullptr;
+    if (cudaMallocFromPoolAsync((void**)&p, (size_t)bytes, pool, st) != cudaSuccess) return false;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return false;
+    *out = p;
+    return true;
+}
+
+}  // namespace
+
 ja_status_t ja_launch_staged(StagedPlan* plan, cudaStream_t st, bool* launched) {
     *launched = false;
     ja_status_t s;
-    if (!plan->scratch || (!plan->everywhere && st != plan->home)) {
-        // a capture cannot take memory or wait: the caller's other form runs there until a call outside has been made
+    if (!plan->scratch) {
+        // a call that a capture records takes no memory: the caller's other form runs there until a call outside has been made
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return JA_OK;
-        if (plan->scratch) {
-            JA_CUDA(cudaStreamSynchronize(plan->home));
-            plan->everywhere = true;
-        } else {
-            const int64_t bytes = (int64_t)(plan->a_bytes + plan->b_bytes);
-            cudaMemPool_t pool;
-            if ((s = ja_library_pool(&pool)) != JA_OK) return s;
-            char* taken = nullptr;
-            if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES || cudaMallocFromPoolAsync((void**)&taken, (size_t)bytes, pool, st) != cudaSuccess) {
-                cudaGetLastError();    // no memory for it: the other form
-                g_staged_bytes -= bytes;
-                return JA_OK;
-            }
-            char *a = plan->a_bytes ? taken : plan->a_base, *b = plan->b_bytes ? taken + plan->a_bytes : plan->b_base;
-            if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) {
-                cudaFreeAsync(taken, st);
-                g_staged_bytes -= bytes;
-                return s;
-            }
-            // kept only now: a plan that has scratch has maps of it
-            cudaGetDevice(&plan->device);
-            plan->scratch = taken;
-            plan->home = st;
-            plan->copies.c[0].dst = a;
-            plan->copies.c[1].dst = b;
+        const int64_t bytes = (int64_t)(plan->a_bytes + plan->b_bytes);
+        char* taken = nullptr;
+        if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES || !take_scratch(bytes, &taken)) {
+            cudaGetLastError();    // no memory for it: the other form
+            g_staged_bytes -= bytes;
+            return JA_OK;
         }
+        char *a = plan->a_bytes ? taken : plan->a_base, *b = plan->b_bytes ? taken + plan->a_bytes : plan->b_base;
+        if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) {
+            cudaFree(taken);
+            g_staged_bytes -= bytes;
+            return s;
+        }
+        // kept only now: a plan that has scratch has maps of it
+        cudaGetDevice(&plan->device);
+        plan->scratch = taken;
+        plan->copies.c[0].dst = a;
+        plan->copies.c[1].dst = b;
     }
     const Copies& c = plan->copies;
     const bool cut = (plan->a_bytes && c.c[0].x.nblk[1] > 1) || (plan->b_bytes && c.c[1].x.nblk[1] > 1);

@@ -100,3 +100,64 @@ def test_one_plan_on_two_streams_and_many_calls_in_a_row():
             spec.execute([ra, rb], res)
             other.synchronize()
         _check(res, a, b, BF)
+
+
+def test_streams_ordered_by_events_alone():
+    """The second stream's call neither waits on the host for the first stream nor starts before it."""
+    a, b, ra, rb, res, spec = _problem(ES(1300, 2), ES(1501, 1), ES(1401, 3), BF)
+    a2, b2, ra2, rb2, res2, spec2 = _problem(ES(30, 1), ES(4001, 1), ES(3501, 1), BF)
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    for p in ((ra, rb, res, spec), (ra2, rb2, res2, spec2)):   # the key tables and the modules, which the host does wait for
+        ja.Spec("ij,jk->ik", p[3].parts).execute([p[0], p[1]], p[2])
+    torch.cuda.synchronize()
+    payloads = {r: r.payload.clone() for r in (ra, rb)}
+    for r in payloads:
+        r.payload.fill_(float("nan"))
+    res.payload.fill_(float("nan"))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(first):
+        torch.cuda._sleep(400_000_000)             # a fifth of a second
+        spec2.execute([ra2, rb2], res2)
+        spec.execute([ra, rb], res)                # of operands that are not there yet
+        for r, x in payloads.items():
+            r.payload.copy_(x)
+        done = first.record_event()
+    second.wait_event(done)
+    with torch.cuda.stream(second):
+        spec.execute([ra, rb], res)
+        spec2.execute([ra2, rb2], res2)
+    assert not done.query()                        # the host is here before the first stream is done
+    second.synchronize()
+    _check(res, a, b, BF)
+    _check(res2, a2, b2, BF)
+
+
+def test_first_stream_may_be_gone():
+    from cuda.bindings import runtime as rt
+    a, b, ra, rb, res, spec = _problem(ES(1300, 2), ES(1501, 1), ES(1401, 3), BF)
+    err, gone = rt.cudaStreamCreateWithFlags(rt.cudaStreamNonBlocking)
+    torch.cuda.synchronize()
+    spec.execute([ra, rb], res, stream=int(gone))
+    assert rt.cudaStreamSynchronize(gone)[0] == rt.cudaStreamDestroy(gone)[0] == err == rt.cudaError_t.cudaSuccess
+    _check(res, a, b, BF)
+    res.payload.fill_(float("nan"))
+    before = ja.ja_launch_count()
+    spec.execute([ra, rb], res)
+    assert ja.ja_launch_count() - before == 2
+    _check(res, a, b, BF)
+
+
+def test_capture_on_another_stream_than_the_first_call():
+    a, b, ra, rb, res, spec = _problem(ES(1000, 1), ES(2001, 1), ES(1501, 1), BF)
+    spec.execute([ra, rb], res)
+    torch.cuda.synchronize()
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    before = ja.ja_launch_count()
+    with torch.cuda.graph(g, stream=st):
+        spec.execute([ra, rb], res)
+    assert ja.ja_launch_count() - before == 2      # the copy and the product, as outside
+    for _ in range(2):
+        res.payload.fill_(float("nan"))
+        torch.cuda.current_stream().synchronize()
+        g.replay()
+        _check(res, a, b, BF)
