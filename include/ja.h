@@ -156,9 +156,10 @@ ja_status_t ja_relation_get_keys(const ja_relation_t* rel, int32_t* coords, int6
  * Supported forms (letters are free; shapes of the signature matter):
  *   "ij,jk->ik"            MUL / SUM        bf16, f16 or f32 operands (one dtype for all three relations), f32 accumulate.
  *                                            bf16 / f16: tensor cores under every tiling
- *                                            (operands fetched by TMA on uniform blocks with 16-byte rows, by plain
- *                                            asynchronous loads otherwise; plain ALUs only where blocks are smaller than
- *                                            64 cells a side); f32: plain ALUs
+ *                                            (operands fetched by TMA on uniform blocks with 16-byte rows; otherwise by TMA
+ *                                            from copies in scratch memory or by plain asynchronous loads, whichever is
+ *                                            expected to be faster; plain ALUs only where blocks are smaller than 64 cells a
+ *                                            side); f32: plain ALUs
  *   "ij,jk,ik->ik"         MATMUL_ADD / SUM   } fused chains: the accumulator of the contraction goes through the
  *   "ij,jk->ik"            MATMUL_ROPE / SUM  } next join-agg before its single rounding and store; bf16 or f16 relations
  *   "ij,jk,jk->ik"         SWIGLU_UP / SUM    } on uniform blocks only (JA_ERR_UNSUPPORTED otherwise: run the chain)
@@ -182,7 +183,12 @@ ja_status_t ja_relation_get_keys(const ja_relation_t* rel, int32_t* coords, int6
  * denominator of every query row (f32, tiled like the first three indices of outputs[0]) -- with it two results over
  * disjoint key ranges combine by the online-softmax aggregation: O = w1 O1 + w2 O2, w_i = exp(lse_i - lse).
  * The first call for a given (spec, relations) tuple builds and caches tables on the device (a few
- * synchronous cudaMalloc / cudaMemcpy); later calls only launch. */
+ * synchronous cudaMalloc / cudaMemcpy); later calls only launch.
+ * A 16-bit product that runs on copies keeps its scratch (at most 1 GiB a tuple and 4 GiB a process; beyond that, and where there is no
+ * memory, it runs on plain loads) from its first call outside a capture on. The scratch serves every stream and, from then on, captures; a
+ * capture before that records the form on plain loads. It is given back once the spec or one of the relations is destroyed, the graphs
+ * that recorded it are destroyed, and the work that uses it has ended: a graph stays valid when the spec goes (the relations must outlive
+ * it). None of this waits for a caller's stream. The memory stays in the library's pool until ja_exchange_trim. */
 ja_status_t ja_execute(const ja_spec_t* spec, const ja_relation_t* const* inputs, int32_t n_inputs,
                        ja_relation_t* const* outputs, int32_t n_outputs, void* cuda_stream);
 
@@ -335,6 +341,9 @@ ja_status_t ja_debug_attention_rows(const ja_relation_t* rel, int32_t* fits, int
 ja_status_t ja_debug_cell_offset(const ja_relation_t* rel, int32_t moving, const int64_t* coord, int64_t* offset);
 /* Which form of the general join-agg a spec would run on (no CUDA call): 0 none, 1 32-bit coordinates and counts, 2 64-bit ones. */
 ja_status_t ja_debug_general_form(const ja_spec_t* spec, int32_t* form);
+
+/* Bytes of the scratch that products on copies hold now: their plans, the graphs that recorded them, work that has not ended. */
+int64_t ja_debug_scratch_bytes(void);
 
 /* Number of kernels this library has launched since load (for launch accounting by callers). */
 int64_t ja_launch_count(void);

@@ -89,6 +89,7 @@ def _load() -> ctypes.CDLL:
     lib.ja_last_error.restype = ctypes.c_char_p
     lib.ja_version.restype = ctypes.c_char_p
     lib.ja_launch_count.restype = ctypes.c_int64
+    lib.ja_debug_scratch_bytes.restype = ctypes.c_int64
     return lib
 
 
@@ -374,3 +375,8 @@ def ja_debug_general_form(spec: int) -> int:
     form = ctypes.c_int32()
     _check(LIB.ja_debug_general_form(ctypes.c_void_p(spec), ctypes.byref(form)))
     return form.value
+
+
+def ja_debug_scratch_bytes() -> int:
+    """Bytes of scratch that products on copies hold: plans, graphs that recorded them, and work that has not ended."""
+    return int(LIB.ja_debug_scratch_bytes())

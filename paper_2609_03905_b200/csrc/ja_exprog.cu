@@ -1711,6 +1711,7 @@ ja_status_t ja_library_pool(cudaMemPool_t* out) {
 }
 
 extern "C" ja_status_t ja_exchange_trim(void) {
+    ja_staged_free_retired();
     std::lock_guard<std::mutex> lk(g_pool_mu);
     for (auto& kv : g_pools) JA_CUDA(cudaMemPoolTrimTo(kv.second, 0));
     return JA_OK;

@@ -267,6 +267,7 @@ extern "C" ja_status_t ja_relation_destroy(ja_relation_t* rel) {
     if (!rel) return JA_OK;
     forget_relayout_plans(rel->id);   // cached copy plans of relayouts from / to this relation (device tables) go with it
     forget_exec_plans(rel->id);       // and the launch state (tensor maps, rotation tables) of every spec that ran on it
+    ja_staged_free_retired();
     if (rel->d_tables) cudaFree(rel->d_tables);
     delete rel;
     return JA_OK;
@@ -520,6 +521,7 @@ extern "C" ja_status_t ja_spec_destroy(ja_spec_t* spec) {
         g_specs.erase(spec);
     }
     delete spec;
+    ja_staged_free_retired();
     return JA_OK;
 }
 

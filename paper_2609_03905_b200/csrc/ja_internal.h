@@ -222,6 +222,7 @@ struct StagedPlan;
 struct TmaOperand;
 ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StagedPlan>* out, double* est_us);
 ja_status_t ja_launch_staged(StagedPlan* plan, cudaStream_t st, bool* launched);
+void ja_staged_free_retired();   // frees the scratch that no plan and no graph has any more and no launch uses
 // what it runs on: plans for operands whose bases are set before the first launch
 ja_status_t ja_gemm_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<GemmTcPlan>* out, bool* eligible);
 ja_status_t ja_gemm_tc_set_bases(GemmTcPlan* plan, char* a, char* b);

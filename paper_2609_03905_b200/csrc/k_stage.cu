@@ -4,8 +4,8 @@
 //
 // The copy moves 2 bytes per byte of the operand; fed piece by piece (k_contract_tc.cu) the tensor cores wait for the loaders' instruction
 // streams instead. The copies live in scratch that the plan takes from the library's pool at its first call and keeps: at most 1 GiB a plan
-// and 4 GiB altogether, given back with the spec or the relations. Two calls of one plan that were not ordered behind one another
-// would already race on its output.
+// and 4 GiB altogether, given back when the spec or the relations go and with them the last graph that recorded a call. Two calls of one
+// plan that were not ordered behind one another would already race on its output.
 //
 // These two launches do not start inside the ones before them. With scratch taken and returned by every call between such launches,
 // [8000, 5001] x [5001, 5003] in a queue of twenty calls stopped the stream for good; every wait inside the kernels is bounded, so
@@ -17,6 +17,7 @@
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <vector>
 
 #include "ja_device.cuh"
 #include "ja_launch.cuh"
@@ -139,8 +140,124 @@ size_t plan_copy(const ja_relation* r, Copy* c) {
 
 }  // namespace
 
-static std::atomic<int64_t> g_staged_bytes{0};   // scratch of all plans
+namespace {
+
 constexpr int64_t MAX_PLAN_BYTES = (int64_t)1 << 30, MAX_ALL_BYTES = (int64_t)4 << 30;
+std::atomic<int64_t> g_staged_bytes{0};   // scratch of all plans, until it is freed
+
+// Calls that a capture of any thread may forbid, made while this lives: on streams of the library's own and on memory that no capture knows
+struct OutsideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Scratch belongs to its plan and to every graph that recorded a call on it (a user object of the graph). Whoever lets go of it last retires
+// it without a CUDA call, which the driver does not allow there, and a later call of the library frees it, once the calls outside
+// graphs have ended: an event for each stream that has seen one. A graph lets go when its own launches have ended. So no destructor
+// waits for the device, nor meets a capture that forbids it.
+struct Scratch {
+    char* at;
+    int64_t bytes;
+    cudaStream_t own;                                  // the library's stream that it was taken on
+    std::map<unsigned long long, cudaEvent_t> used;    // by stream id
+};
+struct Retired {
+    std::mutex mu;
+    std::vector<Scratch*> list;
+    std::atomic<int> n{0};
+};
+Retired& retired() {
+    static Retired* r = new Retired;   // never destroyed: a graph's last reference may go at exit
+    return *r;
+}
+void retire(Scratch* s) {
+    Retired& r = retired();
+    std::lock_guard<std::mutex> lk(r.mu);
+    r.list.push_back(s);
+    ++r.n;
+}
+void CUDART_CB let_go(void* owner) { delete static_cast<std::shared_ptr<Scratch>*>(owner); }
+
+// wait: for calls that have not ended
+void free_retired(bool wait) {
+    Retired& r = retired();
+    if (r.n.load() == 0) return;
+    std::vector<Scratch*> mine;
+    {
+        std::lock_guard<std::mutex> lk(r.mu);
+        mine.swap(r.list);
+        r.n = 0;
+    }
+    const OutsideCaptures relaxed;
+    for (Scratch* s : mine) {
+        bool ended = true;
+        for (auto& u : s->used) ended = ended && (wait ? cudaEventSynchronize(u.second) : cudaEventQuery(u.second)) == cudaSuccess;
+        if (!ended) {
+            cudaGetLastError();
+            retire(s);
+            continue;
+        }
+        for (auto& u : s->used) cudaEventDestroy(u.second);
+        cudaFreeAsync(s->at, s->own);
+        cudaStreamSynchronize(s->own);
+        g_staged_bytes -= s->bytes;
+        delete s;
+    }
+}
+
+// Memory of the library's pool that is good for every stream, and for captures, when this returns: it is taken on a stream of the
+// library's own, where nothing else runs, so the wait for it is no wait for any caller's work. Empty where there is none.
+std::shared_ptr<Scratch> take_scratch(int64_t bytes) {
+    static std::mutex mu;
+    static std::map<int, cudaStream_t> own;
+    const OutsideCaptures relaxed;
+    int dev = 0;
+    cudaMemPool_t pool;
+    if (cudaGetDevice(&dev) != cudaSuccess || ja_library_pool(&pool) != JA_OK) return nullptr;
+    free_retired(false);
+    if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES) free_retired(true);   // (which form a call takes must not hang on how far the GPU is)
+    std::lock_guard<std::mutex> lk(mu);
+    char* p = nullptr;
+    cudaStream_t& st = own[dev];
+    if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) st = nullptr;
+    if (g_staged_bytes.load() <= MAX_ALL_BYTES && st && cudaMallocFromPoolAsync((void**)&p, (size_t)bytes, pool, st) == cudaSuccess &&
+        cudaStreamSynchronize(st) == cudaSuccess)
+        return std::shared_ptr<Scratch>(new Scratch{p, bytes, st, {}}, retire);
+    cudaGetLastError();
+    g_staged_bytes -= bytes;
+    return nullptr;
+}
+
+// The event that calls on this stream are recorded with; those of streams that have drained make room. nullptr where there is none.
+cudaEvent_t event_of(Scratch* s, cudaStream_t st) {
+    unsigned long long id = 0;
+    if (cudaStreamGetId(st, &id) != cudaSuccess) return nullptr;
+    auto it = s->used.find(id);
+    if (it != s->used.end()) return it->second;
+    const OutsideCaptures relaxed;
+    for (auto u = s->used.begin(); u != s->used.end();) {
+        if (cudaEventQuery(u->second) != cudaSuccess) {
+            ++u;
+            continue;
+        }
+        cudaEventDestroy(u->second);
+        u = s->used.erase(u);
+    }
+    cudaGetLastError();
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
+    return s->used[id] = e;
+}
+
+}  // namespace
+
+void ja_staged_free_retired() { free_retired(false); }
+
+extern "C" int64_t ja_debug_scratch_bytes(void) {
+    free_retired(false);
+    return g_staged_bytes.load();
+}
 
 struct StagedPlan {
     Copies copies;           // of A and of B
@@ -148,18 +265,8 @@ struct StagedPlan {
     char *a_base, *b_base;   // of the operands that are used as they lie
     std::shared_ptr<GemmTcPlan> gemm;
     std::shared_ptr<StreamTcPlan> stream;
-    char* scratch = nullptr;
-    int device = 0;
-    ~StagedPlan() {
-        if (!scratch) return;
-        int now = 0;
-        cudaGetDevice(&now);
-        cudaSetDevice(device);
-        cudaDeviceSynchronize();    // pool memory is freed without one
-        cudaFree(scratch);
-        cudaSetDevice(now);
-        g_staged_bytes -= (int64_t)(a_bytes + b_bytes);
-    }
+    std::shared_ptr<Scratch> scratch;
+    unsigned long long recorded = 0;   // the capture whose graph has been made an owner
 };
 
 ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_relation* C, std::shared_ptr<StagedPlan>* out, double* est_us) {
@@ -228,70 +335,55 @@ ja_status_t ja_staged_plan(const ja_relation* A, const ja_relation* B, const ja_
     return JA_OK;
 }
 
-namespace {
-
-// Calls that a capture of any thread may forbid, made while this lives: on streams of the library's own and on memory that no capture knows
-struct OutsideCaptures {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
-
-// Memory of the library's pool that is good for every stream, and for captures, when this returns. It is taken on a stream of the
-// library's own: nothing runs there, so the wait for it is no wait for any caller's work.
-bool take_scratch(int64_t bytes, char** out) {
-    static std::mutex mu;
-    static std::map<int, cudaStream_t> own;
-    const OutsideCaptures relaxed;
-    int dev = 0;
-    cudaMemPool_t pool;
-    if (cudaGetDevice(&dev) != cudaSuccess || ja_library_pool(&pool) != JA_OK) return false;
-    std::lock_guard<std::mutex> lk(mu);
-    cudaStream_t& st = own[dev];
-    if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
-        st = nullptr;
-        return false;
-    }
-    char* p = nullptr;
-    if (cudaMallocFromPoolAsync((void**)&p, (size_t)bytes, pool, st) != cudaSuccess) return false;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return false;
-    *out = p;
-    return true;
-}
-
-}  // namespace
-
 ja_status_t ja_launch_staged(StagedPlan* plan, cudaStream_t st, bool* launched) {
     *launched = false;
     ja_status_t s;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long cap_id = 0;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamGetCaptureInfo(st, &cap, &cap_id, &graph) != cudaSuccess) {
+        cudaGetLastError();   // the question's own error; the launch will tell
+        return JA_OK;
+    }
     if (!plan->scratch) {
         // a call that a capture records takes no memory: the caller's other form runs there until a call outside has been made
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return JA_OK;
-        const int64_t bytes = (int64_t)(plan->a_bytes + plan->b_bytes);
-        char* taken = nullptr;
-        if (g_staged_bytes.fetch_add(bytes) + bytes > MAX_ALL_BYTES || !take_scratch(bytes, &taken)) {
-            cudaGetLastError();    // no memory for it: the other form
-            g_staged_bytes -= bytes;
-            return JA_OK;
-        }
-        char *a = plan->a_bytes ? taken : plan->a_base, *b = plan->b_bytes ? taken + plan->a_bytes : plan->b_base;
-        if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) {
-            cudaFree(taken);
-            g_staged_bytes -= bytes;
-            return s;
-        }
+        if (cap != cudaStreamCaptureStatusNone) return JA_OK;
+        const std::shared_ptr<Scratch> taken = take_scratch((int64_t)(plan->a_bytes + plan->b_bytes));
+        if (!taken) return JA_OK;   // no memory for it: the other form
+        char *a = plan->a_bytes ? taken->at : plan->a_base, *b = plan->b_bytes ? taken->at + plan->a_bytes : plan->b_base;
+        if ((s = plan->gemm ? ja_gemm_tc_set_bases(plan->gemm.get(), a, b) : ja_stream_tc_set_bases(plan->stream.get(), a, b)) != JA_OK) return s;
         // kept only now: a plan that has scratch has maps of it
-        cudaGetDevice(&plan->device);
         plan->scratch = taken;
         plan->copies.c[0].dst = a;
         plan->copies.c[1].dst = b;
+    }
+    cudaEvent_t event = nullptr;
+    if (cap == cudaStreamCaptureStatusNone) {
+        if (!(event = event_of(plan->scratch.get(), st))) {
+            cudaGetLastError();
+            return JA_OK;
+        }
+    } else if (plan->recorded != cap_id) {
+        auto* owner = new std::shared_ptr<Scratch>(plan->scratch);
+        cudaUserObject_t held;
+        if (cudaUserObjectCreate(&held, owner, let_go, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+            delete owner;
+            cudaGetLastError();
+            return JA_OK;
+        }
+        if (cudaGraphRetainUserObject(graph, held, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+            cudaUserObjectRelease(held, 1);
+            cudaGetLastError();
+            return JA_OK;
+        }
+        plan->recorded = cap_id;
     }
     const Copies& c = plan->copies;
     const bool cut = (plan->a_bytes && c.c[0].x.nblk[1] > 1) || (plan->b_bytes && c.c[1].x.nblk[1] > 1);
     JA_CUDA(ja_launch_kernel_after(cut ? stage_kernel<true> : stage_kernel<false>, dim3((unsigned)(c.c[0].ctas + c.c[1].ctas)), THREADS, 0, 1, st, c));
     ja_count_launch();
     s = plan->gemm ? ja_launch_gemm_tc(*plan->gemm, st) : ja_launch_stream_tc(*plan->stream, st);
+    if (event) JA_CUDA(cudaEventRecord(event, st));
     *launched = s == JA_OK;
     return s;
 }

@@ -1,6 +1,8 @@
 """Products of 16-bit relations that TMA cannot address as they lie, on copies that it can (k_stage.cu), and the stores that go with them, against
 an fp64 product of the same 16-bit inputs. Tolerance: gpu_util.TOL, ten half-ulps of the stored type; f32 accumulation does not show
 beside it."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -161,3 +163,70 @@ def test_capture_on_another_stream_than_the_first_call():
         torch.cuda.current_stream().synchronize()
         g.replay()
         _check(res, a, b, BF)
+
+
+def _drops_to(held):
+    """Graphs are destroyed by the driver in its own time."""
+    torch.cuda.synchronize()
+    for _ in range(500):
+        if ja.ja_debug_scratch_bytes() <= held:
+            return True
+        time.sleep(0.02)
+    return False
+
+
+def test_graph_outlives_its_spec():
+    """The scratch that a graph recorded is the graph's as well: not handed to the next plan, and given back when the graph goes."""
+    held = ja.ja_debug_scratch_bytes()
+    a, b, ra, rb, res, spec = _problem(ES(1000, 1), ES(2001, 1), ES(1501, 1), BF)
+    spec.execute([ra, rb], res)
+    torch.cuda.synchronize()
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        spec.execute([ra, rb], res)
+        spec.execute([ra, rb], res)
+    mine = ja.ja_debug_scratch_bytes() - held
+    assert mine > 0
+    spec.close()
+    assert ja.ja_debug_scratch_bytes() == held + mine
+    a2, b2, ra2, rb2, res2, spec2 = _problem(ES(1000, 1), ES(2001, 1), ES(1501, 1), BF)
+    a2, rb2 = -a2, upload(-b2, [ES(2001, 1), ES(1501, 1)])
+    spec2.execute([ra2, rb2], res2)
+    assert ja.ja_debug_scratch_bytes() == held + 2 * mine
+    res.payload.fill_(float("nan"))
+    g.replay()
+    _check(res, a, b, BF)
+    spec2.execute([ra2, rb2], res2)
+    _check(res2, a2, b2, BF)
+    spec2.close()
+    g.replay()                                     # under way when the graph goes
+    del g
+    assert _drops_to(held)
+    _check(res, a, b, BF)
+
+
+def test_spec_dropped_while_a_capture_runs_and_with_its_work_under_way():
+    held = ja.ja_debug_scratch_bytes()
+    a, b, ra, rb, res, spec = _problem(ES(1000, 1), ES(2001, 1), ES(1501, 1), BF)
+    a2, b2, ra2, rb2, res2, dropped = _problem(ES(1300, 2), ES(1501, 1), ES(1401, 3), BF)
+    spec.execute([ra, rb], res)
+    dropped.execute([ra2, rb2], res2)
+    torch.cuda.synchronize()
+    res2.payload.fill_(float("nan"))
+    torch.cuda.current_stream().synchronize()
+    other, st, g = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        spec.execute([ra, rb], res)
+        with torch.cuda.stream(other):
+            torch.cuda._sleep(200_000_000)
+            dropped.execute([ra2, rb2], res2)
+        both = ja.ja_debug_scratch_bytes()
+        dropped.close()
+        assert ja.ja_debug_scratch_bytes() == both          # its work has not ended
+    res.payload.fill_(float("nan"))
+    g.replay()
+    _check(res, a, b, BF)
+    _check(res2, a2, b2, BF)
+    spec.close()
+    del g
+    assert _drops_to(held)
