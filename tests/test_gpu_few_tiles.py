@@ -49,23 +49,24 @@ def test_few_rows(m, gi, k, gj, n, gk, dtype):
 @pytest.mark.parametrize("m,gi,k,gj,n,gk", [(512, 4, 4096, 8, 1024, 8), (1024, 8, 4096, 8, 2048, 4), (256, 2, 2048, 2, 4096, 8), (1280, 1, 1024, 1, 3840, 1),
                                             (600, 1, 1376, 8, 512, 1), (2560, 10, 512, 1, 1920, 1)])
 @pytest.mark.parametrize("fn", ["mul", "matmul_add", "swiglu_up", "matmul_rope"])
-def test_split_tiles(m, gi, k, gj, n, gk, fn):
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_split_tiles(m, gi, k, gj, n, gk, fn, dtype):
     ti, tj, tk = ES(m, gi), ES(k, gj), ES(n, gk)
     if fn != "mul" and ((n // gk) % 128 or (k // gj) % 8):
         pytest.skip("the fused forms take whole 128-column blocks and rows of whole 16 bytes")
-    a, b, ra, rb, res, spec = _problem(ti, tj, tk, BF)
+    a, b, ra, rb, res, spec = _problem(ti, tj, tk, dtype)
     parts, scale = {"i": ti, "j": tj, "k": tk}, k ** -0.5
-    b = (b.float() * scale).to(BF)
+    b = (b.float() * scale).to(dtype)
     rb = upload(b, [tj, tk])
     ref = si.to_f64(a) @ si.to_f64(b)
     if fn == "mul":
         spec.execute([ra, rb], res)
     elif fn == "matmul_add":
-        x = si.normal((m, n), 0.0, 1.0, BF, 37, 42)
+        x = si.normal((m, n), 0.0, 1.0, dtype, 37, 42)
         ref = ref + si.to_f64(x)
         ja.Spec("ij,jk,ik->ik", parts, fn).execute([ra, rb, upload(x, [ti, tk])], res)
     elif fn == "swiglu_up":
-        b2 = (si.normal((k, n), 0.0, 1.0, BF, 37, 43).float() * scale).to(BF)
+        b2 = (si.normal((k, n), 0.0, 1.0, dtype, 37, 43).float() * scale).to(dtype)
         ref = ref / (1.0 + np.exp(-ref)) * (si.to_f64(a) @ si.to_f64(b2))
         ja.Spec("ij,jk,jk->ik", parts, fn).execute([ra, rb, upload(b2, [tj, tk])], res)
     else:
@@ -77,8 +78,8 @@ def test_split_tiles(m, gi, k, gj, n, gk, fn):
         ja.Spec("ij,jk->ik", parts, fn, (10000.0, float(s_len), float(d))).execute([ra, rb], res)
     got = download(res)
     check_status()
-    assert relfro(got, ref) <= TOL[BF]
-    assert np.abs(got - ref).max() <= 2.0 ** -6 * np.abs(ref).max()
+    assert relfro(got, ref) <= TOL[dtype]
+    assert np.abs(got - ref).max() <= 2.0 ** (-6 if dtype == BF else -9) * np.abs(ref).max()
 
 
 # the join alone over ONE contracted block: few tiles, which as an aggregated product would be split, in partial relations of both cell sizes

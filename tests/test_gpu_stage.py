@@ -230,3 +230,27 @@ def test_spec_dropped_while_a_capture_runs_and_with_its_work_under_way():
     spec.close()
     del g
     assert _drops_to(held)
+
+
+@pytest.mark.parametrize("ti,tj,tk", [(ES(1000, 1), ES(2001, 1), ES(1501, 1)), ([0, 100, 1301], [0, 130, 1931], [0, 135, 271, 1400]),
+                                      (ES(1640, 3), list(range(0, 1407, 7)), ES(1520, 2)), (ES(65, 5), ES(3999, 1), ES(3000, 5))])
+@pytest.mark.parametrize("dtype", [BF, F16])
+def test_values_that_are_not_finite_stay_in_their_row_and_column(ti, tj, tk, dtype):
+    """and what lies between the blocks of a payload reaches no cell."""
+    a, b, ra, rb, res, spec = _problem(ti, tj, tk, dtype)
+    for x, r in ((a, ra), (b, rb)):
+        between = torch.from_numpy(blocked.pack(np.ones(x.shape, np.uint16), r.splits) == 0).cuda()
+        r.payload[:between.numel()][between] = float("nan")
+    before = ja.ja_launch_count()
+    spec.execute([ra, rb], res)
+    assert ja.ja_launch_count() - before >= 2
+    _check(res, a, b, dtype)
+    a[5, 17], b[9, 33], b[tj[-1] - 1, 40], a[11, tj[-1] - 1] = float("inf"), float("nan"), float("-inf"), float("nan")
+    ra, rb = upload(a, [ti, tj]), upload(b, [tj, tk])
+    spec.execute([ra, rb], res)
+    got = download(res)
+    with np.errstate(invalid="ignore"):
+        ref = si.to_f64(a) @ si.to_f64(b)
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+    ok = np.isfinite(ref)
+    assert relfro(got[ok], ref[ok]) <= TOL[dtype] and np.array_equal(np.sign(got[np.isinf(ref)]), np.sign(ref[np.isinf(ref)]))
