@@ -527,7 +527,11 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     int m0, m_end, n0, n_end;
     tile_range(p.A.r, p.cut_m, BM, band * p.group_m + tin % rows_in_band, m0, m_end);
     tile_range(p.B.r, p.cut_n, BN, tin / rows_in_band, n0, n_end);
-    if (m0 >= m_end || n0 >= n_end) return;   // an interval shorter than the longest one (the whole cluster leaves)
+    const bool early = p.split == 1;          // launched to start inside the launch before it (clusters are not)
+    if (m0 >= m_end || n0 >= n_end) {         // an interval shorter than the longest one (the whole cluster leaves)
+        if (early) ja_wait_for_stream();
+        return;
+    }
     const int bx[MAX_BATCH] = {(int)blockIdx.z, (int)blockIdx.y};
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
@@ -549,7 +553,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    if (p.split == 1) {   // launched to start inside the kernel before it
+    if (early) {
         ja_wait_for_stream();
         ja_let_next_start();
     }
