@@ -316,7 +316,7 @@ ja_status_t ja_repartition_noalloc(int32_t rank, const int64_t* extents, const i
 ja_status_t ja_stream_status(void* cuda_stream, ja_status_t* device_status);
 
 /* ---- switches and test hooks (no counterpart in the paper) ---------------------------------------------------------
- * Every device-side wait of the kernels is bounded (default 2 s; JA_WAIT_CAP=<nanoseconds> in the environment). The
+ * Every wait of the kernels on a barrier in shared memory is bounded (default 2 s; JA_WAIT_CAP=<nanoseconds> in the environment). The
  * environment (JA_* variables: the wait limit and switches that force a kernel form or a schedule) is read ONCE, when the
  * library is first used; ja_debug_set changes a value afterwards. Names: "wait_cap_ns", "attn_mma_sync", "attn_one_tile",
  * "attn_persistent", "attn_section", "attn_variant", "gemm_cta_group", "gemm_group_m", "gemm_heavy_first", "gemm_split",

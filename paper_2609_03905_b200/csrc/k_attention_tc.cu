@@ -221,6 +221,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         wait_ctl_init(abort_flag, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -229,7 +230,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_wait_for_stream();
     ja_let_next_start();
     const uint32_t tS[2] = {tmem_base, tmem_base + 128};
     const uint32_t tO[2] = {tmem_base + 256, tmem_base + 384};
@@ -692,6 +692,7 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
         wait_ctl_init(abort_flag, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -700,7 +701,6 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_wait_for_stream();
     ja_let_next_start();
 
     if (warp == 0) {

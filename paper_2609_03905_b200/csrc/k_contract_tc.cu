@@ -545,6 +545,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
         wait_ctl_init(ctl, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (early) ja_wait_for_stream();
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(BN * ACC) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -553,10 +554,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    if (early) {
-        ja_wait_for_stream();
-        ja_let_next_start();
-    }
+    if (early) ja_let_next_start();
 
     const int chunks = (p.K + BK - 1) / BK;
     const int c0 = (int)((int64_t)chunks * rank / split), c1 = (int)((int64_t)chunks * (rank + 1) / split);

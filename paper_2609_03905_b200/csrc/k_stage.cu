@@ -7,9 +7,7 @@
 // and 4 GiB altogether, given back when the spec or the relations go and with them the last graph that recorded a call. Two calls of one
 // plan that were not ordered behind one another would already race on its output.
 //
-// These two launches do not start inside the ones before them. With scratch taken and returned by every call between such launches,
-// [8000, 5001] x [5001, 5003] in a queue of twenty calls stopped the stream for good; every wait inside the kernels is bounded, so
-// what never ended were the launches' own waits.
+// These two launches do not start inside the ones before them, for the reason that ja_launch.cuh gives.
 #include <cuda.h>
 #include <string.h>
 

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
         wait_ctl_init(ctl, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(p.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -78,7 +79,6 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_wait_for_stream();
     ja_let_next_start();
 
     // ---- this CTA's columns and its slice of the contracted index ----
