@@ -36,6 +36,15 @@ template <typename T> __device__ __forceinline__ T* ja_after_wait(T* p) {
 }
 __device__ __forceinline__ void ja_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Whether a launch of `ctas` equal CTAs, `places` of which fit an SM, gains by letting a launch like it in at its start. Where the launch
+// takes half of the places or more and yet leaves one on every SM, some of the next one's CTAs find a place beside it and the rest go where
+// its own end first, so that SMs end up with more of them than their share: 320 CTAs at four places 1.09 to 1.29 times as long (f32 contractions of
+// 100 to 1000 cells), 240 at three 1.04 to 1.29, 296 in clusters of four 1.20. With 240 CTAs at four places they all fit beside it, with 480
+// an SM has no place beyond its share: 0.84 to 0.99, as for every other size from 4 to 4096.
+inline bool ja_let_next_pays(int64_t ctas, int64_t sms, int64_t places) {
+    return !(2 * ctas >= sms * places && ctas <= sms * (places - 1));
+}
+
 struct JaLaunch {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];

@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "ja_device.cuh"
 #include "ja_launch.cuh"
@@ -39,6 +40,7 @@ struct Params {
     Rel A, B, C;
     int32_t M, N, K, batch[MAX_BATCH];
     int32_t tiles_m, tiles_n, split;
+    int32_t let_next;                   // the next launch may start as this one does (set at launch)
     int32_t c_dtype;
 };
 
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(NT) contract_f32_kernel(const __grid_constant_
     wa.init(p.A, batch_at(p.A, bx), tid, m0, c0 * TK);
     wb.init(p.B, batch_at(p.B, bx), tid, n0, c0 * TK);
     ja_wait_for_stream();
-    ja_let_next_start();
+    if (p.let_next) ja_let_next_start();
     uint64_t acc2[U][U / 2];                    // pairs of neighbouring columns
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -318,14 +320,18 @@ __global__ void __launch_bounds__(NT) contract_f32_kernel(const __grid_constant_
 }
 
 template <int T, bool KCA, int WA, bool KCB, int WB, bool EQ>
-ja_status_t launch(const Params& p, cudaStream_t st) {
-    static bool configured[64] = {};
+ja_status_t launch(Params p, cudaStream_t st) {
+    static std::atomic<int> places_of[64], sms_of[64];   // CTAs that an SM holds; SMs
     int dev = 0;
     cudaGetDevice(&dev);
-    if (!configured[dev & 63]) {
+    int places = places_of[dev & 63].load();
+    if (!places) {
         JA_CUDA(cudaFuncSetAttribute(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<T>::SMEM));
-        configured[dev & 63] = true;
+        JA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&places, contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, NT, Cfg<T>::SMEM));
+        sms_of[dev & 63].store(ja_sm_count());
+        places_of[dev & 63].store(places = std::max(places, 1));
     }
+    p.let_next = ja_let_next_pays((int64_t)p.tiles_m * p.tiles_n * p.split * p.batch[0] * p.batch[1], sms_of[dev & 63].load(), places);
     JA_CUDA(ja_launch_kernel(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, dim3((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]), NT,
                              Cfg<T>::SMEM, (unsigned)p.split, st, p));
     return JA_OK;

@@ -119,3 +119,25 @@ def test_an_index_of_more_than_2_to_30_cells():
     for lo, hi, at in ((0, 1 << 30, 0), (1 << 30, n, 2 << 30)):       # the two blocks: [2, 2^30] cells, then [2, 64]
         w = hi - lo
         assert torch.equal(out.payload[lo:hi], x.payload[at: at + w].float() + x.payload[at + w: at + 2 * w].float())
+
+
+# a queue of products, each of the one before it: launches that let the next one in at their start, and ones that do not (32 x 32 tiles:
+# 296 to 444 at four CTAs an SM, 222 to 296 at three)
+@pytest.mark.parametrize("b,cut", [(60, 1), (74, 1), (80, 1), (111, 1), (112, 1), (55, 2), (60, 2), (75, 2)])
+def test_queue_of_products(b, cut):
+    n = 61
+    sb, sn = ES(b, 1), ES(n, cut)
+    x = si.normal((b, n, n), 0.0, 1.0, F32, 33, 50)
+    w = (si.normal((b, n, n), 0.0, 1.0, F32, 33, 51) * n ** -0.5).contiguous()
+    cur, rw = upload(x, [sb, sn, sn]), upload(w, [sb, sn, sn])
+    spec = ja.Spec("bij,bjk->bik", {"b": sb, "i": sn, "j": sn, "k": sn})
+    steps = [cur] + [empty_like_tiling([b, n, n], [sb, sn, sn], F32, fill=float("nan")) for _ in range(6)]
+    for _ in range(2):
+        for s, d in zip(steps, steps[1:]):
+            spec.execute([s, rw], d)
+    want = si.to_f64(x)
+    for _ in range(6):
+        want = want @ si.to_f64(w)
+    got = download(steps[-1])
+    check_status()
+    assert relfro(got, want) <= 6 * TOL[F32]
