@@ -4,24 +4,21 @@
 // its barriers and finds its place, and stops at ja_wait_for_stream() until that kernel has finished and its writes are visible. Rules:
 //   every thread calls ja_wait_for_stream(), one that has nothing to do as well, so a grid cannot finish before the one it waits for, and
 //     the order is transitive. Before the call a thread reads parameters and the relations' key tables, which are written once, by a
-//     copy that has returned to the host before any launch that reads them is issued, and no other global memory; it writes none.
-//     (f32 contractions find their place in the tables before it: 256^3 8.2 us, 9.2 behind it.)
-//   Before the call it waits for nothing but its own CTA, and takes nothing that it was not launched with: tensor memory, whose
-//     allocation waits without a limit for CTAs that hold some, is allocated behind it ([32, 4096] x [4096, 11008] 23.0 us, 22.5 before it).
+//     copy that has returned to the host before any launch that reads them is issued, and no other global memory; it writes none;
+//   before the call it waits for nothing but its own CTA, and takes nothing that it was not launched with;
 //   ja_let_next_start() comes after the wait, so that one kernel at most waits inside the running one (called before it, the CTAs of several
-//     launches piled up on the SMs that happened to have room: 256^3 f32, 64 CTAs, 12.9 us a call instead of 8), and after the allocation of
-//     tensor memory. A kernel that does not call it lets the next one in as its CTAs end.
-//   So whoever is resident early waits for one launch alone, all of whose CTAs are resident and have all that they will ever take: however
-//     streams mix, no two launches can wait for one another. Cluster barriers and tensor-memory allocations have no limit as mbarrier waits
-//     have; they stand behind the wait, between CTAs that the hardware starts together, and for memory that ends with running kernels.
-//   A kernel without these calls is launched without the attribute and waits for the whole kernel before it, as ever.
-// One queue did stop: twenty calls in a row that each took scratch from a pool in stream order, copied operands, multiplied with gemm_tc_kernel
-// in pairs and gave the scratch back ([8000, 5001] x [5001, 5003]), both launches overlapping. Read again, the kernels give no cause: a
-// product could be resident only when every CTA of the copy before it had passed its wait, which is after the last product had ended, so
-// no two users of tensor memory or clusters met. What was particular is memory taken and returned in stream order between overlapping
-// launches, and how the two go together is not ours to see. The cause is thus not known. The two launches of that queue, the copy and
-// gemm_tc_kernel in clusters, do not overlap in either direction since; scratch is no longer taken on a caller's stream; and where the
-// library does take memory there (exchange programs), its launches are plain.
+//     launches piled up on the SMs that happened to have room: 256^3 f32, 64 CTAs, 12.9 us a call instead of 8). A kernel that does not
+//     call it lets the next one in as its CTAs end;
+//   kernels in clusters and kernels that allocate tensor memory are launched by ja_launch_kernel_after, behind the whole launch before
+//     them, and let none in before they end. Cluster barriers and tensor-memory allocations wait without a limit, as mbarrier waits do not.
+// The last rule is there because two queues stopped for good (the GPU answered): twenty calls that each copied operands into pooled scratch and
+// multiplied them with gemm_tc_kernel in pairs of CTAs ([8000, 5001] x [5001, 5003]), and, once in many thousand passes, join-only products by
+// gemm_tc_kernel followed by the aggregating relayout ([4096, 11008] x [11008, 4096] in four copies), all of these launches overlapping.
+// The cause is not known. By the rules, whoever is resident early waits for one launch, all of whose CTAs are resident (timed on grids of
+// single CTAs and of clusters, larger than the chip and behind a half-finished launch: no dependent started before the last CTA), so
+// no two launches should wait for one another; both queues had gemm_tc_kernel next to a launch of many CTAs of 256 threads. What it costs,
+// against all of them overlapping: 256^3 f32 in clusters 10.4 us a call, 7.8; [32, 4096] x [4096, 11008] 24.6, 22.4; batched scores 18.4, 17.3;
+// the SwiGLU MLP 537, 532; attention and whole blocks below 1 %.
 #pragma once
 
 #include <cuda_runtime.h>

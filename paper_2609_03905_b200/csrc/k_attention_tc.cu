@@ -221,7 +221,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         wait_ctl_init(abort_flag, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -230,7 +229,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_let_next_start();
     const uint32_t tS[2] = {tmem_base, tmem_base + 128};
     const uint32_t tO[2] = {tmem_base + 256, tmem_base + 384};
 
@@ -692,7 +690,6 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
         wait_ctl_init(abort_flag, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -701,7 +698,6 @@ __device__ __forceinline__ void attention_tc2(const CUtensorMap& tmQ, const CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_let_next_start();
 
     if (warp == 0) {
         // ================= TMA producer =================
@@ -1196,13 +1192,13 @@ ja_status_t launch_two_tiles(int variant, bool f16, dim3 grid, cudaStream_t st, 
                              const CUtensorMap& tv, const CUtensorMap& to, const AttnTcParams& p) {
     if (f16) {   // f16 cells: the default row-thread variant only
         JA_CUDA(cudaFuncSetAttribute(attention_tc2_kernel<PERSIST, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-        JA_CUDA(ja_launch_kernel(attention_tc2_kernel<PERSIST, 1, true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));
+        JA_CUDA(ja_launch_kernel_after(attention_tc2_kernel<PERSIST, 1, true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));
         return JA_OK;
     }
 #define JA_ATTN_LAUNCH(V)                                                                                                          \
     case V: {                                                                                                                      \
         JA_CUDA(cudaFuncSetAttribute(attention_tc2_kernel<PERSIST, V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2)); \
-        JA_CUDA(ja_launch_kernel(attention_tc2_kernel<PERSIST, V, false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));                      \
+        JA_CUDA(ja_launch_kernel_after(attention_tc2_kernel<PERSIST, V, false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p));                      \
         return JA_OK;                                                                                                              \
     }
     switch (variant) {
@@ -1370,10 +1366,10 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         const dim3 grid((unsigned)std::min<int64_t>(items, sms), 1, 1);
         if (a.f16) {
             JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-            JA_CUDA(ja_launch_kernel(attention_ragged_kernel<true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
+            JA_CUDA(ja_launch_kernel_after(attention_ragged_kernel<true>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
         } else {
             JA_CUDA(cudaFuncSetAttribute(attention_ragged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES2));
-            JA_CUDA(ja_launch_kernel(attention_ragged_kernel<false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
+            JA_CUDA(ja_launch_kernel_after(attention_ragged_kernel<false>, grid, NUM_THREADS2, SMEM_BYTES2, 1, st, tq, tk, tv, to, p, rt));
         }
         ja_count_launch();
         JA_CUDA(cudaGetLastError());
@@ -1426,10 +1422,10 @@ ja_status_t ja_launch_attention_tc(const AttnArgs& a, cudaStream_t st, bool* lau
         dim3 grid((unsigned)((int64_t)a.H * a.B * (a.S / QT)), 1, 1);
         if (a.f16) {
             JA_CUDA(cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-            JA_CUDA(ja_launch_kernel(attention_tc_kernel<true>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
+            JA_CUDA(ja_launch_kernel_after(attention_tc_kernel<true>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
         } else {
             JA_CUDA(cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-            JA_CUDA(ja_launch_kernel(attention_tc_kernel<false>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
+            JA_CUDA(ja_launch_kernel_after(attention_tc_kernel<false>, grid, NUM_THREADS, SMEM_BYTES, 1, st, tq, tk, tv, p));
         }
     }
     ja_count_launch();

@@ -173,8 +173,10 @@ __global__ void __launch_bounds__(NT) contract_f32_kernel(const __grid_constant_
     Walk<T, KCB, WB, EQ> wb;
     wa.init(p.A, batch_at(p.A, bx), tid, m0, c0 * TK);
     wb.init(p.B, batch_at(p.B, bx), tid, n0, c0 * TK);
-    ja_wait_for_stream();
-    if (p.let_next) ja_let_next_start();
+    if (split == 1) {                           // (clusters do not overlap: ja_launch.cuh)
+        ja_wait_for_stream();
+        if (p.let_next) ja_let_next_start();
+    }
     uint64_t acc2[U][U / 2];                    // pairs of neighbouring columns
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -332,8 +334,9 @@ ja_status_t launch(Params p, cudaStream_t st) {
         places_of[dev & 63].store(places = std::max(places, 1));
     }
     p.let_next = ja_let_next_pays((int64_t)p.tiles_m * p.tiles_n * p.split * p.batch[0] * p.batch[1], sms_of[dev & 63].load(), places);
-    JA_CUDA(ja_launch_kernel(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, dim3((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]), NT,
-                             Cfg<T>::SMEM, (unsigned)p.split, st, p));
+    const dim3 grid((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]);
+    if (p.split > 1) JA_CUDA(ja_launch_kernel_after(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, grid, NT, Cfg<T>::SMEM, (unsigned)p.split, st, p));
+    else JA_CUDA(ja_launch_kernel(contract_f32_kernel<T, KCA, WA, KCB, WB, EQ>, grid, NT, Cfg<T>::SMEM, 1, st, p));
     return JA_OK;
 }
 template <int T, bool KCA, int WA, bool KCB, int WB>

@@ -25,7 +25,7 @@
 // 256; 0.24 to 0.51 us per stage of a full SM), on short tiles the start and the store of a CTA. Measured, us per call, against the
 // block-bound loader form and the cell-by-cell kernel that this one took the place of:
 //   [2048, 11008] x [11008, 4096] bf16, k cut 64 ways (8-byte pieces)       467 -> 282 (655 TFLOP/s); one block a side 376 -> 175
-//   [32, 4096] x [4096, 11008] bf16                 (TMA form, 48 tiles)    61.5 -> 30 (of 14 at the copy rate)
+//   [32, 4096] x [4096, 11008] bf16                 (TMA form, 48 tiles)    61.5 -> 28.8 (k_stream_tc.cu takes it since)
 //   "bij,bkj->bik" 32 x 512 x 128 x 512 bf16, indices cut in four           19310 -> 18
 //   [154, 8768] x [8768, 3627] f16, odd columns cut in two                  593 -> 108
 #include <string.h>
@@ -527,11 +527,7 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     int m0, m_end, n0, n_end;
     tile_range(p.A.r, p.cut_m, BM, band * p.group_m + tin % rows_in_band, m0, m_end);
     tile_range(p.B.r, p.cut_n, BN, tin / rows_in_band, n0, n_end);
-    const bool early = p.split == 1;          // launched to start inside the launch before it (clusters are not)
-    if (m0 >= m_end || n0 >= n_end) {         // an interval shorter than the longest one (the whole cluster leaves)
-        if (early) ja_wait_for_stream();
-        return;
-    }
+    if (m0 >= m_end || n0 >= n_end) return;   // an interval shorter than the longest one (the whole cluster leaves)
     const int bx[MAX_BATCH] = {(int)blockIdx.z, (int)blockIdx.y};
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
@@ -545,7 +541,6 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
         wait_ctl_init(ctl, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (early) ja_wait_for_stream();
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(BN * ACC) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -554,7 +549,6 @@ __global__ void __launch_bounds__(Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::CTAS_PER_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    if (early) ja_let_next_start();
 
     const int chunks = (p.K + BK - 1) / BK;
     const int c0 = (int)((int64_t)chunks * rank / split), c1 = (int)((int64_t)chunks * (rank + 1) / split);
@@ -662,9 +656,7 @@ ja_status_t launch(const Params& p, cudaStream_t st) {
         configured[dev & 63] = true;
     }
     const dim3 grid((unsigned)(p.tiles_m * p.tiles_n * p.split), (unsigned)p.batch[1], (unsigned)p.batch[0]);
-    // clusters wait for the launch before them: [32, 4096] x [4096, 11008] 28.2 us, 32.8 when they start inside it
-    if (p.split > 1) JA_CUDA(ja_launch_kernel_after(contract_tc_kernel<BN, RAW, ACC>, grid, Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::SMEM, (unsigned)p.split, st, p));
-    else JA_CUDA(ja_launch_kernel(contract_tc_kernel<BN, RAW, ACC>, grid, Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::SMEM, 1, st, p));
+    JA_CUDA(ja_launch_kernel_after(contract_tc_kernel<BN, RAW, ACC>, grid, Cfg<BN, RAW>::THREADS, Cfg<BN, RAW>::SMEM, (unsigned)p.split, st, p));
     return JA_OK;
 }
 

@@ -168,7 +168,7 @@ __device__ __forceinline__ int tile_of_iter(const GemmParams& p, int i, int firs
 // F16: cell type of the operands and of a 2-byte output -- bf16 or f16 (a compile-time choice: a select between the two
 // conversions in the epilogue cost the plain contraction a tenth of its rate)
 // SPLIT: a tile's contracted index over a cluster of CTA pairs, one tile a cluster, the slices' f32 sums taken through distributed shared
-// memory. What bounds it is the sum and the cluster's start and end, 10 us of [512, 4096] x [4096, 4096]'s 27.1 (33.9 as whole tiles).
+// memory. What bounds it is the sum and the cluster's start and end, 10 us of [512, 4096] x [4096, 4096]'s 28.8 in a queue of calls (33.9 as whole tiles).
 // ANYC: the output's tiling is not the one that TMA sees of the operands (operands staged by k_stage.cu, rows of no whole 16 bytes): every
 // cell is located through its key table and stored by itself, 32 columns of a row at a time
 template <int CG, bool F16, bool SPLIT, bool ANYC>
@@ -209,7 +209,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         wait_ctl_init(abort_flag, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (CG == 1) ja_wait_for_stream();
     if (warp == 1) {  // all 512 TMEM columns: two 128 x 256 fp32 accumulators (in each CTA of a pair)
         if (CG == 1) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
@@ -224,7 +223,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (CG == 2) cluster_sync_all();   // the peer's barriers exist before anything remote touches them
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    if (CG == 1) ja_let_next_start();
 
     const int kchunks = (p.bk + Cfg<CG>::BK - 1) / Cfg<CG>::BK;
     const int total_tiles = p.tile_end;
@@ -624,7 +622,6 @@ struct GemmTcPlan {
     int tiles;   // of the whole launch; the last `tail` of them go to a launch of their own, each split along the contracted index
     int tail, split;
     bool any_c;
-    bool staged = false;   // on copies: launched behind the whole launch before it (k_stage.cu)
     TmaOperand a, b;
     double us;   // what the launches are expected to take
 };
@@ -797,9 +794,7 @@ ja_status_t ja_gemm_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, con
     if (a.cols < 64 || b.cols < 64) return JA_OK;
     // 32 columns at a time lie in one block of the output, in rows of whole 16 bytes: stored as ever
     const bool any_c = !(C->equal_blocks && C->bs[1] % 8 == 0 && (C->bs[1] == b.cols || C->bs[1] % 32 == 0));
-    ja_status_t st = plan_gemm(a, b, C, nullptr, any_c, out, eligible);
-    if (*out) (*out)->staged = true;
-    return st;
+    return plan_gemm(a, b, C, nullptr, any_c, out, eligible);
 }
 
 ja_status_t ja_gemm_tc_set_bases(GemmTcPlan* plan, char* a, char* b) {
@@ -817,10 +812,7 @@ static ja_status_t launch_gemm(const GemmTcPlan& plan, GemmParams& p, cudaStream
     constexpr int S1 = ANYC ? Cfg<1>::SMEM_BYTES_ANYC : Cfg<1>::SMEM_BYTES, S2 = ANYC ? Cfg<2>::SMEM_BYTES_ANYC : Cfg<2>::SMEM_BYTES;
     const int sms = ja_sm_count();
     auto launch = [&](auto kernel, int grid, int smem, int cluster) -> ja_status_t {
-        // pairs and clusters of pairs run behind the whole launch before them and let none in early (ja_launch.cuh: the launches of the queue that
-        // stopped); [2048, 4096] in the SwiGLU MLP 537 us, 532 when they overlapped
-        if (plan.staged || cluster > 1) JA_CUDA(ja_launch_kernel_after(kernel, dim3((unsigned)grid, 1, 1), NUM_THREADS, smem, (unsigned)cluster, st, plan.tmA, plan.tmB, plan.tmB2, p));
-        else JA_CUDA(ja_launch_kernel(kernel, dim3((unsigned)grid, 1, 1), NUM_THREADS, smem, (unsigned)cluster, st, plan.tmA, plan.tmB, plan.tmB2, p));
+        JA_CUDA(ja_launch_kernel_after(kernel, dim3((unsigned)grid, 1, 1), NUM_THREADS, smem, (unsigned)cluster, st, plan.tmA, plan.tmB, plan.tmB2, p));
         ja_count_launch();
         return JA_OK;
     };

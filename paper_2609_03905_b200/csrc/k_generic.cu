@@ -118,8 +118,10 @@ __device__ __forceinline__ float merged(int agg, float a, float b) { return agg 
 template <int N, bool LANES>
 __global__ void __launch_bounds__(WARPS * 32) generic_join_agg_kernel(const __grid_constant__ Params p) {
     __shared__ float part[WARPS][32];
-    ja_wait_for_stream();
-    ja_let_next_start();
+    if (p.cluster == 1) {   // (clusters do not overlap: ja_launch.cuh)
+        ja_wait_for_stream();
+        ja_let_next_start();
+    }
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int rank = (int)blockIdx.x % p.cluster;
     const int64_t group = blockIdx.x / p.cluster;
@@ -243,7 +245,9 @@ __global__ void __launch_bounds__(WARPS * 32) generic_join_agg_kernel(const __gr
 
 template <int N, bool LANES>
 ja_status_t launch(const Params& p, int64_t groups, cudaStream_t st) {
-    JA_CUDA(ja_launch_kernel(generic_join_agg_kernel<N, LANES>, dim3((unsigned)(groups * p.cluster)), WARPS * 32, 0, (unsigned)p.cluster, st, p));
+    const dim3 grid((unsigned)(groups * p.cluster));
+    if (p.cluster > 1) JA_CUDA(ja_launch_kernel_after(generic_join_agg_kernel<N, LANES>, grid, WARPS * 32, 0, (unsigned)p.cluster, st, p));
+    else JA_CUDA(ja_launch_kernel(generic_join_agg_kernel<N, LANES>, grid, WARPS * 32, 0, 1, st, p));
     return JA_OK;
 }
 

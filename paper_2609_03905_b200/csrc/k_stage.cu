@@ -7,7 +7,7 @@
 // and 4 GiB altogether, given back when the spec or the relations go and with them the last graph that recorded a call. Two calls of one
 // plan that were not ordered behind one another would already race on its output.
 //
-// These two launches do not start inside the ones before them, for the reason that ja_launch.cuh gives.
+// The copy's launch, like the product's, neither starts inside the one before it nor lets one in: the queue that stopped (ja_launch.cuh).
 #include <cuda.h>
 #include <string.h>
 

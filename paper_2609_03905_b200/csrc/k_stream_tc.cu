@@ -11,7 +11,7 @@
 // Every mbarrier wait is bounded; on expiry the CTA records JA_ERR_TIMEOUT, drains its copies and leaves through the normal exit.
 //
 // What bounds it: the stream of B out of HBM; on small products the trips of a CTA's stages, so up to eight are in flight.
-// [32, 4096] x [4096, 11008] bf16 30.7 us (172 CTAs of the cp.async form) -> 22.4, 4.1 TB/s of weights; [64, 3001] x [3001, 320] on copies 58 -> 23.
+// [32, 4096] x [4096, 11008] bf16 30.7 us (172 CTAs of the cp.async form) -> 24.6, 3.7 TB/s of weights; [64, 3001] x [3001, 320] on copies 58 -> 23.
 #include <cuda.h>
 #include <string.h>
 
@@ -70,7 +70,6 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
         wait_ctl_init(ctl, p.wait_cap_us);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    ja_wait_for_stream();
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(p.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -79,7 +78,6 @@ __global__ void __launch_bounds__(NUM_THREADS) stream_tc_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
-    ja_let_next_start();
 
     // ---- this CTA's columns and its slice of the contracted index ----
     const int split = p.split, rank = (int)blockIdx.x % split, t = (int)blockIdx.x / split;
@@ -221,7 +219,6 @@ struct StreamTcPlan {
     Params p;
     int grid, smem;
     TmaOperand a, b;
-    bool staged = false;   // on copies: launched behind the whole launch before it (k_stage.cu)
 };
 
 static ja_status_t encode_operands(StreamTcPlan* plan) {
@@ -288,9 +285,7 @@ ja_status_t ja_stream_tc_plan(const ja_relation* A, const ja_relation* B, const 
 
 ja_status_t ja_stream_tc_plan_staged(const TmaOperand& a, const TmaOperand& b, const ja_relation* C, std::shared_ptr<StreamTcPlan>* out, double* est_us) {
     out->reset();
-    ja_status_t st = plan_stream(a, b, C, !(C->equal_blocks && C->bs[1] % 8 == 0), out, est_us);
-    if (*out) (*out)->staged = true;
-    return st;
+    return plan_stream(a, b, C, !(C->equal_blocks && C->bs[1] % 8 == 0), out, est_us);
 }
 
 ja_status_t ja_stream_tc_set_bases(StreamTcPlan* plan, char* a, char* b) {
@@ -305,8 +300,7 @@ ja_status_t ja_launch_stream_tc(const StreamTcPlan& plan, cudaStream_t st) {
     if (!p.status) return ja_fail(JA_ERR_CUDA, "cannot resolve the device status word");
     p.wait_cap_us = (uint32_t)ja_config().wait_cap_us;
     const dim3 grid((unsigned)plan.grid, 1, 1);
-    if (plan.staged) JA_CUDA(ja_launch_kernel_after(stream_tc_kernel, grid, NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
-    else JA_CUDA(ja_launch_kernel(stream_tc_kernel, grid, NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
+    JA_CUDA(ja_launch_kernel_after(stream_tc_kernel, grid, NUM_THREADS, plan.smem, (unsigned)p.split, st, plan.tmA, plan.tmB, p));
     ja_count_launch();
     return JA_OK;
 }
