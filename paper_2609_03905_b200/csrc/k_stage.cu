@@ -26,8 +26,9 @@ namespace {
 // A thread writes one 16-byte word of `rows_per_cta` / 8 rows. The word's cells lie in one interval of the column index (two aligned words of
 // the row, shifted together), in two around a split point (two such pairs, merged), or, where intervals are shorter than a word, in
 // more (cell by cell). Words that hold no wanted cell are not read; a payload is 128-byte aligned and padded, so a word that holds one
-// never leaves it. Bound by memory: neighbouring threads read neighbouring words, several rows in flight per thread. CUT: there are
-// split points (and twice the registers a row, so half the rows).
+// never leaves it. Neighbouring threads read neighbouring words, several rows in flight per thread. CUT: there are split points (and
+// twice the registers a row, so half the rows). What bounds that form is its instructions and their latency, two loads, a shift and a
+// merge a word: 45 MB in 172-cell blocks 27 us, DRAM 23 % busy, issue slots 41 %.
 constexpr int WORDS = 32, THREADS = 256, STEP = THREADS / WORDS;
 // one operand's copy; both operands' are one launch
 struct Copy {
