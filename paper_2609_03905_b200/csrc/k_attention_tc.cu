@@ -532,7 +532,8 @@ __device__ __forceinline__ float row_exp_pack128(const uint32_t (&v)[128], float
 //   running counters (items; key steps per tile). Otherwise one CTA per item, handed out by the hardware in grid order.
 //   What lies between two items of a row warp was 6400 cycles (a key step is 3400): the TMA stores of the output are now waited for
 //   where their tile is written again, the producer hands out items worked out, and a CTA's first item is its own number.
-//   B4 S2048 171.0 -> 169.5 us, five packed sequences 111.8 -> 110.0 (a loop of calls, at the power limit's clock).
+//   B4 S2048 171.0 -> 169.5 us, five packed sequences 111.8 -> 110.0 (a loop of calls on one box, at the power limit's clock; boxes differ by
+//   as much).
 //   Traces of the row warps at that point: per key step 220 cycles to the scores, 240 for the load, 500 for the maximum, 280 for the P
 //   tile, 1530 for the exponentials and the store of P. Tiles taking turns at the exponentials (+3 %: by itself a warp's take as long),
 //   and P in tensor memory with one S tile that passes between the two (+4 %, packed +11 %: each waits for the other's load) were built,
